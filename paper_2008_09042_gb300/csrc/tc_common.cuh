@@ -87,28 +87,77 @@ static __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap*
       : "memory");
 }
 
-// The MMA issue asm carries no memory clobber: the barrier waits, fences and
-// commits around it (all volatile asm with memory clobbers) order it, and a
-// clobber here would make the compiler reload state between back-to-back MMAs.
+// MMAs and commits are issued by a whole warp: every lane runs the issue loop
+// and elect.sync picks the issuing one inside the asm.  All operands are then
+// warp-uniform values, which the compiler keeps in uniform registers; issued
+// from one thread of a divergent branch, each MMA costs 53-60 SM cycles for
+// moving its descriptors there, whatever its N (measured: a stage of eight
+// N = 64 and eight N = 32 kind::tf32 MMAs takes 53 cycles per MMA that way and 39
+// this way; the tensor core itself needs 32).  The callers must be converged
+// (a wait is followed by a vote, see mbar_wait_warp).
+// The asm carries no memory clobber: the barrier waits, fences and commits
+// around it (all volatile asm with memory clobbers) order it, and a clobber here
+// would make the compiler reload state between back-to-back MMAs.
 static __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
 // As mma_bf16 with the accumulate flag fixed to 1.
 static __device__ __forceinline__ void mma_bf16_acc(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
-  asm volatile("tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 1;" ::"r"(tmem_d), "l"(adesc), "l"(bdesc),
-               "r"(idesc));
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 1;\n\t}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc));
+}
+
+static __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+// As mma_tf32 with the accumulate flag fixed to 1.
+static __device__ __forceinline__ void mma_tf32_acc(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;\n\t}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc));
+}
+
+// D += A B^T with A (128 x 8, TF32) read from tensor memory.
+static __device__ __forceinline__ void mma_tf32_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc,
+                                                       uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, 1;\n\t}" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(idesc));
 }
 
 static __device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   mpi_ptx::smem_addr(bar))
-               : "memory");
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          mpi_ptx::smem_addr(bar))
+      : "memory");
+}
+
+// A bounded wait by a whole warp: the lanes agree on the outcome and leave converged.
+static __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, long long limit) {
+  return __all_sync(0xffffffffu, mpi_ptx::mbar_wait(bar, parity, err, limit));
 }
 
 static __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

@@ -12,7 +12,7 @@
 //
 // CTA = 6 warps: warp 0 streams 128-pixel x 64-element tiles of U with TMA
 // (128-byte swizzle) into a ring of shared-memory stages; warp 1 owns the TMEM
-// accumulator and one thread issues tcgen05.mma (M = 128, N = padded 2C or 4C,
+// accumulator and issues tcgen05.mma (M = 128, N = padded 2C or 4C,
 // K = 16 per instruction); warps 2-5 read the accumulator with tcgen05.ld
 // (warp w owns TMEM lanes 32 (w % 4) ..) and apply the epilogue, one pixel per
 // thread.  The epilogue warps first write the coefficient operand into shared
@@ -65,7 +65,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bfull + 1);
   __shared__ int s_failed;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform: the roles below do not diverge
   // Launched with programmatic stream serialization: set-up and the TMA stream of
   // the (constant) basis start at once; only the epilogue warps, which read
   // the coefficients and per-pixel data and write the outputs, wait for the
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // warp-uniform (the MMA operands)
 
   const int n_tiles = (a.N + kTileM - 1) / kTileM;
   if (warp == 0 && lane == 0) {
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
       for (int g = (it > stages ? it - stages : 0); g < it; ++g)
         mpi_ptx::mbar_wait(&full[g % stages], (uint32_t)((g / stages) & 1), nullptr, a.wait_cycles);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer
     // A descriptor of base + off is desc(base) + (off >> 4): the 14-bit start
     // address field holds every shared-memory address, so the sum never carries.
@@ -130,18 +131,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
     const uint32_t b_chunk = (uint32_t)(a.n_gemm * 128) >> 4;  // descriptor step per K chunk
     RingPos r;
     int tc = 0;
-    bool ok = mpi_ptx::mbar_wait(bfull, 0, a.err, a.wait_cycles);
+    bool ok = mbar_wait_warp(bfull, 0, a.err, a.wait_cycles);
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++tc) {
       const int buf = tc & 1;
       const uint32_t tacc = tmem + (uint32_t)(buf * a.half_cols);
-      if (!mpi_ptx::mbar_wait(&acc_empty[buf], (uint32_t)(((tc >> 1) & 1) ^ 1), a.err, a.wait_cycles)) {
+      if (!mbar_wait_warp(&acc_empty[buf], (uint32_t)(((tc >> 1) & 1) ^ 1), a.err, a.wait_cycles)) {
         ok = false;
         break;
       }
       fence_after();
       for (int kc = 0; kc < a.KC; ++kc) {
         const int s = r.s;
-        if (!mpi_ptx::mbar_wait(&full[s], r.ph, a.err, a.wait_cycles)) {
+        if (!mbar_wait_warp(&full[s], r.ph, a.err, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -160,8 +161,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
     }
     // all MMAs issued by this thread have completed once `drain` fires
     mma_commit(drain);
-    mpi_ptx::mbar_wait(drain, 0, a.err, a.wait_cycles);
-    if (!ok) s_failed = 1;
+    mbar_wait_warp(drain, 0, a.err, a.wait_cycles);
+    if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2) {
     mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
     build_coef_smem<false>(a, sB, Kp, MODE == EX_JFWD, tid - 64, bfull);

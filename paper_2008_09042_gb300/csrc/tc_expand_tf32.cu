@@ -50,20 +50,6 @@ constexpr int kStageBytes32 = kBoxesPerStage * kBoxBytes32;
 constexpr int kThreads32 = 320;   // warp 0 TMA, 1 MMA, 2-5 epilogue, 6-9 converters
 constexpr size_t kSmemMax = 232448 - 128;  // 227 KB less room for the static shared word
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void mma_tf32_acc(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
-  asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;" ::"r"(tmem_d), "l"(adesc), "l"(bdesc),
-               "r"(idesc));
-}
-
 // 32 consecutive 32-bit TMEM columns of this warp's 32 lanes, one row per thread.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
   asm volatile(
@@ -76,15 +62,9 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) 
       : "memory");
 }
 
-// D += A B^T with A (128 x 8, TF32) read from tensor memory.
-__device__ __forceinline__ void mma_tf32_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc) {
-  asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, 1;" ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc),
-               "r"(idesc));
-}
-
 // Roles: warp 0 lane 0 loads U tiles (TMA ring of `stages` 16 KB slots); warps
 // 6-9 write each landed tile's lo part to the stage's TMEM slot (signalled on
-// `conv`); warp 1 lane 0 issues the U_hi MMAs of a chunk once it has landed
+// `conv`); warp 1 issues the U_hi MMAs of a chunk once it has landed
 // and the U_lo MMAs once its lo part is in TMEM, then commits the stage back to
 // the producer (`empty`); warps 2-5 run the fused epilogue from a
 // double-buffered accumulator.  A stage holds two 32-element boxes (64 K
@@ -139,7 +119,8 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bfull + 1);
   __shared__ int s_failed;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform: the roles below do not diverge
   // Launched with programmatic stream serialization: set-up and the TMA stream of
   // the (constant) basis start at once; only the epilogue warps, which read
   // the coefficients and per-pixel data and write the outputs, wait for the
@@ -170,7 +151,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // warp-uniform (the MMA operands)
   const uint32_t tmem_lo = tmem + (uint32_t)(2 * a.half_cols);  // lo(U) slots, 32 columns per stage
   const int n_tiles = (a.N + kTileM - 1) / kTileM;
   // ring stages this CTA processes (its tiles x ceil(KC / 2)), numbered g = 0 .. G-1;
@@ -244,7 +225,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
       kc += kBoxesPerStage;
       if (kc >= a.KC) kc = 0;
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer: per 8-element K step, U_hi x [A_hi; A_lo] and U_lo x A_hi.
     // A descriptor of base + off is desc(base) + (off >> 4): the 14-bit start
     // address field holds every shared-memory address, so the sum never carries.
@@ -255,18 +236,18 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
     const uint32_t b_chunk = (uint32_t)(2 * a.n_gemm * 128) >> 4;  // descriptor step per K chunk
     RingPos r;
     int tc = 0;
-    bool ok = mpi_ptx::mbar_wait(bfull, 0, a.err, a.wait_cycles);
+    bool ok = mbar_wait_warp(bfull, 0, a.err, a.wait_cycles);
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++tc) {
       const int buf = tc & 1;
       const uint32_t tacc = tmem + (uint32_t)(buf * a.half_cols);
-      if (!mpi_ptx::mbar_wait(&acc_empty[buf], (uint32_t)(((tc >> 1) & 1) ^ 1), a.err, a.wait_cycles)) {
+      if (!mbar_wait_warp(&acc_empty[buf], (uint32_t)(((tc >> 1) & 1) ^ 1), a.err, a.wait_cycles)) {
         ok = false;
         break;
       }
       fence_after();
       for (int kc = 0; kc < a.KC; kc += kBoxesPerStage) {
         const int s = r.s;
-        if (!mpi_ptx::mbar_wait(&full[s], r.ph, a.err, a.wait_cycles)) {
+        if (!mbar_wait_warp(&full[s], r.ph, a.err, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -285,7 +266,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
           mma_tf32_acc(tacc, ad + kBoxDesc + 4, bd + b_chunk + 4, idesc_hi);
           mma_tf32_acc(tacc, ad + kBoxDesc + 6, bd + b_chunk + 6, idesc_hi);
         }
-        if (!mpi_ptx::mbar_wait(&conv[s], r.ph, a.err, a.wait_cycles)) {
+        if (!mbar_wait_warp(&conv[s], r.ph, a.err, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -307,8 +288,8 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
       if (ok) mma_commit(&acc_full[buf]);
     }
     mma_commit(drain);
-    mpi_ptx::mbar_wait(drain, 0, a.err, a.wait_cycles);
-    if (!ok) s_failed = 1;
+    mbar_wait_warp(drain, 0, a.err, a.wait_cycles);
+    if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2 && warp <= 5) {
     mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
     build_coef_smem<true>(a, sB, Kp, MODE == EX_JFWD, tid - 64, bfull);
@@ -368,7 +349,7 @@ __global__ void __launch_bounds__(128, 1) k_tf32_reading(float* __restrict__ out
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
-  if (tid == 0) {
+  if (warp == 0) {
     mma_tf32(tmem, sdesc_sw128(mpi_ptx::smem_addr(sA)), sdesc_sw128(mpi_ptx::smem_addr(sB)), idesc_tf32(kTileM, 16), 0);
     mma_commit(done);
   }

@@ -101,17 +101,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) 
       : "memory");
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-__device__ __forceinline__ void mma_tf32_tmem_a(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc) {
-  asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, 1;" ::"r"(d), "r"(a), "l"(b), "r"(idesc));
-}
-
 // Barrier over the `n` epilogue threads (named barrier 1) that also returns
 // whether any of them passed `flag` != 0.
 __device__ __forceinline__ bool epi_bar_any(int flag, int n) {
@@ -194,7 +183,8 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
   __shared__ float2 s_tw[N1];  // w_N1^(j1 k2) at [j1 R + k2]
   __shared__ int s_failed;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform: the roles below do not diverge
   // the operand and the per-coil data are written by the previous kernels
   mpi_ptx::pdl_wait();
   mpi_ptx::pdl_trigger();
@@ -227,7 +217,7 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // warp-uniform (the MMA operands)
   const uint32_t tmem_scr = tmem + (uint32_t)NG;           // adjoint: DFT scratch
   const uint32_t tmem_lo = tmem + 2u * NG;                 // lo(T) slots: 64 columns per stage (FP32)
   // this CTA: position block blockIdx.x, coils blockIdx.y, blockIdx.y + gridDim.y, ...
@@ -284,23 +274,23 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
       if (lane == 0) mpi_ptx::mbar_arrive(&conv[r.s]);
       r.next(stages);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer
     const uint64_t a0 = sdesc_sw128(mpi_ptx::smem_addr(sA));
     const uint64_t b0 = sdesc_sw128(mpi_ptx::smem_addr(sB));
     RingPos r;
-    bool ok = mpi_ptx::mbar_wait(bfull, 0, a.err, a.wait_cycles);
+    bool ok = mbar_wait_warp(bfull, 0, a.err, a.wait_cycles);
     for (int tc = 0; tc < my_tiles && ok; ++tc) {
       const int buf = NACC == 2 ? (tc & 1) : 0;
       const uint32_t par = NACC == 2 ? (uint32_t)((tc >> 1) & 1) : (uint32_t)(tc & 1);
       const uint32_t tacc = tmem + (uint32_t)(buf * NG);
-      if (!mpi_ptx::mbar_wait(&acc_empty[buf], par ^ 1u, a.err, a.wait_cycles)) {
+      if (!mbar_wait_warp(&acc_empty[buf], par ^ 1u, a.err, a.wait_cycles)) {
         ok = false;
         break;
       }
       fence_after();
       const int s = r.s;
-      if (!mpi_ptx::mbar_wait(&full[s], r.ph, a.err, a.wait_cycles)) {
+      if (!mbar_wait_warp(&full[s], r.ph, a.err, a.wait_cycles)) {
         ok = false;
         break;
       }
@@ -319,7 +309,7 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
             mma_tf32(tacc, adk, bdk, idesc, (h | ks) != 0);
             mma_tf32(tacc, adk, bdk + lo_off, idesc, 1);
           }
-        if (!mpi_ptx::mbar_wait(&conv[s], r.ph, a.err, a.wait_cycles)) {
+        if (!mbar_wait_warp(&conv[s], r.ph, a.err, a.wait_cycles)) {
           ok = false;
           break;
         }
@@ -340,8 +330,8 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
       r.next(stages);
     }
     mma_commit(drain);
-    mpi_ptx::mbar_wait(drain, 0, a.err, a.wait_cycles);
-    if (!ok) s_failed = 1;
+    mbar_wait_warp(drain, 0, a.err, a.wait_cycles);
+    if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= kEpi0) {
     // ---------------- epilogue: 2 warps per lane quarter (sub 0, 1)
     const int e = warp - kEpi0;

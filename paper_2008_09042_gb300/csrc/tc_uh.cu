@@ -61,19 +61,6 @@ struct UhArgs {
   long long wait_cycles;
 };
 
-__device__ __forceinline__ void mma_tf32_uh(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-}
-
-// D += A B^T with A (128 x 8 TF32) in tensor memory.
-__device__ __forceinline__ void mma_tf32_uh_tmem(uint32_t d, uint32_t ta, uint64_t bd, uint32_t idesc) {
-  asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, 1;" ::"r"(d), "r"(ta), "l"(bd), "r"(idesc));
-}
-
 __device__ __forceinline__ void tmem_st32_uh(uint32_t taddr, const float (&v)[32]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -111,7 +98,8 @@ __global__ void __launch_bounds__(kUhThreads, 1) k_uh_tc(const __grid_constant__
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   __shared__ int s_failed;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform: the roles below do not diverge
   mpi_ptx::pdl_trigger();
   if (tid == 0) {
     s_failed = 0;
@@ -134,7 +122,7 @@ __global__ void __launch_bounds__(kUhThreads, 1) k_uh_tc(const __grid_constant__
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // warp-uniform (the MMA operands)
   const int mb = (int)blockIdx.y, split = (int)blockIdx.x;
   // this CTA's stages [g0, g1) along the pixels (g1 > g0: the host keeps S <= T)
   const int g0 = (int)((long long)a.T * split / a.S);
@@ -170,7 +158,7 @@ __global__ void __launch_bounds__(kUhThreads, 1) k_uh_tc(const __grid_constant__
       for (int h = (g > stages ? g - stages : 0); h < g; ++h)  // fills still in flight (bounded)
         mpi_ptx::mbar_wait(&full[h % stages], (uint32_t)((h / stages) & 1), nullptr, a.wait_cycles);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer
     const uint32_t idesc_hi = BF ? idesc_bf16(kTileM, 2 * Cp) : idesc_tf32(kTileM, 4 * Cp);
     const uint32_t idesc_lo = idesc_tf32(kTileM, 2 * Cp);
@@ -179,8 +167,8 @@ __global__ void __launch_bounds__(kUhThreads, 1) k_uh_tc(const __grid_constant__
     bool ok = true;
     for (int g = 0; g < G; ++g) {
       const int s = r.s;
-      if (!mpi_ptx::mbar_wait(&full[s], r.ph, a.err, a.wait_cycles) ||
-          !mpi_ptx::mbar_wait(&conv[s], r.ph, a.err, a.wait_cycles)) {
+      if (!mbar_wait_warp(&full[s], r.ph, a.err, a.wait_cycles) ||
+          !mbar_wait_warp(&conv[s], r.ph, a.err, a.wait_cycles)) {
         ok = false;
         break;
       }
@@ -196,8 +184,8 @@ __global__ void __launch_bounds__(kUhThreads, 1) k_uh_tc(const __grid_constant__
           if (BF) {
             mma_bf16(tmem, ad + 2 * ks, bd + 2 * ks, idesc_hi, acc);
           } else {
-            mma_tf32_uh(tmem, ad + 2 * ks, bd + 2 * ks, idesc_hi, acc);
-            mma_tf32_uh_tmem(tmem, tmem + (uint32_t)(a.lo_base + s * 64 + 32 * h + 8 * ks), bd + 2 * ks, idesc_lo);
+            mma_tf32(tmem, ad + 2 * ks, bd + 2 * ks, idesc_hi, acc);
+            mma_tf32_tmem_a(tmem, tmem + (uint32_t)(a.lo_base + s * 64 + 32 * h + 8 * ks), bd + 2 * ks, idesc_lo);
           }
         }
       }
@@ -206,8 +194,8 @@ __global__ void __launch_bounds__(kUhThreads, 1) k_uh_tc(const __grid_constant__
     }
     if (ok) mma_commit(acc_full);
     mma_commit(drain);
-    mpi_ptx::mbar_wait(drain, 0, a.err, a.wait_cycles);
-    if (!ok) s_failed = 1;
+    mbar_wait_warp(drain, 0, a.err, a.wait_cycles);
+    if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2) {
     // ---------------- converters, then the epilogue
     mpi_ptx::pdl_wait();
