@@ -218,53 +218,75 @@ static __device__ __forceinline__ float tf32_hi(float v) { return __uint_as_floa
 // so that the tensor core reads it exactly.  An FP32 lo would be truncated by
 // the tensor core, and the truncation of every lo towards zero biases a long
 // sum of products; rounded, the error (at most 2^-11 of lo, 2^-22 of x) is
-// unbiased.
+// unbiased.  Rounding the sign-magnitude bits (add half a unit of the last kept
+// place, clear the rest) is the value of cvt.rna.tf32 for every finite x and
+// runs at the full integer rate.  For an infinite x, hi(x) is infinite and so
+// is (or becomes NaN) the product it enters, whatever lo is.
 static __device__ __forceinline__ float tf32_lo(float v) {
   const float lo = v - tf32_hi(v);
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(lo));
-  return __uint_as_float(r);
+  return __uint_as_float((__float_as_uint(lo) + 0x1000u) & 0xFFFFE000u);
 }
 
 // The coefficient operand, written straight into shared memory in the swizzled
-// K-major layout by the four epilogue warps (etid = 0..127) while the first
-// tiles of U are still in flight.  Per coil c, row 2c is [Re a_c, -Im a_c] and
-// row 2c+1 is [Im a_c, Re a_c] over K = [0, q) | [q, 2q), so that accumulator
+// K-major layout by `nthr` threads of whole warps (etid = 0 .. nthr - 1) while the
+// first tiles of U are still in flight.  Per coil c, row 2c is [Re a_c, -Im a_c]
+// and row 2c+1 is [Im a_c, Re a_c] over K = [0, q) | [q, 2q), so that accumulator
 // columns 2c, 2c+1 hold Re and Im of s_c; rows [half, half + 2C) hold dalpha
 // for the Jacobian; everything else is zero.  SPLIT (the 3xTF32 kernel): rows
 // [0, n_gemm) hold hi of those values and rows [n_gemm, 2 n_gemm) their lo
 // parts, as FP32; otherwise one block of BF16 rows.  Each step writes whole
 // 16-byte swizzle units (4 FP32 or 8 BF16 consecutive K values of a row pair).
+// Nothing multiplies before this is done, so it is on the critical path of every
+// launch: the tasks of a thread are walked without divisions and their loads are
+// issued a batch at a time (one round trip to L2 per batch).  With four warps, a
+// division per task and its loads in turn, it took 7,700 SM cycles for 16 coils
+// of q = 128 and 14,000 for 32, out of 28,000-36,000 for the whole expansion.
 // Ends with the writes made visible to the tensor core and one arrival per
 // warp on `ready`.
 template <bool SPLIT>
 static __device__ void build_coef_smem(const TcArgs& a, unsigned char* sB, int Kp, bool with_dalpha, int etid,
-                                       uint64_t* ready) {
+                                       int nthr, uint64_t* ready) {
   constexpr int E = SPLIT ? 4 : 8;        // K values per 16-byte unit
   constexpr int esize = SPLIT ? 4 : 2;
+  constexpr int BATCH = SPLIT ? 4 : 2;    // tasks whose loads are in flight together
   const int rows = SPLIT ? 2 * a.n_gemm : a.n_gemm;
   const int units = Kp / E;               // units along K per row
-  const int per_blk = a.C * units;
-  const int n_data = (with_dalpha ? 2 : 1) * per_blk;
-  // zero rows: [2C, half) always, [half + 2C, n_gemm) for the Jacobian, [2C, n_gemm) otherwise
-  const int z0 = with_dalpha ? a.half - 2 * a.C : a.n_gemm - 2 * a.C;
-  const int z1 = with_dalpha ? a.n_gemm - a.half - 2 * a.C : 0;
-  const int n_zero = (z0 + z1) * units;
-  for (int task = etid; task < n_data + n_zero; task += 128) {
-    if (task < n_data) {
-      const int blk = task >= per_blk;
-      const int t2 = task - blk * per_blk;
-      const int c = t2 / units, u = t2 - c * units;
-      const float2* src = (blk ? a.dalpha : a.alpha) + (size_t)c * a.q;
-      const int r0 = (blk ? a.half : 0) + 2 * c, k0 = u * E;
+  const int n_coil = (with_dalpha ? 2 : 1) * a.C;  // coils of alpha, then of dalpha
+  const int dc = nthr / units, du = nthr - dc * units;
+  int c = etid / units, u = etid - c * units;      // this thread's next task (coil, unit)
+  while (c < n_coil) {
+    float2 al[BATCH][E];
+    int tc[BATCH], tu[BATCH];
+#pragma unroll
+    for (int j = 0; j < BATCH; ++j) {
+      tc[j] = c;
+      tu[j] = u;
+      if (c < n_coil) {
+        const float2* src = c < a.C ? a.alpha + (size_t)c * a.q : a.dalpha + (size_t)(c - a.C) * a.q;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int k = u * E + e + a.k_off;
+          al[j][e] = make_float2(0.f, 0.f);
+          if (k < 2 * a.q) al[j][e] = src[k < a.q ? k : k - a.q];
+        }
+      }
+      c += dc;
+      u += du;
+      if (u >= units) {
+        u -= units;
+        ++c;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < BATCH; ++j) {
+      if (tc[j] >= n_coil) break;
+      const int r0 = tc[j] < a.C ? 2 * tc[j] : a.half + 2 * (tc[j] - a.C), k0 = tu[j] * E;
       float re[E], im[E];  // rows r0 and r0 + 1
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const int k = k0 + e + a.k_off;
-        float2 al = make_float2(0.f, 0.f);
-        if (k < 2 * a.q) al = src[k < a.q ? k : k - a.q];
-        re[e] = k < a.q ? al.x : (k < 2 * a.q ? -al.y : 0.f);
-        im[e] = k < a.q ? al.y : (k < 2 * a.q ? al.x : 0.f);
+        const bool first = k0 + e + a.k_off < a.q;  // past 2 q the loaded value is zero
+        re[e] = first ? al[j][e].x : -al[j][e].y;
+        im[e] = first ? al[j][e].y : al[j][e].x;
       }
       if (SPLIT) {
         float4 h0, h1, l0, l1;
@@ -288,14 +310,17 @@ static __device__ void build_coef_smem(const TcArgs& a, unsigned char* sB, int K
         *reinterpret_cast<uint4*>(sB + sw128_offset_e(r0, k0, rows, esize)) = v0;
         *reinterpret_cast<uint4*>(sB + sw128_offset_e(r0 + 1, k0, rows, esize)) = v1;
       }
-    } else {
-      const int t2 = task - n_data;
-      const int zr = t2 / units, u = t2 - zr * units;
-      const int r = zr < z0 ? 2 * a.C + zr : a.half + 2 * a.C + (zr - z0);
-      const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(sB + sw128_offset_e(r, u * E, rows, esize)) = zero;
-      if (SPLIT) *reinterpret_cast<uint4*>(sB + sw128_offset_e(r + a.n_gemm, u * E, rows, esize)) = zero;
     }
+  }
+  // zero rows: [2C, half) always, [half + 2C, n_gemm) for the Jacobian, [2C, n_gemm) otherwise
+  const int z0 = with_dalpha ? a.half - 2 * a.C : a.n_gemm - 2 * a.C;
+  const int z1 = with_dalpha ? a.n_gemm - a.half - 2 * a.C : 0;
+  for (int t = etid; t < (z0 + z1) * units; t += nthr) {
+    const int zr = t / units, zu = t - zr * units;
+    const int r = zr < z0 ? 2 * a.C + zr : a.half + 2 * a.C + (zr - z0);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(sB + sw128_offset_e(r, zu * E, rows, esize)) = zero;
+    if (SPLIT) *reinterpret_cast<uint4*>(sB + sw128_offset_e(r + a.n_gemm, zu * E, rows, esize)) = zero;
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
   __syncwarp();

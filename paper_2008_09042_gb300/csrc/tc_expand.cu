@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
     if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2) {
     mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
-    build_coef_smem<false>(a, sB, Kp, MODE == EX_JFWD, tid - 64, bfull);
+    build_coef_smem<false>(a, sB, Kp, MODE == EX_JFWD, tid - 64, 128, bfull);
     tc_epilogue<MODE>(a, tmem, warp, lane, acc_full, acc_empty, n_tiles, &s_failed);
   }
   fence_before();

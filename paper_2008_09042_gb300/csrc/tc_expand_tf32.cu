@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
       mpi_ptx::mbar_init(&acc_empty[b], 4);
     }
     mpi_ptx::mbar_init(drain, 1);
-    mpi_ptx::mbar_init(bfull, 4);  // one arrival per epilogue warp once the coefficient operand is written
+    mpi_ptx::mbar_init(bfull, 8);  // one arrival per epilogue and converter warp once the coefficient operand is written
     mpi_ptx::fence_mbar_init();
   }
   if (warp == 1) {
@@ -159,6 +159,13 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int G = my_tiles * ((a.KC + kBoxesPerStage - 1) / kBoxesPerStage);
 
+  if (warp >= 2) {
+    // ---------------- epilogue and converter warps first write the coefficient
+    // operand, which every MMA waits for (one inlined copy for both: small
+    // launches are short enough for the code they fetch to count)
+    mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
+    build_coef_smem<true>(a, sB, Kp, MODE == EX_JFWD, tid - 64, 256, bfull);
+  }
   if (warp == 0 && lane == 0) {
     // ---------------- producer: TMA tiles of U
     RingPos r;
@@ -291,8 +298,6 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
     mbar_wait_warp(drain, 0, a.err, a.wait_cycles);
     if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2 && warp <= 5) {
-    mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
-    build_coef_smem<true>(a, sB, Kp, MODE == EX_JFWD, tid - 64, bfull);
     tc_epilogue<MODE, true>(a, tmem, warp, lane, acc_full, acc_empty, n_tiles, &s_failed);
   }
   fence_before();

@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
       mpi_ptx::mbar_init(&acc_empty[b], MODE == kTxFwd ? 4 : kNEpi);
     }
     mpi_ptx::mbar_init(drain, 1);
-    mpi_ptx::mbar_init(bfull, 4);
+    mpi_ptx::mbar_init(bfull, kNEpi);
     mpi_ptx::fence_mbar_init();
   }
   if (warp == 1) {
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kTxThreads, 1) k_tucker_x1(const __grid_consta
     constexpr int NT = kNEpi * 32;
     const int et = e * 32 + lane;  // 0 .. NT - 1
     const int b = (int)blockIdx.x * kTileM + row;
-    if (e < 4) build_coef_smem<TF>(a.coef, sB, kKp, false, et, bfull);
+    build_coef_smem<TF>(a.coef, sB, kKp, false, et, NT, bfull);
     for (int i = et; i < N1; i += NT) s_tw[i] = a.tw[((i / R) * (i % R)) % N1];
     // forward: this block's image values with the centring sign and the scale;
     // adjoint: a zeroed accumulator ([z][position])
