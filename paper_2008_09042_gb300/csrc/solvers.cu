@@ -181,83 +181,10 @@ __global__ void k_fill(float2* __restrict__ x, float2 v, long n) {
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) x[i] = v;
 }
 
-// ---------------------------------------------------------------- TV prox (FGP)
-
+// The grid of a solve's TV prox (tv.cu): nd = 2 (y, x) or 3 (z, y, x).
 struct Grid3 {
-  int nz, ny, nx, nd;  // nd = 2 (y, x) or 3 (z, y, x)
+  int nz, ny, nx, nd;
 };
-
-// axis d of a component: 0 = x, 1 = y, 2 = z (stride 1, nx, nx*ny)
-__device__ __forceinline__ void coords(const Grid3& g, long i, int& x, int& y, int& z) {
-  x = (int)(i % g.nx);
-  long t = i / g.nx;
-  y = (int)(t % g.ny);
-  z = (int)(t / g.ny);
-}
-
-// x = b - lam D^H R, with (D^H R)_i = sum_d (R_d[i - e_d] if i_d >= 1) - (R_d[i] if i_d <= n_d - 2)
-// lam = 1 / S[S_RHO] (rho_slot >= 0) or lam_host.
-__global__ void k_tv_primal(const float2* __restrict__ b, const float2* __restrict__ R, Grid3 g, long N,
-                            const double* __restrict__ S, int use_rho, float lam_host, float2* __restrict__ x) {
-  const float lam = use_rho ? (float)(1.0 / S[S_RHO]) : lam_host;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long)gridDim.x * blockDim.x) {
-    int cx, cy, cz;
-    coords(g, i, cx, cy, cz);
-    float2 dh = make_float2(0.f, 0.f);
-    const int pos[3] = {cx, cy, cz};
-    const int len[3] = {g.nx, g.ny, g.nz};
-    const long stride[3] = {1, g.nx, (long)g.nx * g.ny};
-    for (int d = 0; d < g.nd; ++d) {
-      const float2* Rd = R + (size_t)d * N;
-      if (pos[d] >= 1) {
-        const float2 v = Rd[i - stride[d]];
-        dh.x += v.x;
-        dh.y += v.y;
-      }
-      if (pos[d] <= len[d] - 2) {
-        const float2 v = Rd[i];
-        dh.x -= v.x;
-        dh.y -= v.y;
-      }
-    }
-    const float2 bv = b[i];
-    x[i] = make_float2(bv.x - lam * dh.x, bv.y - lam * dh.y);
-  }
-}
-
-// Pn = proj(R + D x * rho / L); R = Pn + c (Pn - P); P = Pn
-__global__ void k_tv_dual(const float2* __restrict__ x, float2* __restrict__ P, float2* __restrict__ R, Grid3 g,
-                          long N, const double* __restrict__ S, int use_rho, float lam_host, float c) {
-  const float L = 4.0f * g.nd;
-  const float step = use_rho ? (float)(S[S_RHO] / L) : 1.0f / (L * lam_host);
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long)gridDim.x * blockDim.x) {
-    int cx, cy, cz;
-    coords(g, i, cx, cy, cz);
-    const int pos[3] = {cx, cy, cz};
-    const int len[3] = {g.nx, g.ny, g.nz};
-    const long stride[3] = {1, g.nx, (long)g.nx * g.ny};
-    const float2 xi = x[i];
-    float2 pn[3];
-    float mag2 = 0.f;
-    for (int d = 0; d < g.nd; ++d) {
-      float2 gd = make_float2(0.f, 0.f);
-      if (pos[d] <= len[d] - 2) {
-        const float2 xn = x[i + stride[d]];
-        gd = make_float2(xn.x - xi.x, xn.y - xi.y);
-      }
-      const float2 rv = R[(size_t)d * N + i];
-      pn[d] = make_float2(fmaf(step, gd.x, rv.x), fmaf(step, gd.y, rv.y));
-      mag2 += pn[d].x * pn[d].x + pn[d].y * pn[d].y;
-    }
-    const float inv = 1.0f / fmaxf(1.0f, sqrtf(mag2));
-    for (int d = 0; d < g.nd; ++d) {
-      const float2 p_old = P[(size_t)d * N + i];
-      const float2 pv = make_float2(pn[d].x * inv, pn[d].y * inv);
-      P[(size_t)d * N + i] = pv;
-      R[(size_t)d * N + i] = make_float2(pv.x + c * (pv.x - p_old.x), pv.y + c * (pv.y - p_old.y));
-    }
-  }
-}
 
 // ------------------------------------------------------------ ball projection
 
@@ -554,30 +481,6 @@ Grid3 grid_of(const mpi_plan* plan) {
   g.nx = plan->nx;
   g.nd = plan->ndim == 3 ? 3 : 2;
   return g;
-}
-
-// z = prox_{lam TV}(b) by n_iter FGP iterations; P, R are [nd][N] scratch, x the output.
-mpi_status tv_prox_run(Solver& sv, const Grid3& g, long N, const float2* b, int n_iter, int use_rho, float lam,
-                       float2* P, float2* R, float2* x) {
-  mpi_ctx* ctx = sv.ctx;
-  TRY(sv.fill(P, make_float2(0.f, 0.f), (long)g.nd * N));
-  TRY(sv.fill(R, make_float2(0.f, 0.f), (long)g.nd * N));
-  double t = 1.0;
-  for (int it = 0; it < n_iter; ++it) {
-    MPI_PROF(ctx, KF_SOLVER);
-    k_tv_primal<<<grid_for(N), kVecThreads, 0, ctx->stream>>>(b, R, g, N, sv.S, use_rho, lam, x);
-    MPI_LAUNCH_CHECK(ctx, "k_tv_primal");
-    const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-    const float c = (float)((t - 1.0) / tn);
-    MPI_PROF(ctx, KF_SOLVER);
-    k_tv_dual<<<grid_for(N), kVecThreads, 0, ctx->stream>>>(x, P, R, g, N, sv.S, use_rho, lam, c);
-    MPI_LAUNCH_CHECK(ctx, "k_tv_dual");
-    t = tn;
-  }
-  MPI_PROF(ctx, KF_SOLVER);
-  k_tv_primal<<<grid_for(N), kVecThreads, 0, ctx->stream>>>(b, P, g, N, sv.S, use_rho, lam, x);
-  MPI_LAUNCH_CHECK(ctx, "k_tv_primal");
-  return MPI_OK;
 }
 
 }  // namespace
@@ -894,9 +797,8 @@ mpi_status admm_body(mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mp
   const long N1 = plans[0]->N, M = plans[0]->M, CM1 = (long)C * M;
   const long N = (long)T * N1, TC = (long)T * C, CM = TC * M, CMs = std::max(CM, 1L);
   float2 *p = base, *p_prev = p + N, *u0 = p_prev + N, *z0 = u0 + N, *rhs = z0 + N, *t = rhs + N;
-  float2 *r = t + N, *d = r + N, *Ad = d + N, *tvx = Ad + N, *P = tvx + N, *R = P + (size_t)g.nd * N;
-  float2 *uk = R + (size_t)g.nd * N, *zk = uk + CMs, *Apk = zk + CMs, *Apk_prev = Apk + CMs, *wk = Apk_prev + CMs;
-  (void)tvx;
+  float2 *r = t + N, *d = r + N, *Ad = d + N, *tv = Ad + N;
+  float2 *uk = tv + tv_scratch_elems(g.nd, N), *zk = uk + CMs, *Apk = zk + CMs, *Apk_prev = Apk + CMs, *wk = Apk_prev + CMs;
   double* fball = dx;
   double* bpart = fball + TC;
   TRY(sv.fill(p, make_float2(0.f, 0.f), N));
@@ -925,8 +827,7 @@ mpi_status admm_body(mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mp
 
   for (int it = 0; it < prm->n_outer; ++it) {
     // z0 = prox_{TV/rho}(p + u0)
-    TRY(sv.lincomb(t, p, 1.f, u0, 1.f, N));
-    TRY(tv_prox_run(sv, g, N, t, prm->n_tv, 1, 0.f, P, R, z0));
+    TRY(launch_tv_prox(ctx, g.nz, g.ny, g.nx, g.nd, p, u0, nullptr, sv.S + S_RHO, 0.f, prm->n_tv, tv, z0));
     // zk = Pi(F S p + uk)
     if (CM > 0) {
       MPI_PROF(ctx, KF_SOLVER);
@@ -1035,15 +936,16 @@ mpi_status image_solve_impl(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     g->C = C;
     g->prec = prec;
     g->key = key;
-    // image side: 10 N + 2 nd N; k-space: 5 CM; inputs y (CM), alpha (Cq); output p (N)
-    const size_t elems = 10 * N + 2 * (size_t)gr.nd * N + 5 * CMs + CMs + Cq + N;
+    // image side: 9 N and the TV scratch; k-space: 5 CM; inputs y (CM), alpha (Cq); output p (N)
+    const size_t image = 9 * N + tv_scratch_elems(gr.nd, N);
+    const size_t elems = image + 5 * CMs + CMs + Cq + N;
     const size_t extra = 2 * (size_t)TC + (size_t)TC * kRedBlocks + 3 * (size_t)prm->n_outer + TC + 8;
     mpi_status st = alloc_solver(ctx, g->mem, elems, extra, g->sv, &g->base, &g->dbase);
     if (st) {
       delete g;
       return st;
     }
-    float2* io = g->base + 10 * N + 2 * (size_t)gr.nd * N + 5 * CMs;
+    float2* io = g->base + image + 5 * CMs;
     g->in_y = io;
     g->in_alpha = io + CMs;
     g->out_p = g->in_alpha + Cq;
@@ -1132,11 +1034,12 @@ extern "C" mpi_status mpi_tv_prox(mpi_ctx* ctx, const mpi_plan* plan, const mpi_
   Solver sv;
   float2* base;
   double* dx;
-  TRY(alloc_solver(ctx, mem, 2 * (size_t)g.nd * N, 0, sv, &base, &dx));
+  TRY(alloc_solver(ctx, mem, tv_scratch_elems(g.nd, N), 0, sv, &base, &dx));
   if (lam == 0) {
     TRY(sv.lincomb((float2*)x, (const float2*)v, 1.f, nullptr, 0.f, N));
   } else {
-    TRY(tv_prox_run(sv, g, N, (const float2*)v, n_iter, 0, (float)lam, base, base + (size_t)g.nd * N, (float2*)x));
+    TRY(launch_tv_prox(ctx, g.nz, g.ny, g.nx, g.nd, (const float2*)v, nullptr, nullptr, nullptr, (float)lam, n_iter,
+                       base, (float2*)x));
   }
   return cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "tv_prox");
 }
