@@ -1,0 +1,891 @@
+// MPI-L (scaled ADMM, Eqs. 8-11) on 2D Cartesian grids with a dense basis, one
+// slice or several frames that share the maps: the solve's passes fused.
+//
+// The coefficients alpha are fixed for a solve, so its maps s_k = U alpha_k are
+// expanded once, by the same expansion the operator calls run, and every operator
+// of the solve multiplies by them: C N complex values (8.4 MB at 256^2 and 16
+// coils, which stay in L2) instead of the basis (67 MB) per application.  What is
+// left of an operator are FFT passes over C N values, a few microseconds each, so
+// the point-wise steps and the sums live in those passes:
+//   k_maps_cols<fwd>    v = s p (sign, scale) formed on load, DFT along y; in the
+//                       CG the new direction d = r + beta d is formed there too
+//   k_rows_normal       DFT along x, sampling mask, inverse DFT along x (the
+//                       normal operator never leaves k-space rows); not run where
+//                       every row is sampled whole or not at all, since it is
+//                       then a multiplication by nx
+//   k_maps_cols<inv>    inverse DFT along y, times conj(s) on store
+//   k_coil_sum          sum over coils, + d, and the CG's <d, A d>
+//   k_cg_update         x, r, |r|^2
+// and an outer step adds the ball projection inside the scatter of the k-space
+// rows (k_rows_scatter_ball), the dual update of the data blocks and their
+// residual norms inside the gather (k_rows_gather_dual) and the image's dual
+// update with the choice of rho (k_admm_dual).
+//   The CG starts from the previous p, whose F_s S p is at hand (Apk), so its first
+// residual is one adjoint:  r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p.
+//   rho's rescaling of the scaled duals is applied where they are read (ufac).
+//   Reductions: FP64 partial sums per CTA; the last CTA to arrive adds them in a
+// fixed order, so results do not depend on which one that is.
+// At 256^2, 16 coils, q = 128 an outer step (5 CG, 10 TV iterations) went from 725
+// to ~150 us, in 37 launches instead of 124.
+#include <math.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "admm.h"
+#include "dft_reg.cuh"
+#include "fft_tile.cuh"
+#include "ptx.cuh"
+
+namespace {
+
+using namespace mpi_fft;
+
+constexpr int kThreads = 256;      // column and reduction kernels
+constexpr int kElemThreads = 256;  // element-wise kernels
+constexpr int kMaxElemBlocks = 1024;
+constexpr int kBallBlocks = 8;     // CTAs per coil of the ball norms
+
+// device scalars
+enum { S_RR = 0, S_A, S_BETA, S_RHO, S_UFAC, S_NUM };
+
+// ------------------------------------------------------------- reductions
+
+template <int NV>
+__device__ __forceinline__ void block_sums(double (&v)[NV], double* sh) {
+#pragma unroll
+  for (int j = 0; j < NV; ++j)
+    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __syncthreads();
+  if (lane == 0)
+#pragma unroll
+    for (int j = 0; j < NV; ++j) sh[warp * NV + j] = v[j];
+  __syncthreads();
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      double s = 0.0;
+      for (int w = 0; w < nw; ++w) s += sh[w * NV + j];
+      v[j] = s;
+    }
+}
+
+// Sums of v over the `nblk` CTAs that share `partials` and `counter` (zero before,
+// zero after); true in every thread of the last CTA to arrive, where thread 0's v
+// then holds the sums.  `blk`: this CTA's place among them.
+template <int NV>
+__device__ __forceinline__ bool group_sums(double (&v)[NV], double* partials, unsigned* counter, int blk, int nblk,
+                                           double* sh) {
+  __shared__ int last;
+  block_sums(v, sh);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) partials[(size_t)blk * NV + j] = v[j];
+    __threadfence();
+    last = atomicAdd(counter, 1u) == (unsigned)nblk - 1;
+    if (last) *counter = 0;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    v[j] = 0.0;
+    for (int i = threadIdx.x; i < nblk; i += blockDim.x) v[j] += __ldcg(partials + (size_t)i * NV + j);
+  }
+  block_sums(v, sh);
+  return true;
+}
+
+// ------------------------------------------------------------ column passes
+
+struct MapsCols {
+  float2* W;            // [T][C][N]
+  const float2* S;      // maps [C][N]
+  const float2* v;      // forward: image [T][N], or the CG's old direction
+  const float2* r;      // forward, next CG direction d = r + beta d_old (null: v itself)
+  float2* dnew;         // where that direction goes
+  const double* sc;
+  int C, nx;
+  size_t N;
+  float scale;
+  const uint8_t* rmask;  // [T][ny]: 1 where the k-space row has samples
+  const float2* tw;
+};
+
+template <int L>
+struct RegSplit {
+  static constexpr int R1 = 0, R2 = 0;
+};
+template <> struct RegSplit<64> { static constexpr int R1 = 8, R2 = 8; };
+template <> struct RegSplit<96> { static constexpr int R1 = 8, R2 = 12; };
+template <> struct RegSplit<128> { static constexpr int R1 = 8, R2 = 16; };
+template <> struct RegSplit<192> { static constexpr int R1 = 16, R2 = 12; };
+template <> struct RegSplit<256> { static constexpr int R1 = 16, R2 = 16; };
+
+constexpr int maps_cols_tile(int L) { return (L == 64 || L == 96 || L == 128 || L == 192 || L == 256) ? 32 : 8; }
+
+// R values of one thread: rows y0 + step m of column x, formed from the image and
+// the map (forward) or read from the rows with samples (inverse).  All loads are
+// issued before the first use or store: a CTA has 8 warps and there are only
+// T C nx / 32 of them, so what a thread has in flight sets the time (the loads in
+// turn, with the store of the new direction between them: 30 us per pass at
+// 256^2 and 16 coils; batched: see the file header).
+template <int R, bool INV>
+__device__ __forceinline__ void maps_load(const MapsCols& a, int t, int c, int tc, int y0, int step, int x, int L,
+                                          float2 (&u)[R]) {
+  const size_t n0 = (size_t)y0 * a.nx + x, ns = (size_t)step * a.nx;
+  if (INV) {
+    const float2* W = a.W + (size_t)tc * a.N + n0;
+    const uint8_t* rm = a.rmask + (size_t)t * L + y0;
+    uint8_t keep[R];
+#pragma unroll
+    for (int m = 0; m < R; ++m) keep[m] = rm[step * m];
+#pragma unroll
+    for (int m = 0; m < R; ++m) u[m] = keep[m] ? W[ns * m] : make_float2(0.f, 0.f);
+    return;
+  }
+  const float2* S = a.S + (size_t)c * a.N + n0;
+  const float2* v = a.v + (size_t)t * a.N + n0;
+  float2 s[R];
+#pragma unroll
+  for (int m = 0; m < R; ++m) u[m] = v[ns * m];
+#pragma unroll
+  for (int m = 0; m < R; ++m) s[m] = S[ns * m];
+  if (a.r) {  // the CG's next direction, kept by the first coil's CTAs
+    const float2* r = a.r + (size_t)t * a.N + n0;
+    const float beta = (float)a.sc[S_BETA];
+    float2 rv[R];
+#pragma unroll
+    for (int m = 0; m < R; ++m) rv[m] = r[ns * m];
+#pragma unroll
+    for (int m = 0; m < R; ++m) u[m] = make_float2(fmaf(beta, u[m].x, rv[m].x), fmaf(beta, u[m].y, rv[m].y));
+    if (c == 0) {
+      float2* d = a.dnew + (size_t)t * a.N + n0;
+#pragma unroll
+      for (int m = 0; m < R; ++m) d[ns * m] = u[m];
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < R; ++m) {
+    const float2 e = cmul(s[m], u[m]);
+    const float sg = ((x + y0 + step * m) & 1) ? -a.scale : a.scale;
+    u[m] = make_float2(e.x * sg, e.y * sg);
+  }
+}
+
+// The R transformed values of rows y0 + step m: forward, to the rows with samples;
+// inverse, times conj(s) (the maps `s` loaded ahead by the caller).
+template <int R, bool INV>
+__device__ __forceinline__ void maps_store(const MapsCols& a, int t, int tc, int y0, int step, int x, int L,
+                                           const float2 (&u)[R], const float2 (&s)[R]) {
+  float2* W = a.W + (size_t)tc * a.N + (size_t)y0 * a.nx + x;
+  const size_t ns = (size_t)step * a.nx;
+  const uint8_t* rm = a.rmask + (size_t)t * L + y0;
+#pragma unroll
+  for (int m = 0; m < R; ++m) {
+    if (INV)
+      W[ns * m] = make_float2(s[m].x * u[m].x + s[m].y * u[m].y, s[m].x * u[m].y - s[m].y * u[m].x);
+    else if (rm[step * m])
+      W[ns * m] = u[m];
+  }
+}
+
+template <int R>
+__device__ __forceinline__ void maps_prefetch(const MapsCols& a, int c, int y0, int step, int x, float2 (&s)[R]) {
+  const float2* S = a.S + (size_t)c * a.N + (size_t)y0 * a.nx + x;
+  const size_t ns = (size_t)step * a.nx;
+#pragma unroll
+  for (int m = 0; m < R; ++m) s[m] = S[ns * m];
+}
+
+// The pass along y of one (frame, coil) and a tile of adjacent columns, with the
+// products by the maps: the register two-step FFT (see k_fft_cols_reg) for lengths
+// that have a split, else Stockham lines in shared memory.
+template <int L, bool INV>
+__global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
+  constexpr int R1 = RegSplit<L>::R1, R2 = RegSplit<L>::R2;
+  constexpr int TILE = maps_cols_tile(L);
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const int x_tiles = (a.nx + TILE - 1) / TILE;
+  const int tc = (int)blockIdx.x / x_tiles, x0 = ((int)blockIdx.x - tc * x_tiles) * TILE;
+  const int t = tc / a.C, c = tc - t * a.C;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if constexpr (R1 > 0) {
+    __shared__ float2 sY[L * 32];  // [k1][r][column]
+    __shared__ float2 tw[L];
+    for (int i = tid; i < L; i += kThreads) tw[i] = a.tw[i];
+    const int x = x0 + lane;
+    const bool ok = x < a.nx;
+    float2 u1[(R2 + 7) / 8][R1];
+#pragma unroll
+    for (int it = 0; it < (R2 + 7) / 8; ++it) {
+      const int q = w + 8 * it;
+      if (ok && q < R2) maps_load<R1, INV>(a, t, c, tc, q, R2, x, L, u1[it]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < (R2 + 7) / 8; ++it) {
+      const int q = w + 8 * it;
+      if (q >= R2) break;
+      float2 (&u)[R1] = u1[it];
+      if (INV)  // the inverse on conjugated values
+#pragma unroll
+        for (int m = 0; m < R1; ++m) u[m].y = -u[m].y;
+      mpi_dft::dft_r<R1>(u);
+#pragma unroll
+      for (int k1 = 1; k1 < R1; ++k1) u[k1] = mpi_dft::cmulf(u[k1], tw[q * k1]);
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) sY[(k1 * R2 + q) * 32 + lane] = u[k1];
+    }
+    float2 s[(R1 + 7) / 8][R2];
+    if (INV)
+#pragma unroll
+      for (int it = 0; it < (R1 + 7) / 8; ++it)
+        if (ok && w + 8 * it < R1) maps_prefetch<R2>(a, c, w + 8 * it, R1, x, s[it]);
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < (R1 + 7) / 8; ++it) {
+      const int k1 = w + 8 * it;
+      if (k1 >= R1) break;
+      float2 u[R2];
+#pragma unroll
+      for (int q = 0; q < R2; ++q) u[q] = sY[(k1 * R2 + q) * 32 + lane];
+      mpi_dft::dft_r<R2>(u);
+      if (INV)
+#pragma unroll
+        for (int q = 0; q < R2; ++q) u[q].y = -u[q].y;
+      if (ok) maps_store<R2, INV>(a, t, tc, k1, R1, x, L, u, s[it]);
+    }
+  } else {
+    constexpr int ST = col_stride(L, TILE);
+    constexpr int RSTEP = kThreads / TILE;
+    constexpr int PER = (L + RSTEP - 1) / RSTEP;  // rows r0 + RSTEP u of the thread's column
+    constexpr int LAST = L - RSTEP * (PER - 1);   // threads with r0 below this have a last row
+    __shared__ float2 tw[L];
+    __shared__ float2 buf[TILE * ST];
+    for (int i = tid; i < L; i += kThreads) tw[i] = a.tw[i];
+    const int cx = tid % TILE, r0 = tid / TILE, x = x0 + cx;
+    const bool ok = x < a.nx, all = r0 < LAST;
+    float2 v[PER], e[1];
+    if (ok) {
+      if constexpr (PER > 1) {
+        float2 (&v1)[PER - 1] = reinterpret_cast<float2 (&)[PER - 1]>(v);
+        maps_load<PER - 1, INV>(a, t, c, tc, r0, RSTEP, x, L, v1);
+      }
+      if (all) {
+        maps_load<1, INV>(a, t, c, tc, r0 + RSTEP * (PER - 1), RSTEP, x, L, e);
+        v[PER - 1] = e[0];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+      if (r0 + RSTEP * u < L) buf[cx * ST + pad8(r0 + RSTEP * u)] = ok ? v[u] : make_float2(0.f, 0.f);
+    __syncthreads();
+    fft_tile_lines<L, INV, TILE, ST>(buf, tw, w, lane);
+    __syncthreads();
+    if (!ok) return;
+    float2 s[PER];
+    if (INV)
+#pragma unroll
+      for (int u = 0; u < PER; ++u)
+        if (r0 + RSTEP * u < L) s[u] = a.S[(size_t)c * a.N + (size_t)(r0 + RSTEP * u) * a.nx + x];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      if (r0 + RSTEP * u >= L) continue;
+      const float2 o[1] = {buf[cx * ST + pad8(r0 + RSTEP * u)]}, so[1] = {s[u]};
+      maps_store<1, INV>(a, t, tc, r0 + RSTEP * u, RSTEP, x, L, o, so);
+    }
+  }
+}
+
+// --------------------------------------------------------------- row passes
+
+struct MapsRows {
+  float2* W;                 // [T][C][ny][NX]
+  int TC, C, ny, M;
+  const uint8_t* rmask;      // [T][ny]
+  const uint8_t* mask;       // [T][ny][NX]
+  const int32_t* idx;        // [T][M]
+  const int32_t* row_ptr;    // [T][ny + 1]
+  const float2* tw;
+  float ksign;
+  const float2* y;           // data [T][C][M]
+  float2 *ap, *uk, *zk;      // F_s S p, the scaled duals, the projections [T][C][M]
+  const double* f;           // ball factors [T][C]
+  const double* sc;
+  double* partials;
+};
+
+// The normal operator in k-space: F_x, mask, F_x^H of every row with samples.
+template <int NX>
+__global__ void __launch_bounds__(kRowWarps * 32) k_rows_normal(MapsRows a) {
+  __shared__ float2 tw[NX];
+  __shared__ float2 buf[kRowWarps][padded_len(NX)];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = a.tw[i];
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float2* b = buf[warp];
+  const int total = a.TC * a.ny;
+  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
+    const int tc = gr / a.ny, row = gr - tc * a.ny, t = tc / a.C;
+    if (!a.rmask[(size_t)t * a.ny + row]) continue;  // warp-uniform
+    float2* src = a.W + (size_t)gr * NX;
+    const uint8_t* mk = a.mask + ((size_t)t * a.ny + row) * NX;
+    constexpr int PL = (NX + 31) / 32;
+    float2 v[PL];
+    uint8_t keep[PL];
+#pragma unroll
+    for (int u = 0; u < PL; ++u)
+      if (lane + 32 * u < NX) {
+        v[u] = src[lane + 32 * u];
+        keep[u] = mk[lane + 32 * u];
+      }
+#pragma unroll
+    for (int u = 0; u < PL; ++u)
+      if (lane + 32 * u < NX) b[pad8(lane + 32 * u)] = v[u];
+    __syncwarp();
+    Fft<NX, false>::go(b, tw, lane);
+#pragma unroll
+    for (int u = 0; u < PL; ++u)
+      if (lane + 32 * u < NX && !keep[u]) b[pad8(lane + 32 * u)] = make_float2(0.f, 0.f);
+    __syncwarp();
+    Fft<NX, true>::go(b, tw, lane);
+    for (int i = lane; i < NX; i += 32) src[i] = b[pad8(i)];
+    __syncwarp();  // the buffer is refilled for the next row
+  }
+}
+
+// z_k = y + f_k (F_s S p + u_k - y), the l2-ball projection, and the zero-filled
+// rows of z_k - u_k - F_s S p through the inverse DFT along x.
+template <int NX>
+__global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_ball(MapsRows a) {
+  __shared__ float2 tw[NX];
+  __shared__ float2 buf[kRowWarps][padded_len(NX)];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = a.tw[i];
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float fu = (float)a.sc[S_UFAC];
+  float2* b = buf[warp];
+  const int total = a.TC * a.ny;
+  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
+    const int tc = gr / a.ny, row = gr - tc * a.ny, t = tc / a.C;
+    const int32_t* rp = a.row_ptr + (size_t)t * (a.ny + 1) + row;
+    const int m0 = rp[0], m1 = rp[1];
+    if (m1 <= m0) continue;  // warp-uniform
+    const float fc = (float)a.f[tc];
+    for (int i = lane; i < padded_len(NX); i += 32) b[i] = make_float2(0.f, 0.f);
+    __syncwarp();
+    for (int m = m0 + lane; m < m1; m += 32) {
+      const int kx = a.idx[(size_t)t * a.M + m] - row * NX;
+      const float sg = ((kx + row) & 1) ? -a.ksign : a.ksign;
+      const size_t i = (size_t)tc * a.M + m;
+      const float2 ap = a.ap[i], u0 = a.uk[i], yv = a.y[i];
+      const float2 u = make_float2(fu * u0.x, fu * u0.y);
+      const float2 z = make_float2(yv.x + fc * (ap.x + u.x - yv.x), yv.y + fc * (ap.y + u.y - yv.y));
+      a.zk[i] = z;
+      b[pad8(kx)] = make_float2((z.x - u.x - ap.x) * sg, (z.y - u.y - ap.y) * sg);
+    }
+    __syncwarp();
+    Fft<NX, true>::go(b, tw, lane);
+    float2* dst = a.W + (size_t)gr * NX;
+    for (int i = lane; i < NX; i += 32) dst[i] = b[pad8(i)];
+    __syncwarp();
+  }
+}
+
+// F_s S p of every row (DFT along x, gather) with the data blocks' dual update
+// u_k += F_s S p - z_k; per CTA the sums |F_s S p - z_k|^2 and |F_s S (p - p_prev)|^2.
+template <int NX>
+__global__ void __launch_bounds__(kRowWarps * 32) k_rows_gather_dual(MapsRows a) {
+  __shared__ float2 tw[NX];
+  __shared__ float2 buf[kRowWarps][padded_len(NX)];
+  __shared__ double sh[2 * kRowWarps];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = a.tw[i];
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float fu = (float)a.sc[S_UFAC];
+  float2* b = buf[warp];
+  double sums[2] = {0.0, 0.0};
+  const int total = a.TC * a.ny;
+  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
+    const int tc = gr / a.ny, row = gr - tc * a.ny, t = tc / a.C;
+    const int32_t* rp = a.row_ptr + (size_t)t * (a.ny + 1) + row;
+    const int m0 = rp[0], m1 = rp[1];
+    if (m1 <= m0) continue;  // warp-uniform
+    const float2* src = a.W + (size_t)gr * NX;
+    for (int i = lane; i < NX; i += 32) b[pad8(i)] = src[i];
+    __syncwarp();
+    Fft<NX, false>::go(b, tw, lane);
+    for (int m = m0 + lane; m < m1; m += 32) {
+      const int kx = a.idx[(size_t)t * a.M + m] - row * NX;
+      const float sg = ((kx + row) & 1) ? -a.ksign : a.ksign;
+      const size_t i = (size_t)tc * a.M + m;
+      const float2 e = b[pad8(kx)], old = a.ap[i], z = a.zk[i];
+      const float2 ap = make_float2(e.x * sg, e.y * sg);
+      float2 u = a.uk[i];
+      u = make_float2(fu * u.x + ap.x - z.x, fu * u.y + ap.y - z.y);
+      a.ap[i] = ap;
+      a.uk[i] = u;
+      const double rx = (double)ap.x - z.x, ry = (double)ap.y - z.y;
+      const double sx = (double)ap.x - old.x, sy = (double)ap.y - old.y;
+      sums[0] += rx * rx + ry * ry;
+      sums[1] += sx * sx + sy * sy;
+    }
+    __syncwarp();
+  }
+  block_sums(sums, sh);
+  if (threadIdx.x == 0) {
+    a.partials[2 * (size_t)blockIdx.x] = sums[0];
+    a.partials[2 * (size_t)blockIdx.x + 1] = sums[1];
+  }
+}
+
+// ------------------------------------------------------- element-wise passes
+
+struct CoilSum {
+  const float2* W;  // conj(s_k) w_k [T][C][N]
+  int C, nx;
+  size_t N, total;  // total = T N
+  float scale;
+  float2 *d, *Ad;                        // normal: A d = sum + d
+  const float2 *z0, *u0, *p;             // residual: sum + z0 - ufac u0 - p
+  float2 *r, *p_prev;                    //   into r and d; p kept as p_prev
+  double *sc, *partials;
+  unsigned* counter;
+};
+
+// sum over coils of conj(s_k) w_k with sign and scale.  NORMAL: A d and the CG
+// step a = |r|^2 / <d, A d>; else the CG's first residual and |r|^2.
+template <bool NORMAL>
+__global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
+  __shared__ double sh[kElemThreads / 32];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const float fu = NORMAL ? 1.f : (float)a.sc[S_UFAC];
+  double s[1] = {0.0};
+  for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < a.total; i += (size_t)gridDim.x * kElemThreads) {
+    const size_t t = i / a.N, n = i - t * a.N;
+    const float2* w = a.W + t * a.C * a.N + n;
+    float2 acc = make_float2(0.f, 0.f);
+    int c = 0;
+    for (; c + 8 <= a.C; c += 8) {
+      float2 v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = w[(size_t)(c + j) * a.N];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        acc.x += v[j].x;
+        acc.y += v[j].y;
+      }
+    }
+    for (; c < a.C; ++c) {
+      const float2 v = w[(size_t)c * a.N];
+      acc.x += v.x;
+      acc.y += v.y;
+    }
+    const int y = (int)(n / a.nx), x = (int)(n - (size_t)y * a.nx);
+    const float sg = ((x + y) & 1) ? -a.scale : a.scale;
+    float2 o = make_float2(acc.x * sg, acc.y * sg);
+    if (NORMAL) {
+      const float2 d = a.d[i];
+      o = make_float2(o.x + d.x, o.y + d.y);
+      a.Ad[i] = o;
+      s[0] += (double)d.x * o.x + (double)d.y * o.y;
+    } else {
+      const float2 z = a.z0[i], u = a.u0[i], p = a.p[i];
+      o = make_float2(o.x + z.x - fu * u.x - p.x, o.y + z.y - fu * u.y - p.y);
+      a.r[i] = o;
+      a.d[i] = o;
+      a.p_prev[i] = p;
+      s[0] += (double)o.x * o.x + (double)o.y * o.y;
+    }
+  }
+  if (!group_sums(s, a.partials, a.counter, (int)blockIdx.x, (int)gridDim.x, sh) || threadIdx.x) return;
+  if (NORMAL)
+    a.sc[S_A] = s[0] > 0.0 ? a.sc[S_RR] / s[0] : 0.0;
+  else
+    a.sc[S_RR] = s[0];
+}
+
+// x += a d, r -= a A d, and beta = |r|^2 / |r_old|^2.
+__global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__ x, float2* __restrict__ r,
+                                                            const float2* __restrict__ d,
+                                                            const float2* __restrict__ Ad, size_t n, double* sc,
+                                                            double* partials, unsigned* counter) {
+  __shared__ double sh[kElemThreads / 32];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const float a = (float)sc[S_A];
+  double s[1] = {0.0};
+  for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
+    const float2 dv = d[i], av = Ad[i];
+    float2 xv = x[i], rv = r[i];
+    xv.x = fmaf(a, dv.x, xv.x);
+    xv.y = fmaf(a, dv.y, xv.y);
+    rv.x = fmaf(-a, av.x, rv.x);
+    rv.y = fmaf(-a, av.y, rv.y);
+    x[i] = xv;
+    r[i] = rv;
+    s[0] += (double)rv.x * rv.x + (double)rv.y * rv.y;
+  }
+  if (!group_sums(s, partials, counter, (int)blockIdx.x, (int)gridDim.x, sh) || threadIdx.x) return;
+  sc[S_BETA] = sc[S_RR] > 0.0 ? s[0] / sc[S_RR] : 0.0;
+  sc[S_RR] = s[0];
+}
+
+// f_k = eps_k / max(|F_s S p + u_k - y|, eps_k): kBallBlocks CTAs per (frame, coil).
+__global__ void __launch_bounds__(kThreads) k_ball_norm(const float2* __restrict__ ap, const float2* __restrict__ uk,
+                                                        const float2* __restrict__ y, int M,
+                                                        const double* __restrict__ eps, const double* __restrict__ sc,
+                                                        double* __restrict__ f, double* partials, unsigned* counters) {
+  __shared__ double sh[kThreads / 32];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const int c = blockIdx.y;
+  const float fu = (float)sc[S_UFAC];
+  double s[1] = {0.0};
+  for (int m = blockIdx.x * kThreads + threadIdx.x; m < M; m += gridDim.x * kThreads) {
+    const size_t i = (size_t)c * M + m;
+    const float2 av = ap[i], uv = uk[i], yv = y[i];
+    const double dx = (double)av.x + (double)(fu * uv.x) - yv.x, dy = (double)av.y + (double)(fu * uv.y) - yv.y;
+    s[0] += dx * dx + dy * dy;
+  }
+  if (!group_sums(s, partials + (size_t)c * kBallBlocks, counters + c, (int)blockIdx.x, (int)gridDim.x, sh) ||
+      threadIdx.x)
+    return;
+  f[c] = eps[c] / fmax(sqrt(s[0]), eps[c]);
+}
+
+// u_0 += p - z_0; the residual norms of both blocks (row_part: the data blocks'
+// sums per CTA) and the balancing of rho (He et al. 2000).
+__global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__ u0, const float2* __restrict__ p,
+                                                            const float2* __restrict__ z0,
+                                                            const float2* __restrict__ p_prev, size_t n, double* sc,
+                                                            double* partials, unsigned* counter,
+                                                            const double* __restrict__ row_part, int n_row, double mu,
+                                                            double tau, double* __restrict__ hist) {
+  __shared__ double sh[2 * kElemThreads / 32];
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const float fu = (float)sc[S_UFAC];
+  double s[2] = {0.0, 0.0};
+  for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
+    const float2 pv = p[i], zv = z0[i], qv = p_prev[i];
+    const float2 uv = u0[i];
+    u0[i] = make_float2(fu * uv.x + pv.x - zv.x, fu * uv.y + pv.y - zv.y);
+    const double rx = (double)pv.x - zv.x, ry = (double)pv.y - zv.y;
+    const double dx = (double)pv.x - qv.x, dy = (double)pv.y - qv.y;
+    s[0] += rx * rx + ry * ry;
+    s[1] += dx * dx + dy * dy;
+  }
+  if (!group_sums(s, partials, counter, (int)blockIdx.x, (int)gridDim.x, sh)) return;
+  double d[2] = {0.0, 0.0};
+  for (int i = threadIdx.x; i < n_row; i += kElemThreads) {
+    d[0] += row_part[2 * (size_t)i];
+    d[1] += row_part[2 * (size_t)i + 1];
+  }
+  block_sums(d, sh);
+  if (threadIdx.x) return;
+  const double prim = sqrt(s[0] + d[0]), rho = sc[S_RHO], dual = rho * sqrt(s[1] + d[1]);
+  hist[0] = prim;
+  hist[1] = dual;
+  hist[2] = rho;
+  double f = 1.0;
+  if (prim > mu * dual) {
+    sc[S_RHO] = rho * tau;
+    f = 1.0 / tau;
+  } else if (dual > mu * prim) {
+    sc[S_RHO] = rho / tau;
+    f = tau;
+  }
+  sc[S_UFAC] = f;
+}
+
+__global__ void k_admm_start(double* sc, double rho0) {
+  sc[S_RHO] = rho0;
+  sc[S_UFAC] = 1.0;
+}
+
+// mask[t][idx[t][m]] = 1
+__global__ void k_sample_mask(const int32_t* __restrict__ idx, int M, size_t N, uint8_t* __restrict__ mask) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m < M) mask[(size_t)blockIdx.y * N + idx[(size_t)blockIdx.y * M + m]] = 1;
+}
+
+// --------------------------------------------------------------- launchers
+
+template <bool INV>
+mpi_status launch_maps_cols(mpi_ctx* ctx, int L, const MapsCols& a, int TC) {
+  const int tile = maps_cols_tile(L);
+  const unsigned blocks = (unsigned)((size_t)TC * ((a.nx + tile - 1) / tile));
+  MPI_PROF(ctx, KF_FFT_LINES);
+  switch (L) {
+#define MPI_COLS(n)                                                                              \
+  case n:                                                                                        \
+    launch_pdl(ctx, k_maps_cols<n, INV>, dim3(blocks), dim3(kThreads), 0, a);                    \
+    break;
+    MPI_COLS(16) MPI_COLS(32) MPI_COLS(48) MPI_COLS(64) MPI_COLS(96) MPI_COLS(128) MPI_COLS(192) MPI_COLS(256)
+    MPI_COLS(320) MPI_COLS(512)
+#undef MPI_COLS
+    default:
+      return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+  }
+  MPI_LAUNCH_CHECK(ctx, INV ? "k_maps_cols<inv>" : "k_maps_cols<fwd>");
+  return MPI_OK;
+}
+
+enum RowPass { ROWS_NORMAL, ROWS_SCATTER, ROWS_GATHER };
+
+mpi_status launch_maps_rows(mpi_ctx* ctx, int nx, RowPass pass, const MapsRows& a, unsigned blocks) {
+  MPI_PROF(ctx, KF_FFT_ROWS);
+  switch (nx) {
+#define MPI_ROWS(n)                                                                                             \
+  case n:                                                                                                       \
+    if (pass == ROWS_NORMAL) launch_pdl(ctx, k_rows_normal<n>, dim3(blocks), dim3(kRowWarps * 32), 0, a);       \
+    else if (pass == ROWS_SCATTER)                                                                              \
+      launch_pdl(ctx, k_rows_scatter_ball<n>, dim3(blocks), dim3(kRowWarps * 32), 0, a);                        \
+    else launch_pdl(ctx, k_rows_gather_dual<n>, dim3(blocks), dim3(kRowWarps * 32), 0, a);                      \
+    break;
+    MPI_ROWS(16) MPI_ROWS(32) MPI_ROWS(48) MPI_ROWS(64) MPI_ROWS(96) MPI_ROWS(128) MPI_ROWS(192) MPI_ROWS(256)
+    MPI_ROWS(320) MPI_ROWS(512)
+#undef MPI_ROWS
+    default:
+      return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+  }
+  MPI_LAUNCH_CHECK(ctx, pass == ROWS_NORMAL ? "k_rows_normal"
+                                            : (pass == ROWS_SCATTER ? "k_rows_scatter_ball" : "k_rows_gather_dual"));
+  return MPI_OK;
+}
+
+float axis_sign(int n) { return ((n / 2) & 1) ? -1.f : 1.f; }
+
+unsigned elem_blocks(size_t n) {
+  return (unsigned)std::min<size_t>((n + kElemThreads - 1) / kElemThreads, kMaxElemBlocks);
+}
+
+unsigned row_blocks(const mpi_ctx* ctx, size_t rows) {
+  return (unsigned)std::min<size_t>((rows + kRowWarps - 1) / kRowWarps, 16 * (size_t)std::max(ctx->num_sms, 1));
+}
+
+#define TRY(x)                       \
+  do {                               \
+    mpi_status st__ = (x);           \
+    if (st__ != MPI_OK) return st__; \
+  } while (0)
+
+}  // namespace
+
+bool admm_maps_supported(const mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mpi_basis* basis, int C,
+                         mpi_precision prec) {
+  if (ctx->line_kernel || basis->ctx != ctx || basis->tucker || basis->N != plans[0]->N || plans[0]->M < 1)
+    return false;
+  const bool bf = prec == MPI_PREC_BF16 || prec == MPI_PREC_MIXED;
+  if (!bf && prec != MPI_PREC_FP32 && prec != MPI_PREC_FP32_SIMT) return false;
+  if (bf && (!basis->Ubf || C > 128)) return false;
+  for (int t = 0; t < T; ++t)
+    if (plans[t]->ctx != ctx || plans[t]->kind != MPI_TRAJ_CARTESIAN || plans[t]->ndim != 2) return false;
+  const size_t rows = (size_t)T * C * plans[0]->ny;
+  return rows < 0x7fffffffu && (size_t)T * C <= 65535 && T <= 65535;
+}
+
+size_t admm_maps_layout(const mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mpi_basis* basis, int C,
+                        const mpi_admm_params* prm, mpi_precision prec, void* mem, AdmmMaps* m) {
+  const size_t N = plans[0]->N, M = plans[0]->M, TN = (size_t)T * N, CM = (size_t)T * C * M;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    char* p = (char*)mem + off;
+    off += (bytes + 255) & ~(size_t)255;
+    return p;
+  };
+  auto cplx = [&](size_t n) { return (float2*)take(n * sizeof(float2)); };
+  m->in_y = cplx(CM);
+  m->in_alpha = cplx((size_t)C * basis->q);
+  m->in_eps = (double*)take((size_t)T * C * sizeof(double));
+  m->hist = (double*)take(3 * (size_t)std::max(prm->n_outer, 1) * sizeof(double));
+  m->S = cplx(C * N);
+  m->S_cg = prec == MPI_PREC_MIXED ? cplx(C * N) : m->S;
+  m->W = cplx((size_t)T * C * N);
+  m->zero_begin = (char*)mem + off;  // cleared when a solve starts
+  m->p = cplx(TN);
+  m->u0 = cplx(TN);
+  m->ap = cplx(CM);
+  m->uk = cplx(CM);
+  m->counters = (unsigned*)take(((size_t)T * C + 4) * sizeof(unsigned));
+  m->zero_bytes = (char*)mem + off - m->zero_begin;
+  m->zk = cplx(CM);
+  float2** img[] = {&m->z0, &m->r, &m->d[0], &m->d[1], &m->Ad, &m->p_prev};
+  for (float2** b : img) *b = cplx(TN);
+  m->tv = cplx(tv_scratch_elems(T > 1 ? 3 : 2, (long)TN));
+  m->sc = (double*)take(S_NUM * sizeof(double));
+  m->fball = (double*)take((size_t)T * C * sizeof(double));
+  m->ball_part = (double*)take((size_t)T * C * kBallBlocks * sizeof(double));
+  m->part = (double*)take(2 * (size_t)kMaxElemBlocks * sizeof(double));
+  m->row_part = (double*)take(2 * (size_t)row_blocks(ctx, (size_t)T * C * plans[0]->ny) * sizeof(double));
+  m->idx = (int32_t*)take((size_t)T * M * sizeof(int32_t));
+  m->row_ptr = (int32_t*)take((size_t)T * (plans[0]->ny + 1) * sizeof(int32_t));
+  m->rmask = (uint8_t*)take((size_t)T * plans[0]->ny);
+  m->mask = (uint8_t*)take(TN);
+  return off;
+}
+
+mpi_status admm_maps_tables(mpi_ctx* ctx, const mpi_plan* const* plans, int T, AdmmMaps* m) {
+  const int ny = plans[0]->ny, nx = plans[0]->nx, M = plans[0]->M;
+  const size_t N = plans[0]->N;
+  std::vector<int32_t> rp((size_t)T * (ny + 1));
+  std::vector<uint8_t> has((size_t)T * ny);
+  cudaError_t e = cudaMemsetAsync(m->mask, 0, (size_t)T * N, ctx->stream);
+  for (int t = 0; t < T && e == cudaSuccess; ++t) {
+    e = cudaMemcpyAsync(m->idx + (size_t)t * M, plans[t]->idx, (size_t)M * sizeof(int32_t), cudaMemcpyDeviceToDevice,
+                        ctx->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(rp.data() + (size_t)t * (ny + 1), plans[t]->row_ptr, (size_t)(ny + 1) * sizeof(int32_t),
+                          cudaMemcpyDeviceToHost, ctx->stream);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) return cuda_check(ctx, e, "image solver tables");
+  m->whole_rows = true;
+  for (int t = 0; t < T; ++t)
+    for (int r = 0; r < ny; ++r) {
+      const int n = rp[(size_t)t * (ny + 1) + r + 1] - rp[(size_t)t * (ny + 1) + r];
+      has[(size_t)t * ny + r] = n > 0;
+      m->whole_rows &= n == 0 || n == nx;
+    }
+  e = cudaMemcpyAsync(m->row_ptr, rp.data(), rp.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(m->rmask, has.data(), has.size(), cudaMemcpyHostToDevice, ctx->stream);
+  if (e != cudaSuccess) return cuda_check(ctx, e, "image solver tables");
+  MPI_PROF(ctx, KF_SOLVER);
+  k_sample_mask<<<dim3((unsigned)((M + 255) / 256), (unsigned)T), 256, 0, ctx->stream>>>(m->idx, M, N, m->mask);
+  MPI_LAUNCH_CHECK(ctx, "k_sample_mask");
+  return cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "image solver tables");  // rp and has are read until here
+}
+
+mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mpi_basis* basis, int C,
+                            const mpi_admm_params* prm, mpi_precision prec, const AdmmMaps& m) {
+  const int ny = plans[0]->ny, nx = plans[0]->nx, M = plans[0]->M, TC = T * C;
+  const size_t N = plans[0]->N, TN = (size_t)T * N;
+  const float scale = 1.0f / sqrtf((float)N);
+  const unsigned eblk = elem_blocks(TN), rblk = row_blocks(ctx, (size_t)TC * ny);
+  unsigned* ball_count = m.counters;
+  unsigned* count = m.counters + TC;
+  TRY(cuda_check(ctx, cudaMemsetAsync(m.zero_begin, 0, m.zero_bytes, ctx->stream), "image solver start"));
+  MPI_PROF(ctx, KF_SOLVER);
+  k_admm_start<<<1, 1, 0, ctx->stream>>>(m.sc, prm->rho0);
+  MPI_LAUNCH_CHECK(ctx, "k_admm_start");
+  // MIXED: BF16 maps in the CG iterations; FP32 ones for the constraint-side
+  // products and the CG's first residual
+  TRY(mpi_basis_expand(ctx, basis, (const mpi_c32*)m.in_alpha, C, (mpi_c32*)m.S,
+                       prec == MPI_PREC_MIXED ? MPI_PREC_FP32 : prec));
+  if (m.S_cg != m.S) TRY(mpi_basis_expand(ctx, basis, (const mpi_c32*)m.in_alpha, C, (mpi_c32*)m.S_cg, MPI_PREC_BF16));
+
+  MapsCols cols{};
+  cols.W = m.W;
+  cols.sc = m.sc;
+  cols.C = C;
+  cols.nx = nx;
+  cols.N = N;
+  cols.scale = scale;
+  cols.rmask = m.rmask;
+  cols.tw = twiddle_table(ctx, ny);
+  auto cols_fwd = [&](const float2* S, const float2* v, const float2* r, float2* dnew) {
+    MapsCols a = cols;
+    a.S = S;
+    a.v = v;
+    a.r = r;
+    a.dnew = dnew;
+    return launch_maps_cols<false>(ctx, ny, a, TC);
+  };
+  auto cols_inv = [&](const float2* S) {
+    MapsCols a = cols;
+    a.S = S;
+    a.v = m.p;  // not read
+    return launch_maps_cols<true>(ctx, ny, a, TC);
+  };
+  MapsRows rows{};
+  rows.W = m.W;
+  rows.TC = TC;
+  rows.C = C;
+  rows.ny = ny;
+  rows.M = M;
+  rows.rmask = m.rmask;
+  rows.mask = m.mask;
+  rows.idx = m.idx;
+  rows.row_ptr = m.row_ptr;
+  rows.tw = twiddle_table(ctx, nx);
+  rows.ksign = axis_sign(nx) * axis_sign(ny);
+  rows.y = m.in_y;
+  rows.ap = m.ap;
+  rows.uk = m.uk;
+  rows.zk = m.zk;
+  rows.f = m.fball;
+  rows.sc = m.sc;
+  rows.partials = m.row_part;
+  CoilSum sum{};
+  sum.W = m.W;
+  sum.C = C;
+  sum.nx = nx;
+  sum.N = N;
+  sum.total = TN;
+  sum.Ad = m.Ad;
+  sum.z0 = m.z0;
+  sum.u0 = m.u0;
+  sum.p = m.p;
+  sum.r = m.r;
+  sum.p_prev = m.p_prev;
+  sum.sc = m.sc;
+  sum.partials = m.part;
+  sum.counter = count;
+
+  for (int it = 0; it < prm->n_outer; ++it) {
+    // z_0 = prox_{TV/rho}(p + u_0), z_k = Pi(F_s S p + u_k)
+    TRY(launch_tv_prox(ctx, T > 1 ? T : 1, ny, nx, T > 1 ? 3 : 2, m.p, m.u0, m.sc + S_UFAC, m.sc + S_RHO, 0.f,
+                       prm->n_tv, m.tv, m.z0));
+    MPI_PROF(ctx, KF_SOLVER);
+    launch_pdl(ctx, k_ball_norm, dim3(kBallBlocks, (unsigned)TC), dim3(kThreads), 0, m.ap, m.uk, m.in_y, M, m.in_eps,
+               m.sc, m.fball, m.ball_part, ball_count);
+    MPI_LAUNCH_CHECK(ctx, "k_ball_norm");
+    TRY(launch_maps_rows(ctx, nx, ROWS_SCATTER, rows, rblk));
+    // r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p
+    TRY(cols_inv(m.S));
+    int cur = 0;
+    sum.scale = scale;
+    sum.d = m.d[cur];
+    MPI_PROF(ctx, KF_SOLVER);
+    launch_pdl(ctx, k_coil_sum<false>, dim3(eblk), dim3(kElemThreads), 0, sum);
+    MPI_LAUNCH_CHECK(ctx, "k_coil_sum<residual>");
+    for (int k = 0; k < prm->n_cg; ++k) {
+      if (k) {
+        TRY(cols_fwd(m.S_cg, m.d[cur], m.r, m.d[cur ^ 1]));
+        cur ^= 1;
+      } else {
+        TRY(cols_fwd(m.S_cg, m.d[cur], nullptr, nullptr));
+      }
+      if (!m.whole_rows) TRY(launch_maps_rows(ctx, nx, ROWS_NORMAL, rows, rblk));
+      TRY(cols_inv(m.S_cg));
+      sum.scale = m.whole_rows ? scale * (float)nx : scale;  // F_x^H F_x = nx on whole rows
+      sum.d = m.d[cur];
+      MPI_PROF(ctx, KF_SOLVER);
+      launch_pdl(ctx, k_coil_sum<true>, dim3(eblk), dim3(kElemThreads), 0, sum);
+      MPI_LAUNCH_CHECK(ctx, "k_coil_sum<normal>");
+      MPI_PROF(ctx, KF_SOLVER);
+      launch_pdl(ctx, k_cg_update, dim3(eblk), dim3(kElemThreads), 0, m.p, m.r, m.d[cur], m.Ad, TN, m.sc, m.part, count);
+      MPI_LAUNCH_CHECK(ctx, "k_cg_update");
+    }
+    // u += A p - z, the residuals, rho
+    TRY(cols_fwd(m.S, m.p, nullptr, nullptr));
+    TRY(launch_maps_rows(ctx, nx, ROWS_GATHER, rows, rblk));
+    MPI_PROF(ctx, KF_SOLVER);
+    launch_pdl(ctx, k_admm_dual, dim3(eblk), dim3(kElemThreads), 0, m.u0, m.p, m.z0, m.p_prev, TN, m.sc, m.part, count,
+               m.row_part, (int)rblk, prm->mu, prm->tau, m.hist + 3 * (size_t)it);
+    MPI_LAUNCH_CHECK(ctx, "k_admm_dual");
+  }
+  return MPI_OK;
+}

@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "admm.h"
 #include "mpi_internal.h"
 
 namespace {
@@ -936,32 +937,52 @@ mpi_status image_solve_impl(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     g->C = C;
     g->prec = prec;
     g->key = key;
-    // image side: 9 N and the TV scratch; k-space: 5 CM; inputs y (CM), alpha (Cq); output p (N)
-    const size_t image = 9 * N + tv_scratch_elems(gr.nd, N);
-    const size_t elems = image + 5 * CMs + CMs + Cq + N;
-    const size_t extra = 2 * (size_t)TC + (size_t)TC * kRedBlocks + 3 * (size_t)prm->n_outer + TC + 8;
-    mpi_status st = alloc_solver(ctx, g->mem, elems, extra, g->sv, &g->base, &g->dbase);
-    if (st) {
-      delete g;
-      return st;
+    mpi_status st = MPI_OK;
+    // 2D Cartesian with a dense basis: the fused solve with the maps kept (admm.cu),
+    // where its buffers (T C N complex values and C N of maps beside the state) fit
+    AdmmMaps maps{};
+    bool fused = admm_maps_supported(ctx, plans, T, basis, C, prec);
+    if (fused && cudaMalloc(&g->mem.p, admm_maps_layout(ctx, plans, T, basis, C, prm, prec, nullptr, &maps)) !=
+                     cudaSuccess) {
+      cudaGetLastError();
+      g->mem.p = nullptr;
+      fused = false;
     }
-    float2* io = g->base + image + 5 * CMs;
-    g->in_y = io;
-    g->in_alpha = io + CMs;
-    g->out_p = g->in_alpha + Cq;
-    double* scratch = g->dbase;                                     // fball, bpart
-    g->hist = scratch + 2 * (size_t)TC + (size_t)TC * kRedBlocks;  // [n_outer][3]
-    g->in_eps = g->hist + 3 * (size_t)prm->n_outer;
     g->work = ctx->work;
-    for (int t = 0; t < T && st == MPI_OK; ++t) st = tune_line_passes(ctx, plans[t], C);
-    if (st) {
-      delete g;
-      return st;
+    if (fused) {
+      admm_maps_layout(ctx, plans, T, basis, C, prm, prec, g->mem.p, &maps);
+      g->in_y = maps.in_y;
+      g->in_alpha = maps.in_alpha;
+      g->in_eps = maps.in_eps;
+      g->out_p = maps.p;
+      g->hist = maps.hist;
+      st = admm_maps_tables(ctx, plans, T, &maps);
+      if (st == MPI_OK)
+        st = capture(ctx, g, [&]() { return admm_maps_record(ctx, plans, T, basis, C, prm, prec, maps); });
+    } else {
+      // image side: 9 N and the TV scratch; k-space: 5 CM; inputs y (CM), alpha (Cq); output p (N)
+      const size_t image = 9 * N + tv_scratch_elems(gr.nd, N);
+      const size_t elems = image + 5 * CMs + CMs + Cq + N;
+      const size_t extra = 2 * (size_t)TC + (size_t)TC * kRedBlocks + 3 * (size_t)prm->n_outer + TC + 8;
+      st = alloc_solver(ctx, g->mem, elems, extra, g->sv, &g->base, &g->dbase);
+      if (st) {
+        delete g;
+        return st;
+      }
+      float2* io = g->base + image + 5 * CMs;
+      g->in_y = io;
+      g->in_alpha = io + CMs;
+      g->out_p = g->in_alpha + Cq;
+      double* scratch = g->dbase;                                     // fball, bpart
+      g->hist = scratch + 2 * (size_t)TC + (size_t)TC * kRedBlocks;  // [n_outer][3]
+      g->in_eps = g->hist + 3 * (size_t)prm->n_outer;
+      for (int t = 0; t < T && st == MPI_OK; ++t) st = tune_line_passes(ctx, plans[t], C);
+      if (st == MPI_OK)
+        st = capture(ctx, g, [&]() {
+          return admm_body(ctx, plans, T, basis, C, prm, prec, g->sv, g->base, scratch, (const mpi_c32*)g->in_alpha,
+                           g->in_y, g->in_eps, g->out_p, g->hist);
+        });
     }
-    st = capture(ctx, g, [&]() {
-      return admm_body(ctx, plans, T, basis, C, prm, prec, g->sv, g->base, scratch, (const mpi_c32*)g->in_alpha,
-                       g->in_y, g->in_eps, g->out_p, g->hist);
-    });
     if (st) {
       delete g;
       return st;
