@@ -15,7 +15,10 @@
 // and output); the rows stream the same basis tiles in step, so the basis is
 // read from DRAM about once per group instead of once per slice.  Each slice's
 // per-coil images live in a batch-owned buffer between the expansion and the
-// slice's FFT passes.  How many CTAs each row gets is chosen at creation by
+// FFT passes.  From kGroupedPasses slices on, the FFT passes take all coils of a
+// group's slices in one launch too (per run of slices whose pass along y is tuned
+// to the same kernel, so that a slice's values stay those of its own call), with a
+// table of every coil's sampling.  How many CTAs each row gets is chosen at creation by
 // timing the candidates (an autotuner decision the context records).
 #include <algorithm>
 #include <cstdio>
@@ -33,6 +36,7 @@ struct mpi_batch {
   int64_t kernels = 0;  // kernels per replay
   void* buf = nullptr;   // per-coil images of one group [sum C][N]
   void* rows = nullptr;  // row tables of every group (device)
+  void* tabs = nullptr;  // sampling tables and row masks of the grouped passes (device)
   int groups = 0;        // grouped launches per direction
 };
 
@@ -47,12 +51,25 @@ mpi_status record_slice(mpi_ctx* ctx, const mpi_batch_slice& s, int kind, mpi_pr
   return st;
 }
 
+// Slices a group needs for its FFT passes to be grouped.  A launch of its own costs a
+// slice 5-14 us per pass (8-32 coils of 128^2 to 320^2), much of it fixed: 16 slices
+// of 128^2 took 90 us in 16 row passes and 22 in one, of 320^2 219 and 131.  Two or
+// three slices save a few microseconds at most and keep the passes of their own calls.
+constexpr int kGroupedPasses = 4;
+
 struct Group {
   std::vector<int> idx;  // slices, in recording order
   int Cmax = 0;
   long sumC = 0;
   size_t fwd_rows = 0, adj_rows = 0;  // offsets (rows) into the device row table
   int row_ctas = 0;
+  // grouped passes: runs of slices (first, count in coils) per direction and kernel
+  struct Run {
+    int kernel, first, coils;
+  };
+  std::vector<Run> fwd, inv;  // empty: the passes run slice by slice
+  const CoilSamples* tab = nullptr;
+  const uint8_t* row_has = nullptr;
 };
 
 bool groupable(const mpi_batch_slice& s, mpi_precision prec) {
@@ -64,20 +81,30 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
                         const ExpandRow* rows, float2* buf) {
   const mpi_batch_slice& s0 = sl[g.idx[0]];
   const long N = s0.plan->N;
-  const int nr = (int)g.idx.size();
+  const int nr = (int)g.idx.size(), ny = s0.plan->ny, nx = s0.plan->nx;
   mpi_status st = MPI_OK;
   if (kind & MPI_BATCH_FORWARD) {
     st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, rows + g.fwd_rows, nr, g.Cmax, prec, g.row_ctas);
+    for (const Group::Run& r : g.fwd)
+      if (st == MPI_OK)
+        st = launch_fft_cols_group(ctx, r.kernel, buf + r.first * N, r.coils, ny, nx, false,
+                                   g.row_has ? g.row_has + (size_t)r.first * ny : nullptr);
+    if (st == MPI_OK && !g.fwd.empty()) st = launch_rows_group(ctx, buf, (int)g.sumC, ny, nx, false, g.tab);
     long off = 0;
-    for (int i = 0; i < nr && st == MPI_OK; ++i) {
+    for (int i = 0; i < nr && st == MPI_OK && g.fwd.empty(); ++i) {
       const mpi_batch_slice& s = sl[g.idx[i]];
       st = plan_image_to_kspace(ctx, s.plan, buf + off * N, s.C, (float2*)s.y);
       off += s.C;
     }
   }
   if (st == MPI_OK && (kind & MPI_BATCH_ADJOINT)) {
+    if (!g.inv.empty()) st = launch_rows_group(ctx, buf, (int)g.sumC, ny, nx, true, g.tab);
+    for (const Group::Run& r : g.inv)
+      if (st == MPI_OK)
+        st = launch_fft_cols_group(ctx, r.kernel, buf + r.first * N, r.coils, ny, nx, true,
+                                   g.row_has ? g.row_has + (size_t)r.first * ny : nullptr);
     long off = 0;
-    for (int i = 0; i < nr && st == MPI_OK; ++i) {
+    for (int i = 0; i < nr && st == MPI_OK && g.inv.empty(); ++i) {
       const mpi_batch_slice& s = sl[g.idx[i]];
       st = plan_kspace_to_image(ctx, s.plan, (const float2*)s.y, s.C, buf + off * N);
       off += s.C;
@@ -85,6 +112,66 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
     if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_ADJ, rows + g.adj_rows, nr, g.Cmax, prec, g.row_ctas);
   }
   return st;
+}
+
+// Runs of the group's slices (already in an order that keeps equal kernels
+// together) whose pass along y runs the same kernel.
+std::vector<Group::Run> pass_runs(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g, bool inverse) {
+  std::vector<Group::Run> runs;
+  int off = 0;
+  for (int i : g.idx) {
+    const int k = fft_cols_kernel(ctx, sl[i].plan, sl[i].C, inverse);
+    if (runs.empty() || runs.back().kernel != k) runs.push_back({k, off, 0});
+    runs.back().coils += sl[i].C;
+    off += sl[i].C;
+  }
+  return runs;
+}
+
+// The grouped passes' tables: every coil's sampling (idx, row_ptr, its samples) and,
+// where some slice has rows without samples, every coil's row mask.
+mpi_status group_tables(mpi_ctx* ctx, const mpi_batch_slice* sl, std::vector<Group>& groups, void** out) {
+  std::vector<size_t> tab_off, mask_off;
+  size_t bytes = 0;
+  for (const Group& g : groups) {
+    if (g.fwd.empty()) continue;
+    tab_off.push_back(bytes);
+    bytes += ((size_t)g.sumC * sizeof(CoilSamples) + 255) & ~(size_t)255;
+    mask_off.push_back(bytes);
+    bytes += ((size_t)g.sumC * sl[g.idx[0]].plan->ny + 255) & ~(size_t)255;
+  }
+  if (!bytes) return MPI_OK;
+  cudaError_t e = cudaMalloc(out, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return set_err(ctx, MPI_ERR_OOM, "batch: group tables");
+  }
+  std::vector<unsigned char> host(bytes, 1);
+  size_t k = 0;
+  for (Group& g : groups) {
+    if (g.fwd.empty()) continue;
+    CoilSamples* tab = (CoilSamples*)(host.data() + tab_off[k]);
+    const int ny = sl[g.idx[0]].plan->ny;
+    long off = 0;
+    bool masked = false;
+    for (int i : g.idx) {
+      const mpi_batch_slice& s = sl[i];
+      unsigned char* m = host.data() + mask_off[k] + (size_t)off * ny;
+      if (s.plan->row_has) {
+        masked = true;
+        e = cudaMemcpy(m, s.plan->row_has, ny, cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_check(ctx, e, "batch: group tables");
+        for (int c = 1; c < s.C; ++c) std::copy(m, m + ny, m + (size_t)c * ny);
+      }
+      for (int c = 0; c < s.C; ++c)
+        tab[off + c] = CoilSamples{s.plan->idx, s.plan->row_ptr, (float2*)s.y + (size_t)c * s.plan->M};
+      off += s.C;
+    }
+    g.tab = (const CoilSamples*)((char*)*out + tab_off[k]);
+    g.row_has = masked ? (const uint8_t*)*out + mask_off[k] : nullptr;
+    ++k;
+  }
+  return cuda_check(ctx, cudaMemcpy(*out, host.data(), bytes, cudaMemcpyHostToDevice), "batch: group tables");
 }
 
 // CTAs per row for a group's expansion: every candidate timed over three
@@ -200,6 +287,19 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     ++i;
   }
 
+  // grouped passes: slices in the order of the kernels their passes along y run
+  for (Group& g : groups) {
+    if ((int)g.idx.size() < kGroupedPasses || ctx->line_kernel) continue;
+    std::stable_sort(g.idx.begin(), g.idx.end(), [&](int a, int b) {
+      const mpi_batch_slice &x = slices[a], &y = slices[b];
+      const int fa = fft_cols_kernel(ctx, x.plan, x.C, false), fb = fft_cols_kernel(ctx, y.plan, y.C, false);
+      if (fa != fb) return fa < fb;
+      return fft_cols_kernel(ctx, x.plan, x.C, true) < fft_cols_kernel(ctx, y.plan, y.C, true);
+    });
+    g.fwd = pass_runs(ctx, slices, g, false);
+    g.inv = pass_runs(ctx, slices, g, true);
+  }
+
   mpi_batch* bt = new mpi_batch();
   bt->ctx = ctx;
   bt->n = n;
@@ -236,6 +336,11 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     e = cudaMemcpy(bt->rows, host.data(), nrows * sizeof(ExpandRow), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
       mpi_status st = cuda_check(ctx, e, "batch: row tables");
+      mpi_batch_destroy(bt);
+      return st;
+    }
+    mpi_status st = group_tables(ctx, slices, groups, &bt->tabs);
+    if (st) {
       mpi_batch_destroy(bt);
       return st;
     }
@@ -312,12 +417,13 @@ extern "C" int mpi_batch_group_count(const mpi_batch* bt) { return bt ? bt->grou
 
 extern "C" mpi_status mpi_batch_destroy(mpi_batch* bt) {
   if (!bt) return MPI_ERR_ARG;
-  if (bt->ctx && (bt->buf || bt->rows)) cudaStreamSynchronize(bt->ctx->stream);  // a replay may still run
+  if (bt->ctx && (bt->buf || bt->rows || bt->tabs)) cudaStreamSynchronize(bt->ctx->stream);  // a replay may still run
   ctx_release(&bt->ctx);
   if (bt->exec) cudaGraphExecDestroy(bt->exec);
   if (bt->graph) cudaGraphDestroy(bt->graph);
   if (bt->buf) cudaFree(bt->buf);
   if (bt->rows) cudaFree(bt->rows);
+  if (bt->tabs) cudaFree(bt->tabs);
   delete bt;
   return MPI_OK;
 }

@@ -28,11 +28,12 @@ using namespace mpi_fft;
 // most of them without samples, and one CTA each would make the pass bound by
 // CTA launches).  Forward: FFT along x, k-side centring sign, gather the row's
 // samples (contiguous in the sorted list); rows without samples are skipped.
-template <int NX>
+// TAB (a batch's group of slices): coil c has its own sampling and data block, tab[c].
+template <int NX, bool TAB = false>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(
     const float2* __restrict__ data, int C, int n_rows, int ny, const int32_t* __restrict__ idx,
     const int32_t* __restrict__ row_ptr, float2* __restrict__ y, int M, float ksign,
-    const float2* __restrict__ tw_g) {
+    const float2* __restrict__ tw_g, const CoilSamples* __restrict__ tab) {
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   __shared__ float2 tw[NX];
@@ -44,6 +45,11 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(
   const int total = C * n_rows;
   for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
     const int c = gr / n_rows, row = gr - c * n_rows;
+    if (TAB) {
+      idx = tab[c].idx;
+      row_ptr = tab[c].row_ptr;
+    }
+    float2* yc = TAB ? tab[c].y : y + (size_t)c * M;
     const int m0 = row_ptr[row], m1 = row_ptr[row + 1];
     if (m1 <= m0) continue;  // warp-uniform
     const float2* src = data + ((size_t)c * n_rows + row) * NX;
@@ -63,7 +69,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(
       const int kx = (int)(idx[m] - rbase);
       const float sg = ((kx + rpar) & 1) ? -ksign : ksign;
       const float2 t = b[pad8(kx)];
-      y[(size_t)c * M + m] = make_float2(t.x * sg, t.y * sg);
+      yc[m] = make_float2(t.x * sg, t.y * sg);
     }
     __syncwarp();  // the buffer is refilled for the next row
   }
@@ -72,11 +78,11 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(
 // Adjoint: zero-fill the row from its samples (with the k-side sign), inverse
 // FFT.  Rows without samples are not written: the pass along y that follows
 // reads them as zeros.  Same row striding.
-template <int NX>
+template <int NX, bool TAB = false>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_inv(
     const float2* __restrict__ y, int C, int n_rows, int ny, const int32_t* __restrict__ idx,
     const int32_t* __restrict__ row_ptr, float2* __restrict__ data, int M, float ksign,
-    const float2* __restrict__ tw_g) {
+    const float2* __restrict__ tw_g, const CoilSamples* __restrict__ tab) {
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   __shared__ float2 tw[NX];
@@ -88,6 +94,11 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_inv(
   const int total = C * n_rows;
   for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
     const int c = gr / n_rows, row = gr - c * n_rows;
+    if (TAB) {
+      idx = tab[c].idx;
+      row_ptr = tab[c].row_ptr;
+    }
+    const float2* yc = TAB ? tab[c].y : y + (size_t)c * M;
     const int m0 = row_ptr[row], m1 = row_ptr[row + 1];
     float2* dst = data + ((size_t)c * n_rows + row) * NX;
     if (m1 <= m0) continue;  // warp-uniform
@@ -98,7 +109,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_inv(
     for (int m = m0 + lane; m < m1; m += 32) {
       const int kx = (int)(idx[m] - rbase);
       const float sg = ((kx + rpar) & 1) ? -ksign : ksign;
-      const float2 t = y[(size_t)c * M + m];
+      const float2 t = yc[m];
       b[pad8(kx)] = make_float2(t.x * sg, t.y * sg);
     }
     __syncwarp();
@@ -1158,7 +1169,7 @@ mpi_status launch_rows_fwd_gather(mpi_ctx* ctx, const mpi_plan* plan, const floa
 #define MPI_ROWS_CASE(n)                                                                          \
   case n:                                                                                         \
     launch_pdl(ctx, k_rows_fwd_gather<n>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, data, C, n_rows, \
-               plan->ny, plan->idx, plan->row_ptr, y, plan->M, ks, tw);                           \
+               plan->ny, plan->idx, plan->row_ptr, y, plan->M, ks, tw, nullptr);                  \
     break;
   MPI_PROF(ctx, KF_FFT_ROWS);
   switch (plan->nx) {
@@ -1192,7 +1203,7 @@ mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const flo
 #define MPI_ROWS_CASE(n)                                                                          \
   case n:                                                                                         \
     launch_pdl(ctx, k_rows_scatter_inv<n>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, y, C, n_rows, \
-               plan->ny, plan->idx, plan->row_ptr, data, plan->M, ks, tw);                        \
+               plan->ny, plan->idx, plan->row_ptr, data, plan->M, ks, tw, nullptr);               \
     break;
   MPI_PROF(ctx, KF_FFT_ROWS);
   switch (plan->nx) {
@@ -1211,6 +1222,69 @@ mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const flo
   }
 #undef MPI_ROWS_CASE
   MPI_LAUNCH_CHECK(ctx, "k_rows_scatter_inv");
+  return MPI_OK;
+}
+
+// ------------------------------------------------- passes of a batch's group
+
+int fft_cols_kernel(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse) {
+  const int ny = plan->ny, nx = plan->nx;
+  const long plane = (long)ny * nx;
+  const float2* tw = twiddle_table(ctx, ny);
+  const int t = inverse ? lines_choose<true>(ctx, nullptr, ny, nx, nx, C, 1, plane, 0, tw, plan->row_has, 1)
+                        : lines_choose<false>(ctx, nullptr, ny, nx, nx, C, 1, plane, 0, tw, plan->row_has, 1);
+  return t ? t : lines_tile(ctx, ny, nx, C);
+}
+
+mpi_status launch_fft_cols_group(mpi_ctx* ctx, int kernel, float2* data, int coils, int ny, int nx, bool inverse,
+                                 const uint8_t* row_has) {
+  const float2* tw = twiddle_table(ctx, ny);
+  const int cols = kernel < 0 ? 32 : kernel;
+  const long blocks = (long)coils * ((nx + cols - 1) / cols);
+  if (!tw || blocks > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "grouped FFT pass");
+  MPI_PROF(ctx, KF_FFT_LINES);
+  const long plane = (long)ny * nx;
+  const bool ok =
+      inverse ? lines_launch_tile<true>(ctx, kernel, ny, blocks, data, nx, nx, coils, 1, plane, 0, tw, row_has, coils)
+              : lines_launch_tile<false>(ctx, kernel, ny, blocks, data, nx, nx, coils, 1, plane, 0, tw, row_has, coils);
+  if (!ok) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+  MPI_LAUNCH_CHECK(ctx, inverse ? "k_fft_lines<y,inv,group>" : "k_fft_lines<y,fwd,group>");
+  return MPI_OK;
+}
+
+mpi_status launch_rows_group(mpi_ctx* ctx, float2* data, int coils, int ny, int nx, bool inverse,
+                             const CoilSamples* tab) {
+  if ((long)coils * ny > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "too many k-space rows");
+  const long blocks = std::min(((long)coils * ny + kRowWarps - 1) / kRowWarps, 16L * std::max(ctx->num_sms, 1));
+  const float ks = axis_sign(nx) * axis_sign(ny);
+  const float2* tw = twiddle_table(ctx, nx);
+  if (!tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+  MPI_PROF(ctx, KF_FFT_ROWS);
+#define MPI_ROWS_CASE(n)                                                                                          \
+  case n:                                                                                                         \
+    if (inverse)                                                                                                  \
+      launch_pdl(ctx, k_rows_scatter_inv<n, true>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, nullptr, coils, \
+                 ny, ny, nullptr, nullptr, data, 0, ks, tw, tab);                                                 \
+    else                                                                                                          \
+      launch_pdl(ctx, k_rows_fwd_gather<n, true>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, data, coils,   \
+                 ny, ny, nullptr, nullptr, nullptr, 0, ks, tw, tab);                                              \
+    break;
+  switch (nx) {
+    MPI_ROWS_CASE(16)
+    MPI_ROWS_CASE(32)
+    MPI_ROWS_CASE(48)
+    MPI_ROWS_CASE(64)
+    MPI_ROWS_CASE(96)
+    MPI_ROWS_CASE(128)
+    MPI_ROWS_CASE(192)
+    MPI_ROWS_CASE(256)
+    MPI_ROWS_CASE(320)
+    MPI_ROWS_CASE(512)
+    default:
+      return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+  }
+#undef MPI_ROWS_CASE
+  MPI_LAUNCH_CHECK(ctx, inverse ? "k_rows_scatter_inv<group>" : "k_rows_fwd_gather<group>");
   return MPI_OK;
 }
 

@@ -418,6 +418,21 @@ mpi_status launch_rows_fwd_gather(mpi_ctx* ctx, const mpi_plan* plan, const floa
 mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, int C,
                                    float2* data);
 
+// Passes of a batch's group of 2D slices on one grid: all their coils [coils][ny][nx]
+// in one launch.  fft_cols_kernel is the line kernel that the pass along y of a
+// slice with C coils runs (tuned or by rule); launch_fft_cols_group runs that one, with
+// row_has [coils][ny]; launch_rows_group gathers or scatters by a table per coil.
+struct CoilSamples {
+  const int32_t* idx;
+  const int32_t* row_ptr;
+  float2* y;  // the coil's samples
+};
+int fft_cols_kernel(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse);
+mpi_status launch_fft_cols_group(mpi_ctx* ctx, int kernel, float2* data, int coils, int ny, int nx, bool inverse,
+                                 const uint8_t* row_has);
+mpi_status launch_rows_group(mpi_ctx* ctx, float2* data, int coils, int ny, int nx, bool inverse,
+                             const CoilSamples* tab);
+
 // ------------------------------------------------------------- NUFFT (radial)
 
 mpi_status nufft_plan_init(mpi_ctx* ctx, mpi_plan* plan, const float* traj_host);
