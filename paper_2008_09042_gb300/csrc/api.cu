@@ -568,6 +568,15 @@ extern "C" mpi_status mpi_plan_create(mpi_ctx* ctx, const mpi_plan_desc* d, mpi_
     if (e == cudaSuccess && any_empty) e = cudaMalloc(&plan->row_has, row_has.size());
     if (e == cudaSuccess && any_empty)
       e = cudaMemcpy(plan->row_has, row_has.data(), row_has.size(), cudaMemcpyHostToDevice);
+    std::vector<int32_t> list;
+    for (int r = 0; r < plan->n_rows; ++r)
+      if (row_has[r]) list.push_back(r);
+    plan->n_list = (int)list.size();
+    if (e == cudaSuccess && any_empty && !list.empty()) {
+      e = cudaMalloc(&plan->row_list, list.size() * sizeof(int32_t));
+      if (e == cudaSuccess)
+        e = cudaMemcpy(plan->row_list, list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    }
     if (e == cudaSuccess && d->ndim == 3) {
       // per kz plane, the rows with samples (the pipelined plane passes keep
       // only those rows of a plane in shared memory)
@@ -649,7 +658,7 @@ extern "C" mpi_status mpi_plan_destroy(mpi_plan* plan) {
     solver_cache_forget(plan->ctx, plan);
     ctx_release(&plan->ctx);
   }
-  void* ptrs[] = {plan->idx,        plan->row_ptr,     plan->row_has,    plan->plane_rows, plan->plane_nrows,
+  void* ptrs[] = {plan->idx,        plan->row_ptr,     plan->row_has,    plan->row_list,   plan->plane_rows, plan->plane_nrows,
                   plan->plane_slot, plan->traj,        plan->gstart,     plan->gw,         plan->deap,
                   plan->cell_ptr,   plan->cell_rank,   plan->cell_sx,    plan->cell_w,     plan->cell_dense,
                   plan->tile_items, plan->tile_samples};

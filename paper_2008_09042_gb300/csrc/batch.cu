@@ -70,6 +70,7 @@ struct Group {
   std::vector<Run> fwd, inv;  // empty: the passes run slice by slice
   const CoilSamples* tab = nullptr;
   const uint8_t* row_has = nullptr;
+  int n_list = 0;  // the most rows with samples that any slice has
 };
 
 bool groupable(const mpi_batch_slice& s, mpi_precision prec) {
@@ -89,7 +90,7 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
       if (st == MPI_OK)
         st = launch_fft_cols_group(ctx, r.kernel, buf + r.first * N, r.coils, ny, nx, false,
                                    g.row_has ? g.row_has + (size_t)r.first * ny : nullptr);
-    if (st == MPI_OK && !g.fwd.empty()) st = launch_rows_group(ctx, buf, (int)g.sumC, ny, nx, false, g.tab);
+    if (st == MPI_OK && !g.fwd.empty()) st = launch_rows_group(ctx, buf, (int)g.sumC, ny, nx, false, g.tab, g.n_list);
     long off = 0;
     for (int i = 0; i < nr && st == MPI_OK && g.fwd.empty(); ++i) {
       const mpi_batch_slice& s = sl[g.idx[i]];
@@ -98,7 +99,7 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
     }
   }
   if (st == MPI_OK && (kind & MPI_BATCH_ADJOINT)) {
-    if (!g.inv.empty()) st = launch_rows_group(ctx, buf, (int)g.sumC, ny, nx, true, g.tab);
+    if (!g.inv.empty()) st = launch_rows_group(ctx, buf, (int)g.sumC, ny, nx, true, g.tab, g.n_list);
     for (const Group::Run& r : g.inv)
       if (st == MPI_OK)
         st = launch_fft_cols_group(ctx, r.kernel, buf + r.first * N, r.coils, ny, nx, true,
@@ -164,7 +165,9 @@ mpi_status group_tables(mpi_ctx* ctx, const mpi_batch_slice* sl, std::vector<Gro
         for (int c = 1; c < s.C; ++c) std::copy(m, m + ny, m + (size_t)c * ny);
       }
       for (int c = 0; c < s.C; ++c)
-        tab[off + c] = CoilSamples{s.plan->idx, s.plan->row_ptr, (float2*)s.y + (size_t)c * s.plan->M};
+        tab[off + c] = CoilSamples{s.plan->idx,      s.plan->row_ptr, s.plan->row_list,
+                                   s.plan->n_list, (float2*)s.y + (size_t)c * s.plan->M};
+      g.n_list = std::max(g.n_list, s.plan->n_list);
       off += s.C;
     }
     g.tab = (const CoilSamples*)((char*)*out + tab_off[k]);

@@ -1,8 +1,8 @@
 // Small DFTs held in registers (one thread, complex float2 values):
-// X[k] = sum_n x[n] exp(-2 pi i n k / R) for R = 3, 4, 8, 12, 16, with the
-// constants of the roots of unity written out (cos and sin of multiples of
-// pi / 8 and pi / 6).  Shared by the fused Tucker kernels and the register
-// column FFT.
+// X[k] = sum_n x[n] exp(-2 pi i n k / R) for R = 3, 4, 5, 8, 12, 16, 20, 32, with
+// the constants of the roots of unity written out (cos and sin of multiples of
+// pi / 16, pi / 10 and pi / 6).  Shared by the fused Tucker kernels and the register
+// row and column FFTs.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -127,11 +127,98 @@ __host__ __device__ __forceinline__ void dft16(float2 (&v)[16]) {
   }
 }
 
+__host__ __device__ __forceinline__ void dft5(float2 (&v)[5]) {
+  // c1 = cos(2 pi / 5), c2 = cos(4 pi / 5), s1 = sin(2 pi / 5), s2 = sin(4 pi / 5)
+  const float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;
+  const float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;
+  const float2 a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
+  const float2 a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
+  const float2 x0 = v[0];
+  const float2 r1 = make_float2(x0.x + c1 * a1.x + c2 * a2.x, x0.y + c1 * a1.y + c2 * a2.y);
+  const float2 r2 = make_float2(x0.x + c2 * a1.x + c1 * a2.x, x0.y + c2 * a1.y + c1 * a2.y);
+  const float2 i1 = make_float2(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y);
+  const float2 i2 = make_float2(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y);
+  v[0] = make_float2(x0.x + a1.x + a2.x, x0.y + a1.y + a2.y);
+  v[1] = make_float2(r1.x + i1.y, r1.y - i1.x);
+  v[4] = make_float2(r1.x - i1.y, r1.y + i1.x);
+  v[2] = make_float2(r2.x + i2.y, r2.y - i2.x);
+  v[3] = make_float2(r2.x - i2.y, r2.y + i2.x);
+}
+
+// exp(-2 pi i m / 20) and exp(-2 pi i m / 32) for constant m (folded when unrolled)
+__host__ __device__ __forceinline__ float2 root20(int m) {
+  const float c[6] = {1.f, 0.95105651629515357f, 0.80901699437494742f, 0.58778525229247313f, 0.30901699437494742f, 0.f};
+  // cos(2 pi m / 20), sin(2 pi m / 20) for 0 <= m <= 12
+  const float co = m <= 5 ? c[m] : (m <= 10 ? -c[10 - m] : -c[m - 10]);
+  const float si = m <= 5 ? c[5 - m] : (m <= 10 ? c[m - 5] : -c[15 - m]);
+  return make_float2(co, -si);
+}
+__host__ __device__ __forceinline__ float2 root32(int m) {
+  const float c[9] = {1.f,
+                      0.98078528040323045f,
+                      0.92387953251128676f,
+                      0.83146961230254524f,
+                      0.70710678118654752f,
+                      0.55557023301960222f,
+                      0.38268343236508977f,
+                      0.19509032201612827f,
+                      0.f};
+  // cos(2 pi m / 32), sin(2 pi m / 32) for 0 <= m <= 24
+  const float co = m <= 8 ? c[m] : (m <= 16 ? -c[16 - m] : -c[m - 16]);
+  const float si = m <= 8 ? c[8 - m] : (m <= 16 ? c[m - 8] : -c[24 - m]);
+  return make_float2(co, -si);
+}
+
+// 20 = 4 x 5: n = 4 n2 + n1, k = k1 + 5 k2; 5-point DFTs over n2, twiddles
+// exp(-2 pi i n1 k1 / 20), 4-point DFTs over n1.
+__host__ __device__ __forceinline__ void dft20(float2 (&v)[20]) {
+  float2 y[4][5];
+#pragma unroll
+  for (int n1 = 0; n1 < 4; ++n1) {
+#pragma unroll
+    for (int n2 = 0; n2 < 5; ++n2) y[n1][n2] = v[4 * n2 + n1];
+    dft5(y[n1]);
+#pragma unroll
+    for (int k1 = 1; k1 < 5; ++k1)
+      if (n1) y[n1][k1] = cmulf(y[n1][k1], root20(n1 * k1));
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < 5; ++k1) {
+    dft4(y[0][k1], y[1][k1], y[2][k1], y[3][k1]);
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) v[k1 + 5 * k2] = y[k2][k1];
+  }
+}
+
+// 32 = 4 x 8: n = 4 n2 + n1, k = k1 + 8 k2; 8-point DFTs over n2, twiddles
+// exp(-2 pi i n1 k1 / 32), 4-point DFTs over n1.
+__host__ __device__ __forceinline__ void dft32(float2 (&v)[32]) {
+  float2 y[4][8];
+#pragma unroll
+  for (int n1 = 0; n1 < 4; ++n1) {
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2) y[n1][n2] = v[4 * n2 + n1];
+    dft8(y[n1]);
+#pragma unroll
+    for (int k1 = 1; k1 < 8; ++k1)
+      if (n1) y[n1][k1] = cmulf(y[n1][k1], root32(n1 * k1));
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < 8; ++k1) {
+    dft4(y[0][k1], y[1][k1], y[2][k1], y[3][k1]);
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) v[k1 + 8 * k2] = y[k2][k1];
+  }
+}
+
 template <int R>
 __host__ __device__ __forceinline__ void dft_r(float2 (&v)[R]) {
-  if constexpr (R == 8) dft8(v);
+  if constexpr (R == 4) dft4(v[0], v[1], v[2], v[3]);
+  else if constexpr (R == 8) dft8(v);
   else if constexpr (R == 12) dft12(v);
-  else dft16(v);
+  else if constexpr (R == 16) dft16(v);
+  else if constexpr (R == 20) dft20(v);
+  else dft32(v);
 }
 
 

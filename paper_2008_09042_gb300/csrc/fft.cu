@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "dft_reg.cuh"
+#include "fft_rows.cuh"
 #include "fft_tile.cuh"
 #include "mpi_internal.h"
 #include "ptx.cuh"
@@ -23,98 +24,152 @@ namespace {
 
 using namespace mpi_fft;
 
-// One warp per (coil, k-space row), the warps striding over all rows (the grid
-// is capped at a few CTAs per SM: volumes have hundreds of thousands of rows,
-// most of them without samples, and one CTA each would make the pass bound by
-// CTA launches).  Forward: FFT along x, k-side centring sign, gather the row's
-// samples (contiguous in the sorted list); rows without samples are skipped.
+// Rows along x of a Cartesian plan.  A warp takes R of a coil's k-space rows with
+// samples (row_list; null: every row) through the register FFT of fft_rows.cuh,
+// the warps striding over all of them (the grid is capped at a few CTAs per SM:
+// volumes have hundreds of thousands of rows, and one CTA each would make the pass
+// bound by CTA launches).  256^2, 16 coils, warm L2: 7 us with a Stockham line per
+// warp, 5 this way; 288 coils of 320^2 in one launch 131 -> 85 us (gather), 118 -> 85
+// (scatter), of which the 236 MB they read or write take 35 at HBM's rate.
+//
+// Forward: FFT along x, k-side centring sign, gather the row's samples (contiguous
+// in the sorted list); rows without samples are not touched.
 // TAB (a batch's group of slices): coil c has its own sampling and data block, tab[c].
+struct RowsArgs {
+  int C, n_rows, ny, M;
+  int n_list;  // rows with samples (TAB: the most that any coil has)
+  const int32_t* row_list;
+  const int32_t* idx;
+  const int32_t* row_ptr;
+  float ksign;
+  const float2* tw;
+  const CoilSamples* tab;
+};
+
 template <int NX, bool TAB = false>
-__global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(
-    const float2* __restrict__ data, int C, int n_rows, int ny, const int32_t* __restrict__ idx,
-    const int32_t* __restrict__ row_ptr, float2* __restrict__ y, int M, float ksign,
-    const float2* __restrict__ tw_g, const CoilSamples* __restrict__ tab) {
+__global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(const float2* __restrict__ data,
+                                                                    float2* __restrict__ y, RowsArgs a) {
+  using F = Rows<NX>;
+  __shared__ float2 buf[kRowWarps][F::kSmem];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  __shared__ float2 tw[NX];
-  __shared__ float2 buf[kRowWarps][padded_len(NX)];
-  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = tw_g[i];
-  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* b = buf[warp];
-  const int total = C * n_rows;
-  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
-    const int c = gr / n_rows, row = gr - c * n_rows;
-    if (TAB) {
-      idx = tab[c].idx;
-      row_ptr = tab[c].row_ptr;
+  const int per = (a.n_list + F::R - 1) / F::R, total = a.C * per;
+  for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
+    const int c = gi / per, j0 = (gi - c * per) * F::R;
+    const int n_list = TAB ? a.tab[c].n_list : a.n_list;
+    const int32_t* list = TAB ? a.tab[c].row_list : a.row_list;
+    const int32_t* idx = TAB ? a.tab[c].idx : a.idx;
+    const int32_t* row_ptr = TAB ? a.tab[c].row_ptr : a.row_ptr;
+    float2* yc = TAB ? a.tab[c].y : y + (size_t)c * a.M;
+    if (j0 >= n_list) continue;  // warp-uniform
+    // the group's rows, their (kz + ky) parities and the range of their samples
+    int row[F::R], rpar[F::R], m0 = 0, m1 = 0;
+#pragma unroll
+    for (int r = 0; r < F::R; ++r) {
+      const bool in = j0 + r < n_list;
+      row[r] = in ? (list ? list[j0 + r] : j0 + r) : 0x7fffffff;
+      rpar[r] = in ? (row[r] / a.ny + row[r] % a.ny) & 1 : 0;
     }
-    float2* yc = TAB ? tab[c].y : y + (size_t)c * M;
-    const int m0 = row_ptr[row], m1 = row_ptr[row + 1];
-    if (m1 <= m0) continue;  // warp-uniform
-    const float2* src = data + ((size_t)c * n_rows + row) * NX;
-    constexpr int PL = (NX + 31) / 32;
-    float2 v[PL];
+    m0 = row_ptr[row[0]];
+    m1 = row_ptr[(list ? list[min(j0 + F::R, n_list) - 1] : min(j0 + F::R, n_list) - 1) + 1];
+    float2 v[F::T1][F::A];
 #pragma unroll
-    for (int u = 0; u < PL; ++u)
-      if (lane + 32 * u < NX) v[u] = src[lane + 32 * u];
+    for (int i = 0; i < F::T1; ++i) {
+      const int j = j0 + (lane + 32 * i) / F::P;
+      if (j < n_list) {
+        const float2* src = data + ((size_t)c * a.n_rows + (list ? list[j] : j)) * NX + lane % F::P;
 #pragma unroll
-    for (int u = 0; u < PL; ++u)
-      if (lane + 32 * u < NX) b[pad8(lane + 32 * u)] = v[u];
+        for (int e = 0; e < F::A; ++e) v[i][e] = src[F::P * e];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < F::T1; ++i) {
+      const int r = (lane + 32 * i) / F::P;
+      if (j0 + r < n_list) F::template step1<false>(v[i], r, lane % F::P, b, a.tw);
+    }
     __syncwarp();
-    Fft<NX, false>::go(b, tw, lane);
-    const int rpar = (row / ny + row % ny) & 1;  // (kz + ky) parity
-    const size_t rbase = (size_t)row * NX;
-    for (int m = m0 + lane; m < m1; m += 32) {
-      const int kx = (int)(idx[m] - rbase);
-      const float sg = ((kx + rpar) & 1) ? -ksign : ksign;
-      const float2 t = b[pad8(kx)];
-      yc[m] = make_float2(t.x * sg, t.y * sg);
+#pragma unroll
+    for (int i = 0; i < F::T2; ++i) {
+      const int t = lane + 32 * i, r = t / F::A, k1 = t % F::A;
+      if (r < F::R && j0 + r < n_list) {
+        float2 u[F::P];
+        F::template step2<false>(u, r, k1, b);
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) b[r * F::S + k1 * (F::P + 1) + k] = u[k];
+      }
     }
-    __syncwarp();  // the buffer is refilled for the next row
+    __syncwarp();
+    F::samples(row, m0, m1, lane, [&](int m) { return idx[m]; }, [](int) { return 0; },
+               [&](int m, int r, int kx, int) {
+      const float sg = ((kx + rpar[r]) & 1) ? -a.ksign : a.ksign;
+      const float2 t = b[F::out_at(r, kx)];
+      yc[m] = make_float2(t.x * sg, t.y * sg);
+    });
+    __syncwarp();  // the buffer is refilled for the next rows
   }
 }
 
 // Adjoint: zero-fill the row from its samples (with the k-side sign), inverse
 // FFT.  Rows without samples are not written: the pass along y that follows
-// reads them as zeros.  Same row striding.
+// reads them as zeros.
 template <int NX, bool TAB = false>
-__global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_inv(
-    const float2* __restrict__ y, int C, int n_rows, int ny, const int32_t* __restrict__ idx,
-    const int32_t* __restrict__ row_ptr, float2* __restrict__ data, int M, float ksign,
-    const float2* __restrict__ tw_g, const CoilSamples* __restrict__ tab) {
+__global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_inv(const float2* __restrict__ y,
+                                                                     float2* __restrict__ data, RowsArgs a) {
+  using F = Rows<NX>;
+  __shared__ float2 buf[kRowWarps][F::kSmem];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  __shared__ float2 tw[NX];
-  __shared__ float2 buf[kRowWarps][padded_len(NX)];
-  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = tw_g[i];
-  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* b = buf[warp];
-  const int total = C * n_rows;
-  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
-    const int c = gr / n_rows, row = gr - c * n_rows;
-    if (TAB) {
-      idx = tab[c].idx;
-      row_ptr = tab[c].row_ptr;
+  const int per = (a.n_list + F::R - 1) / F::R, total = a.C * per;
+  for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
+    const int c = gi / per, j0 = (gi - c * per) * F::R;
+    const int n_list = TAB ? a.tab[c].n_list : a.n_list;
+    const int32_t* list = TAB ? a.tab[c].row_list : a.row_list;
+    const int32_t* idx = TAB ? a.tab[c].idx : a.idx;
+    const int32_t* row_ptr = TAB ? a.tab[c].row_ptr : a.row_ptr;
+    const float2* yc = TAB ? a.tab[c].y : y + (size_t)c * a.M;
+    if (j0 >= n_list) continue;  // warp-uniform
+    // the group's rows, their (kz + ky) parities and the range of their samples
+    int row[F::R], rpar[F::R], m0 = 0, m1 = 0;
+#pragma unroll
+    for (int r = 0; r < F::R; ++r) {
+      const bool in = j0 + r < n_list;
+      row[r] = in ? (list ? list[j0 + r] : j0 + r) : 0x7fffffff;
+      rpar[r] = in ? (row[r] / a.ny + row[r] % a.ny) & 1 : 0;
     }
-    const float2* yc = TAB ? tab[c].y : y + (size_t)c * M;
-    const int m0 = row_ptr[row], m1 = row_ptr[row + 1];
-    float2* dst = data + ((size_t)c * n_rows + row) * NX;
-    if (m1 <= m0) continue;  // warp-uniform
-    for (int i = lane; i < padded_len(NX); i += 32) b[i] = make_float2(0.f, 0.f);
+    m0 = row_ptr[row[0]];
+    m1 = row_ptr[(list ? list[min(j0 + F::R, n_list) - 1] : min(j0 + F::R, n_list) - 1) + 1];
+    for (int i = lane; i < F::kSmem; i += 32) b[i] = make_float2(0.f, 0.f);
     __syncwarp();
-    const int rpar = (row / ny + row % ny) & 1;
-    const size_t rbase = (size_t)row * NX;
-    for (int m = m0 + lane; m < m1; m += 32) {
-      const int kx = (int)(idx[m] - rbase);
-      const float sg = ((kx + rpar) & 1) ? -ksign : ksign;
-      const float2 t = yc[m];
-      b[pad8(kx)] = make_float2(t.x * sg, t.y * sg);
+    F::samples(row, m0, m1, lane, [&](int m) { return idx[m]; }, [&](int m) { return yc[m]; },
+               [&](int, int r, int kx, float2 t) {
+      const float sg = ((kx + rpar[r]) & 1) ? -a.ksign : a.ksign;
+      b[F::in_at(r, kx)] = make_float2(t.x * sg, t.y * sg);
+    });
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < F::T1; ++i) {  // a lane's task reads and writes the same places
+      const int r = (lane + 32 * i) / F::P, p = lane % F::P;
+      float2 v[F::A];
+#pragma unroll
+      for (int e = 0; e < F::A; ++e) v[e] = b[r * F::S + e * (F::P + 1) + p];
+      F::template step1<true>(v, r, p, b, a.tw);
     }
     __syncwarp();
-    Fft<NX, true>::go(b, tw, lane);
-    for (int i = lane; i < NX; i += 32) dst[i] = b[pad8(i)];
+#pragma unroll
+    for (int i = 0; i < F::T2; ++i) {
+      const int t = lane + 32 * i, r = t / F::A, k1 = t % F::A;
+      if (r < F::R && j0 + r < n_list) {
+        float2 u[F::P];
+        F::template step2<true>(u, r, k1, b);
+        float2* dst = data + ((size_t)c * a.n_rows + (list ? list[j0 + r] : j0 + r)) * NX + k1;
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) dst[F::A * k] = u[k];
+      }
+    }
     __syncwarp();
   }
 }
@@ -282,6 +337,7 @@ bool cols_reg_launch(mpi_ctx* ctx, int L, float2* data, int nx, long stride, int
     MPI_CREG(128, 8, 16)
     MPI_CREG(192, 16, 12)
     MPI_CREG(256, 16, 16)
+    MPI_CREG(320, 16, 20)
     default:
       return false;
   }
@@ -427,7 +483,7 @@ int lines_choose(mpi_ctx* ctx, float2* data, int L, int nx, long stride, int n_s
   // a caller's fixed choice (mpi_ctx_set_line_kernel), where this pass has it
   if (ctx->line_kernel) {
     const int t = ctx->line_kernel;
-    const bool ok = t == -1 ? (L == 64 || L == 96 || L == 128 || L == 192 || L == 256) && stride == nx && inner == 1
+    const bool ok = t == -1 ? (L == 64 || L == 96 || L == 128 || L == 192 || L == 256 || L == 320) && stride == nx && inner == 1
                             : (t == 8 || (t == 16 && L <= 256) || (t == 32 && L <= 128));
     if (ok) tile = t;
   }
@@ -1157,22 +1213,27 @@ mpi_status launch_plane_yx(mpi_ctx* ctx, const mpi_plan* plan, float2* data, int
   return set_err(ctx, MPI_ERR_UNSUPPORTED, "plane pass: shape");
 }
 
-mpi_status launch_rows_fwd_gather(mpi_ctx* ctx, const mpi_plan* plan, const float2* data, int C,
-                                  float2* y) {
-  if (plan->M == 0 || C == 0) return MPI_OK;
-  const int n_rows = plan->n_rows;
-  if ((long)C * n_rows > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "too many k-space rows");
-  const long blocks = std::min(((long)C * n_rows + kRowWarps - 1) / kRowWarps, 16L * std::max(ctx->num_sms, 1));
-  const float ks = axis_sign(plan->nx) * axis_sign(plan->ny) * (plan->ndim == 3 ? axis_sign(plan->nz) : 1.f);
-  const float2* tw = twiddle_table(ctx, plan->nx);
-  if (!tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
-#define MPI_ROWS_CASE(n)                                                                          \
-  case n:                                                                                         \
-    launch_pdl(ctx, k_rows_fwd_gather<n>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, data, C, n_rows, \
-               plan->ny, plan->idx, plan->row_ptr, y, plan->M, ks, tw, nullptr);                  \
-    break;
+namespace {
+
+// Launch of the row pass for rows of nx values; y is only read by the scatter.
+template <bool INV, bool TAB>
+mpi_status rows_launch(mpi_ctx* ctx, int nx, float2* data, float2* y, const RowsArgs& a, const char* name) {
+  long groups = 0;
+#define MPI_ROWS_CASE(n)                                                                                           \
+  case n: {                                                                                                        \
+    groups = (long)a.C * ((a.n_list + Rows<n>::R - 1) / Rows<n>::R);                                               \
+    if (groups > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "too many k-space rows");                         \
+    const long blocks = std::min((groups + kRowWarps - 1) / kRowWarps, 16L * std::max(ctx->num_sms, 1));            \
+    if (INV)                                                                                                       \
+      launch_pdl(ctx, k_rows_scatter_inv<n, TAB>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, y, data, a);     \
+    else                                                                                                           \
+      launch_pdl(ctx, k_rows_fwd_gather<n, TAB>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, data, y, a);      \
+    break;                                                                                                         \
+  }
+  if (a.C == 0 || a.n_list == 0) return MPI_OK;
+  if (!a.tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
   MPI_PROF(ctx, KF_FFT_ROWS);
-  switch (plan->nx) {
+  switch (nx) {
     MPI_ROWS_CASE(16)
     MPI_ROWS_CASE(32)
     MPI_ROWS_CASE(48)
@@ -1187,42 +1248,35 @@ mpi_status launch_rows_fwd_gather(mpi_ctx* ctx, const mpi_plan* plan, const floa
       return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
   }
 #undef MPI_ROWS_CASE
-  MPI_LAUNCH_CHECK(ctx, "k_rows_fwd_gather");
+  MPI_LAUNCH_CHECK(ctx, name);
   return MPI_OK;
+}
+
+RowsArgs rows_args(const mpi_ctx* ctx, const mpi_plan* plan, int C) {
+  RowsArgs a{};
+  a.C = C;
+  a.n_rows = plan->n_rows;
+  a.ny = plan->ny;
+  a.M = plan->M;
+  a.n_list = plan->n_list;
+  a.row_list = plan->row_list;
+  a.idx = plan->idx;
+  a.row_ptr = plan->row_ptr;
+  a.ksign = axis_sign(plan->nx) * axis_sign(plan->ny) * (plan->ndim == 3 ? axis_sign(plan->nz) : 1.f);
+  a.tw = twiddle_table(ctx, plan->nx);
+  return a;
+}
+
+}  // namespace
+
+mpi_status launch_rows_fwd_gather(mpi_ctx* ctx, const mpi_plan* plan, const float2* data, int C,
+                                  float2* y) {
+  return rows_launch<false, false>(ctx, plan->nx, (float2*)data, y, rows_args(ctx, plan, C), "k_rows_fwd_gather");
 }
 
 mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, int C,
                                    float2* data) {
-  if (C == 0) return MPI_OK;
-  const int n_rows = plan->n_rows;
-  if ((long)C * n_rows > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "too many k-space rows");
-  const long blocks = std::min(((long)C * n_rows + kRowWarps - 1) / kRowWarps, 16L * std::max(ctx->num_sms, 1));
-  const float ks = axis_sign(plan->nx) * axis_sign(plan->ny) * (plan->ndim == 3 ? axis_sign(plan->nz) : 1.f);
-  const float2* tw = twiddle_table(ctx, plan->nx);
-  if (!tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
-#define MPI_ROWS_CASE(n)                                                                          \
-  case n:                                                                                         \
-    launch_pdl(ctx, k_rows_scatter_inv<n>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, y, C, n_rows, \
-               plan->ny, plan->idx, plan->row_ptr, data, plan->M, ks, tw, nullptr);               \
-    break;
-  MPI_PROF(ctx, KF_FFT_ROWS);
-  switch (plan->nx) {
-    MPI_ROWS_CASE(16)
-    MPI_ROWS_CASE(32)
-    MPI_ROWS_CASE(48)
-    MPI_ROWS_CASE(64)
-    MPI_ROWS_CASE(96)
-    MPI_ROWS_CASE(128)
-    MPI_ROWS_CASE(192)
-    MPI_ROWS_CASE(256)
-    MPI_ROWS_CASE(320)
-    MPI_ROWS_CASE(512)
-    default:
-      return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
-  }
-#undef MPI_ROWS_CASE
-  MPI_LAUNCH_CHECK(ctx, "k_rows_scatter_inv");
-  return MPI_OK;
+  return rows_launch<true, false>(ctx, plan->nx, data, (float2*)y, rows_args(ctx, plan, C), "k_rows_scatter_inv");
 }
 
 // ------------------------------------------------- passes of a batch's group
@@ -1253,85 +1307,74 @@ mpi_status launch_fft_cols_group(mpi_ctx* ctx, int kernel, float2* data, int coi
 }
 
 mpi_status launch_rows_group(mpi_ctx* ctx, float2* data, int coils, int ny, int nx, bool inverse,
-                             const CoilSamples* tab) {
-  if ((long)coils * ny > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "too many k-space rows");
-  const long blocks = std::min(((long)coils * ny + kRowWarps - 1) / kRowWarps, 16L * std::max(ctx->num_sms, 1));
-  const float ks = axis_sign(nx) * axis_sign(ny);
-  const float2* tw = twiddle_table(ctx, nx);
-  if (!tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
-  MPI_PROF(ctx, KF_FFT_ROWS);
-#define MPI_ROWS_CASE(n)                                                                                          \
-  case n:                                                                                                         \
-    if (inverse)                                                                                                  \
-      launch_pdl(ctx, k_rows_scatter_inv<n, true>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, nullptr, coils, \
-                 ny, ny, nullptr, nullptr, data, 0, ks, tw, tab);                                                 \
-    else                                                                                                          \
-      launch_pdl(ctx, k_rows_fwd_gather<n, true>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, data, coils,   \
-                 ny, ny, nullptr, nullptr, nullptr, 0, ks, tw, tab);                                              \
-    break;
-  switch (nx) {
-    MPI_ROWS_CASE(16)
-    MPI_ROWS_CASE(32)
-    MPI_ROWS_CASE(48)
-    MPI_ROWS_CASE(64)
-    MPI_ROWS_CASE(96)
-    MPI_ROWS_CASE(128)
-    MPI_ROWS_CASE(192)
-    MPI_ROWS_CASE(256)
-    MPI_ROWS_CASE(320)
-    MPI_ROWS_CASE(512)
-    default:
-      return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
-  }
-#undef MPI_ROWS_CASE
-  MPI_LAUNCH_CHECK(ctx, inverse ? "k_rows_scatter_inv<group>" : "k_rows_fwd_gather<group>");
-  return MPI_OK;
+                             const CoilSamples* tab, int n_list) {
+  RowsArgs a{};
+  a.C = coils;
+  a.n_rows = a.ny = ny;
+  a.n_list = n_list;
+  a.ksign = axis_sign(nx) * axis_sign(ny);
+  a.tw = twiddle_table(ctx, nx);
+  a.tab = tab;
+  return inverse ? rows_launch<true, true>(ctx, nx, data, nullptr, a, "k_rows_scatter_inv<group>")
+                 : rows_launch<false, true>(ctx, nx, data, nullptr, a, "k_rows_fwd_gather<group>");
 }
 
 namespace {
 
-// In-place FFT of contiguous lines of length L, one warp per line.  Elements
-// outside [load_lo, load_hi) are taken as zero without being read (the radial
-// forward's padded columns), and only [keep_lo, keep_hi) of each transformed
-// line is stored back (the radial adjoint keeps the columns that its cropping
-// pass along y reads).
+// In-place FFT of contiguous lines of length L by the register steps of
+// fft_rows.cuh, R lines per warp.  Elements outside [load_lo, load_hi) are taken
+// as zero without being read (the radial forward's padded columns), and only
+// [keep_lo, keep_hi) of each transformed line is stored back (the radial adjoint
+// keeps the columns that its cropping pass along y reads).
 template <int L, bool INV>
 __global__ void __launch_bounds__(kRowWarps * 32) k_fft_rows_inplace(float2* __restrict__ data, long n_rows,
                                                                     const float2* __restrict__ tw_g, int load_lo,
                                                                     int load_hi, int keep_lo, int keep_hi) {
+  using F = Rows<L>;
+  __shared__ float2 buf[kRowWarps][F::kSmem];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  __shared__ float2 tw[L];
-  __shared__ float2 buf[kRowWarps][padded_len(L)];
-  for (int i = threadIdx.x; i < L; i += blockDim.x) tw[i] = tw_g[i];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long row = (long)blockIdx.x * kRowWarps + warp;
-  float2* src = data + (size_t)(row < n_rows ? row : 0) * L;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
   float2* b = buf[warp];
-  if (row < n_rows) {
+  const long row0 = ((long)blockIdx.x * kRowWarps + warp) * F::R;
+  float2 v[F::T1][F::A];
 #pragma unroll
-    for (int i = lane; i < L; i += 32)
-      b[pad8(i)] = (i >= load_lo && i < load_hi) ? src[i] : make_float2(0.f, 0.f);
+  for (int i = 0; i < F::T1; ++i) {
+    const long row = row0 + (lane + 32 * i) / F::P;
+    const float2* src = data + (size_t)row * L;
+#pragma unroll
+    for (int e = 0; e < F::A; ++e) {
+      const int n = p + F::P * e;
+      v[i][e] = (row < n_rows && n >= load_lo && n < load_hi) ? src[n] : make_float2(0.f, 0.f);
+    }
   }
-  __syncthreads();
-  if (row >= n_rows) return;
-  Fft<L, INV>::go(b, tw, lane);
 #pragma unroll
-  for (int i = lane; i < L; i += 32)
-    if (i >= keep_lo && i < keep_hi) src[i] = b[pad8(i)];
+  for (int i = 0; i < F::T1; ++i) F::template step1<INV>(v[i], (lane + 32 * i) / F::P, p, b, tw_g);
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < F::T2; ++i) {
+    const int t = lane + 32 * i, r = t / F::A, k1 = t % F::A;
+    if (r >= F::R || row0 + r >= n_rows) continue;
+    float2 u[F::P];
+    F::template step2<INV>(u, r, k1, b);
+    float2* dst = data + (size_t)(row0 + r) * L;
+#pragma unroll
+    for (int k = 0; k < F::P; ++k)
+      if (k1 + F::A * k >= keep_lo && k1 + F::A * k < keep_hi) dst[k1 + F::A * k] = u[k];
+  }
 }
 
 template <bool INV>
 mpi_status rows_inplace_dispatch(mpi_ctx* ctx, float2* data, long n_rows, int L, int load_lo, int load_hi,
                                  int keep_lo, int keep_hi) {
-  const long blocks = (n_rows + kRowWarps - 1) / kRowWarps;
-  if (blocks == 0) return MPI_OK;
+  if (n_rows == 0) return MPI_OK;
   const float2* tw = twiddle_table(ctx, L);
   if (!tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
-#define MPI_RI_CASE(n)                                                                           \
-  case n:                                                                                        \
-    launch_pdl(ctx, k_fft_rows_inplace<n, INV>, dim3((unsigned)blocks), dim3(kRowWarps * 32), 0, data, n_rows, \
-               tw, load_lo, load_hi, keep_lo, keep_hi);                                           \
+#define MPI_RI_CASE(n)                                                                                         \
+  case n:                                                                                                      \
+    launch_pdl(ctx, k_fft_rows_inplace<n, INV>,                                                                \
+               dim3((unsigned)((n_rows + kRowWarps * Rows<n>::R - 1) / (kRowWarps * Rows<n>::R))),             \
+               dim3(kRowWarps * 32), 0, data, n_rows, tw, load_lo, load_hi, keep_lo, keep_hi);                 \
     break;
   MPI_PROF(ctx, KF_FFT_ROWS);
   switch (L) {

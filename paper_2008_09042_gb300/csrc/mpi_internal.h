@@ -89,6 +89,8 @@ struct mpi_plan {
   int32_t* row_ptr = nullptr;
   uint8_t* row_has = nullptr;  // [n_rows]: 1 where the k-space row has samples; null when every row has some
   int n_rows = 0;
+  int32_t* row_list = nullptr;  // [n_list] the k-space rows with samples; null when every row has some
+  int n_list = 0;
   // 3D: per kz plane, its k-space rows with samples in order of ky:
   // plane_rows [nz][max(plane_kmax, 1)] = {ky, first sample, end of samples, 0}
   // (unused entries ky = -1), plane_nrows [nz] their number, plane_slot
@@ -425,13 +427,15 @@ mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const flo
 struct CoilSamples {
   const int32_t* idx;
   const int32_t* row_ptr;
+  const int32_t* row_list;  // the coil's rows with samples (null: every row) and their number
+  int n_list;
   float2* y;  // the coil's samples
 };
 int fft_cols_kernel(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse);
 mpi_status launch_fft_cols_group(mpi_ctx* ctx, int kernel, float2* data, int coils, int ny, int nx, bool inverse,
                                  const uint8_t* row_has);
 mpi_status launch_rows_group(mpi_ctx* ctx, float2* data, int coils, int ny, int nx, bool inverse,
-                             const CoilSamples* tab);
+                             const CoilSamples* tab, int n_list);
 
 // ------------------------------------------------------------- NUFFT (radial)
 
