@@ -23,10 +23,10 @@
 //   The CG starts from the previous p, whose F_s S p is at hand (Apk), so its first
 // residual is one adjoint:  r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p.
 //   rho's rescaling of the scaled duals is applied where they are read (ufac).
-//   Reductions: FP64 partial sums per CTA; the last CTA to arrive adds them in a
-// fixed order, so results do not depend on which one that is.
+//   Reductions: partial sums per CTA, added in a fixed order by the kernels that use
+// them, so results do not depend on the order the CTAs run in.
 // At 256^2, 16 coils, q = 128 an outer step (5 CG, 10 TV iterations) went from 725
-// to ~150 us, in 37 launches instead of 124.
+// to 245 us, in 33 launches instead of 124.
 #include <math.h>
 
 #include <algorithm>
@@ -34,6 +34,7 @@
 
 #include "admm.h"
 #include "dft_reg.cuh"
+#include "fft_rows.cuh"
 #include "fft_tile.cuh"
 #include "ptx.cuh"
 
@@ -43,59 +44,110 @@ using namespace mpi_fft;
 
 constexpr int kThreads = 256;      // column and reduction kernels
 constexpr int kElemThreads = 256;  // element-wise kernels
-constexpr int kMaxElemBlocks = 1024;
+constexpr int kMaxElemBlocks = 512;  // also the partial sums that a consumer adds
 constexpr int kBallBlocks = 8;     // CTAs per coil of the ball norms
 
 // device scalars
-enum { S_RR = 0, S_A, S_BETA, S_RHO, S_UFAC, S_NUM };
+enum { S_RHO = 0, S_UFAC, S_NUM };
 
 // ------------------------------------------------------------- reductions
+//
+// Sums are kept as pairs of FP32 values (h + l, about 48 bits) of exact differences
+// and products, from the threads to the partial sums: this GPU does two FP64
+// operations per clock and SM, and the fourteen per sample of the data blocks'
+// residuals took longer than everything else in their pass.
 
+struct Sum2 {
+  float h = 0.f, l = 0.f;
+};
+
+// s += p + e, e a small correction of p
+__device__ __forceinline__ void sum2_add(Sum2& s, float p, float e) {
+  const float t = s.h + p, z = t - s.h;
+  s.l += ((s.h - (t - z)) + (p - z)) + e;
+  s.h = t;
+}
+// s += a b
+__device__ __forceinline__ void sum2_mul(Sum2& s, float a, float b) {
+  const float p = a * b;
+  sum2_add(s, p, fmaf(a, b, -p));
+}
+// s += (d + e)^2, e a small correction of d
+__device__ __forceinline__ void sum2_sq(Sum2& s, float d, float e) {
+  const float p = d * d;
+  sum2_add(s, p, fmaf(2.f * d, e, fmaf(d, d, -p)));
+}
+// d + e = a - b exactly
+__device__ __forceinline__ float diff_exact(float a, float b, float& e) {
+  const float d = a - b, t = d - a;
+  e = (a - (d - t)) - (b + t);
+  return d;
+}
+__device__ __forceinline__ void sum2_diff_sq(Sum2& s, float2 a, float2 b) {
+  float e;
+  float d = diff_exact(a.x, b.x, e);
+  sum2_sq(s, d, e);
+  d = diff_exact(a.y, b.y, e);
+  sum2_sq(s, d, e);
+}
+
+// Sum over a warp (valid in every lane).
+__device__ __forceinline__ Sum2 warp_sum(Sum2 s) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, s.h, o), l = __shfl_xor_sync(0xffffffffu, s.l, o);
+    // the lower lane's sum first in both lanes, so that all lanes agree
+    const bool up = threadIdx.x & o;
+    Sum2 a;
+    a.h = up ? h : s.h;
+    a.l = up ? l : s.l;
+    sum2_add(a, up ? s.h : h, up ? s.l : l);
+    s = a;
+  }
+  return s;
+}
+
+__device__ __forceinline__ float2 pack(Sum2 s) { return make_float2(s.h, s.l); }
+__device__ __forceinline__ double to_double(Sum2 s) { return (double)s.h + (double)s.l; }
+
+// Sums over the CTA (valid in thread 0); sh holds NV values per warp.
 template <int NV>
-__device__ __forceinline__ void block_sums(double (&v)[NV], double* sh) {
-#pragma unroll
-  for (int j = 0; j < NV; ++j)
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
+__device__ __forceinline__ void block_sums(const Sum2 (&v)[NV], float2* sh, Sum2 (&out)[NV]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0)
 #pragma unroll
-    for (int j = 0; j < NV; ++j) sh[warp * NV + j] = v[j];
+  for (int j = 0; j < NV; ++j) {
+    const Sum2 w = warp_sum(v[j]);
+    if (lane == 0) sh[warp * NV + j] = pack(w);
+  }
   __syncthreads();
   if (threadIdx.x == 0)
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
-      double s = 0.0;
-      for (int w = 0; w < nw; ++w) s += sh[w * NV + j];
-      v[j] = s;
+      Sum2 s;
+      for (int w = 0; w < nw; ++w) sum2_add(s, sh[w * NV + j].x, sh[w * NV + j].y);
+      out[j] = s;
     }
 }
 
-// Sums of v over the `nblk` CTAs that share `partials` and `counter` (zero before,
-// zero after); true in every thread of the last CTA to arrive, where thread 0's v
-// then holds the sums.  `blk`: this CTA's place among them.
-template <int NV>
-__device__ __forceinline__ bool group_sums(double (&v)[NV], double* partials, unsigned* counter, int blk, int nblk,
-                                           double* sh) {
-  __shared__ int last;
-  block_sums(v, sh);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) partials[(size_t)blk * NV + j] = v[j];
-    __threadfence();
-    last = atomicAdd(counter, 1u) == (unsigned)nblk - 1;
-    if (last) *counter = 0;
+// a / b to FP32 accuracy (0 where b <= 0), with the pairs' low parts.
+__device__ __forceinline__ float pair_ratio(Sum2 a, Sum2 b) {
+  const float bh = b.h + b.l, bl = b.l - (bh - b.h), ah = a.h + a.l, al = a.l - (ah - a.h);
+  if (!(bh > 0.f)) return 0.f;
+  const float q = ah / bh;
+  return q + (fmaf(-q, bh, ah) + fmaf(-q, bl, al)) / bh;
+}
+
+// The sum of n partial sums, by one warp in a fixed order (valid in every lane):
+// the kernels that use a reduction's result add its CTAs' partial sums themselves,
+// which is faster than having the last CTA of the reduction do it (its fence,
+// counter and second round trip were 3 us at the end of every such kernel).
+__device__ __forceinline__ Sum2 partial_sum(const float2* __restrict__ part, int n) {
+  Sum2 s;
+  for (int i = threadIdx.x & 31; i < n; i += 32) {
+    const float2 v = part[i];
+    sum2_add(s, v.x, v.y);
   }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    v[j] = 0.0;
-    for (int i = threadIdx.x; i < nblk; i += blockDim.x) v[j] += __ldcg(partials + (size_t)i * NV + j);
-  }
-  block_sums(v, sh);
-  return true;
+  return warp_sum(s);
 }
 
 // ------------------------------------------------------------ column passes
@@ -106,7 +158,8 @@ struct MapsCols {
   const float2* v;      // forward: image [T][N], or the CG's old direction
   const float2* r;      // forward, next CG direction d = r + beta d_old (null: v itself)
   float2* dnew;         // where that direction goes
-  const double* sc;
+  const float2 *rr, *rr_old;  // partial sums of |r|^2, now and before the last update: beta = rr / rr_old
+  int n_part;
   int C, nx;
   size_t N;
   float scale;
@@ -133,8 +186,8 @@ constexpr int maps_cols_tile(int L) { return (L == 64 || L == 96 || L == 128 || 
 // turn, with the store of the new direction between them: 30 us per pass at
 // 256^2 and 16 coils; batched: see the file header).
 template <int R, bool INV>
-__device__ __forceinline__ void maps_load(const MapsCols& a, int t, int c, int tc, int y0, int step, int x, int L,
-                                          float2 (&u)[R]) {
+__device__ __forceinline__ void maps_load(const MapsCols& a, float beta, int t, int c, int tc, int y0, int step,
+                                          int x, int L, float2 (&u)[R]) {
   const size_t n0 = (size_t)y0 * a.nx + x, ns = (size_t)step * a.nx;
   if (INV) {
     const float2* W = a.W + (size_t)tc * a.N + n0;
@@ -155,7 +208,6 @@ __device__ __forceinline__ void maps_load(const MapsCols& a, int t, int c, int t
   for (int m = 0; m < R; ++m) s[m] = S[ns * m];
   if (a.r) {  // the CG's next direction, kept by the first coil's CTAs
     const float2* r = a.r + (size_t)t * a.N + n0;
-    const float beta = (float)a.sc[S_BETA];
     float2 rv[R];
 #pragma unroll
     for (int m = 0; m < R; ++m) rv[m] = r[ns * m];
@@ -213,6 +265,11 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
   const int tc = (int)blockIdx.x / x_tiles, x0 = ((int)blockIdx.x - tc * x_tiles) * TILE;
   const int t = tc / a.C, c = tc - t * a.C;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  float beta = 0.f;
+  if (!INV && a.r) {  // every warp adds the partial sums (a few per lane, L2 hits)
+    const Sum2 rr = partial_sum(a.rr, a.n_part), old = partial_sum(a.rr_old, a.n_part);
+    beta = pair_ratio(rr, old);
+  }
   if constexpr (R1 > 0) {
     __shared__ float2 sY[L * 32];  // [k1][r][column]
     __shared__ float2 tw[L];
@@ -223,7 +280,7 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
 #pragma unroll
     for (int it = 0; it < (R2 + 7) / 8; ++it) {
       const int q = w + 8 * it;
-      if (ok && q < R2) maps_load<R1, INV>(a, t, c, tc, q, R2, x, L, u1[it]);
+      if (ok && q < R2) maps_load<R1, INV>(a, beta, t, c, tc, q, R2, x, L, u1[it]);
     }
     __syncthreads();
 #pragma unroll
@@ -273,10 +330,10 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
     if (ok) {
       if constexpr (PER > 1) {
         float2 (&v1)[PER - 1] = reinterpret_cast<float2 (&)[PER - 1]>(v);
-        maps_load<PER - 1, INV>(a, t, c, tc, r0, RSTEP, x, L, v1);
+        maps_load<PER - 1, INV>(a, beta, t, c, tc, r0, RSTEP, x, L, v1);
       }
       if (all) {
-        maps_load<1, INV>(a, t, c, tc, r0 + RSTEP * (PER - 1), RSTEP, x, L, e);
+        maps_load<1, INV>(a, beta, t, c, tc, r0 + RSTEP * (PER - 1), RSTEP, x, L, e);
         v[PER - 1] = e[0];
       }
     }
@@ -306,7 +363,9 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
 struct MapsRows {
   float2* W;                 // [T][C][ny][NX]
   int TC, C, ny, M;
-  const uint8_t* rmask;      // [T][ny]
+  const int32_t* row_list;   // [T][ny] rows with samples
+  const int32_t* n_list;     // [T] their number
+  int n_list_max;
   const uint8_t* mask;       // [T][ny][NX]
   const int32_t* idx;        // [T][M]
   const int32_t* row_ptr;    // [T][ny + 1]
@@ -314,49 +373,95 @@ struct MapsRows {
   float ksign;
   const float2* y;           // data [T][C][M]
   float2 *ap, *uk, *zk;      // F_s S p, the scaled duals, the projections [T][C][M]
-  const double* f;           // ball factors [T][C]
+  const float2* ball;        // partial sums of the ball norms [T][C][kBallBlocks]
+  const double* eps;         // ball radii [T][C]
   const double* sc;
-  double* partials;
+  float2* partials;
+};
+
+// One sample's F_s S p, scaled dual and datum or projection.
+struct Sample {
+  float2 ap, uk, yz;
 };
 
 // The normal operator in k-space: F_x, mask, F_x^H of every row with samples.
 template <int NX>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_normal(MapsRows a) {
-  __shared__ float2 tw[NX];
-  __shared__ float2 buf[kRowWarps][padded_len(NX)];
+  using F = Rows<NX>;
+  __shared__ float2 buf[kRowWarps][F::kSmem];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = a.tw[i];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
   float2* b = buf[warp];
-  const int total = a.TC * a.ny;
-  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
-    const int tc = gr / a.ny, row = gr - tc * a.ny, t = tc / a.C;
-    if (!a.rmask[(size_t)t * a.ny + row]) continue;  // warp-uniform
-    float2* src = a.W + (size_t)gr * NX;
-    const uint8_t* mk = a.mask + ((size_t)t * a.ny + row) * NX;
-    constexpr int PL = (NX + 31) / 32;
-    float2 v[PL];
-    uint8_t keep[PL];
+  const int per = (a.n_list_max + F::R - 1) / F::R, total = a.TC * per;
+  for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
+    const int tc = gi / per, j0 = (gi - tc * per) * F::R, t = tc / a.C;
+    const int n_list = a.n_list[t];
+    if (j0 >= n_list) continue;  // warp-uniform
+    const int32_t* list = a.row_list + (size_t)t * a.ny;
+    float2* W = a.W + (size_t)tc * a.ny * NX;
+    float2 v[F::T1][F::A];
 #pragma unroll
-    for (int u = 0; u < PL; ++u)
-      if (lane + 32 * u < NX) {
-        v[u] = src[lane + 32 * u];
-        keep[u] = mk[lane + 32 * u];
+    for (int i = 0; i < F::T1; ++i) {
+      const int j = j0 + (lane + 32 * i) / F::P;
+      if (j < n_list) {
+        const float2* src = W + (size_t)list[j] * NX + p;
+#pragma unroll
+        for (int e = 0; e < F::A; ++e) v[i][e] = src[F::P * e];
       }
+    }
 #pragma unroll
-    for (int u = 0; u < PL; ++u)
-      if (lane + 32 * u < NX) b[pad8(lane + 32 * u)] = v[u];
+    for (int i = 0; i < F::T1; ++i) {
+      const int r = (lane + 32 * i) / F::P;
+      if (j0 + r < n_list) F::template step1<false>(v[i], r, p, b, a.tw);
+    }
     __syncwarp();
-    Fft<NX, false>::go(b, tw, lane);
+    float2 u[F::T2][F::P];
 #pragma unroll
-    for (int u = 0; u < PL; ++u)
-      if (lane + 32 * u < NX && !keep[u]) b[pad8(lane + 32 * u)] = make_float2(0.f, 0.f);
+    for (int i = 0; i < F::T2; ++i) {
+      const int q = lane + 32 * i, r = q / F::A, k1 = q % F::A;
+      if (r < F::R && j0 + r < n_list) {
+        const uint8_t* mk = a.mask + ((size_t)t * a.ny + list[j0 + r]) * NX + k1;
+        uint8_t keep[F::P];
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) keep[k] = mk[F::A * k];
+        F::template step2<false>(u[i], r, k1, b);
+#pragma unroll
+        for (int k = 0; k < F::P; ++k)
+          if (!keep[k]) u[i][k] = make_float2(0.f, 0.f);
+      }
+    }
+    __syncwarp();  // every output is out of the exchange: back in as the inverse's input
+#pragma unroll
+    for (int i = 0; i < F::T2; ++i) {
+      const int q = lane + 32 * i, r = q / F::A, k1 = q % F::A;
+      if (r < F::R && j0 + r < n_list) {
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) b[F::in_at(r, k1 + F::A * k)] = u[i][k];
+      }
+    }
     __syncwarp();
-    Fft<NX, true>::go(b, tw, lane);
-    for (int i = lane; i < NX; i += 32) src[i] = b[pad8(i)];
-    __syncwarp();  // the buffer is refilled for the next row
+#pragma unroll
+    for (int i = 0; i < F::T1; ++i) {
+      const int r = (lane + 32 * i) / F::P;
+      if (j0 + r < n_list) {
+#pragma unroll
+        for (int e = 0; e < F::A; ++e) v[i][e] = b[r * F::S + e * (F::P + 1) + p];
+        F::template step1<true>(v[i], r, p, b, a.tw);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < F::T2; ++i) {
+      const int q = lane + 32 * i, r = q / F::A, k1 = q % F::A;
+      if (r < F::R && j0 + r < n_list) {
+        F::template step2<true>(u[i], r, k1, b);
+        float2* dst = W + (size_t)list[j0 + r] * NX + k1;
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) dst[F::A * k] = u[i][k];
+      }
+    }
+    __syncwarp();  // the buffer is refilled for the next rows
   }
 }
 
@@ -364,38 +469,74 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_normal(MapsRows a) {
 // rows of z_k - u_k - F_s S p through the inverse DFT along x.
 template <int NX>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_ball(MapsRows a) {
-  __shared__ float2 tw[NX];
-  __shared__ float2 buf[kRowWarps][padded_len(NX)];
+  using F = Rows<NX>;
+  __shared__ float2 buf[kRowWarps][F::kSmem];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = a.tw[i];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
   const float fu = (float)a.sc[S_UFAC];
   float2* b = buf[warp];
-  const int total = a.TC * a.ny;
-  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
-    const int tc = gr / a.ny, row = gr - tc * a.ny, t = tc / a.C;
-    const int32_t* rp = a.row_ptr + (size_t)t * (a.ny + 1) + row;
-    const int m0 = rp[0], m1 = rp[1];
-    if (m1 <= m0) continue;  // warp-uniform
-    const float fc = (float)a.f[tc];
-    for (int i = lane; i < padded_len(NX); i += 32) b[i] = make_float2(0.f, 0.f);
+  const int per = (a.n_list_max + F::R - 1) / F::R, total = a.TC * per;
+  for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
+    const int tc = gi / per, j0 = (gi - tc * per) * F::R, t = tc / a.C;
+    const int n_list = a.n_list[t];
+    if (j0 >= n_list) continue;  // warp-uniform
+    const int32_t* list = a.row_list + (size_t)t * a.ny;
+    // f = eps / max(|.|, eps): the root and the quotient corrected by their residues,
+    // so that FP32 arithmetic gives the FP64 value's rounding
+    Sum2 nrm;
+#pragma unroll
+    for (int i = 0; i < kBallBlocks; ++i) {
+      const float2 v = a.ball[(size_t)tc * kBallBlocks + i];
+      sum2_add(nrm, v.x, v.y);
+    }
+    const double eps = a.eps[tc];
+    Sum2 root, radius;
+    root.h = sqrtf(nrm.h);
+    root.l = root.h > 0.f ? 0.5f * (fmaf(-root.h, root.h, nrm.h) + nrm.l) / root.h : 0.f;
+    radius.h = (float)eps;
+    radius.l = (float)(eps - radius.h);
+    const float fc = root.h > radius.h ? pair_ratio(radius, root) : 1.f;
+    for (int i = lane; i < F::kSmem; i += 32) b[i] = make_float2(0.f, 0.f);
     __syncwarp();
-    for (int m = m0 + lane; m < m1; m += 32) {
-      const int kx = a.idx[(size_t)t * a.M + m] - row * NX;
-      const float sg = ((kx + row) & 1) ? -a.ksign : a.ksign;
-      const size_t i = (size_t)tc * a.M + m;
-      const float2 ap = a.ap[i], u0 = a.uk[i], yv = a.y[i];
-      const float2 u = make_float2(fu * u0.x, fu * u0.y);
-      const float2 z = make_float2(yv.x + fc * (ap.x + u.x - yv.x), yv.y + fc * (ap.y + u.y - yv.y));
-      a.zk[i] = z;
-      b[pad8(kx)] = make_float2((z.x - u.x - ap.x) * sg, (z.y - u.y - ap.y) * sg);
+    int row[F::R];  // the group's rows and the range of their samples
+#pragma unroll
+    for (int r = 0; r < F::R; ++r) row[r] = j0 + r < n_list ? list[j0 + r] : 0x7fffffff;
+    const int32_t* rp = a.row_ptr + (size_t)t * (a.ny + 1);
+    const int m0 = rp[row[0]], m1 = rp[list[min(j0 + F::R, n_list) - 1] + 1];
+    const int32_t* idx = a.idx + (size_t)t * a.M;
+    const size_t i0 = (size_t)tc * a.M;
+    F::samples(
+        row, m0, m1, lane, [&](int m) { return idx[m]; },
+        [&](int m) { return Sample{a.ap[i0 + m], a.uk[i0 + m], a.y[i0 + m]}; },
+        [&](int m, int r, int kx, const Sample& d) {
+          const float sg = ((kx + row[r]) & 1) ? -a.ksign : a.ksign;
+          const float2 u = make_float2(fu * d.uk.x, fu * d.uk.y);
+          const float2 z = make_float2(d.yz.x + fc * (d.ap.x + u.x - d.yz.x), d.yz.y + fc * (d.ap.y + u.y - d.yz.y));
+          a.zk[i0 + m] = z;
+          b[F::in_at(r, kx)] = make_float2((z.x - u.x - d.ap.x) * sg, (z.y - u.y - d.ap.y) * sg);
+        });
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < F::T1; ++i) {
+      const int r = (lane + 32 * i) / F::P;
+      float2 v[F::A];
+#pragma unroll
+      for (int e = 0; e < F::A; ++e) v[e] = b[r * F::S + e * (F::P + 1) + p];
+      F::template step1<true>(v, r, p, b, a.tw);
     }
     __syncwarp();
-    Fft<NX, true>::go(b, tw, lane);
-    float2* dst = a.W + (size_t)gr * NX;
-    for (int i = lane; i < NX; i += 32) dst[i] = b[pad8(i)];
+#pragma unroll
+    for (int i = 0; i < F::T2; ++i) {
+      const int q = lane + 32 * i, r = q / F::A, k1 = q % F::A;
+      if (r < F::R && j0 + r < n_list) {
+        float2 u[F::P];
+        F::template step2<true>(u, r, k1, b);
+        float2* dst = a.W + ((size_t)tc * a.ny + list[j0 + r]) * NX + k1;
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) dst[F::A * k] = u[k];
+      }
+    }
     __syncwarp();
   }
 }
@@ -404,48 +545,75 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_ball(MapsRows a
 // u_k += F_s S p - z_k; per CTA the sums |F_s S p - z_k|^2 and |F_s S (p - p_prev)|^2.
 template <int NX>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_gather_dual(MapsRows a) {
-  __shared__ float2 tw[NX];
-  __shared__ float2 buf[kRowWarps][padded_len(NX)];
-  __shared__ double sh[2 * kRowWarps];
+  using F = Rows<NX>;
+  __shared__ float2 buf[kRowWarps][F::kSmem];
+  __shared__ float2 sh[2 * kRowWarps];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  for (int i = threadIdx.x; i < NX; i += blockDim.x) tw[i] = a.tw[i];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
   const float fu = (float)a.sc[S_UFAC];
   float2* b = buf[warp];
-  double sums[2] = {0.0, 0.0};
-  const int total = a.TC * a.ny;
-  for (int gr = blockIdx.x * kRowWarps + warp; gr < total; gr += gridDim.x * kRowWarps) {
-    const int tc = gr / a.ny, row = gr - tc * a.ny, t = tc / a.C;
-    const int32_t* rp = a.row_ptr + (size_t)t * (a.ny + 1) + row;
-    const int m0 = rp[0], m1 = rp[1];
-    if (m1 <= m0) continue;  // warp-uniform
-    const float2* src = a.W + (size_t)gr * NX;
-    for (int i = lane; i < NX; i += 32) b[pad8(i)] = src[i];
-    __syncwarp();
-    Fft<NX, false>::go(b, tw, lane);
-    for (int m = m0 + lane; m < m1; m += 32) {
-      const int kx = a.idx[(size_t)t * a.M + m] - row * NX;
-      const float sg = ((kx + row) & 1) ? -a.ksign : a.ksign;
-      const size_t i = (size_t)tc * a.M + m;
-      const float2 e = b[pad8(kx)], old = a.ap[i], z = a.zk[i];
-      const float2 ap = make_float2(e.x * sg, e.y * sg);
-      float2 u = a.uk[i];
-      u = make_float2(fu * u.x + ap.x - z.x, fu * u.y + ap.y - z.y);
-      a.ap[i] = ap;
-      a.uk[i] = u;
-      const double rx = (double)ap.x - z.x, ry = (double)ap.y - z.y;
-      const double sx = (double)ap.x - old.x, sy = (double)ap.y - old.y;
-      sums[0] += rx * rx + ry * ry;
-      sums[1] += sx * sx + sy * sy;
+  Sum2 sums[2];
+  const int per = (a.n_list_max + F::R - 1) / F::R, total = a.TC * per;
+  for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
+    const int tc = gi / per, j0 = (gi - tc * per) * F::R, t = tc / a.C;
+    const int n_list = a.n_list[t];
+    if (j0 >= n_list) continue;  // warp-uniform
+    const int32_t* list = a.row_list + (size_t)t * a.ny;
+    const float2* W = a.W + (size_t)tc * a.ny * NX;
+    float2 v[F::T1][F::A];
+#pragma unroll
+    for (int i = 0; i < F::T1; ++i) {
+      const int j = j0 + (lane + 32 * i) / F::P;
+      if (j < n_list) {
+        const float2* src = W + (size_t)list[j] * NX + p;
+#pragma unroll
+        for (int e = 0; e < F::A; ++e) v[i][e] = src[F::P * e];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < F::T1; ++i) {
+      const int r = (lane + 32 * i) / F::P;
+      if (j0 + r < n_list) F::template step1<false>(v[i], r, p, b, a.tw);
     }
     __syncwarp();
+#pragma unroll
+    for (int i = 0; i < F::T2; ++i) {
+      const int q = lane + 32 * i, r = q / F::A, k1 = q % F::A;
+      if (r < F::R && j0 + r < n_list) {
+        float2 u[F::P];
+        F::template step2<false>(u, r, k1, b);
+#pragma unroll
+        for (int k = 0; k < F::P; ++k) b[r * F::S + k1 * (F::P + 1) + k] = u[k];
+      }
+    }
+    __syncwarp();
+    int row[F::R];  // the group's rows and the range of their samples
+#pragma unroll
+    for (int r = 0; r < F::R; ++r) row[r] = j0 + r < n_list ? list[j0 + r] : 0x7fffffff;
+    const int32_t* rp = a.row_ptr + (size_t)t * (a.ny + 1);
+    const int m0 = rp[row[0]], m1 = rp[list[min(j0 + F::R, n_list) - 1] + 1];
+    const int32_t* idx = a.idx + (size_t)t * a.M;
+    const size_t i0 = (size_t)tc * a.M;
+    F::samples(
+        row, m0, m1, lane, [&](int m) { return idx[m]; },
+        [&](int m) { return Sample{a.ap[i0 + m], a.uk[i0 + m], a.zk[i0 + m]}; },
+        [&](int m, int r, int kx, const Sample& d) {
+          const float sg = ((kx + row[r]) & 1) ? -a.ksign : a.ksign;
+          const float2 e = b[F::out_at(r, kx)];
+          const float2 ap = make_float2(e.x * sg, e.y * sg);
+          a.ap[i0 + m] = ap;
+          a.uk[i0 + m] = make_float2(fu * d.uk.x + ap.x - d.yz.x, fu * d.uk.y + ap.y - d.yz.y);
+          sum2_diff_sq(sums[0], ap, d.yz);
+          sum2_diff_sq(sums[1], ap, d.ap);
+        });
+    __syncwarp();
   }
-  block_sums(sums, sh);
+  Sum2 out[2];
+  block_sums(sums, sh, out);
   if (threadIdx.x == 0) {
-    a.partials[2 * (size_t)blockIdx.x] = sums[0];
-    a.partials[2 * (size_t)blockIdx.x + 1] = sums[1];
+    a.partials[2 * (size_t)blockIdx.x] = pack(out[0]);
+    a.partials[2 * (size_t)blockIdx.x + 1] = pack(out[1]);
   }
 }
 
@@ -459,19 +627,19 @@ struct CoilSum {
   float2 *d, *Ad;                        // normal: A d = sum + d
   const float2 *z0, *u0, *p;             // residual: sum + z0 - ufac u0 - p
   float2 *r, *p_prev;                    //   into r and d; p kept as p_prev
-  double *sc, *partials;
-  unsigned* counter;
+  const double* sc;
+  float2* partials;  // per CTA: normal, <d, A d>; residual, |r|^2
 };
 
-// sum over coils of conj(s_k) w_k with sign and scale.  NORMAL: A d and the CG
-// step a = |r|^2 / <d, A d>; else the CG's first residual and |r|^2.
+// sum over coils of conj(s_k) w_k with sign and scale.  NORMAL: A d and <d, A d>;
+// else the CG's first residual and |r|^2.
 template <bool NORMAL>
 __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
-  __shared__ double sh[kElemThreads / 32];
+  __shared__ float2 sh[kElemThreads / 32];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const float fu = NORMAL ? 1.f : (float)a.sc[S_UFAC];
-  double s[1] = {0.0};
+  Sum2 s[1];
   for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < a.total; i += (size_t)gridDim.x * kElemThreads) {
     const size_t t = i / a.N, n = i - t * a.N;
     const float2* w = a.W + t * a.C * a.N + n;
@@ -499,103 +667,143 @@ __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
       const float2 d = a.d[i];
       o = make_float2(o.x + d.x, o.y + d.y);
       a.Ad[i] = o;
-      s[0] += (double)d.x * o.x + (double)d.y * o.y;
+      sum2_mul(s[0], d.x, o.x);
+      sum2_mul(s[0], d.y, o.y);
     } else {
       const float2 z = a.z0[i], u = a.u0[i], p = a.p[i];
       o = make_float2(o.x + z.x - fu * u.x - p.x, o.y + z.y - fu * u.y - p.y);
       a.r[i] = o;
       a.d[i] = o;
       a.p_prev[i] = p;
-      s[0] += (double)o.x * o.x + (double)o.y * o.y;
+      sum2_mul(s[0], o.x, o.x);
+      sum2_mul(s[0], o.y, o.y);
     }
   }
-  if (!group_sums(s, a.partials, a.counter, (int)blockIdx.x, (int)gridDim.x, sh) || threadIdx.x) return;
-  if (NORMAL)
-    a.sc[S_A] = s[0] > 0.0 ? a.sc[S_RR] / s[0] : 0.0;
-  else
-    a.sc[S_RR] = s[0];
+  Sum2 out[1];
+  block_sums(s, sh, out);
+  if (threadIdx.x == 0) a.partials[blockIdx.x] = pack(out[0]);
 }
 
-// x += a d, r -= a A d, and beta = |r|^2 / |r_old|^2.
+// x += a d, r -= a A d with a = |r|^2 / <d, A d>, and the new |r|^2 (partial sums in
+// and out; rr and rr_new are different buffers).
 __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__ x, float2* __restrict__ r,
                                                             const float2* __restrict__ d,
-                                                            const float2* __restrict__ Ad, size_t n, double* sc,
-                                                            double* partials, unsigned* counter) {
-  __shared__ double sh[kElemThreads / 32];
+                                                            const float2* __restrict__ Ad, size_t n,
+                                                            const float2* __restrict__ rr,
+                                                            const float2* __restrict__ dad, int n_part,
+                                                            float2* __restrict__ rr_new) {
+  __shared__ float2 sh[kElemThreads / 32];
+  __shared__ float s_a;
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  const float a = (float)sc[S_A];
-  double s[1] = {0.0};
-  for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
-    const float2 dv = d[i], av = Ad[i];
-    float2 xv = x[i], rv = r[i];
+  if (threadIdx.x < 32) {
+    const Sum2 num = partial_sum(rr, n_part), den = partial_sum(dad, n_part);
+    if (threadIdx.x == 0) s_a = pair_ratio(num, den);
+  }
+  const size_t i0 = (size_t)blockIdx.x * kElemThreads + threadIdx.x, step = (size_t)gridDim.x * kElemThreads;
+  float2 dv, av, xv, rv;  // the first element's loads while the step size is formed
+  if (i0 < n) {
+    dv = d[i0];
+    av = Ad[i0];
+    xv = x[i0];
+    rv = r[i0];
+  }
+  __syncthreads();
+  const float a = s_a;
+  Sum2 s[1];
+  for (size_t i = i0; i < n; i += step) {
+    if (i != i0) {
+      dv = d[i];
+      av = Ad[i];
+      xv = x[i];
+      rv = r[i];
+    }
     xv.x = fmaf(a, dv.x, xv.x);
     xv.y = fmaf(a, dv.y, xv.y);
     rv.x = fmaf(-a, av.x, rv.x);
     rv.y = fmaf(-a, av.y, rv.y);
     x[i] = xv;
     r[i] = rv;
-    s[0] += (double)rv.x * rv.x + (double)rv.y * rv.y;
+    sum2_mul(s[0], rv.x, rv.x);
+    sum2_mul(s[0], rv.y, rv.y);
   }
-  if (!group_sums(s, partials, counter, (int)blockIdx.x, (int)gridDim.x, sh) || threadIdx.x) return;
-  sc[S_BETA] = sc[S_RR] > 0.0 ? s[0] / sc[S_RR] : 0.0;
-  sc[S_RR] = s[0];
+  Sum2 out[1];
+  block_sums(s, sh, out);
+  if (threadIdx.x == 0) rr_new[blockIdx.x] = pack(out[0]);
 }
 
-// f_k = eps_k / max(|F_s S p + u_k - y|, eps_k): kBallBlocks CTAs per (frame, coil).
+// |F_s S p + u_k - y|^2 of every (frame, coil): kBallBlocks partial sums each.
 __global__ void __launch_bounds__(kThreads) k_ball_norm(const float2* __restrict__ ap, const float2* __restrict__ uk,
                                                         const float2* __restrict__ y, int M,
-                                                        const double* __restrict__ eps, const double* __restrict__ sc,
-                                                        double* __restrict__ f, double* partials, unsigned* counters) {
-  __shared__ double sh[kThreads / 32];
+                                                        const double* __restrict__ sc, float2* __restrict__ partials) {
+  __shared__ float2 sh[kThreads / 32];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const int c = blockIdx.y;
   const float fu = (float)sc[S_UFAC];
-  double s[1] = {0.0};
+  Sum2 s[1];
   for (int m = blockIdx.x * kThreads + threadIdx.x; m < M; m += gridDim.x * kThreads) {
     const size_t i = (size_t)c * M + m;
     const float2 av = ap[i], uv = uk[i], yv = y[i];
-    const double dx = (double)av.x + (double)(fu * uv.x) - yv.x, dy = (double)av.y + (double)(fu * uv.y) - yv.y;
-    s[0] += dx * dx + dy * dy;
+    float e1, e2;  // ap + fu uk - y = d + e1 + e2 exactly
+    float d = diff_exact(av.x, -(fu * uv.x), e1);
+    d = diff_exact(d, yv.x, e2);
+    sum2_sq(s[0], d, e1 + e2);
+    d = diff_exact(av.y, -(fu * uv.y), e1);
+    d = diff_exact(d, yv.y, e2);
+    sum2_sq(s[0], d, e1 + e2);
   }
-  if (!group_sums(s, partials + (size_t)c * kBallBlocks, counters + c, (int)blockIdx.x, (int)gridDim.x, sh) ||
-      threadIdx.x)
-    return;
-  f[c] = eps[c] / fmax(sqrt(s[0]), eps[c]);
+  Sum2 out[1];
+  block_sums(s, sh, out);
+  if (threadIdx.x == 0) partials[(size_t)c * kBallBlocks + blockIdx.x] = pack(out[0]);
 }
 
 // u_0 += p - z_0; the residual norms of both blocks (row_part: the data blocks'
-// sums per CTA) and the balancing of rho (He et al. 2000).
+// sums per CTA) and the balancing of rho (He et al. 2000), by the last CTA to
+// arrive at `counter` (zero before and after), which adds the partial sums in order.
 __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__ u0, const float2* __restrict__ p,
                                                             const float2* __restrict__ z0,
                                                             const float2* __restrict__ p_prev, size_t n, double* sc,
-                                                            double* partials, unsigned* counter,
-                                                            const double* __restrict__ row_part, int n_row, double mu,
+                                                            float2* partials, unsigned* counter,
+                                                            const float2* __restrict__ row_part, int n_row, double mu,
                                                             double tau, double* __restrict__ hist) {
-  __shared__ double sh[2 * kElemThreads / 32];
+  __shared__ float2 sh[2 * kElemThreads / 32];
+  __shared__ int last;
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const float fu = (float)sc[S_UFAC];
-  double s[2] = {0.0, 0.0};
+  Sum2 s[2];
   for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
     const float2 pv = p[i], zv = z0[i], qv = p_prev[i];
     const float2 uv = u0[i];
     u0[i] = make_float2(fu * uv.x + pv.x - zv.x, fu * uv.y + pv.y - zv.y);
-    const double rx = (double)pv.x - zv.x, ry = (double)pv.y - zv.y;
-    const double dx = (double)pv.x - qv.x, dy = (double)pv.y - qv.y;
-    s[0] += rx * rx + ry * ry;
-    s[1] += dx * dx + dy * dy;
+    sum2_diff_sq(s[0], pv, zv);
+    sum2_diff_sq(s[1], pv, qv);
   }
-  if (!group_sums(s, partials, counter, (int)blockIdx.x, (int)gridDim.x, sh)) return;
-  double d[2] = {0.0, 0.0};
-  for (int i = threadIdx.x; i < n_row; i += kElemThreads) {
-    d[0] += row_part[2 * (size_t)i];
-    d[1] += row_part[2 * (size_t)i + 1];
+  Sum2 out[2];
+  block_sums(s, sh, out);
+  if (threadIdx.x == 0) {
+    partials[2 * (size_t)blockIdx.x] = pack(out[0]);
+    partials[2 * (size_t)blockIdx.x + 1] = pack(out[1]);
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    if (last) *counter = 0;
   }
-  block_sums(d, sh);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  s[0] = s[1] = Sum2();
+  for (unsigned i = threadIdx.x; i < gridDim.x + n_row; i += kElemThreads) {
+    const float2* q = i < gridDim.x ? partials + 2 * (size_t)i : row_part + 2 * (size_t)(i - gridDim.x);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float2 v = __ldcg(q + j);
+      sum2_add(s[j], v.x, v.y);
+    }
+  }
+  block_sums(s, sh, out);
   if (threadIdx.x) return;
-  const double prim = sqrt(s[0] + d[0]), rho = sc[S_RHO], dual = rho * sqrt(s[1] + d[1]);
+  const double prim = sqrt(to_double(out[0])), rho = sc[S_RHO], dual = rho * sqrt(to_double(out[1]));
   hist[0] = prim;
   hist[1] = dual;
   hist[2] = rho;
@@ -672,8 +880,16 @@ unsigned elem_blocks(size_t n) {
   return (unsigned)std::min<size_t>((n + kElemThreads - 1) / kElemThreads, kMaxElemBlocks);
 }
 
-unsigned row_blocks(const mpi_ctx* ctx, size_t rows) {
-  return (unsigned)std::min<size_t>((rows + kRowWarps - 1) / kRowWarps, 16 * (size_t)std::max(ctx->num_sms, 1));
+// CTAs of a row pass over TC coils with at most n_list rows each, R rows per warp
+unsigned row_blocks(const mpi_ctx* ctx, size_t TC, int n_list, int nx) {
+  int R = 1;
+#define MPI_ROWS(n) \
+  if (nx == n) R = Rows<n>::R;
+  MPI_ROWS(16) MPI_ROWS(32) MPI_ROWS(48) MPI_ROWS(64) MPI_ROWS(96) MPI_ROWS(128) MPI_ROWS(192) MPI_ROWS(256)
+  MPI_ROWS(320) MPI_ROWS(512)
+#undef MPI_ROWS
+  const size_t groups = TC * (size_t)((n_list + R - 1) / R);
+  return (unsigned)std::min<size_t>((groups + kRowWarps - 1) / kRowWarps, 16 * (size_t)std::max(ctx->num_sms, 1));
 }
 
 #define TRY(x)                       \
@@ -719,19 +935,22 @@ size_t admm_maps_layout(const mpi_ctx* ctx, const mpi_plan* const* plans, int T,
   m->u0 = cplx(TN);
   m->ap = cplx(CM);
   m->uk = cplx(CM);
-  m->counters = (unsigned*)take(((size_t)T * C + 4) * sizeof(unsigned));
+  m->counters = (unsigned*)take(sizeof(unsigned));
   m->zero_bytes = (char*)mem + off - m->zero_begin;
   m->zk = cplx(CM);
   float2** img[] = {&m->z0, &m->r, &m->d[0], &m->d[1], &m->Ad, &m->p_prev};
   for (float2** b : img) *b = cplx(TN);
   m->tv = cplx(tv_scratch_elems(T > 1 ? 3 : 2, (long)TN));
   m->sc = (double*)take(S_NUM * sizeof(double));
-  m->fball = (double*)take((size_t)T * C * sizeof(double));
-  m->ball_part = (double*)take((size_t)T * C * kBallBlocks * sizeof(double));
-  m->part = (double*)take(2 * (size_t)kMaxElemBlocks * sizeof(double));
-  m->row_part = (double*)take(2 * (size_t)row_blocks(ctx, (size_t)T * C * plans[0]->ny) * sizeof(double));
+  m->ball_part = cplx((size_t)T * C * kBallBlocks);
+  m->part = cplx(5 * (size_t)kMaxElemBlocks);  // |r|^2 twice, <d, A d>, the dual's two
+  int n_list = 0;
+  for (int t = 0; t < T; ++t) n_list = std::max(n_list, plans[t]->n_list);
+  m->row_part = cplx(2 * (size_t)row_blocks(ctx, (size_t)T * C, n_list, plans[0]->nx));
   m->idx = (int32_t*)take((size_t)T * M * sizeof(int32_t));
   m->row_ptr = (int32_t*)take((size_t)T * (plans[0]->ny + 1) * sizeof(int32_t));
+  m->row_list = (int32_t*)take((size_t)T * plans[0]->ny * sizeof(int32_t));
+  m->n_list = (int32_t*)take((size_t)T * sizeof(int32_t));
   m->rmask = (uint8_t*)take((size_t)T * plans[0]->ny);
   m->mask = (uint8_t*)take(TN);
   return off;
@@ -742,6 +961,7 @@ mpi_status admm_maps_tables(mpi_ctx* ctx, const mpi_plan* const* plans, int T, A
   const size_t N = plans[0]->N;
   std::vector<int32_t> rp((size_t)T * (ny + 1));
   std::vector<uint8_t> has((size_t)T * ny);
+  std::vector<int32_t> list((size_t)T * ny, 0), count(T, 0);
   cudaError_t e = cudaMemsetAsync(m->mask, 0, (size_t)T * N, ctx->stream);
   for (int t = 0; t < T && e == cudaSuccess; ++t) {
     e = cudaMemcpyAsync(m->idx + (size_t)t * M, plans[t]->idx, (size_t)M * sizeof(int32_t), cudaMemcpyDeviceToDevice,
@@ -757,15 +977,20 @@ mpi_status admm_maps_tables(mpi_ctx* ctx, const mpi_plan* const* plans, int T, A
     for (int r = 0; r < ny; ++r) {
       const int n = rp[(size_t)t * (ny + 1) + r + 1] - rp[(size_t)t * (ny + 1) + r];
       has[(size_t)t * ny + r] = n > 0;
+      if (n > 0) list[(size_t)t * ny + count[t]++] = r;
       m->whole_rows &= n == 0 || n == nx;
     }
   e = cudaMemcpyAsync(m->row_ptr, rp.data(), rp.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(m->row_list, list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(m->n_list, count.data(), count.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->rmask, has.data(), has.size(), cudaMemcpyHostToDevice, ctx->stream);
   if (e != cudaSuccess) return cuda_check(ctx, e, "image solver tables");
   MPI_PROF(ctx, KF_SOLVER);
   k_sample_mask<<<dim3((unsigned)((M + 255) / 256), (unsigned)T), 256, 0, ctx->stream>>>(m->idx, M, N, m->mask);
   MPI_LAUNCH_CHECK(ctx, "k_sample_mask");
-  return cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "image solver tables");  // rp and has are read until here
+  return cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "image solver tables");  // the host tables are read until here
 }
 
 mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mpi_basis* basis, int C,
@@ -773,9 +998,10 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   const int ny = plans[0]->ny, nx = plans[0]->nx, M = plans[0]->M, TC = T * C;
   const size_t N = plans[0]->N, TN = (size_t)T * N;
   const float scale = 1.0f / sqrtf((float)N);
-  const unsigned eblk = elem_blocks(TN), rblk = row_blocks(ctx, (size_t)TC * ny);
-  unsigned* ball_count = m.counters;
-  unsigned* count = m.counters + TC;
+  int n_list = 0;
+  for (int t = 0; t < T; ++t) n_list = std::max(n_list, plans[t]->n_list);
+  const unsigned eblk = elem_blocks(TN), rblk = row_blocks(ctx, TC, n_list, nx);
+  float2 *rr[2] = {m.part, m.part + kMaxElemBlocks}, *dad = m.part + 2 * kMaxElemBlocks;
   TRY(cuda_check(ctx, cudaMemsetAsync(m.zero_begin, 0, m.zero_bytes, ctx->stream), "image solver start"));
   MPI_PROF(ctx, KF_SOLVER);
   k_admm_start<<<1, 1, 0, ctx->stream>>>(m.sc, prm->rho0);
@@ -788,19 +1014,22 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
 
   MapsCols cols{};
   cols.W = m.W;
-  cols.sc = m.sc;
+  cols.n_part = (int)eblk;
   cols.C = C;
   cols.nx = nx;
   cols.N = N;
   cols.scale = scale;
   cols.rmask = m.rmask;
   cols.tw = twiddle_table(ctx, ny);
+  int par = 0;  // which of rr holds |r|^2
   auto cols_fwd = [&](const float2* S, const float2* v, const float2* r, float2* dnew) {
     MapsCols a = cols;
     a.S = S;
     a.v = v;
     a.r = r;
     a.dnew = dnew;
+    a.rr = rr[par];
+    a.rr_old = rr[par ^ 1];
     return launch_maps_cols<false>(ctx, ny, a, TC);
   };
   auto cols_inv = [&](const float2* S) {
@@ -815,7 +1044,9 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   rows.C = C;
   rows.ny = ny;
   rows.M = M;
-  rows.rmask = m.rmask;
+  rows.row_list = m.row_list;
+  rows.n_list = m.n_list;
+  rows.n_list_max = n_list;
   rows.mask = m.mask;
   rows.idx = m.idx;
   rows.row_ptr = m.row_ptr;
@@ -825,7 +1056,8 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   rows.ap = m.ap;
   rows.uk = m.uk;
   rows.zk = m.zk;
-  rows.f = m.fball;
+  rows.ball = m.ball_part;
+  rows.eps = m.in_eps;
   rows.sc = m.sc;
   rows.partials = m.row_part;
   CoilSum sum{};
@@ -841,16 +1073,14 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   sum.r = m.r;
   sum.p_prev = m.p_prev;
   sum.sc = m.sc;
-  sum.partials = m.part;
-  sum.counter = count;
 
   for (int it = 0; it < prm->n_outer; ++it) {
     // z_0 = prox_{TV/rho}(p + u_0), z_k = Pi(F_s S p + u_k)
     TRY(launch_tv_prox(ctx, T > 1 ? T : 1, ny, nx, T > 1 ? 3 : 2, m.p, m.u0, m.sc + S_UFAC, m.sc + S_RHO, 0.f,
                        prm->n_tv, m.tv, m.z0));
     MPI_PROF(ctx, KF_SOLVER);
-    launch_pdl(ctx, k_ball_norm, dim3(kBallBlocks, (unsigned)TC), dim3(kThreads), 0, m.ap, m.uk, m.in_y, M, m.in_eps,
-               m.sc, m.fball, m.ball_part, ball_count);
+    launch_pdl(ctx, k_ball_norm, dim3(kBallBlocks, (unsigned)TC), dim3(kThreads), 0, m.ap, m.uk, m.in_y, M,
+               m.sc, m.ball_part);
     MPI_LAUNCH_CHECK(ctx, "k_ball_norm");
     TRY(launch_maps_rows(ctx, nx, ROWS_SCATTER, rows, rblk));
     // r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p
@@ -858,6 +1088,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     int cur = 0;
     sum.scale = scale;
     sum.d = m.d[cur];
+    sum.partials = rr[par];
     MPI_PROF(ctx, KF_SOLVER);
     launch_pdl(ctx, k_coil_sum<false>, dim3(eblk), dim3(kElemThreads), 0, sum);
     MPI_LAUNCH_CHECK(ctx, "k_coil_sum<residual>");
@@ -872,19 +1103,22 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
       TRY(cols_inv(m.S_cg));
       sum.scale = m.whole_rows ? scale * (float)nx : scale;  // F_x^H F_x = nx on whole rows
       sum.d = m.d[cur];
+      sum.partials = dad;
       MPI_PROF(ctx, KF_SOLVER);
       launch_pdl(ctx, k_coil_sum<true>, dim3(eblk), dim3(kElemThreads), 0, sum);
       MPI_LAUNCH_CHECK(ctx, "k_coil_sum<normal>");
       MPI_PROF(ctx, KF_SOLVER);
-      launch_pdl(ctx, k_cg_update, dim3(eblk), dim3(kElemThreads), 0, m.p, m.r, m.d[cur], m.Ad, TN, m.sc, m.part, count);
+      launch_pdl(ctx, k_cg_update, dim3(eblk), dim3(kElemThreads), 0, m.p, m.r, m.d[cur], m.Ad, TN, rr[par], dad,
+                 (int)eblk, rr[par ^ 1]);
       MPI_LAUNCH_CHECK(ctx, "k_cg_update");
+      par ^= 1;
     }
     // u += A p - z, the residuals, rho
     TRY(cols_fwd(m.S, m.p, nullptr, nullptr));
     TRY(launch_maps_rows(ctx, nx, ROWS_GATHER, rows, rblk));
     MPI_PROF(ctx, KF_SOLVER);
-    launch_pdl(ctx, k_admm_dual, dim3(eblk), dim3(kElemThreads), 0, m.u0, m.p, m.z0, m.p_prev, TN, m.sc, m.part, count,
-               m.row_part, (int)rblk, prm->mu, prm->tau, m.hist + 3 * (size_t)it);
+    launch_pdl(ctx, k_admm_dual, dim3(eblk), dim3(kElemThreads), 0, m.u0, m.p, m.z0, m.p_prev, TN, m.sc,
+               m.part + 3 * kMaxElemBlocks, m.counters, m.row_part, (int)rblk, prm->mu, prm->tau, m.hist + 3 * (size_t)it);
     MPI_LAUNCH_CHECK(ctx, "k_admm_dual");
   }
   return MPI_OK;

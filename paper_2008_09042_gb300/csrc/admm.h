@@ -17,8 +17,9 @@ struct AdmmMaps {
   unsigned* counters;
   char* zero_begin;
   size_t zero_bytes;
-  double *sc, *fball, *ball_part, *part, *row_part;
-  int32_t *idx, *row_ptr;
+  double* sc;
+  float2 *ball_part, *part, *row_part;  // partial sums as pairs
+  int32_t *idx, *row_ptr, *row_list, *n_list;
   uint8_t *rmask, *mask;
   bool whole_rows;  // every k-space row of every frame is sampled whole or not at all
 };
