@@ -603,6 +603,85 @@ __global__ void __launch_bounds__(kLineWarps * 32, (L * 8 <= 2048) ? 4 : (L * 8 
   }
 }
 
+// The windowed pass along y as a two-step register FFT (G = R1 R2, see
+// k_fft_cols_reg), 16 adjacent columns per CTA (two rows per warp step): one write
+// and read of shared memory per element instead of one per radix stage and two
+// transposes, and the padded rows are never loaded.  256^2, 12 coils, G = 512:
+// 17.6 -> 12.4 us.  Tiles wholly outside the window are not launched.
+template <int R1, int R2, bool INV>
+__global__ void __launch_bounds__(256) k_fft_cols_win(float2* __restrict__ grid, int C, LineWin win, int x_first,
+                                                      int x_tiles, const float2* __restrict__ tw_g) {
+  constexpr int L = R1 * R2, TILE = 16;
+  extern __shared__ float2 sY[];  // [k1][r][column]
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const int tid = threadIdx.x, col = tid % TILE, s0 = tid / TILE;
+  const int c = (int)blockIdx.x / x_tiles, gx = x_first + ((int)blockIdx.x - c * x_tiles) * TILE + col;
+  const int xi = gx - win.o;
+  const bool colin = gx < L && xi >= 0 && xi < win.n;  // else a column of zeros: nothing reads or keeps it
+  float2* gcol = grid + (size_t)c * L * L + gx;
+  const float fx = colin ? win.deap[xi] / (float)win.n : 0.f;
+#pragma unroll
+  for (int it = 0; it < (R2 + 15) / 16; ++it) {
+    const int r = s0 + 16 * it;
+    if (r >= R2) break;
+    float2 v[R1];
+    if (!INV) {
+      const float2* src = win.src + (size_t)c * win.n * win.n + xi;
+      float f[R1];
+#pragma unroll
+      for (int m = 0; m < R1; ++m) {
+        const int yi = r + R2 * m - win.o;
+        const bool in = colin && yi >= 0 && yi < win.n;
+        v[m] = in ? src[(size_t)yi * win.n] : make_float2(0.f, 0.f);
+        f[m] = in ? win.deap[yi] * fx : 0.f;
+      }
+#pragma unroll
+      for (int m = 0; m < R1; ++m) {
+        const float g = ((gx + r + R2 * m) & 1) ? -f[m] : f[m];
+        v[m] = make_float2(v[m].x * g, v[m].y * g);
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < R1; ++m) {
+        const float2 e = colin ? gcol[(size_t)(r + R2 * m) * L] : make_float2(0.f, 0.f);
+        v[m] = make_float2(e.x, -e.y);  // the inverse on conjugated values
+      }
+    }
+    float2 w[R1];
+#pragma unroll
+    for (int k1 = 1; k1 < R1; ++k1) w[k1] = __ldg(tw_g + r * k1);
+    mpi_dft::dft_r<R1>(v);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) sY[(k1 * R2 + r) * TILE + col] = k1 ? mpi_dft::cmulf(v[k1], w[k1]) : v[0];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < (R1 + 15) / 16; ++it) {
+    const int k1 = s0 + 16 * it;
+    if (k1 >= R1 || !colin) break;
+    float2 u[R2];
+#pragma unroll
+    for (int r = 0; r < R2; ++r) u[r] = sY[(k1 * R2 + r) * TILE + col];
+    mpi_dft::dft_r<R2>(u);
+    if (!INV) {
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) gcol[(size_t)(k1 + R1 * k2) * L] = u[k2];
+    } else {
+      float2* dst = win.dst + (size_t)c * win.n * win.n + xi;
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) {
+        const int gy = k1 + R1 * k2, yi = gy - win.o;
+        if (yi >= 0 && yi < win.n) {
+          float f = win.deap[yi] * fx;
+          if ((gx + gy) & 1) f = -f;
+          dst[(size_t)yi * win.n] = make_float2(u[k2].x * f, -u[k2].y * f);
+        }
+      }
+    }
+  }
+}
+
 float axis_sign(int n) { return ((n / 2) & 1) ? -1.f : 1.f; }
 
 // The passes along y and x of one (coil, kz) plane of a 3D volume in one CTA,
@@ -1063,22 +1142,37 @@ mpi_status launch_fft_cols_window(mpi_ctx* ctx, float2* grid, int C, int G, cons
     else                                                                                                   \
       launch_pdl(ctx, k_fft_lines_win<L, false>, dim3((unsigned)blocks), dim3(kLineWarps * 32), 0, grid, C, win, tw); \
     break;
+  // register two-step pass: the 16-column tiles that meet the window
+  const int x_first = win.o / 16 * 16, x_tiles = (win.o + n - x_first + 15) / 16;
+  const long wblocks = (long)C * x_tiles;
+#define MPI_WIN_REG(L, r1, r2)                                                                                      \
+  case L: {                                                                                                         \
+    const size_t smem = (size_t)L * 16 * sizeof(float2);                                                            \
+    auto kern = inverse ? k_fft_cols_win<r1, r2, true> : k_fft_cols_win<r1, r2, false>;                             \
+    if (smem > 48 * 1024) { /* more than a launch may ask for without it */                                        \
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);           \
+      if (e != cudaSuccess) return cuda_check(ctx, e, "windowed pass attributes");                                  \
+    }                                                                                                               \
+    launch_pdl(ctx, kern, dim3((unsigned)wblocks), dim3(256), smem, grid, C, win, x_first, x_tiles, tw);             \
+    break;                                                                                                          \
+  }
   MPI_PROF(ctx, KF_FFT_LINES);
   switch (G) {
     MPI_WIN_CASE(16)
     MPI_WIN_CASE(32)
     MPI_WIN_CASE(48)
-    MPI_WIN_CASE(64)
-    MPI_WIN_CASE(96)
-    MPI_WIN_CASE(128)
-    MPI_WIN_CASE(192)
-    MPI_WIN_CASE(256)
-    MPI_WIN_CASE(320)
-    MPI_WIN_CASE(512)
+    MPI_WIN_REG(64, 8, 8)
+    MPI_WIN_REG(96, 8, 12)
+    MPI_WIN_REG(128, 8, 16)
+    MPI_WIN_REG(192, 16, 12)
+    MPI_WIN_REG(256, 16, 16)
+    MPI_WIN_REG(320, 16, 20)
+    MPI_WIN_REG(512, 16, 32)
     default:
       return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
   }
 #undef MPI_WIN_CASE
+#undef MPI_WIN_REG
   MPI_LAUNCH_CHECK(ctx, "k_fft_lines_win");
   return MPI_OK;
 }

@@ -81,13 +81,18 @@ __global__ void k_nufft_deap(int n, int G, int W, double beta, float* __restrict
 constexpr int kInterpTile = 32;    // first-tap tile of the shared-memory interpolation
 constexpr int kInterpChunk = 256;  // samples per interpolation work item (one per thread)
 
-// Interpolation through shared memory: CTA (item, coil) takes a chunk of at
-// most kInterpChunk of the samples whose first tap lies in one 32 x 32 tile
-// (the plan's tile-sorted list).  Each thread loads its sample's first tap
-// and weights (before waiting on the kernel that writes the grid), the CTA
-// copies the grid cells the chunk reads, (32 + W - 1)^2 from the tile's corner
-// (periodic), into shared memory with coalesced loads, and each thread forms
-// its sample's W x W sum there.
+// Interpolation through shared memory: CTA (item, group of kInterpCoils coils) takes
+// a chunk of at most kInterpChunk of the samples whose first tap lies in one 32 x 32
+// tile (the plan's tile-sorted list).  Each thread loads its sample's first tap
+// and weights (before waiting on the kernel that writes the grid) and forms the
+// addresses of its share of the grid cells that the chunk reads, (32 + W - 1)^2 from
+// the tile's corner (periodic); then, coil by coil, the CTA copies those cells to
+// shared memory, the next coil's loads in flight while each thread forms its
+// sample's W x W sum there.  The set-up (divisions by the tile width, wraps,
+// scattered weights) was most of the kernel when every CTA did one coil:
+// 256^2, 12 coils, 64 spokes 26.2 -> 22.4 us.
+constexpr int kInterpCoils = 4;
+
 template <int W>
 __global__ void __launch_bounds__(kInterpChunk) k_nufft_interp_tiled(const float2* __restrict__ grid, int C, int G,
                                                                      int M, const int32_t* __restrict__ gstart,
@@ -97,51 +102,86 @@ __global__ void __launch_bounds__(kInterpChunk) k_nufft_interp_tiled(const float
                                                                      float2* __restrict__ y) {
   mpi_ptx::pdl_trigger();
   constexpr int TT = kInterpTile + W - 1;
+  constexpr int PER = (TT * TT + kInterpChunk - 1) / kInterpChunk;  // cells per thread
   __shared__ float2 tile[TT * TT];
-  const int it = blockIdx.x, c = blockIdx.y;
+  const int it = blockIdx.x, c0 = blockIdx.y * kInterpCoils, c1 = min(c0 + kInterpCoils, C);
   const int t = items[3 * it], s0 = items[3 * it + 1], cnt = items[3 * it + 2];
   const int tpr = (G + kInterpTile - 1) / kInterpTile;
   const int oy = (t / tpr) * kInterpTile, ox = (t % tpr) * kInterpTile;
   const bool active = (int)threadIdx.x < cnt;
   const int m = samples[s0 + (active ? (int)threadIdx.x : 0)];
   const int sx = gstart[2 * m], sy = gstart[2 * m + 1];
+  // weights with the k-side sign (-1)^(gx + gy) folded in: (-1)^b and the sample's own
+  // parity along x, (-1)^a along y (G is even, so wrapping keeps the parity)
+  const int odd = (sx + sy) & 1;
   float wx[W], wy[W];
 #pragma unroll
   for (int a = 0; a < W; ++a) {
     wx[a] = gw[(size_t)(2 * m) * W + a];
     wy[a] = gw[(size_t)(2 * m + 1) * W + a];
+    if ((a + odd) & 1) wx[a] = -wx[a];
+    if (a & 1) wy[a] = -wy[a];
+  }
+  int off[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int e = threadIdx.x + kInterpChunk * j, r = e / TT, q = e - r * TT;
+    off[j] = e < TT * TT ? ((oy + r) % G) * G + (ox + q) % G : 0;
   }
   mpi_ptx::pdl_wait();
-  const float2* gc = grid + (size_t)c * G * G;
-  for (int e = threadIdx.x; e < TT * TT; e += blockDim.x) {
-    const int r = e / TT, q = e % TT;
-    tile[e] = gc[(size_t)((oy + r) % G) * G + (ox + q) % G];
-  }
-  __syncthreads();
-  if (!active) return;
+  const float2* gc = grid + (size_t)c0 * G * G;
+  float2 cell[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) cell[j] = gc[off[j]];
   const float2* tp = tile + (sy - oy) * TT + (sx - ox);
-  const bool odd = (sx + sy) & 1;  // (-1)^(gx + gy); G is even, so wrapping keeps the parity
-  float2 acc = make_float2(0.f, 0.f);
+  for (int c = c0; c < c1; ++c) {
+    if (c > c0) __syncthreads();  // the previous coil's tile has been read
 #pragma unroll
-  for (int a = 0; a < W; ++a) {
-    float2 racc = make_float2(0.f, 0.f);
+    for (int j = 0; j < PER; ++j)
+      if (threadIdx.x + kInterpChunk * j < TT * TT) tile[threadIdx.x + kInterpChunk * j] = cell[j];
+    gc += (size_t)G * G;
+    if (c + 1 < c1) {
 #pragma unroll
-    for (int b = 0; b < W; ++b) {
-      const float2 g = tp[a * TT + b];
-      const float w = (((a + b) & 1) != odd) ? -wx[b] : wx[b];
-      racc.x = fmaf(w, g.x, racc.x);
-      racc.y = fmaf(w, g.y, racc.y);
+      for (int j = 0; j < PER; ++j) cell[j] = gc[off[j]];
     }
-    acc.x = fmaf(wy[a], racc.x, acc.x);
-    acc.y = fmaf(wy[a], racc.y, acc.y);
+    __syncthreads();
+    if (!active) continue;
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int a = 0; a < W; ++a) {
+      float2 racc = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int b = 0; b < W; ++b) {
+        const float2 g = tp[a * TT + b];
+        racc.x = fmaf(wx[b], g.x, racc.x);
+        racc.y = fmaf(wx[b], g.y, racc.y);
+      }
+      acc.x = fmaf(wy[a], racc.x, acc.x);
+      acc.y = fmaf(wy[a], racc.y, acc.y);
+    }
+    y[(size_t)c * M + m] = make_float2(acc.x * ksign, acc.y * ksign);
   }
-  y[(size_t)c * M + m] = make_float2(acc.x * ksign, acc.y * ksign);
 }
 
-constexpr int kSpreadCoils = 4;   // coils a spreading thread accumulates (one group of four)
+constexpr int kSpreadCoils = 4;   // coils of a group; a spreading thread accumulates up to kSpreadGroups of them
+constexpr int kSpreadGroups = 3;
 constexpr int kSpreadDense = 24;  // cells with more samples in their window go to the warp kernel
 
-int spread_coils_padded(int C) { return (C + 3) / 4 * 4; }
+// Groups per spreading thread for C coils on a G x G grid: as many as leave 131,072
+// threads (some 860 per SM; a 192^2 grid with 5 coils is slower with two groups per
+// thread, 11.5 against 9.3 us), at most kSpreadGroups, in as few passes over the
+// samples and with as few padded coils as that allows.
+int spread_groups(int C, int G) {
+  const int g = (C + kSpreadCoils - 1) / kSpreadCoils;
+  int ng = std::min(kSpreadGroups, g);
+  while (ng > 1 && (long)G * G * ((g + ng - 1) / ng) < 131072) --ng;
+  const int z = (g + ng - 1) / ng;
+  return (g + z - 1) / z;
+}
+int spread_coils_padded(int C, int G) {
+  const int per = kSpreadCoils * spread_groups(C, G);
+  return (C + per - 1) / per * per;
+}
 
 // ys[cell_rank[m]][c] = ksign * y[c][m] for c < C, zero for C <= c < Cp (C
 // padded to a multiple of four): the samples in first-tap-cell order, the
@@ -179,79 +219,89 @@ __device__ __forceinline__ void spread_row_ranges(const int32_t* __restrict__ rp
 }
 
 // One sample's term: weight phi_x(b) phi_y(a) with b = gx - sx (mod G) read
-// from the sample's own first tap, times four coils of ys.
-template <int W>
+// from the sample's own first tap, times the 4 NG coils of ys from yc.
+template <int W, int NG>
 __device__ __forceinline__ void spread_term(const float* __restrict__ cell_w, const int32_t* __restrict__ cell_sx,
                                             const float4* __restrict__ yc, int ystride, int k, int gx, int a,
-                                            int G, float acc[8]) {
+                                            int G, float (&acc)[8 * NG]) {
   int b = gx - cell_sx[k];
   if (b < 0) b += G;
   const float w = cell_w[k * 2 * W + b] * cell_w[k * 2 * W + W + a];
-  const float4 u = yc[k * ystride], v = yc[k * ystride + 1];
-  acc[0] = fmaf(w, u.x, acc[0]);
-  acc[1] = fmaf(w, u.y, acc[1]);
-  acc[2] = fmaf(w, u.z, acc[2]);
-  acc[3] = fmaf(w, u.w, acc[3]);
-  acc[4] = fmaf(w, v.x, acc[4]);
-  acc[5] = fmaf(w, v.y, acc[5]);
-  acc[6] = fmaf(w, v.z, acc[6]);
-  acc[7] = fmaf(w, v.w, acc[7]);
+#pragma unroll
+  for (int g = 0; g < 2 * NG; ++g) {
+    const float4 u = yc[(size_t)k * ystride + g];
+    acc[4 * g + 0] = fmaf(w, u.x, acc[4 * g + 0]);
+    acc[4 * g + 1] = fmaf(w, u.y, acc[4 * g + 1]);
+    acc[4 * g + 2] = fmaf(w, u.z, acc[4 * g + 2]);
+    acc[4 * g + 3] = fmaf(w, u.w, acc[4 * g + 3]);
+  }
 }
 
+template <int NG>
 __device__ __forceinline__ void spread_store(float2* __restrict__ grid, int C, int G, int c0, int gy, int gx,
-                                             const float acc[8]) {
+                                             const float (&acc)[8 * NG]) {
   const float s = ((gx + gy) & 1) ? -1.f : 1.f;  // the k-side sign (-1)^(gx + gy)
 #pragma unroll
-  for (int j = 0; j < kSpreadCoils; ++j)
+  for (int j = 0; j < kSpreadCoils * NG; ++j)
     if (c0 + j < C) grid[((size_t)(c0 + j) * G + gy) * G + gx] = make_float2(s * acc[2 * j], s * acc[2 * j + 1]);
 }
 
-// Output-driven spreading, sparse cells: thread (gy, gx, coil group) sums the
+// Output-driven spreading, sparse cells: thread (gy, gx, 4 NG coils) sums the
 // samples whose W x W footprint covers its cell, i.e. whose first tap is
 // (gy - a, gx - b) (mod G) for 0 <= a, b < W, and stores the cell once; no
 // atomics.  A cell whose window holds more than kSpreadDense samples is left
-// to k_nufft_spread_dense (its thread would hold the CTA up).
-template <int W>
-__global__ void __launch_bounds__(256, 4) k_nufft_spread(const float4* __restrict__ ys, int C, int Cp, int G,
-                                                         const int32_t* __restrict__ cell_ptr,
-                                                         const int32_t* __restrict__ cell_sx,
-                                                         const float* __restrict__ cell_w,
-                                                         float2* __restrict__ grid) {
+// to k_nufft_spread_dense (its thread would hold the CTA up).  Finding a cell's
+// samples (the CSR ranges of W rows) costs about as much as adding a few coils of
+// them, so a thread takes up to three groups of four coils: at 256^2, 12 coils,
+// 64 spokes 54 us (both kernels) -> 40.
+template <int W, int NG>
+__global__ void __launch_bounds__(256) k_nufft_spread(const float4* __restrict__ ys, int C, int Cp, int G,
+                                                      const int32_t* __restrict__ cell_ptr,
+                                                      const int32_t* __restrict__ cell_sx,
+                                                      const float* __restrict__ cell_w,
+                                                      float2* __restrict__ grid) {
   mpi_ptx::pdl_trigger();
   const int gx = blockIdx.x * 32 + threadIdx.x, gy = blockIdx.y * 8 + threadIdx.y;
-  const int c0 = blockIdx.z * kSpreadCoils;
-  mpi_ptx::pdl_wait();
+  const int c0 = blockIdx.z * kSpreadCoils * NG;
   if (gx >= G || gy >= G) return;
-  int n = 0;
+  // the plan's ranges do not depend on earlier work
+  int lo[W], hi[W], n = 0;
 #pragma unroll
   for (int a = 0; a < W; ++a) {
     int sy = gy - a;
     if (sy < 0) sy += G;
     int r[4];
     spread_row_ranges<W>(cell_ptr + sy * G, gx, G, r);
+    lo[a] = r[0];
+    hi[a] = r[1];
     n += r[1] - r[0] + r[3] - r[2];
   }
   if (n > kSpreadDense) return;
+  mpi_ptx::pdl_wait();
   const int ystride = Cp / 2;
   const float4* yc = ys + c0 / 2;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float acc[8 * NG] = {};
   if (n > 0) {
-    for (int a = 0; a < W; ++a) {  // the ranges again (L1 hits), rather than W x 4 live registers
-      int sy = gy - a;
-      if (sy < 0) sy += G;
-      int r[4];
-      spread_row_ranges<W>(cell_ptr + sy * G, gx, G, r);
-      for (int k = r[0]; k < r[1]; ++k) spread_term<W>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
-      for (int k = r[2]; k < r[3]; ++k) spread_term<W>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
+#pragma unroll
+    for (int a = 0; a < W; ++a)
+      for (int k = lo[a]; k < hi[a]; ++k) spread_term<W, NG>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
+    if (gx < W - 1) {  // the window wraps past column 0: the rows' second ranges
+      for (int a = 0; a < W; ++a) {
+        int sy = gy - a;
+        if (sy < 0) sy += G;
+        int r[4];
+        spread_row_ranges<W>(cell_ptr + sy * G, gx, G, r);
+        for (int k = r[2]; k < r[3]; ++k) spread_term<W, NG>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
+      }
     }
   }
-  spread_store(grid, C, G, c0, gy, gx, acc);
+  spread_store<NG>(grid, C, G, c0, gy, gx, acc);
 }
 
 // Output-driven spreading, dense cells (the plan's list of cells whose window
-// holds more than kSpreadDense samples): warp (cell, coil group), the lanes
+// holds more than kSpreadDense samples): warp (cell, 4 NG coils), the lanes
 // taking every 32nd sample of each row range, then a butterfly sum.
-template <int W>
+template <int W, int NG>
 __global__ void __launch_bounds__(256) k_nufft_spread_dense(const float4* __restrict__ ys, int C, int Cp, int G,
                                                             const int32_t* __restrict__ cell_ptr,
                                                             const int32_t* __restrict__ cell_sx,
@@ -261,27 +311,27 @@ __global__ void __launch_bounds__(256) k_nufft_spread_dense(const float4* __rest
   mpi_ptx::pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int c0 = blockIdx.y * kSpreadCoils;
+  const int c0 = blockIdx.y * kSpreadCoils * NG;
   mpi_ptx::pdl_wait();
   if (i >= n_dense) return;
   const int cell = dense[i], gy = cell / G, gx = cell % G;
   const int ystride = Cp / 2;
   const float4* yc = ys + c0 / 2;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float acc[8 * NG] = {};
 #pragma unroll
   for (int a = 0; a < W; ++a) {
     int sy = gy - a;
     if (sy < 0) sy += G;
     int r[4];
     spread_row_ranges<W>(cell_ptr + sy * G, gx, G, r);
-    for (int k = r[0] + lane; k < r[1]; k += 32) spread_term<W>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
-    for (int k = r[2] + lane; k < r[3]; k += 32) spread_term<W>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
+    for (int k = r[0] + lane; k < r[1]; k += 32) spread_term<W, NG>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
+    for (int k = r[2] + lane; k < r[3]; k += 32) spread_term<W, NG>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
   }
 #pragma unroll
-  for (int j = 0; j < 8; ++j)
+  for (int j = 0; j < 8 * NG; ++j)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-  if (lane == 0) spread_store(grid, C, G, c0, gy, gx, acc);
+  if (lane == 0) spread_store<NG>(grid, C, G, c0, gy, gx, acc);
 }
 
 float axis_sign(int n) { return ((n / 2) & 1) ? -1.f : 1.f; }
@@ -296,7 +346,7 @@ mpi_status launch_fft_rows_inplace(mpi_ctx* ctx, float2* data, long n_rows, int 
                                    int load_hi = -1, int keep_lo = 0, int keep_hi = -1);
 
 size_t nufft_grid_elems(const mpi_plan* plan, int C) {
-  return (size_t)C * plan->G * plan->G + (size_t)spread_coils_padded(C) * plan->M;
+  return (size_t)C * plan->G * plan->G + (size_t)spread_coils_padded(C, plan->G) * plan->M;
 }
 
 mpi_status nufft_plan_init(mpi_ctx* ctx, mpi_plan* plan, const float* traj_host) {
@@ -411,7 +461,7 @@ mpi_status nufft_forward(mpi_ctx* ctx, const mpi_plan* plan, const float2* v, in
   if (st) return st;
   if (M == 0) return MPI_OK;
   const float ks = axis_sign(G) * axis_sign(G);
-  const dim3 igrid((unsigned)plan->n_tile_items, (unsigned)C);
+  const dim3 igrid((unsigned)plan->n_tile_items, (unsigned)((C + kInterpCoils - 1) / kInterpCoils));
   MPI_PROF(ctx, KF_NUFFT);
   switch (plan->W) {
 #define MPI_W_CASE(w)                                                                                \
@@ -436,34 +486,34 @@ mpi_status nufft_adjoint(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, in
     if (e != cudaSuccess) return cuda_check(ctx, e, "grid clear");
   } else {
     const float ks = axis_sign(G) * axis_sign(G);
-    const int Cp = spread_coils_padded(C);
+    const int Cp = spread_coils_padded(C, G);
     float2* ys = grid + total;  // nufft_grid_elems reserves the sorted copy after the grid
     MPI_PROF(ctx, KF_NUFFT);
     launch_pdl(ctx, k_nufft_sort_y, dim3(blocks_for((size_t)M * Cp, 256)), dim3(256), 0, y, C, Cp, M,
                plan->cell_rank, ks, ys);
     MPI_LAUNCH_CHECK(ctx, "k_nufft_sort_y");
-    const unsigned groups = (unsigned)(Cp / kSpreadCoils);
+    const int ng = spread_groups(C, G);
+    const unsigned groups = (unsigned)(Cp / (kSpreadCoils * ng));
     const dim3 sgrid((unsigned)((G + 31) / 32), (unsigned)((G + 7) / 8), groups);
     const dim3 dgrid((unsigned)((plan->n_dense + 7) / 8), groups);
     const float4* ys4 = (const float4*)ys;
-    switch (plan->W) {
-#define MPI_W_CASE(w)                                                                                      \
-  case w:                                                                                                  \
-    MPI_PROF(ctx, KF_NUFFT);                                                                               \
-    launch_pdl(ctx, k_nufft_spread<w>, sgrid, dim3(32, 8), 0, ys4, C, Cp, G, plan->cell_ptr, plan->cell_sx,  \
-               plan->cell_w, grid);                                                                        \
-    if (plan->n_dense > 0) {                                                                               \
-      MPI_LAUNCH_CHECK(ctx, "k_nufft_spread");                                                             \
-      MPI_PROF(ctx, KF_NUFFT);                                                                             \
-      launch_pdl(ctx, k_nufft_spread_dense<w>, dgrid, dim3(256), 0, ys4, C, Cp, G, plan->cell_ptr,          \
-                 plan->cell_sx, plan->cell_w, plan->cell_dense, plan->n_dense, grid);                      \
-    }                                                                                                      \
-    break;
-      MPI_W_CASE(2) MPI_W_CASE(3) MPI_W_CASE(4) MPI_W_CASE(5) MPI_W_CASE(6) MPI_W_CASE(7) MPI_W_CASE(8)
+#define MPI_SPREAD(w, g)                                                                                    \
+  if (plan->W == w && ng == g) {                                                                            \
+    MPI_PROF(ctx, KF_NUFFT);                                                                                \
+    launch_pdl(ctx, k_nufft_spread<w, g>, sgrid, dim3(32, 8), 0, ys4, C, Cp, G, plan->cell_ptr, plan->cell_sx, \
+               plan->cell_w, grid);                                                                         \
+    if (plan->n_dense > 0) {                                                                                \
+      MPI_LAUNCH_CHECK(ctx, "k_nufft_spread");                                                              \
+      MPI_PROF(ctx, KF_NUFFT);                                                                              \
+      launch_pdl(ctx, k_nufft_spread_dense<w, g>, dgrid, dim3(256), 0, ys4, C, Cp, G, plan->cell_ptr,        \
+                 plan->cell_sx, plan->cell_w, plan->cell_dense, plan->n_dense, grid);                       \
+    }                                                                                                       \
+  }
+#define MPI_W_CASE(w) MPI_SPREAD(w, 1) MPI_SPREAD(w, 2) MPI_SPREAD(w, 3)
+    if (plan->W < 2 || plan->W > 8) return set_err(ctx, MPI_ERR_ARG, "kernel width");
+    MPI_W_CASE(2) MPI_W_CASE(3) MPI_W_CASE(4) MPI_W_CASE(5) MPI_W_CASE(6) MPI_W_CASE(7) MPI_W_CASE(8)
 #undef MPI_W_CASE
-      default:
-        return set_err(ctx, MPI_ERR_ARG, "kernel width");
-    }
+#undef MPI_SPREAD
     MPI_LAUNCH_CHECK(ctx, "k_nufft_spread");
   }
   // only the columns of the centred window reach the cropping pass along y
