@@ -176,8 +176,11 @@ template <> struct RegSplit<96> { static constexpr int R1 = 8, R2 = 12; };
 template <> struct RegSplit<128> { static constexpr int R1 = 8, R2 = 16; };
 template <> struct RegSplit<192> { static constexpr int R1 = 16, R2 = 12; };
 template <> struct RegSplit<256> { static constexpr int R1 = 16, R2 = 16; };
+template <> struct RegSplit<320> { static constexpr int R1 = 16, R2 = 20; };
 
-constexpr int maps_cols_tile(int L) { return (L == 64 || L == 96 || L == 128 || L == 192 || L == 256) ? 32 : 8; }
+constexpr int maps_cols_tile(int L) {
+  return (L == 64 || L == 96 || L == 128 || L == 192 || L == 256 || L == 320) ? 16 : 8;
+}
 
 // R values of one thread: rows y0 + step m of column x, formed from the image and
 // the map (forward) or read from the rows with samples (inverse).  All loads are
@@ -271,45 +274,44 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
     beta = pair_ratio(rr, old);
   }
   if constexpr (R1 > 0) {
-    __shared__ float2 sY[L * 32];  // [k1][r][column]
-    __shared__ float2 tw[L];
-    for (int i = tid; i < L; i += kThreads) tw[i] = a.tw[i];
-    const int x = x0 + lane;
+    constexpr int G = kThreads / TILE;  // rows r (step 1) or k1 (step 2) at a time
+    __shared__ float2 sY[L * TILE];     // [k1][r][column]
+    const int ci = tid % TILE, g = tid / TILE, x = x0 + ci;
     const bool ok = x < a.nx;
-    float2 u1[(R2 + 7) / 8][R1];
+    float2 u1[(R2 + G - 1) / G][R1];
 #pragma unroll
-    for (int it = 0; it < (R2 + 7) / 8; ++it) {
-      const int q = w + 8 * it;
+    for (int it = 0; it < (R2 + G - 1) / G; ++it) {
+      const int q = g + G * it;
       if (ok && q < R2) maps_load<R1, INV>(a, beta, t, c, tc, q, R2, x, L, u1[it]);
     }
-    __syncthreads();
 #pragma unroll
-    for (int it = 0; it < (R2 + 7) / 8; ++it) {
-      const int q = w + 8 * it;
+    for (int it = 0; it < (R2 + G - 1) / G; ++it) {
+      const int q = g + G * it;
       if (q >= R2) break;
       float2 (&u)[R1] = u1[it];
+      float2 tw[R1];
+#pragma unroll
+      for (int k1 = 1; k1 < R1; ++k1) tw[k1] = __ldg(a.tw + q * k1);
       if (INV)  // the inverse on conjugated values
 #pragma unroll
         for (int m = 0; m < R1; ++m) u[m].y = -u[m].y;
       mpi_dft::dft_r<R1>(u);
 #pragma unroll
-      for (int k1 = 1; k1 < R1; ++k1) u[k1] = mpi_dft::cmulf(u[k1], tw[q * k1]);
-#pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) sY[(k1 * R2 + q) * 32 + lane] = u[k1];
+      for (int k1 = 0; k1 < R1; ++k1) sY[(k1 * R2 + q) * TILE + ci] = k1 ? mpi_dft::cmulf(u[k1], tw[k1]) : u[0];
     }
-    float2 s[(R1 + 7) / 8][R2];
+    float2 s[(R1 + G - 1) / G][R2];
     if (INV)
 #pragma unroll
-      for (int it = 0; it < (R1 + 7) / 8; ++it)
-        if (ok && w + 8 * it < R1) maps_prefetch<R2>(a, c, w + 8 * it, R1, x, s[it]);
+      for (int it = 0; it < (R1 + G - 1) / G; ++it)
+        if (ok && g + G * it < R1) maps_prefetch<R2>(a, c, g + G * it, R1, x, s[it]);
     __syncthreads();
 #pragma unroll
-    for (int it = 0; it < (R1 + 7) / 8; ++it) {
-      const int k1 = w + 8 * it;
+    for (int it = 0; it < (R1 + G - 1) / G; ++it) {
+      const int k1 = g + G * it;
       if (k1 >= R1) break;
       float2 u[R2];
 #pragma unroll
-      for (int q = 0; q < R2; ++q) u[q] = sY[(k1 * R2 + q) * 32 + lane];
+      for (int q = 0; q < R2; ++q) u[q] = sY[(k1 * R2 + q) * TILE + ci];
       mpi_dft::dft_r<R2>(u);
       if (INV)
 #pragma unroll

@@ -16,8 +16,9 @@
 // read from DRAM about once per group instead of once per slice.  Each slice's
 // per-coil images live in a batch-owned buffer between the expansion and the
 // FFT passes.  From kGroupedPasses slices on, the FFT passes take all coils of a
-// group's slices in one launch too (per run of slices whose pass along y is tuned
-// to the same kernel, so that a slice's values stay those of its own call), with a
+// group's slices in one launch too (per run of slices whose pass along y is of the
+// same kind, register or Stockham, so that a slice's values stay those of its own
+// call; its width is timed for the group), with a
 // table of every coil's sampling.  How many CTAs each row gets is chosen at creation by
 // timing the candidates (an autotuner decision the context records).
 #include <algorithm>
@@ -65,7 +66,8 @@ struct Group {
   int row_ctas = 0;
   // grouped passes: runs of slices (first, count in coils) per direction and kernel
   struct Run {
-    int kernel, first, coils;
+    bool registers;
+    int first, coils, kernel;
   };
   std::vector<Run> fwd, inv;  // empty: the passes run slice by slice
   const CoilSamples* tab = nullptr;
@@ -115,14 +117,14 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
   return st;
 }
 
-// Runs of the group's slices (already in an order that keeps equal kernels
-// together) whose pass along y runs the same kernel.
+// Runs of the group's slices (already in an order that keeps equal kinds together)
+// whose pass along y is of the same kind.
 std::vector<Group::Run> pass_runs(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g, bool inverse) {
   std::vector<Group::Run> runs;
   int off = 0;
   for (int i : g.idx) {
-    const int k = fft_cols_kernel(ctx, sl[i].plan, sl[i].C, inverse);
-    if (runs.empty() || runs.back().kernel != k) runs.push_back({k, off, 0});
+    const bool k = fft_cols_in_registers(ctx, sl[i].plan, sl[i].C, inverse);
+    if (runs.empty() || runs.back().registers != k) runs.push_back({k, off, 0, 0});
     runs.back().coils += sl[i].C;
     off += sl[i].C;
   }
@@ -290,14 +292,14 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     ++i;
   }
 
-  // grouped passes: slices in the order of the kernels their passes along y run
+  // grouped passes: slices in the order of the kinds of their passes along y
   for (Group& g : groups) {
     if ((int)g.idx.size() < kGroupedPasses || ctx->line_kernel) continue;
     std::stable_sort(g.idx.begin(), g.idx.end(), [&](int a, int b) {
       const mpi_batch_slice &x = slices[a], &y = slices[b];
-      const int fa = fft_cols_kernel(ctx, x.plan, x.C, false), fb = fft_cols_kernel(ctx, y.plan, y.C, false);
+      const bool fa = fft_cols_in_registers(ctx, x.plan, x.C, false), fb = fft_cols_in_registers(ctx, y.plan, y.C, false);
       if (fa != fb) return fa < fb;
-      return fft_cols_kernel(ctx, x.plan, x.C, true) < fft_cols_kernel(ctx, y.plan, y.C, true);
+      return fft_cols_in_registers(ctx, x.plan, x.C, true) < fft_cols_in_registers(ctx, y.plan, y.C, true);
     });
     g.fwd = pass_runs(ctx, slices, g, false);
     g.inv = pass_runs(ctx, slices, g, true);
@@ -349,6 +351,13 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     }
     for (Group& g : groups) {
       mpi_status st = tune_group(ctx, slices, g, prec, (const ExpandRow*)bt->rows);
+      const mpi_plan* pl = slices[g.idx[0]].plan;
+      for (int dir = 0; dir < 2; ++dir)
+        for (Group::Run& r : dir ? g.inv : g.fwd)
+          if (st == MPI_OK)
+            st = tune_fft_cols_group(ctx, r.registers, (float2*)bt->buf + (size_t)r.first * pl->N, r.coils, pl->ny,
+                                     pl->nx, dir == 1, g.row_has ? g.row_has + (size_t)r.first * pl->ny : nullptr,
+                                     &r.kernel);
       if (st) {
         mpi_batch_destroy(bt);
         return st;

@@ -13,6 +13,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "dft_reg.cuh"
 #include "fft_rows.cuh"
@@ -57,7 +58,10 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_fwd_gather(const float2
   float2* b = buf[warp];
   const int per = (a.n_list + F::R - 1) / F::R, total = a.C * per;
   for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
-    const int c = gi / per, j0 = (gi - c * per) * F::R;
+    // a group's data may exceed L2: last coil first, so that this pass and the one along
+    // y meet at the coils that are still there
+    const int gq = TAB ? total - 1 - gi : gi;
+    const int c = gq / per, j0 = (gq - c * per) * F::R;
     const int n_list = TAB ? a.tab[c].n_list : a.n_list;
     const int32_t* list = TAB ? a.tab[c].row_list : a.row_list;
     const int32_t* idx = TAB ? a.tab[c].idx : a.idx;
@@ -125,7 +129,10 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_inv(const float
   float2* b = buf[warp];
   const int per = (a.n_list + F::R - 1) / F::R, total = a.C * per;
   for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
-    const int c = gi / per, j0 = (gi - c * per) * F::R;
+    // a group's data may exceed L2: last coil first, so that this pass and the one along
+    // y meet at the coils that are still there
+    const int gq = TAB ? total - 1 - gi : gi;
+    const int c = gq / per, j0 = (gq - c * per) * F::R;
     const int n_list = TAB ? a.tab[c].n_list : a.n_list;
     const int32_t* list = TAB ? a.tab[c].row_list : a.row_list;
     const int32_t* idx = TAB ? a.tab[c].idx : a.idx;
@@ -255,36 +262,36 @@ int lines_tile(const mpi_ctx* ctx, int L, int nx, int n_slabs) {
 }
 
 // The pass along y as a two-step FFT in registers: L = R1 R2 points per
-// column, y = r + R2 m.  A CTA takes 32 adjacent columns (one per lane) of one
-// (coil, z) plane.  Step 1: for each r, the R1 values y = r + R2 m are loaded
-// (rows of 32 columns: coalesced), transformed (R1-point DFT in registers) and
-// twiddled by w_L^(r k1) into shared memory [k1][r][column].  Step 2: for each
-// k1, the R2 values are read back, transformed (R2-point DFT) and stored to
+// column, y = r + R2 m.  A CTA takes TILE adjacent columns (32: a warp per r; 16: half
+// a warp) of one (coil, z) plane.  Step 1: for each r, the R1 values y = r + R2 m are
+// loaded (row segments of TILE columns: coalesced), transformed (R1-point DFT in
+// registers) and twiddled by w_L^(r k1) into shared memory [k1][r][column].  Step 2:
+// for each k1, the R2 values are read back, transformed (R2-point DFT) and stored to
 // rows k = k1 + R1 k2.  One shared-memory write and read per element (the
 // Stockham passes take one per radix stage plus two transposes).  The inverse
 // is the forward of the conjugated data, conjugated back.  Row mask as in
 // k_fft_lines: inverse, rows without samples are read as zeros; forward, only
-// rows with samples are stored.
-template <int R1, int R2, bool INV>
+// rows with samples are stored.  32 columns make longer bursts for volumes that do
+// not fit in L2; 16 make twice the CTAs, each with half the work: 16 coils of
+// 256^2, 128 CTAs of 32 columns on 152 SMs 7.0 us, 256 of 16 columns 4.9.  The width does
+// not change a column's arithmetic.
+template <int R1, int R2, bool INV, int TILE>
 __global__ void __launch_bounds__(256, 2) k_fft_cols_reg(float2* __restrict__ data, int nx, int n_slabs, long plane,
                                                       const float2* __restrict__ tw_g,
                                                       const uint8_t* __restrict__ rmask, int mask_nz) {
-  constexpr int L = R1 * R2;
-  __shared__ float2 sY[L * 32];  // [k1][r][column]
-  __shared__ float2 tw[L];
+  constexpr int L = R1 * R2, GROUPS = 256 / TILE;
+  __shared__ float2 sY[L * TILE];  // [k1][r][column]
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  for (int i = tid; i < L; i += 256) tw[i] = tw_g[i];
-  const int x_tiles = (nx + 31) / 32;
-  const int slab = (int)blockIdx.x / x_tiles, x0 = ((int)blockIdx.x - slab * x_tiles) * 32;
-  const bool ok = x0 + lane < nx;
-  float2* col = data + (size_t)slab * plane + x0 + lane;
+  const int tid = threadIdx.x, col_i = tid % TILE, w = tid / TILE;
+  const int x_tiles = (nx + TILE - 1) / TILE;
+  const int slab = (int)blockIdx.x / x_tiles, x0 = ((int)blockIdx.x - slab * x_tiles) * TILE;
+  const bool ok = x0 + col_i < nx;
+  float2* col = data + (size_t)slab * plane + x0 + col_i;
   const uint8_t* rm = rmask ? rmask + (size_t)(slab % mask_nz) * L : nullptr;
-  __syncthreads();
 #pragma unroll
-  for (int it = 0; it < (R2 + 7) / 8; ++it) {
-    const int r = w + 8 * it;
+  for (int it = 0; it < (R2 + GROUPS - 1) / GROUPS; ++it) {
+    const int r = w + GROUPS * it;
     if (r >= R2) break;
     float2 v[R1];
 #pragma unroll
@@ -294,20 +301,21 @@ __global__ void __launch_bounds__(256, 2) k_fft_cols_reg(float2* __restrict__ da
       if (ok && !(INV && rm && !rm[y])) t = col[(size_t)y * nx];
       v[m] = INV ? make_float2(t.x, -t.y) : t;
     }
+    float2 tw[R1];
+#pragma unroll
+    for (int k1 = 1; k1 < R1; ++k1) tw[k1] = __ldg(tw_g + r * k1);
     mpi_dft::dft_r<R1>(v);
 #pragma unroll
-    for (int k1 = 1; k1 < R1; ++k1) v[k1] = mpi_dft::cmulf(v[k1], tw[r * k1]);
-#pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) sY[(k1 * R2 + r) * 32 + lane] = v[k1];
+    for (int k1 = 0; k1 < R1; ++k1) sY[(k1 * R2 + r) * TILE + col_i] = k1 ? mpi_dft::cmulf(v[k1], tw[k1]) : v[0];
   }
   __syncthreads();
 #pragma unroll
-  for (int it = 0; it < (R1 + 7) / 8; ++it) {
-    const int k1 = w + 8 * it;
+  for (int it = 0; it < (R1 + GROUPS - 1) / GROUPS; ++it) {
+    const int k1 = w + GROUPS * it;
     if (k1 >= R1) break;
     float2 u[R2];
 #pragma unroll
-    for (int r = 0; r < R2; ++r) u[r] = sY[(k1 * R2 + r) * 32 + lane];
+    for (int r = 0; r < R2; ++r) u[r] = sY[(k1 * R2 + r) * TILE + col_i];
     mpi_dft::dft_r<R2>(u);
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) {
@@ -317,19 +325,29 @@ __global__ void __launch_bounds__(256, 2) k_fft_cols_reg(float2* __restrict__ da
   }
 }
 
+// Line kernels by choice: 8, 16, 32 lines per CTA (Stockham), or the register pass
+// along y with 32 (-1) or 16 (-16) columns per CTA.
+constexpr int kRegCols32 = -1, kRegCols16 = -16;
+int kernel_cols(int choice) { return choice == kRegCols32 ? 32 : (choice == kRegCols16 ? 16 : choice); }
+
 // Launch of the register pass along y for length L; false where L has no
 // (R1, R2) split or the geometry is not a y pass (lines of stride nx in
 // planes of `outer_stride`).
 template <bool INV>
-bool cols_reg_launch(mpi_ctx* ctx, int L, float2* data, int nx, long stride, int n_slabs, int inner,
+bool cols_reg_launch(mpi_ctx* ctx, int choice, int L, float2* data, int nx, long stride, int n_slabs, int inner,
                      long outer_stride, const float2* tw, const uint8_t* rmask, int mask_nz) {
   if (stride != nx || inner != 1) return false;
-  const long blocks = (long)n_slabs * ((nx + 31) / 32);
+  const int cols = kernel_cols(choice);
+  const long blocks = (long)n_slabs * ((nx + cols - 1) / cols);
   if (blocks == 0 || blocks > 0x7fffffffL) return false;
 #define MPI_CREG(n, r1, r2)                                                                                   \
   case n:                                                                                                    \
-    launch_pdl(ctx, k_fft_cols_reg<r1, r2, INV>, dim3((unsigned)blocks), dim3(256), 0, data, nx, n_slabs,       \
-               outer_stride, tw, rmask, mask_nz);                                                            \
+    if (cols == 32)                                                                                          \
+      launch_pdl(ctx, k_fft_cols_reg<r1, r2, INV, 32>, dim3((unsigned)blocks), dim3(256), 0, data, nx, n_slabs, \
+                 outer_stride, tw, rmask, mask_nz);                                                          \
+    else                                                                                                     \
+      launch_pdl(ctx, k_fft_cols_reg<r1, r2, INV, 16>, dim3((unsigned)blocks), dim3(256), 0, data, nx, n_slabs, \
+                 outer_stride, tw, rmask, mask_nz);                                                          \
     return true;
   switch (L) {
     MPI_CREG(64, 8, 8)
@@ -344,14 +362,14 @@ bool cols_reg_launch(mpi_ctx* ctx, int L, float2* data, int nx, long stride, int
 #undef MPI_CREG
 }
 
-// Launch of one line pass with tile width `tile` (8, 16 or 32 lines, or -1
-// for the register pass along y); false when the length / tile pair is not
+// Launch of one line pass with kernel `tile` (8, 16 or 32 lines, or a register
+// pass along y); false when the length / tile pair is not
 // compiled.
 template <bool INV>
 bool lines_launch_tile(mpi_ctx* ctx, int tile, int L, long blocks, float2* data, int nx, long stride, int n_slabs,
                        int inner, long outer_stride, long inner_stride, const float2* tw, const uint8_t* rmask,
                        int mask_nz) {
-  if (tile == -1) return cols_reg_launch<INV>(ctx, L, data, nx, stride, n_slabs, inner, outer_stride, tw, rmask, mask_nz);
+  if (tile < 0) return cols_reg_launch<INV>(ctx, tile, L, data, nx, stride, n_slabs, inner, outer_stride, tw, rmask, mask_nz);
 #define MPI_LINES_CASE(n)                                                                                     \
   case n:                                                                                                     \
     if (tile == 32 && n <= 128)                                                                               \
@@ -422,10 +440,10 @@ int lines_autotune(mpi_ctx* ctx, const long (&key)[10], int L, float2* data, int
   rec.n = 0;
   rec.choice = 0;
   float best = 1e30f;
-  const int cands[4] = {8, 16, 32, -1};
+  const int cands[5] = {8, 16, 32, kRegCols32, kRegCols16};
   for (int tile : cands) {
     if (tile > 0 && (long)L * tile / (kLineWarps * 32) > 16) continue;
-    const int cols = tile < 0 ? 32 : tile;  // columns per CTA
+    const int cols = kernel_cols(tile);  // columns per CTA
     const long blocks = (long)n_slabs * ((nx + cols - 1) / cols);
     if (blocks > 0x7fffffffL) continue;
     if (!lines_launch_tile<INV>(ctx, tile, L, blocks, scratch, nx, stride, n_slabs, inner, outer_stride,
@@ -453,12 +471,12 @@ int lines_autotune(mpi_ctx* ctx, const long (&key)[10], int L, float2* data, int
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (!rec.choice || cudaGetLastError() != cudaSuccess) return 0;
-  char buf[256];
+  char buf[320];
   auto tname = [](int t, char* b, size_t n) {
-    if (t < 0) snprintf(b, n, "register two-step");
+    if (t < 0) snprintf(b, n, "register two-step, %d columns", kernel_cols(t));
     else snprintf(b, n, "%d lines", t);
   };
-  char tn[32];
+  char tn[48];
   tname(rec.choice, tn, sizeof tn);
   int len = snprintf(buf, sizeof buf, "FFT line pass L=%d %s stride=%ld lines=%ld%s: %s (", L, INV ? "inverse" : "forward",
                      stride, (long)n_slabs * nx, rmask ? " row-masked" : "", tn);
@@ -507,7 +525,7 @@ mpi_status lines_dispatch(mpi_ctx* ctx, const char* name, float2* data, int L, i
   int tile = lines_choose<INV>(ctx, data, L, nx, stride, n_slabs, inner, outer_stride, inner_stride, tw, rmask,
                                mask_nz);
   if (!tile) tile = lines_tile(ctx, L, nx, n_slabs);
-  const int tw_cols = tile < 0 ? 32 : tile;
+  const int tw_cols = kernel_cols(tile);
   const int x_tiles = (nx + tw_cols - 1) / tw_cols;
   const long blocks = (long)n_slabs * x_tiles;
   if (blocks > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "too many FFT tiles");
@@ -1375,19 +1393,57 @@ mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const flo
 
 // ------------------------------------------------- passes of a batch's group
 
-int fft_cols_kernel(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse) {
+bool fft_cols_in_registers(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse) {
   const int ny = plan->ny, nx = plan->nx;
   const long plane = (long)ny * nx;
   const float2* tw = twiddle_table(ctx, ny);
   const int t = inverse ? lines_choose<true>(ctx, nullptr, ny, nx, nx, C, 1, plane, 0, tw, plan->row_has, 1)
                         : lines_choose<false>(ctx, nullptr, ny, nx, nx, C, 1, plane, 0, tw, plan->row_has, 1);
-  return t ? t : lines_tile(ctx, ny, nx, C);
+  return t < 0;
+}
+
+// The widest Stockham tile, or 32 register columns, unless tuning finds a faster width.
+mpi_status tune_fft_cols_group(mpi_ctx* ctx, bool registers, float2* data, int coils, int ny, int nx, bool inverse,
+                               const uint8_t* row_has, int* kernel) {
+  std::vector<int> cands;
+  if (registers) cands = {kRegCols32, kRegCols16};
+  else
+    for (int t : {32, 16, 8})
+      if ((long)ny * t / (kLineWarps * 32) <= 16 && (t == 8 || (t == 16 && ny <= 256) || (t == 32 && ny <= 128)))
+        cands.push_back(t);
+  *kernel = cands[0];
+  if (!ctx->autotune || cands.size() < 2) return MPI_OK;
+  cudaEvent_t e0, e1;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+    cudaGetLastError();
+    return set_err(ctx, MPI_ERR_CUDA, "grouped batch: tuning events");
+  }
+  mpi_status st = MPI_OK;
+  float best = 1e30f;
+  for (int k : cands) {
+    st = launch_fft_cols_group(ctx, k, data, coils, ny, nx, inverse, row_has);  // warm-up
+    cudaEventRecord(e0, ctx->stream);
+    for (int r = 0; r < 3 && st == MPI_OK; ++r)
+      st = launch_fft_cols_group(ctx, k, data, coils, ny, nx, inverse, row_has);
+    cudaEventRecord(e1, ctx->stream);
+    float ms = 0.f;
+    if (st == MPI_OK && (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+      st = cuda_check(ctx, cudaGetLastError(), "grouped batch tuning");
+    if (st) break;
+    if (ms < best) {
+      best = ms;
+      *kernel = k;
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  return st;
 }
 
 mpi_status launch_fft_cols_group(mpi_ctx* ctx, int kernel, float2* data, int coils, int ny, int nx, bool inverse,
                                  const uint8_t* row_has) {
   const float2* tw = twiddle_table(ctx, ny);
-  const int cols = kernel < 0 ? 32 : kernel;
+  const int cols = kernel_cols(kernel);
   const long blocks = (long)coils * ((nx + cols - 1) / cols);
   if (!tw || blocks > 0x7fffffffL) return set_err(ctx, MPI_ERR_SHAPE, "grouped FFT pass");
   MPI_PROF(ctx, KF_FFT_LINES);

@@ -68,8 +68,8 @@ struct mpi_ctx {
     long key[10];
     int choice;
     int n;
-    int cand[4];
-    float us[4];
+    int cand[5];
+    float us[5];
     std::string what;
   };
   std::vector<TuneRecord> tuned;
@@ -421,9 +421,11 @@ mpi_status launch_rows_scatter_inv(mpi_ctx* ctx, const mpi_plan* plan, const flo
                                    float2* data);
 
 // Passes of a batch's group of 2D slices on one grid: all their coils [coils][ny][nx]
-// in one launch.  fft_cols_kernel is the line kernel that the pass along y of a
-// slice with C coils runs (tuned or by rule); launch_fft_cols_group runs that one, with
-// row_has [coils][ny]; launch_rows_group gathers or scatters by a table per coil.
+// in one launch.  fft_cols_in_registers: whether the pass along y of a slice with C
+// coils is a register FFT (else Stockham lines), which decides its rounding;
+// tune_fft_cols_group times the widths of that kind on `data` (overwritten);
+// launch_fft_cols_group runs one, with row_has [coils][ny]; launch_rows_group
+// gathers or scatters by a table per coil.
 struct CoilSamples {
   const int32_t* idx;
   const int32_t* row_ptr;
@@ -431,7 +433,9 @@ struct CoilSamples {
   int n_list;
   float2* y;  // the coil's samples
 };
-int fft_cols_kernel(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse);
+bool fft_cols_in_registers(mpi_ctx* ctx, const mpi_plan* plan, int C, bool inverse);
+mpi_status tune_fft_cols_group(mpi_ctx* ctx, bool registers, float2* data, int coils, int ny, int nx, bool inverse,
+                               const uint8_t* row_has, int* kernel);
 mpi_status launch_fft_cols_group(mpi_ctx* ctx, int kernel, float2* data, int coils, int ny, int nx, bool inverse,
                                  const uint8_t* row_has);
 mpi_status launch_rows_group(mpi_ctx* ctx, float2* data, int coils, int ny, int nx, bool inverse,
