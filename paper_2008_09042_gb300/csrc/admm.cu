@@ -55,7 +55,10 @@ enum { S_RHO = 0, S_UFAC, S_NUM };
 // Sums are kept as pairs of FP32 values (h + l, about 48 bits) of exact differences
 // and products, from the threads to the partial sums: this GPU does two FP64
 // operations per clock and SM, and the fourteen per sample of the data blocks'
-// residuals took longer than everything else in their pass.
+// residuals took longer than everything else in their pass.  Every factor of a
+// product is multiplied by sum_scale first, a power of two that brings the data to
+// magnitude one (exact), since squares of FP32 values leave FP32's range long before
+// the values do; ratios of sums do not see it, norms are divided by it.
 
 struct Sum2 {
   float h = 0.f, l = 0.f;
@@ -83,12 +86,20 @@ __device__ __forceinline__ float diff_exact(float a, float b, float& e) {
   e = (a - (d - t)) - (b + t);
   return d;
 }
-__device__ __forceinline__ void sum2_diff_sq(Sum2& s, float2 a, float2 b) {
+// s += |k (a - b)|^2
+__device__ __forceinline__ void sum2_diff_sq(Sum2& s, float k, float2 a, float2 b) {
   float e;
   float d = diff_exact(a.x, b.x, e);
-  sum2_sq(s, d, e);
+  sum2_sq(s, k * d, k * e);
   d = diff_exact(a.y, b.y, e);
-  sum2_sq(s, d, e);
+  sum2_sq(s, k * d, k * e);
+}
+
+// The power of two for the data's largest finite magnitude (its bits, k_data_max);
+// 2^-126 to 2^126, 1 for data that are all zero.
+__device__ __forceinline__ float sum_scale(const unsigned* __restrict__ ymax) {
+  const unsigned bits = *ymax, e = min(max(bits >> 23, 1u), 253u);
+  return bits ? __uint_as_float((254u - e) << 23) : 1.f;
 }
 
 // Sum over a warp (valid in every lane).
@@ -378,6 +389,7 @@ struct MapsRows {
   const float2* ball;        // partial sums of the ball norms [T][C][kBallBlocks]
   const double* eps;         // ball radii [T][C]
   const double* sc;
+  const unsigned* ymax;      // see sum_scale
   float2* partials;
 };
 
@@ -492,7 +504,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_ball(MapsRows a
       const float2 v = a.ball[(size_t)tc * kBallBlocks + i];
       sum2_add(nrm, v.x, v.y);
     }
-    const double eps = a.eps[tc];
+    const double eps = a.eps[tc] * sum_scale(a.ymax);
     Sum2 root, radius;
     root.h = sqrtf(nrm.h);
     root.l = root.h > 0.f ? 0.5f * (fmaf(-root.h, root.h, nrm.h) + nrm.l) / root.h : 0.f;
@@ -553,7 +565,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_gather_dual(MapsRows a)
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
-  const float fu = (float)a.sc[S_UFAC];
+  const float fu = (float)a.sc[S_UFAC], ks = sum_scale(a.ymax);
   float2* b = buf[warp];
   Sum2 sums[2];
   const int per = (a.n_list_max + F::R - 1) / F::R, total = a.TC * per;
@@ -606,8 +618,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_gather_dual(MapsRows a)
           const float2 ap = make_float2(e.x * sg, e.y * sg);
           a.ap[i0 + m] = ap;
           a.uk[i0 + m] = make_float2(fu * d.uk.x + ap.x - d.yz.x, fu * d.uk.y + ap.y - d.yz.y);
-          sum2_diff_sq(sums[0], ap, d.yz);
-          sum2_diff_sq(sums[1], ap, d.ap);
+          sum2_diff_sq(sums[0], ks, ap, d.yz);
+          sum2_diff_sq(sums[1], ks, ap, d.ap);
         });
     __syncwarp();
   }
@@ -630,6 +642,7 @@ struct CoilSum {
   const float2 *z0, *u0, *p;             // residual: sum + z0 - ufac u0 - p
   float2 *r, *p_prev;                    //   into r and d; p kept as p_prev
   const double* sc;
+  const unsigned* ymax;  // see sum_scale
   float2* partials;  // per CTA: normal, <d, A d>; residual, |r|^2
 };
 
@@ -640,7 +653,7 @@ __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
   __shared__ float2 sh[kElemThreads / 32];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  const float fu = NORMAL ? 1.f : (float)a.sc[S_UFAC];
+  const float fu = NORMAL ? 1.f : (float)a.sc[S_UFAC], ks = sum_scale(a.ymax);
   Sum2 s[1];
   for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < a.total; i += (size_t)gridDim.x * kElemThreads) {
     const size_t t = i / a.N, n = i - t * a.N;
@@ -669,16 +682,16 @@ __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
       const float2 d = a.d[i];
       o = make_float2(o.x + d.x, o.y + d.y);
       a.Ad[i] = o;
-      sum2_mul(s[0], d.x, o.x);
-      sum2_mul(s[0], d.y, o.y);
+      sum2_mul(s[0], ks * d.x, ks * o.x);
+      sum2_mul(s[0], ks * d.y, ks * o.y);
     } else {
       const float2 z = a.z0[i], u = a.u0[i], p = a.p[i];
       o = make_float2(o.x + z.x - fu * u.x - p.x, o.y + z.y - fu * u.y - p.y);
       a.r[i] = o;
       a.d[i] = o;
       a.p_prev[i] = p;
-      sum2_mul(s[0], o.x, o.x);
-      sum2_mul(s[0], o.y, o.y);
+      sum2_mul(s[0], ks * o.x, ks * o.x);
+      sum2_mul(s[0], ks * o.y, ks * o.y);
     }
   }
   Sum2 out[1];
@@ -693,6 +706,7 @@ __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__
                                                             const float2* __restrict__ Ad, size_t n,
                                                             const float2* __restrict__ rr,
                                                             const float2* __restrict__ dad, int n_part,
+                                                            const unsigned* __restrict__ ymax,
                                                             float2* __restrict__ rr_new) {
   __shared__ float2 sh[kElemThreads / 32];
   __shared__ float s_a;
@@ -711,7 +725,7 @@ __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__
     rv = r[i0];
   }
   __syncthreads();
-  const float a = s_a;
+  const float a = s_a, ks = sum_scale(ymax);
   Sum2 s[1];
   for (size_t i = i0; i < n; i += step) {
     if (i != i0) {
@@ -726,8 +740,8 @@ __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__
     rv.y = fmaf(-a, av.y, rv.y);
     x[i] = xv;
     r[i] = rv;
-    sum2_mul(s[0], rv.x, rv.x);
-    sum2_mul(s[0], rv.y, rv.y);
+    sum2_mul(s[0], ks * rv.x, ks * rv.x);
+    sum2_mul(s[0], ks * rv.y, ks * rv.y);
   }
   Sum2 out[1];
   block_sums(s, sh, out);
@@ -737,12 +751,14 @@ __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__
 // |F_s S p + u_k - y|^2 of every (frame, coil): kBallBlocks partial sums each.
 __global__ void __launch_bounds__(kThreads) k_ball_norm(const float2* __restrict__ ap, const float2* __restrict__ uk,
                                                         const float2* __restrict__ y, int M,
-                                                        const double* __restrict__ sc, float2* __restrict__ partials) {
+                                                        const double* __restrict__ sc,
+                                                        const unsigned* __restrict__ ymax,
+                                                        float2* __restrict__ partials) {
   __shared__ float2 sh[kThreads / 32];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const int c = blockIdx.y;
-  const float fu = (float)sc[S_UFAC];
+  const float fu = (float)sc[S_UFAC], ks = sum_scale(ymax);
   Sum2 s[1];
   for (int m = blockIdx.x * kThreads + threadIdx.x; m < M; m += gridDim.x * kThreads) {
     const size_t i = (size_t)c * M + m;
@@ -750,10 +766,10 @@ __global__ void __launch_bounds__(kThreads) k_ball_norm(const float2* __restrict
     float e1, e2;  // ap + fu uk - y = d + e1 + e2 exactly
     float d = diff_exact(av.x, -(fu * uv.x), e1);
     d = diff_exact(d, yv.x, e2);
-    sum2_sq(s[0], d, e1 + e2);
+    sum2_sq(s[0], ks * d, ks * (e1 + e2));
     d = diff_exact(av.y, -(fu * uv.y), e1);
     d = diff_exact(d, yv.y, e2);
-    sum2_sq(s[0], d, e1 + e2);
+    sum2_sq(s[0], ks * d, ks * (e1 + e2));
   }
   Sum2 out[1];
   block_sums(s, sh, out);
@@ -768,19 +784,20 @@ __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__
                                                             const float2* __restrict__ p_prev, size_t n, double* sc,
                                                             float2* partials, unsigned* counter,
                                                             const float2* __restrict__ row_part, int n_row, double mu,
-                                                            double tau, double* __restrict__ hist) {
+                                                            double tau, const unsigned* __restrict__ ymax,
+                                                            double* __restrict__ hist) {
   __shared__ float2 sh[2 * kElemThreads / 32];
   __shared__ int last;
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  const float fu = (float)sc[S_UFAC];
+  const float fu = (float)sc[S_UFAC], ks = sum_scale(ymax);
   Sum2 s[2];
   for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
     const float2 pv = p[i], zv = z0[i], qv = p_prev[i];
     const float2 uv = u0[i];
     u0[i] = make_float2(fu * uv.x + pv.x - zv.x, fu * uv.y + pv.y - zv.y);
-    sum2_diff_sq(s[0], pv, zv);
-    sum2_diff_sq(s[1], pv, qv);
+    sum2_diff_sq(s[0], ks, pv, zv);
+    sum2_diff_sq(s[1], ks, pv, qv);
   }
   Sum2 out[2];
   block_sums(s, sh, out);
@@ -805,7 +822,7 @@ __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__
   }
   block_sums(s, sh, out);
   if (threadIdx.x) return;
-  const double prim = sqrt(to_double(out[0])), rho = sc[S_RHO], dual = rho * sqrt(to_double(out[1]));
+  const double prim = sqrt(to_double(out[0])) / ks, rho = sc[S_RHO], dual = rho * (sqrt(to_double(out[1])) / ks);
   hist[0] = prim;
   hist[1] = dual;
   hist[2] = rho;
@@ -823,6 +840,19 @@ __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__
 __global__ void k_admm_start(double* sc, double rho0) {
   sc[S_RHO] = rho0;
   sc[S_UFAC] = 1.0;
+}
+
+// The bits of the largest finite |Re| or |Im| of n values (*ymax cleared before).
+__global__ void __launch_bounds__(kElemThreads) k_data_max(const float2* __restrict__ y, size_t n, unsigned* ymax) {
+  unsigned m = 0;
+  for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
+    const float2 v = y[i];
+    const unsigned a = __float_as_uint(v.x) & 0x7fffffffu, b = __float_as_uint(v.y) & 0x7fffffffu;
+    if (a < 0x7f800000u) m = max(m, a);
+    if (b < 0x7f800000u) m = max(m, b);
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(ymax, m);
 }
 
 // mask[t][idx[t][m]] = 1
@@ -937,7 +967,7 @@ size_t admm_maps_layout(const mpi_ctx* ctx, const mpi_plan* const* plans, int T,
   m->u0 = cplx(TN);
   m->ap = cplx(CM);
   m->uk = cplx(CM);
-  m->counters = (unsigned*)take(sizeof(unsigned));
+  m->counters = (unsigned*)take(2 * sizeof(unsigned));
   m->zero_bytes = (char*)mem + off - m->zero_begin;
   m->zk = cplx(CM);
   float2** img[] = {&m->z0, &m->r, &m->d[0], &m->d[1], &m->Ad, &m->p_prev};
@@ -1008,6 +1038,10 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   MPI_PROF(ctx, KF_SOLVER);
   k_admm_start<<<1, 1, 0, ctx->stream>>>(m.sc, prm->rho0);
   MPI_LAUNCH_CHECK(ctx, "k_admm_start");
+  const unsigned* ymax = m.counters + 1;
+  MPI_PROF(ctx, KF_SOLVER);
+  k_data_max<<<elem_blocks((size_t)TC * M), kElemThreads, 0, ctx->stream>>>(m.in_y, (size_t)TC * M, m.counters + 1);
+  MPI_LAUNCH_CHECK(ctx, "k_data_max");
   // MIXED: BF16 maps in the CG iterations; FP32 ones for the constraint-side
   // products and the CG's first residual
   TRY(mpi_basis_expand(ctx, basis, (const mpi_c32*)m.in_alpha, C, (mpi_c32*)m.S,
@@ -1061,6 +1095,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   rows.ball = m.ball_part;
   rows.eps = m.in_eps;
   rows.sc = m.sc;
+  rows.ymax = ymax;
   rows.partials = m.row_part;
   CoilSum sum{};
   sum.W = m.W;
@@ -1075,6 +1110,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   sum.r = m.r;
   sum.p_prev = m.p_prev;
   sum.sc = m.sc;
+  sum.ymax = ymax;
 
   for (int it = 0; it < prm->n_outer; ++it) {
     // z_0 = prox_{TV/rho}(p + u_0), z_k = Pi(F_s S p + u_k)
@@ -1082,7 +1118,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
                        prm->n_tv, m.tv, m.z0));
     MPI_PROF(ctx, KF_SOLVER);
     launch_pdl(ctx, k_ball_norm, dim3(kBallBlocks, (unsigned)TC), dim3(kThreads), 0, m.ap, m.uk, m.in_y, M,
-               m.sc, m.ball_part);
+               m.sc, ymax, m.ball_part);
     MPI_LAUNCH_CHECK(ctx, "k_ball_norm");
     TRY(launch_maps_rows(ctx, nx, ROWS_SCATTER, rows, rblk));
     // r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p
@@ -1111,7 +1147,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
       MPI_LAUNCH_CHECK(ctx, "k_coil_sum<normal>");
       MPI_PROF(ctx, KF_SOLVER);
       launch_pdl(ctx, k_cg_update, dim3(eblk), dim3(kElemThreads), 0, m.p, m.r, m.d[cur], m.Ad, TN, rr[par], dad,
-                 (int)eblk, rr[par ^ 1]);
+                 (int)eblk, ymax, rr[par ^ 1]);
       MPI_LAUNCH_CHECK(ctx, "k_cg_update");
       par ^= 1;
     }
@@ -1120,7 +1156,8 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     TRY(launch_maps_rows(ctx, nx, ROWS_GATHER, rows, rblk));
     MPI_PROF(ctx, KF_SOLVER);
     launch_pdl(ctx, k_admm_dual, dim3(eblk), dim3(kElemThreads), 0, m.u0, m.p, m.z0, m.p_prev, TN, m.sc,
-               m.part + 3 * kMaxElemBlocks, m.counters, m.row_part, (int)rblk, prm->mu, prm->tau, m.hist + 3 * (size_t)it);
+               m.part + 3 * kMaxElemBlocks, m.counters, m.row_part, (int)rblk, prm->mu, prm->tau, ymax,
+               m.hist + 3 * (size_t)it);
     MPI_LAUNCH_CHECK(ctx, "k_admm_dual");
   }
   return MPI_OK;

@@ -14,7 +14,7 @@ struct AdmmMaps {
   float2* W;         // [T][C][N]
   float2 *p, *u0, *ap, *uk, *zk;
   float2 *z0, *r, *d[2], *Ad, *p_prev, *tv;
-  unsigned* counters;
+  unsigned* counters;  // the dual's arrival counter, the data's largest magnitude
   char* zero_begin;
   size_t zero_bytes;
   double* sc;

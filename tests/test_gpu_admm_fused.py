@@ -100,3 +100,27 @@ def test_fused_solve_without_cg_steps(mp):
     p, h = mp.image_solve(ctx, plan, B, c64(w.random_coefficients(2, 5, seed=2)), y, np.ones(2), n_outer=3, n_cg=0,
                           n_tv=0)
     assert float(p.abs().max()) == 0.0 and np.isfinite(h).all()
+
+
+@pytest.mark.parametrize("exponent", [-90, 90])
+def test_fused_solve_of_data_whose_squares_leave_fp32(mp, exponent):
+    # data and radii scaled by 2^e, rho by 2^-e: the image scales along; |y|^2 is 2^-180 or 2^180
+    ny = nx = 64
+    C, s = 3, 2.0 ** exponent
+    idx = _mask("points", ny, nx, 1)
+    U = w.smooth_orthonormal_basis(ny, nx, 8, seed=3) * np.sqrt(ny * nx)
+    rng = np.random.default_rng(2)
+    alpha = c64(w.random_coefficients(C, 8, seed=4))
+    y = c64((rng.normal(size=(C, len(idx))) + 1j * rng.normal(size=(C, len(idx)))) * s)
+    eps = np.full(C, 0.3 * np.sqrt(len(idx)) * s)
+    out = []
+    for line_kernel in (0, 8):
+        ctx = mp.Context(0)
+        ctx.set_line_kernel(line_kernel)
+        p, h = mp.image_solve(ctx, mp.Plan(ctx, (ny, nx), sample_idx=idx), mp.Basis(ctx, U.T), alpha, y, eps,
+                              n_outer=4, n_cg=3, n_tv=11, rho0=1.0 / s)
+        ctx.synchronize()
+        out.append((f64(p), h))
+    assert float(np.linalg.norm(out[1][0])) > 0
+    assert nrmse(out[0][0], out[1][0]) < 1e-4
+    np.testing.assert_allclose(out[0][1], out[1][1], rtol=1e-3)
