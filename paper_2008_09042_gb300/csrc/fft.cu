@@ -294,11 +294,14 @@ __global__ void __launch_bounds__(256, 2) k_fft_cols_reg(float2* __restrict__ da
     const int r = w + GROUPS * it;
     if (r >= R2) break;
     float2 v[R1];
+    uint8_t keep[R1];  // the mask's loads in flight together, then the values'
+#pragma unroll
+    for (int m = 0; m < R1; ++m) keep[m] = INV && rm ? rm[r + R2 * m] : 1;
 #pragma unroll
     for (int m = 0; m < R1; ++m) {
       const int y = r + R2 * m;
       float2 t = make_float2(0.f, 0.f);
-      if (ok && !(INV && rm && !rm[y])) t = col[(size_t)y * nx];
+      if (ok && keep[m]) t = col[(size_t)y * nx];
       v[m] = INV ? make_float2(t.x, -t.y) : t;
     }
     float2 tw[R1];
@@ -329,6 +332,18 @@ __global__ void __launch_bounds__(256, 2) k_fft_cols_reg(float2* __restrict__ da
 // along y with 32 (-1) or 16 (-16) columns per CTA.
 constexpr int kRegCols32 = -1, kRegCols16 = -16;
 int kernel_cols(int choice) { return choice == kRegCols32 ? 32 : (choice == kRegCols16 ? 16 : choice); }
+
+// Whether lines of length L with this geometry have a register pass.
+bool cols_reg_has(int L, int nx, long stride, int inner) {
+  return stride == nx && inner == 1 && (L == 64 || L == 96 || L == 128 || L == 192 || L == 256 || L == 320);
+}
+
+// Passes along y over at most this many bytes take 16 register columns untimed.  Over
+// 1 to 32 coils of 64^2 to 320^2 (26 MB), masked and not, they were the fastest of the
+// five candidates or within the timer's 0.7 us of it (32 coils of 256^2: 8-line Stockham
+// 11.1 us, 32 columns 8.4, 16 columns 7.7), while timing all five cost a plan's first call
+// 0.2 ms and let noise choose.  Beyond half of L2 a pass runs at HBM's rate and is timed.
+constexpr size_t kRegCols16Bytes = 64u << 20;
 
 // Launch of the register pass along y for length L; false where L has no
 // (R1, R2) split or the geometry is not a y pass (lines of stride nx in
@@ -501,10 +516,12 @@ int lines_choose(mpi_ctx* ctx, float2* data, int L, int nx, long stride, int n_s
   // a caller's fixed choice (mpi_ctx_set_line_kernel), where this pass has it
   if (ctx->line_kernel) {
     const int t = ctx->line_kernel;
-    const bool ok = t == -1 ? (L == 64 || L == 96 || L == 128 || L == 192 || L == 256 || L == 320) && stride == nx && inner == 1
+    const bool ok = t == -1 ? cols_reg_has(L, nx, stride, inner)
                             : (t == 8 || (t == 16 && L <= 256) || (t == 32 && L <= 128));
     if (ok) tile = t;
   }
+  if (!tile && cols_reg_has(L, nx, stride, inner) && (size_t)n_slabs * L * nx * sizeof(float2) <= kRegCols16Bytes)
+    tile = kRegCols16;
   for (const auto& r : ctx->tuned) {
     if (tile) break;
     if (std::equal(r.key, r.key + 10, key)) tile = r.choice;
