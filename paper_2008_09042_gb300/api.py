@@ -14,11 +14,17 @@ from . import _lib
 from ._lib import PREC, check, load
 
 
+_Tensor, _c64 = torch.Tensor, torch.complex64
+
+
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None and t.numel() > 0 else ctypes.c_void_p(0)
+    # a plain int: every entry point declares its pointers as c_void_p
+    return t.data_ptr() if t is not None and t.numel() > 0 else None
 
 
 def _need(t, shape, name):
+    if isinstance(t, _Tensor) and t.dtype is _c64 and t.shape == shape and t.is_cuda and t.is_contiguous():
+        return t
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch tensor")
     if t.dtype != torch.complex64 or not t.is_cuda or not t.is_contiguous():

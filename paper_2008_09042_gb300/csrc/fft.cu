@@ -1246,7 +1246,7 @@ mpi_status launch_fft_cols_window(mpi_ctx* ctx, float2* grid, int C, int G, cons
     const size_t smem = (size_t)L * 16 * sizeof(float2);                                                            \
     auto kern = inverse ? k_fft_cols_win<r1, r2, true> : k_fft_cols_win<r1, r2, false>;                             \
     if (smem > 48 * 1024) { /* more than a launch may ask for without it */                                        \
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);           \
+      cudaError_t e = smem_attr(ctx, (const void*)kern);                                                            \
       if (e != cudaSuccess) return cuda_check(ctx, e, "windowed pass attributes");                                  \
     }                                                                                                               \
     launch_pdl(ctx, kern, dim3((unsigned)wblocks), dim3(256), smem, grid, C, win, x_first, x_tiles, tw);             \

@@ -73,6 +73,7 @@ struct mpi_ctx {
     std::string what;
   };
   std::vector<TuneRecord> tuned;
+  std::vector<const void*> smem_granted;  // kernels that smem_attr has prepared
 };
 
 struct mpi_plan {
@@ -192,6 +193,22 @@ inline cudaError_t launch_pdl(mpi_ctx* ctx, void (*kern)(KArgs...), dim3 grid, d
   cfg.attrs = attr;
   cfg.numAttrs = ctx->pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+// Lets `kern` be launched with any dynamic shared memory that the device has: set on a
+// context's first launch of it, to the same value by every context, rather than to each
+// launch's size before every launch (0.4 us of host time each, on calls of 15 to 50 us).
+inline cudaError_t smem_attr(mpi_ctx* ctx, const void* kern) {
+  for (const void* k : ctx->smem_granted)
+    if (k == kern) return cudaSuccess;
+  int most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess) ctx->smem_granted.push_back(kern);
+  return e;
 }
 
 #define MPI_LAUNCH_CHECK(ctx, what)                                   \

@@ -340,7 +340,7 @@ mpi_status launch_expand_tc(mpi_ctx* ctx, const mpi_basis* b, int mode, const Ex
   cudaError_t e = cudaSuccess;
 #define MPI_TC_CASE(m)                                                                                        \
   case m:                                                                                                     \
-    e = cudaFuncSetAttribute(k_expand_tc<m>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
+    e = smem_attr(ctx, (const void*)k_expand_tc<m>);                                                         \
     if (e != cudaSuccess) return cuda_check(ctx, e, "tc smem attribute");                                    \
     MPI_PROF(ctx, KF_EXPAND);                                                                                \
     launch_pdl(ctx, k_expand_tc<m>, dim3(grid), dim3(kThreads), smem, map, a, stages);                                           \

@@ -630,7 +630,7 @@ mpi_status launch_expand_tf32(mpi_ctx* ctx, const mpi_basis* b, int mode, const 
     return set_err(ctx, MPI_ERR_UNSUPPORTED, "3xTF32 expansion: odd K box count in this mode");
 #define MPI_TF_LAUNCH(m, o)                                                                                   \
   do {                                                                                                        \
-    e = cudaFuncSetAttribute(k_expand_tf32x3<m, o>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem); \
+    e = smem_attr(ctx, (const void*)k_expand_tf32x3<m, o>);                                                     \
     if (e != cudaSuccess) return cuda_check(ctx, e, "tf32 smem attribute");                                  \
     MPI_PROF(ctx, KF_EXPAND);                                                                                \
     launch_pdl(ctx, k_expand_tf32x3<m, o>, grid, dim3(kThreads32), pl.smem, map, a, pl.stages);            \

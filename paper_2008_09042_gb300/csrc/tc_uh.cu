@@ -502,13 +502,13 @@ mpi_status launch_uh_tc(mpi_ctx* ctx, const mpi_basis* b, const float2* V, int C
     const CUtensorMap& um = *(const CUtensorMap*)(bf ? b->umap_bf : b->umap32);
     cudaError_t e;
     if (bf) {
-      e = cudaFuncSetAttribute(k_uh_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+      e = smem_attr(ctx, (const void*)k_uh_tc<true>);
       if (e != cudaSuccess) return cuda_check(ctx, e, "uh smem attribute");
       MPI_PROF(ctx, KF_UHV);
       launch_pdl(ctx, k_uh_tc<true>, grid, dim3(kUhThreads), pl.smem, um, vmap, a);
       MPI_LAUNCH_CHECK(ctx, "k_uh_tc<bf16>");
     } else {
-      e = cudaFuncSetAttribute(k_uh_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+      e = smem_attr(ctx, (const void*)k_uh_tc<false>);
       if (e != cudaSuccess) return cuda_check(ctx, e, "uh smem attribute");
       MPI_PROF(ctx, KF_UHV);
       launch_pdl(ctx, k_uh_tc<false>, grid, dim3(kUhThreads), pl.smem, um, vmap, a);
