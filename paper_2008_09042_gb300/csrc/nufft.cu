@@ -246,23 +246,30 @@ __device__ __forceinline__ void spread_store(float2* __restrict__ grid, int C, i
     if (c0 + j < C) grid[((size_t)(c0 + j) * G + gy) * G + gx] = make_float2(s * acc[2 * j], s * acc[2 * j + 1]);
 }
 
+struct SpreadArgs {
+  const float4* ys;
+  int C, Cp, G;
+  const int32_t* cell_ptr;
+  const int32_t* cell_sx;
+  const float* cell_w;
+  const int32_t* dense;  // the plan's list of dense cells
+  int n_dense;
+  float2* grid;
+};
+
 // Output-driven spreading, sparse cells: thread (gy, gx, 4 NG coils) sums the
 // samples whose W x W footprint covers its cell, i.e. whose first tap is
 // (gy - a, gx - b) (mod G) for 0 <= a, b < W, and stores the cell once; no
 // atomics.  A cell whose window holds more than kSpreadDense samples is left
-// to k_nufft_spread_dense (its thread would hold the CTA up).  Finding a cell's
+// to spread_dense (its thread would hold the CTA up).  Finding a cell's
 // samples (the CSR ranges of W rows) costs about as much as adding a few coils of
 // them, so a thread takes up to three groups of four coils: at 256^2, 12 coils,
-// 64 spokes 54 us (both kernels) -> 40.
+// 64 spokes 54 us (both kinds of cells) -> 40.
 template <int W, int NG>
-__global__ void __launch_bounds__(256) k_nufft_spread(const float4* __restrict__ ys, int C, int Cp, int G,
-                                                      const int32_t* __restrict__ cell_ptr,
-                                                      const int32_t* __restrict__ cell_sx,
-                                                      const float* __restrict__ cell_w,
-                                                      float2* __restrict__ grid) {
-  mpi_ptx::pdl_trigger();
-  const int gx = blockIdx.x * 32 + threadIdx.x, gy = blockIdx.y * 8 + threadIdx.y;
-  const int c0 = blockIdx.z * kSpreadCoils * NG;
+__device__ __forceinline__ void spread_sparse(const SpreadArgs& s, int gx, int gy, int c0) {
+  const int C = s.C, Cp = s.Cp, G = s.G;
+  const int32_t *cell_ptr = s.cell_ptr, *cell_sx = s.cell_sx;
+  const float* cell_w = s.cell_w;
   if (gx >= G || gy >= G) return;
   // the plan's ranges do not depend on earlier work
   int lo[W], hi[W], n = 0;
@@ -279,7 +286,7 @@ __global__ void __launch_bounds__(256) k_nufft_spread(const float4* __restrict__
   if (n > kSpreadDense) return;
   mpi_ptx::pdl_wait();
   const int ystride = Cp / 2;
-  const float4* yc = ys + c0 / 2;
+  const float4* yc = s.ys + c0 / 2;
   float acc[8 * NG] = {};
   if (n > 0) {
 #pragma unroll
@@ -295,28 +302,23 @@ __global__ void __launch_bounds__(256) k_nufft_spread(const float4* __restrict__
       }
     }
   }
-  spread_store<NG>(grid, C, G, c0, gy, gx, acc);
+  spread_store<NG>(s.grid, C, G, c0, gy, gx, acc);
 }
 
 // Output-driven spreading, dense cells (the plan's list of cells whose window
-// holds more than kSpreadDense samples): warp (cell, 4 NG coils), the lanes
+// holds more than kSpreadDense samples): warp (cell i, 4 NG coils), the lanes
 // taking every 32nd sample of each row range, then a butterfly sum.
 template <int W, int NG>
-__global__ void __launch_bounds__(256) k_nufft_spread_dense(const float4* __restrict__ ys, int C, int Cp, int G,
-                                                            const int32_t* __restrict__ cell_ptr,
-                                                            const int32_t* __restrict__ cell_sx,
-                                                            const float* __restrict__ cell_w,
-                                                            const int32_t* __restrict__ dense, int n_dense,
-                                                            float2* __restrict__ grid) {
-  mpi_ptx::pdl_trigger();
+__device__ __forceinline__ void spread_dense(const SpreadArgs& s, int i, int c0) {
+  const int C = s.C, Cp = s.Cp, G = s.G;
+  const int32_t *cell_ptr = s.cell_ptr, *cell_sx = s.cell_sx;
+  const float* cell_w = s.cell_w;
   const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int c0 = blockIdx.y * kSpreadCoils * NG;
   mpi_ptx::pdl_wait();
-  if (i >= n_dense) return;
-  const int cell = dense[i], gy = cell / G, gx = cell % G;
+  if (i >= s.n_dense) return;
+  const int cell = s.dense[i], gy = cell / G, gx = cell % G;
   const int ystride = Cp / 2;
-  const float4* yc = ys + c0 / 2;
+  const float4* yc = s.ys + c0 / 2;
   float acc[8 * NG] = {};
 #pragma unroll
   for (int a = 0; a < W; ++a) {
@@ -331,7 +333,23 @@ __global__ void __launch_bounds__(256) k_nufft_spread_dense(const float4* __rest
   for (int j = 0; j < 8 * NG; ++j)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-  if (lane == 0) spread_store<NG>(grid, C, G, c0, gy, gx, acc);
+  if (lane == 0) spread_store<NG>(s.grid, C, G, c0, gy, gx, acc);
+}
+
+// Both kinds of cells in one launch, the dense ones' CTAs (a warp per cell) first: a
+// grid cell has one kind, so they need no order, and neither fills the chip by itself
+// (the dense cells of a radial trajectory's centre are few and long, most sparse ones
+// are empty).
+template <int W, int NG>
+__global__ void __launch_bounds__(256) k_nufft_spread(SpreadArgs s, int dense_ctas) {
+  mpi_ptx::pdl_trigger();
+  const int c0 = blockIdx.y * kSpreadCoils * NG, warp = threadIdx.x >> 5;
+  if ((int)blockIdx.x < dense_ctas) {
+    spread_dense<W, NG>(s, blockIdx.x * 8 + warp, c0);
+  } else {
+    const int b = blockIdx.x - dense_ctas, tx = (s.G + 31) / 32;
+    spread_sparse<W, NG>(s, b % tx * 32 + (threadIdx.x & 31), b / tx * 8 + warp, c0);
+  }
 }
 
 float axis_sign(int n) { return ((n / 2) & 1) ? -1.f : 1.f; }
@@ -494,21 +512,13 @@ mpi_status nufft_adjoint(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, in
     MPI_LAUNCH_CHECK(ctx, "k_nufft_sort_y");
     const int ng = spread_groups(C, G);
     const unsigned groups = (unsigned)(Cp / (kSpreadCoils * ng));
-    const dim3 sgrid((unsigned)((G + 31) / 32), (unsigned)((G + 7) / 8), groups);
-    const dim3 dgrid((unsigned)((plan->n_dense + 7) / 8), groups);
-    const float4* ys4 = (const float4*)ys;
-#define MPI_SPREAD(w, g)                                                                                    \
-  if (plan->W == w && ng == g) {                                                                            \
-    MPI_PROF(ctx, KF_NUFFT);                                                                                \
-    launch_pdl(ctx, k_nufft_spread<w, g>, sgrid, dim3(32, 8), 0, ys4, C, Cp, G, plan->cell_ptr, plan->cell_sx, \
-               plan->cell_w, grid);                                                                         \
-    if (plan->n_dense > 0) {                                                                                \
-      MPI_LAUNCH_CHECK(ctx, "k_nufft_spread");                                                              \
-      MPI_PROF(ctx, KF_NUFFT);                                                                              \
-      launch_pdl(ctx, k_nufft_spread_dense<w, g>, dgrid, dim3(256), 0, ys4, C, Cp, G, plan->cell_ptr,        \
-                 plan->cell_sx, plan->cell_w, plan->cell_dense, plan->n_dense, grid);                       \
-    }                                                                                                       \
-  }
+    const int dense_ctas = (plan->n_dense + 7) / 8;
+    const dim3 sgrid((unsigned)(dense_ctas + (G + 31) / 32 * ((G + 7) / 8)), groups);
+    const SpreadArgs sa{(const float4*)ys, C, Cp, G, plan->cell_ptr, plan->cell_sx, plan->cell_w, plan->cell_dense,
+                        plan->n_dense, grid};
+    MPI_PROF(ctx, KF_NUFFT);
+#define MPI_SPREAD(w, g) \
+  if (plan->W == w && ng == g) launch_pdl(ctx, k_nufft_spread<w, g>, sgrid, dim3(256), 0, sa, dense_ctas);
 #define MPI_W_CASE(w) MPI_SPREAD(w, 1) MPI_SPREAD(w, 2) MPI_SPREAD(w, 3)
     if (plan->W < 2 || plan->W > 8) return set_err(ctx, MPI_ERR_ARG, "kernel width");
     MPI_W_CASE(2) MPI_W_CASE(3) MPI_W_CASE(4) MPI_W_CASE(5) MPI_W_CASE(6) MPI_W_CASE(7) MPI_W_CASE(8)
