@@ -1202,14 +1202,13 @@ bool rows_supported(const mpi_basis* basis, int Cmax, mpi_precision prec) {
   return false;
 }
 
-mpi_status expand_rows(mpi_ctx* ctx, const mpi_plan* plan0, const mpi_basis* basis, int mode, const ExpandRow* rows,
-                       int nrows, int Cmax, mpi_precision prec, int row_ctas) {
+mpi_status expand_rows(mpi_ctx* ctx, const mpi_plan* plan0, const mpi_basis* basis, int mode, const ExpandRow* ctas,
+                       int n_ctas, int Cmax, mpi_precision prec) {
   if (!rows_supported(basis, Cmax, prec)) return set_err(ctx, MPI_ERR_UNSUPPORTED, "grouped expansion: shape");
-  if (nrows < 1 || nrows > 65535) return set_err(ctx, MPI_ERR_SHAPE, "grouped expansion: row count");
+  if (n_ctas < 1) return set_err(ctx, MPI_ERR_SHAPE, "grouped expansion: CTA count");
   ExpandArgs a = base_args(plan0, basis, Cmax);
-  a.rows = rows;
-  a.nrows = nrows;
-  a.row_ctas = row_ctas;
+  a.rows = ctas;
+  a.n_ctas = n_ctas;
   a.kname = mode == EX_FWD ? "k_expand<grouped fwd>" : "k_expand<grouped adj>";
   if (prec == MPI_PREC_BF16) return launch_expand_tc(ctx, basis, mode, a);
   return launch_expand_tf32(ctx, basis, mode, a);

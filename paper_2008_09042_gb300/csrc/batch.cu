@@ -9,18 +9,18 @@
 // stay valid for the life of the batch.
 //
 // Grouped expansion: consecutive slices on Cartesian plans that share a dense
-// basis (FP32 or BF16, every slice's coils within one tensor-core pass) form a
-// group.  The group's basis expansion is one launch whose grid rows are its
-// slices (a device table gives each row its coefficients, image, per-coil data
-// and output); the rows stream the same basis tiles in step, so the basis is
-// read from DRAM about once per group instead of once per slice.  Each slice's
-// per-coil images live in a batch-owned buffer between the expansion and the
-// FFT passes.  From kGroupedPasses slices on, the FFT passes take all coils of a
-// group's slices in one launch too (per run of slices whose pass along y is of the
-// same kind, register or Stockham, so that a slice's values stay those of its own
-// call; its width is timed for the group), with a
-// table of every coil's sampling.  How many CTAs each row gets is chosen at creation by
-// timing the candidates (an autotuner decision the context records).
+// basis (FP32 or BF16, every slice's coils within one tensor-core pass)
+// form a group.  The group's basis expansion is one launch over its slices (a device
+// table gives each CTA its slice's coefficients, image, per-coil data and output);
+// the slices stream the same basis tiles in step, so the basis is read from DRAM
+// about once per group instead of once per slice.  Each slice's per-coil images live
+// in a batch-owned buffer between the expansion and the FFT passes.  From
+// kGroupedPasses slices on, the FFT passes take all coils of a group's slices in one
+// launch too (per run of slices whose pass along y is of the same kind, register or
+// Stockham, so that a slice's values stay those of its own call; its width is timed
+// for the group), with a table of every coil's sampling.  How many CTAs each slice gets
+// is chosen at creation by timing the candidates (an autotuner decision the context
+// records).
 #include <algorithm>
 #include <cstdio>
 #include <numeric>
@@ -36,7 +36,7 @@ struct mpi_batch {
   int n = 0;
   int64_t kernels = 0;  // kernels per replay
   void* buf = nullptr;   // per-coil images of one group [sum C][N]
-  void* rows = nullptr;  // row tables of every group (device)
+  void* ctas = nullptr;  // CTA tables of every group's expansions (device)
   void* tabs = nullptr;  // sampling tables and row masks of the grouped passes (device)
   int groups = 0;        // grouped launches per direction
 };
@@ -62,8 +62,9 @@ struct Group {
   std::vector<int> idx;  // slices, in recording order
   int Cmax = 0;
   long sumC = 0;
-  size_t fwd_rows = 0, adj_rows = 0;  // offsets (rows) into the device row table
-  int row_ctas = 0;
+  // grouped expansions: the CTAs of a launch and their offsets in the device CTA table
+  size_t fwd_ctas = 0, adj_ctas = 0;
+  int n_ctas = 0;
   // grouped passes: runs of slices (first, count in coils) per direction and kernel
   struct Run {
     bool registers;
@@ -81,13 +82,13 @@ bool groupable(const mpi_batch_slice& s, mpi_precision prec) {
 
 // The group's forward and adjoint expansions, and its slices' FFT passes.
 mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g, int kind, mpi_precision prec,
-                        const ExpandRow* rows, float2* buf) {
+                        const ExpandRow* ctas, float2* buf) {
   const mpi_batch_slice& s0 = sl[g.idx[0]];
   const long N = s0.plan->N;
   const int nr = (int)g.idx.size(), ny = s0.plan->ny, nx = s0.plan->nx;
   mpi_status st = MPI_OK;
   if (kind & MPI_BATCH_FORWARD) {
-    st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, rows + g.fwd_rows, nr, g.Cmax, prec, g.row_ctas);
+    st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, ctas + g.fwd_ctas, g.n_ctas, g.Cmax, prec);
     for (const Group::Run& r : g.fwd)
       if (st == MPI_OK)
         st = launch_fft_cols_group(ctx, r.kernel, buf + r.first * N, r.coils, ny, nx, false,
@@ -112,7 +113,7 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
       st = plan_kspace_to_image(ctx, s.plan, (const float2*)s.y, s.C, buf + off * N);
       off += s.C;
     }
-    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_ADJ, rows + g.adj_rows, nr, g.Cmax, prec, g.row_ctas);
+    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_ADJ, ctas + g.adj_ctas, g.n_ctas, g.Cmax, prec);
   }
   return st;
 }
@@ -179,17 +180,57 @@ mpi_status group_tables(mpi_ctx* ctx, const mpi_batch_slice* sl, std::vector<Gro
   return cuda_check(ctx, cudaMemcpy(*out, host.data(), bytes, cudaMemcpyHostToDevice), "batch: group tables");
 }
 
-// CTAs per row for a group's expansion: every candidate timed over three
-// launches of the group's forward expansion (between events on the context's
-// stream, after one warm-up launch), the fastest kept.
-mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_precision prec,
-                      const ExpandRow* rows) {
+// The CTAs of a group's expansion launches, `total` of them (one per slice at least),
+// shared out in proportion to 1 + skew x (a slice's coil columns, padded to whole
+// MMAs, / 64): a tile of a slice with more coils takes more MMA and epilogue time,
+// and has a shorter ring beside its larger coefficient operand, so equal shares
+// would leave the CTAs of small coil arrays waiting for the large ones'.  With shares
+// that match, all slices also pass through the basis in step, so that it leaves DRAM
+// about once.  A slice's values do not depend on its share.
+void share_ctas(const mpi_batch_slice* sl, const Group& g, int total, float skew, float2* buf, int n_tiles,
+                std::vector<ExpandRow>* fwd, std::vector<ExpandRow>* adj) {
+  const int n = (int)g.idx.size();
+  std::vector<float> w(n);
+  std::vector<int> share(n, 1);
+  for (int i = 0; i < n; ++i) w[i] = 1.f + skew * (float)((2 * sl[g.idx[i]].C + 15) / 16 * 16) / 64.f;
+  for (int used = n; used < total; ++used) {
+    int most = -1;
+    for (int i = 0; i < n; ++i)
+      if (share[i] < n_tiles && (most < 0 || w[i] * share[most] > w[most] * share[i])) most = i;
+    if (most < 0) break;
+    ++share[most];
+  }
+  fwd->clear();
+  adj->clear();
+  long off = 0;
+  const long N = sl[g.idx[0]].plan->N;
+  for (int i = 0; i < n; ++i) {
+    const mpi_batch_slice& s = sl[g.idx[i]];
+    float2* W = buf + off * N;
+    for (int k = 0; k < share[i]; ++k) {
+      fwd->push_back(ExpandRow{(const float2*)s.alpha, (const float2*)s.p, nullptr, W, s.C, k, share[i], 0});
+      adj->push_back(ExpandRow{(const float2*)s.alpha, nullptr, W, (float2*)s.x, s.C, k, share[i], 0});
+    }
+    off += s.C;
+  }
+}
+
+// The most CTAs a group's launch may have.
+int most_ctas(const mpi_ctx* ctx, const Group& g) { return std::max(2 * std::max(ctx->num_sms, 1), (int)g.idx.size()); }
+
+// CTAs of a group's expansions: every candidate timed over three launches of the
+// group's forward expansion (between events on the context's stream, after one
+// warm-up launch), the fastest kept.  FP32 CTAs fill an SM each, BF16 ones half.
+mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_precision prec, ExpandRow* ctas,
+                      float2* buf) {
   const mpi_batch_slice& s0 = sl[g.idx[0]];
-  const int nr = (int)g.idx.size();
-  const int sms = std::max(ctx->num_sms, 1);
-  std::vector<int> cands;
-  for (int c : {std::max(1, sms / nr), std::max(1, 2 * sms / nr), std::max(1, sms / (2 * nr))})
-    if (std::find(cands.begin(), cands.end(), c) == cands.end()) cands.push_back(c);
+  const int nr = (int)g.idx.size(), n_tiles = (int)((s0.plan->N + 127) / 128);
+  const int fill = std::max(ctx->num_sms, 1) * (prec == MPI_PREC_BF16 ? 2 : 1);
+  struct Cand {
+    int total;
+    float skew;
+  };
+  const Cand cands[4] = {{fill, 0.f}, {fill, 1.f}, {fill, 3.f}, {prec == MPI_PREC_BF16 ? fill / 2 : 2 * fill, 1.f}};
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     cudaGetLastError();
@@ -199,14 +240,26 @@ mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_pre
                     std::to_string(s0.plan->N) + ", q=" + std::to_string(s0.basis->q) + ", sumC=" +
                     std::to_string(g.sumC) + ", " + (prec == MPI_PREC_BF16 ? "bf16" : "fp32") + "):";
   float best = 1e30f;
-  int pick = cands[0];
+  int pick = 0;
   mpi_status st = MPI_OK;
-  for (int c : cands) {
-    st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, rows + g.fwd_rows, nr, g.Cmax, prec, c);
+  std::vector<ExpandRow> fwd, adj;
+  auto upload = [&](const Cand& c) {
+    share_ctas(sl, g, c.total, c.skew, buf, n_tiles, &fwd, &adj);
+    cudaError_t e = cudaStreamSynchronize(ctx->stream);  // the launches that read the last table
+    if (e == cudaSuccess)
+      e = cudaMemcpy(ctas + g.fwd_ctas, fwd.data(), fwd.size() * sizeof(ExpandRow), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(ctas + g.adj_ctas, adj.data(), adj.size() * sizeof(ExpandRow), cudaMemcpyHostToDevice);
+    g.n_ctas = (int)fwd.size();
+    return cuda_check(ctx, e, "batch: CTA tables");
+  };
+  for (int k = 0; k < 4; ++k) {
+    st = upload(cands[k]);
+    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, ctas + g.fwd_ctas, g.n_ctas, g.Cmax, prec);
     if (st) break;
     cudaEventRecord(e0, ctx->stream);
     for (int r = 0; r < 3 && st == MPI_OK; ++r)
-      st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, rows + g.fwd_rows, nr, g.Cmax, prec, c);
+      st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, ctas + g.fwd_ctas, g.n_ctas, g.Cmax, prec);
     cudaEventRecord(e1, ctx->stream);
     if (st) break;
     if (cudaEventSynchronize(e1) != cudaSuccess) {
@@ -215,24 +268,24 @@ mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_pre
     }
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    char buf[64];
-    snprintf(buf, sizeof(buf), " %d CTAs/row %.2f us;", c, ms / 3 * 1e3);
-    rec += buf;
+    char line[64];
+    snprintf(line, sizeof(line), " %d CTAs, skew %g: %.2f us;", g.n_ctas, cands[k].skew, ms / 3 * 1e3);
+    rec += line;
     if (ms < best) {
       best = ms;
-      pick = c;
+      pick = k;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (st == MPI_OK) st = upload(cands[pick]);
   if (st) return st;
-  g.row_ctas = pick;
   mpi_ctx::TuneRecord tr{};
   tr.key[0] = -1;  // not a line-pass record
-  tr.choice = pick;
-  char buf[64];
-  snprintf(buf, sizeof(buf), " chose %d (%.2f us)", pick, best / 3 * 1e3);
-  tr.what = rec + buf;
+  tr.choice = g.n_ctas;
+  char line[64];
+  snprintf(line, sizeof(line), " chose %d, skew %g (%.2f us)", g.n_ctas, cands[pick].skew, best / 3 * 1e3);
+  tr.what = rec + line;
   ctx->tuned.push_back(tr);
   return MPI_OK;
 }
@@ -309,40 +362,22 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
   bt->ctx = ctx;
   bt->n = n;
   bt->groups = (int)groups.size();
-  // the group buffer and the row tables
-  size_t buf_elems = 0, nrows = 0;
+  // the group buffer and the CTA tables
+  size_t buf_elems = 0, n_ctas = 0;
   for (Group& g : groups) {
     buf_elems = std::max(buf_elems, (size_t)g.sumC * slices[g.idx[0]].plan->N);
-    g.fwd_rows = nrows;
-    g.adj_rows = nrows + g.idx.size();
-    nrows += 2 * g.idx.size();
+    g.fwd_ctas = n_ctas;
+    g.adj_ctas = n_ctas + most_ctas(ctx, g);
+    n_ctas += 2 * (size_t)most_ctas(ctx, g);
   }
   cudaError_t e = cudaSuccess;
   if (!groups.empty()) {
     e = cudaMalloc(&bt->buf, buf_elems * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMalloc(&bt->rows, nrows * sizeof(ExpandRow));
+    if (e == cudaSuccess) e = cudaMalloc(&bt->ctas, n_ctas * sizeof(ExpandRow));
     if (e != cudaSuccess) {
       cudaGetLastError();
       mpi_batch_destroy(bt);
       return set_err(ctx, MPI_ERR_OOM, "batch: group buffers");
-    }
-    std::vector<ExpandRow> host(nrows);
-    float2* buf = (float2*)bt->buf;
-    for (const Group& g : groups) {
-      long off = 0;
-      const long N = slices[g.idx[0]].plan->N;
-      for (size_t r = 0; r < g.idx.size(); ++r) {
-        const mpi_batch_slice& s = slices[g.idx[r]];
-        host[g.fwd_rows + r] = ExpandRow{(const float2*)s.alpha, (const float2*)s.p, nullptr, buf + off * N, s.C, 0};
-        host[g.adj_rows + r] = ExpandRow{(const float2*)s.alpha, nullptr, buf + off * N, (float2*)s.x, s.C, 0};
-        off += s.C;
-      }
-    }
-    e = cudaMemcpy(bt->rows, host.data(), nrows * sizeof(ExpandRow), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      mpi_status st = cuda_check(ctx, e, "batch: row tables");
-      mpi_batch_destroy(bt);
-      return st;
     }
     mpi_status st = group_tables(ctx, slices, groups, &bt->tabs);
     if (st) {
@@ -350,7 +385,7 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
       return st;
     }
     for (Group& g : groups) {
-      mpi_status st = tune_group(ctx, slices, g, prec, (const ExpandRow*)bt->rows);
+      mpi_status st = tune_group(ctx, slices, g, prec, (ExpandRow*)bt->ctas, (float2*)bt->buf);
       const mpi_plan* pl = slices[g.idx[0]].plan;
       for (int dir = 0; dir < 2; ++dir)
         for (Group::Run& r : dir ? g.inv : g.fwd)
@@ -382,7 +417,7 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
   if (e == cudaSuccess) {
     for (size_t i = 0; i < seq.size() && st == MPI_OK; ++i) {
       if (seq[i].first == 0)
-        st = record_group(ctx, slices, groups[seq[i].second], kind, prec, (const ExpandRow*)bt->rows,
+        st = record_group(ctx, slices, groups[seq[i].second], kind, prec, (const ExpandRow*)bt->ctas,
                           (float2*)bt->buf);
       else
         st = record_slice(ctx, slices[seq[i].second], kind, prec);
@@ -429,12 +464,12 @@ extern "C" int mpi_batch_group_count(const mpi_batch* bt) { return bt ? bt->grou
 
 extern "C" mpi_status mpi_batch_destroy(mpi_batch* bt) {
   if (!bt) return MPI_ERR_ARG;
-  if (bt->ctx && (bt->buf || bt->rows || bt->tabs)) cudaStreamSynchronize(bt->ctx->stream);  // a replay may still run
+  if (bt->ctx && (bt->buf || bt->ctas || bt->tabs)) cudaStreamSynchronize(bt->ctx->stream);  // a replay may still run
   ctx_release(&bt->ctx);
   if (bt->exec) cudaGraphExecDestroy(bt->exec);
   if (bt->graph) cudaGraphDestroy(bt->graph);
   if (bt->buf) cudaFree(bt->buf);
-  if (bt->rows) cudaFree(bt->rows);
+  if (bt->ctas) cudaFree(bt->ctas);
   if (bt->tabs) cudaFree(bt->tabs);
   delete bt;
   return MPI_OK;

@@ -235,15 +235,15 @@ struct ScatterMap {
   bool bf16 = false;  // write BF16 values (the same element offsets) instead of FP32
 };
 
-// One row of a grouped expansion launch (grid row blockIdx.y): a slice that
-// shares the basis, with its own coefficients, image, per-coil data and output.
+// One CTA of a grouped expansion launch: a slice that shares the basis, with its own
+// coefficients, image, per-coil data and output, and the CTA's tiles t0, t0 + step, ...
 struct ExpandRow {
   const float2* alpha;
   const float2* p;
   const float2* w;
   float2* out;
   int C;
-  int pad;
+  int t0, step, pad;
 };
 
 struct ExpandArgs {
@@ -268,11 +268,10 @@ struct ExpandArgs {
   const char* kname = nullptr;  // name of the launch in the per-kernel timing (default: the kernel's)
   ScatterMap sc;                // EX_SCATTER output map
   int accumulate = 0;           // EX_FWD / EX_JFWD: add into out instead of storing (several sets of maps)
-  // Grouped launch (tensor-core kernels): device table of nrows rows, C = the
-  // largest row's coil count; row_ctas CTAs per row (0: the SMs shared out).
+  // Grouped launch (tensor-core kernels): device table of n_ctas CTAs, C = the
+  // largest slice's coil count.
   const ExpandRow* rows = nullptr;
-  int nrows = 0;
-  int row_ctas = 0;
+  int n_ctas = 0;
   // 3xTF32 EX_SCATTER_ADD: split K into this many parts (grid rows, >= 2), each
   // adding its partial products into `out` (scattered as EX_SCATTER), which the
   // caller has zeroed
@@ -336,11 +335,11 @@ mpi_status jacobi_columns(mpi_ctx* ctx, double2* M, int L, int nj, double2* V, d
 // tmp holds q r1 (n2 n3 + r2 n3) complex values.
 mpi_status tucker_project(mpi_ctx* ctx, const float2* T, int q, const int n[3], const int r[3], const float2* F0,
                           const float2* F1, const float2* F2, float2* core, float2* tmp);
-// Grouped batch pieces (api.cu): one expansion launch over the rows of slices
+// Grouped batch pieces (api.cu): one expansion launch over the slices
 // that share `basis` (grid geometry from plan0), and a Cartesian plan's
 // image -> k-space / k-space -> image passes on a caller buffer.
-mpi_status expand_rows(mpi_ctx* ctx, const mpi_plan* plan0, const mpi_basis* basis, int mode, const ExpandRow* rows,
-                       int nrows, int Cmax, mpi_precision prec, int row_ctas);
+mpi_status expand_rows(mpi_ctx* ctx, const mpi_plan* plan0, const mpi_basis* basis, int mode, const ExpandRow* ctas,
+                       int n_ctas, int Cmax, mpi_precision prec);
 bool rows_supported(const mpi_basis* basis, int Cmax, mpi_precision prec);
 mpi_status plan_image_to_kspace(mpi_ctx* ctx, const mpi_plan* plan, float2* v, int C, float2* y);
 mpi_status plan_kspace_to_image(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, int C, float2* w);

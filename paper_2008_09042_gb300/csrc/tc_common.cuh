@@ -43,7 +43,9 @@ struct TcArgs {
   int ksplit;
   int k_off;              // global K index of the coefficient image's first column
   int accumulate;         // EX_FWD / EX_JFWD: add into out instead of storing
-  const ExpandRow* rows;  // grouped launch: row blockIdx.y's pointers and coil count (nullptr: none)
+  const ExpandRow* rows;  // grouped launch: CTA blockIdx.x's slice and tiles (nullptr: none)
+  int t0, tstep;          // this CTA's tiles t0, t0 + tstep, ... (set by the kernel)
+  int smem;               // dynamic shared memory of the launch (3xTF32 kernel, grouped)
   long long wait_cycles;  // bounded-wait limit (SM clock cycles)
   int stall_after;        // fault injection: the producer stops after this many stages (-1: off)
 };
@@ -338,7 +340,7 @@ static __device__ __forceinline__ void tc_epilogue(const TcArgs& a, uint32_t tme
     const int quarter = warp & 3;  // TMEM lanes 32 * quarter ..
     const int row = quarter * 32 + lane;
     int tc = 0;
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++tc) {
+    for (int t = a.t0; t < n_tiles; t += a.tstep, ++tc) {
       const int buf = tc & 1;
       const bool got = mpi_ptx::mbar_wait(&acc_full[buf], (uint32_t)((tc >> 1) & 1), a.err, a.wait_cycles);
       if (!__all_sync(0xffffffffu, got)) {  // warp-uniform decision before the .sync.aligned loads

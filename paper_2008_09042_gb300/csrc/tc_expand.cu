@@ -41,8 +41,12 @@ template <int MODE>
 __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant__ CUtensorMap tmap, TcArgs a_in,
                                                             int stages) {
   TcArgs a = a_in;
-  if (a.rows) {  // grouped launch: this row's slice
-    const ExpandRow r = a.rows[blockIdx.y];
+  a.t0 = (int)blockIdx.x;
+  a.tstep = (int)gridDim.x;
+  if ((MODE == EX_FWD || MODE == EX_ADJ) && a.rows) {  // grouped launch: this CTA's slice
+    const ExpandRow r = a.rows[blockIdx.x];
+    a.t0 = r.t0;
+    a.tstep = r.step;
     a.alpha = r.alpha;
     a.p = r.p;
     a.w = r.w;
@@ -104,7 +108,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
     int it = 0;
     RingPos r;
     bool ok = true;
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+    for (int t = a.t0; t < n_tiles && ok; t += a.tstep) {
       for (int kc = 0; kc < a.KC; ++kc, ++it) {
         if (!mpi_ptx::mbar_wait(&empty[r.s], r.ph ^ 1u, a.err, a.wait_cycles)) {
           ok = false;
@@ -132,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
     RingPos r;
     int tc = 0;
     bool ok = mbar_wait_warp(bfull, 0, a.err, a.wait_cycles);
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++tc) {
+    for (int t = a.t0; t < n_tiles && ok; t += a.tstep, ++tc) {
       const int buf = tc & 1;
       const uint32_t tacc = tmem + (uint32_t)(buf * a.half_cols);
       if (!mbar_wait_warp(&acc_empty[buf], (uint32_t)(((tc >> 1) & 1) ^ 1), a.err, a.wait_cycles)) {
@@ -333,9 +337,7 @@ mpi_status launch_expand_tc(mpi_ctx* ctx, const mpi_basis* b, int mode, const Ex
   if (stages < 2) return set_err(ctx, MPI_ERR_UNSUPPORTED, "BF16 expansion: shared memory");
   const size_t smem = fixed + (size_t)stages * kStageBytes;
   const int n_tiles = (x.N + kTileM - 1) / kTileM;
-  const int nrows = x.rows ? x.nrows : 1;
-  const int per_row = x.rows && x.row_ctas > 0 ? x.row_ctas : std::max(per_sm * std::max(ctx->num_sms, 1) / nrows, 1);
-  const dim3 grid((unsigned)std::min(n_tiles, per_row), (unsigned)nrows);
+  const dim3 grid((unsigned)(x.rows ? x.n_ctas : std::min(n_tiles, per_sm * std::max(ctx->num_sms, 1))));
   const CUtensorMap& map = *(const CUtensorMap*)b->tmap;
   cudaError_t e = cudaSuccess;
 #define MPI_TC_CASE(m)                                                                                        \

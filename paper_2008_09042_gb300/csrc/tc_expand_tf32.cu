@@ -50,6 +50,30 @@ constexpr int kStageBytes32 = kBoxesPerStage * kBoxBytes32;
 constexpr int kThreads32 = 320;   // warp 0 TMA, 1 MMA, 2-5 epilogue, 6-9 converters
 constexpr size_t kSmemMax = 232448 - 128;  // 227 KB less room for the static shared word
 
+constexpr int kMaxStages32 = 6;
+
+// TMEM columns of one accumulator for n_gemm stacked rows (a power of two, 32 or more).
+__host__ __device__ constexpr int tf32_acc_cols(int n_gemm) {
+  int c = 32;
+  while (c < 2 * n_gemm) c <<= 1;
+  return c;
+}
+// Shared memory beside the ring: alignment slack, the stacked coefficient image over
+// K values, 3 barriers per stage and 6 more, the TMEM slot.
+__host__ __device__ constexpr size_t tf32_fixed(int n_gemm, int K) {
+  return 1024 + ((2 * (size_t)n_gemm * K * 4 + 1023) & ~(size_t)1023) + 8 * (3 * kMaxStages32 + 6) + 16;
+}
+// Ring stages that fit in `smem` bytes and, with two accumulators and 64 columns of
+// lo(U) per stage, in the SM's 512 TMEM columns.
+__host__ __device__ constexpr int tf32_stages(int n_gemm, int K, size_t smem) {
+  const size_t fixed = tf32_fixed(n_gemm, K);
+  if (smem < fixed) return 0;
+  const int by_smem = (int)((smem - fixed) / kStageBytes32);
+  const int by_tmem = (512 - 2 * tf32_acc_cols(n_gemm)) / (32 * kBoxesPerStage);
+  const int s = by_smem < by_tmem ? by_smem : by_tmem;
+  return s < kMaxStages32 ? s : kMaxStages32;
+}
+
 // 32 consecutive 32-bit TMEM columns of this warp's 32 lanes, one row per thread.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
   asm volatile(
@@ -79,8 +103,15 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   // rows of a launch stream the same basis tiles in the same order, so all but
   // one of them mostly find each tile in L2.
   TcArgs a = a_in;
-  if (a.rows) {  // grouped launch: this row's slice
-    const ExpandRow r = a.rows[blockIdx.y];
+  a.t0 = (int)blockIdx.x;
+  a.tstep = (int)gridDim.x;
+  if ((MODE == EX_FWD || MODE == EX_ADJ) && a.rows) {  // grouped launch: this CTA's slice, with the operand, accumulators and ring of its own coil count
+    const ExpandRow r = a.rows[blockIdx.x];
+    a.t0 = r.t0;
+    a.tstep = r.step;
+    a.n_gemm = a.half = a.lo_cols = (2 * r.C + 15) / 16 * 16;
+    a.half_cols = tf32_acc_cols(a.n_gemm);
+    stages = tf32_stages(a.n_gemm, a.KC * kKChunk32, (size_t)a.smem);
     a.alpha = r.alpha;
     a.p = r.p;
     a.w = r.w;
@@ -156,7 +187,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   const int n_tiles = (a.N + kTileM - 1) / kTileM;
   // ring stages this CTA processes (its tiles x ceil(KC / 2)), numbered g = 0 .. G-1;
   // with an odd box count KC the last stage of each tile holds one box
-  const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int my_tiles = a.t0 < n_tiles ? (n_tiles - 1 - a.t0) / a.tstep + 1 : 0;
   const int G = my_tiles * ((a.KC + kBoxesPerStage - 1) / kBoxesPerStage);
 
   if (warp >= 2) {
@@ -169,7 +200,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   if (warp == 0 && lane == 0) {
     // ---------------- producer: TMA tiles of U
     RingPos r;
-    int g = 0, kc = 0, t = (int)blockIdx.x;  // kc: first box of the stage
+    int g = 0, kc = 0, t = a.t0;  // kc: first box of the stage
     for (; g < G; ++g) {
       // fault injection (a test of the timeout path): stop issuing copies, so
       // that every consumer's wait on the stages not loaded runs out
@@ -184,7 +215,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
       kc += kBoxesPerStage;
       if (kc >= a.KC) {
         kc = 0;
-        t += (int)gridDim.x;
+        t += a.tstep;
       }
     }
     if (g < G) {
@@ -244,7 +275,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
     RingPos r;
     int tc = 0;
     bool ok = mbar_wait_warp(bfull, 0, a.err, a.wait_cycles);
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++tc) {
+    for (int t = a.t0; t < n_tiles && ok; t += a.tstep, ++tc) {
       const int buf = tc & 1;
       const uint32_t tacc = tmem + (uint32_t)(buf * a.half_cols);
       if (!mbar_wait_warp(&acc_empty[buf], (uint32_t)(((tc >> 1) & 1) ^ 1), a.err, a.wait_cycles)) {
@@ -395,10 +426,8 @@ int round_up_i(int x, int m) { return (x + m - 1) / m * m; }
 
 struct TfPlan {
   int n_gemm, half, half_cols, tmem_cols, stages;
-  size_t b_bytes, smem;
+  size_t smem;
 };
-
-constexpr int kMaxStages32 = 6;
 
 // ksplit > 1: each CTA row takes 1/ksplit of the K boxes, so its coefficient
 // image covers that part of K only.
@@ -407,22 +436,14 @@ bool plan_tf32(const mpi_basis* b, int mode, int C, TfPlan* p, int ksplit = 1) {
   p->half = cols;
   p->n_gemm = mode == EX_JFWD ? 2 * cols : cols;
   if (2 * p->n_gemm > 256) return false;  // the stacked [hi; lo] rows form one MMA's N
-  int acc_cols = 32;
-  while (acc_cols < 2 * p->n_gemm) acc_cols <<= 1;
+  const int K = b->Kp32 / ksplit, acc_cols = tf32_acc_cols(p->n_gemm);
   p->half_cols = acc_cols;
-  p->b_bytes = 2 * (size_t)p->n_gemm * (b->Kp32 / ksplit) * 4;
-  // alignment slack + the stacked coefficient image + 3 barriers per stage and 6 more + TMEM slot
-  const size_t fixed = 1024 + ((p->b_bytes + 1023) & ~(size_t)1023) + 8 * (3 * kMaxStages32 + 6) + 16;
-  if (fixed + 2 * (size_t)kStageBytes32 > kSmemMax) return false;
-  int stages = (int)std::min<size_t>(kMaxStages32, (kSmemMax - fixed) / kStageBytes32);
-  // TMEM: two accumulators, then 64 columns of lo(U) per stage, within the SM's 512
-  stages = std::min(stages, (512 - 2 * acc_cols) / (32 * kBoxesPerStage));
-  if (stages < 2) return false;
-  p->stages = stages;
+  p->stages = tf32_stages(p->n_gemm, K, kSmemMax);
+  if (p->stages < 2) return false;
   int tcols = 32;
-  while (tcols < 2 * acc_cols + 32 * kBoxesPerStage * stages) tcols <<= 1;
+  while (tcols < 2 * acc_cols + 32 * kBoxesPerStage * p->stages) tcols <<= 1;
   p->tmem_cols = tcols;
-  p->smem = fixed + (size_t)stages * kStageBytes32;
+  p->smem = tf32_fixed(p->n_gemm, K) + (size_t)p->stages * kStageBytes32;
   return true;
 }
 
@@ -616,11 +637,17 @@ mpi_status launch_expand_tf32(mpi_ctx* ctx, const mpi_basis* b, int mode, const 
   a.C_total = x.C;
   if (groups > 1) a.C = Cg;
   const int n_tiles = (x.N + kTileM - 1) / kTileM;
-  // one CTA per SM over all groups (or rows of a grouped launch, or K parts)
-  const int nrows = x.rows ? x.nrows : (ks > 1 ? ks : groups);
-  if (x.rows) a.group_coils = 0;
-  const int per_row = x.rows && x.row_ctas > 0 ? x.row_ctas : std::max(std::max(ctx->num_sms, 1) / nrows, 1);
-  const dim3 grid((unsigned)std::min(n_tiles, per_row), (unsigned)nrows);
+  // one CTA per SM over all groups (or K parts)
+  const int nrows = ks > 1 ? ks : groups;
+  const int per_row = std::max(std::max(ctx->num_sms, 1) / nrows, 1);
+  dim3 grid((unsigned)std::min(n_tiles, per_row), (unsigned)nrows);
+  if (x.rows) {  // each CTA lays out its own slice's ring in all of the SM's memory
+    a.group_coils = 0;
+    a.tmem_cols = 512;
+    pl.smem = kSmemMax;
+    a.smem = (int)kSmemMax;
+    grid = dim3((unsigned)x.n_ctas);
+  }
   const CUtensorMap& map = *(const CUtensorMap*)b->tmap32;
   cudaError_t e = cudaSuccess;
   // an odd K box count occurs only for the chain's operand views (whole-box

@@ -59,3 +59,34 @@ def test_grouped_passes_match_single_calls(ny, nx, kinds, coils, kind, prec):
         if kind != "forward":
             assert torch.equal(s["x"], mp.adjoint(ctx, s["plan"], B, s["alpha"], y1, prec))
     batch.close()
+
+
+@pytest.mark.parametrize("n,q,coils", [
+    (320, 160, (32, 8, 16, 1, 32)),  # the largest coefficient operand (a ring of two stages) beside small ones
+    (16, 5, (1, 3, 2)),              # fewer tiles than CTAs
+    (32, 30, tuple(1 + i % 7 for i in range(170))),  # more slices than SMs
+])
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_grouped_expansions_of_mixed_coil_counts(n, q, coils, prec):
+    # every CTA lays out its own slice's operand, accumulators and ring: values as in the slice's own calls
+    import paper_2008_09042_gb300 as mp
+
+    ctx = mp.Context(0)
+    B = mp.Basis(ctx, w.smooth_orthonormal_basis(n, n, q, seed=1).T)
+    slices = []
+    for i, C in enumerate(coils):
+        idx = _idx("points", n, n, i)
+        slices.append(dict(plan=mp.Plan(ctx, (n, n), sample_idx=idx), basis=B,
+                           y=torch.zeros((C, idx.size), dtype=torch.complex64, device="cuda"),
+                           alpha=torch.from_numpy(w.random_coefficients(C, q, seed=i).astype(np.complex64)).cuda(),
+                           p=torch.from_numpy(w.random_image(n * n, seed=i).astype(np.complex64)).cuda(),
+                           x=torch.zeros(n * n, dtype=torch.complex64, device="cuda")))
+    batch = mp.Batch(ctx, slices, kind="pair", prec=prec)
+    assert batch.groups() == 1
+    batch.run()
+    ctx.synchronize()
+    for s in slices:
+        y1 = mp.forward(ctx, s["plan"], B, s["alpha"], s["p"], prec)
+        assert torch.equal(s["y"], y1)
+        assert torch.equal(s["x"], mp.adjoint(ctx, s["plan"], B, s["alpha"], y1, prec))
+    batch.close()
