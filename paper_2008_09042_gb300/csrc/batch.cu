@@ -10,16 +10,17 @@
 //
 // Grouped expansion: consecutive slices on Cartesian plans that share a dense
 // basis (FP32 or BF16, every slice's coils within one tensor-core pass)
-// form a group.  The group's basis expansion is one launch over its slices (a device
-// table gives each CTA its slice's coefficients, image, per-coil data and output);
-// the slices stream the same basis tiles in step, so the basis is read from DRAM
-// about once per group instead of once per slice.  Each slice's per-coil images live
+// form a group.  The group's basis expansion is one launch over its slices (device
+// tables give each CTA its slices' coefficients, images, per-coil data and outputs);
+// the CTAs stream the same basis tiles in step, so the basis is read from DRAM
+// about once per group instead of once per slice, and slices of few coils are bundled,
+// their coefficients stacked into one operand, so that one CTA reads a tile for all.  Each slice's per-coil images live
 // in a batch-owned buffer between the expansion and the FFT passes.  From
 // kGroupedPasses slices on, the FFT passes take all coils of a group's slices in one
 // launch too (per run of slices whose pass along y is of the same kind, register or
 // Stockham, so that a slice's values stay those of its own call; its width is timed
-// for the group), with a table of every coil's sampling.  How many CTAs each slice gets
-// is chosen at creation by timing the candidates (an autotuner decision the context
+// for the group), with a table of every coil's sampling.  How the slices are bundled
+// and how many CTAs each bundle gets is chosen at creation by timing the candidates (an autotuner decision the context
 // records).
 #include <algorithm>
 #include <cstdio>
@@ -36,7 +37,7 @@ struct mpi_batch {
   int n = 0;
   int64_t kernels = 0;  // kernels per replay
   void* buf = nullptr;   // per-coil images of one group [sum C][N]
-  void* ctas = nullptr;  // CTA tables of every group's expansions (device)
+  void* ctas = nullptr;  // CTA and slice tables of every group's expansions (device)
   void* tabs = nullptr;  // sampling tables and row masks of the grouped passes (device)
   int groups = 0;        // grouped launches per direction
 };
@@ -62,9 +63,11 @@ struct Group {
   std::vector<int> idx;  // slices, in recording order
   int Cmax = 0;
   long sumC = 0;
-  // grouped expansions: the CTAs of a launch and their offsets in the device CTA table
-  size_t fwd_ctas = 0, adj_ctas = 0;
-  int n_ctas = 0;
+  // grouped expansions: the launches' CTA and slice tables (device), their CTAs and
+  // the coils of the largest bundle
+  ExpandRow *fwd_ctas = nullptr, *adj_ctas = nullptr;
+  ExpandSeg *fwd_segs = nullptr, *adj_segs = nullptr;
+  int n_ctas = 0, coils = 0;
   // grouped passes: runs of slices (first, count in coils) per direction and kernel
   struct Run {
     bool registers;
@@ -81,14 +84,13 @@ bool groupable(const mpi_batch_slice& s, mpi_precision prec) {
 }
 
 // The group's forward and adjoint expansions, and its slices' FFT passes.
-mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g, int kind, mpi_precision prec,
-                        const ExpandRow* ctas, float2* buf) {
+mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g, int kind, mpi_precision prec, float2* buf) {
   const mpi_batch_slice& s0 = sl[g.idx[0]];
   const long N = s0.plan->N;
   const int nr = (int)g.idx.size(), ny = s0.plan->ny, nx = s0.plan->nx;
   mpi_status st = MPI_OK;
   if (kind & MPI_BATCH_FORWARD) {
-    st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, ctas + g.fwd_ctas, g.n_ctas, g.Cmax, prec);
+    st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, g.fwd_ctas, g.n_ctas, g.coils, prec);
     for (const Group::Run& r : g.fwd)
       if (st == MPI_OK)
         st = launch_fft_cols_group(ctx, r.kernel, buf + r.first * N, r.coils, ny, nx, false,
@@ -113,7 +115,7 @@ mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g,
       st = plan_kspace_to_image(ctx, s.plan, (const float2*)s.y, s.C, buf + off * N);
       off += s.C;
     }
-    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_ADJ, ctas + g.adj_ctas, g.n_ctas, g.Cmax, prec);
+    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_ADJ, g.adj_ctas, g.n_ctas, g.coils, prec);
   }
   return st;
 }
@@ -180,57 +182,106 @@ mpi_status group_tables(mpi_ctx* ctx, const mpi_batch_slice* sl, std::vector<Gro
   return cuda_check(ctx, cudaMemcpy(*out, host.data(), bytes, cudaMemcpyHostToDevice), "batch: group tables");
 }
 
-// The CTAs of a group's expansion launches, `total` of them (one per slice at least),
-// shared out in proportion to 1 + skew x (a slice's coil columns, padded to whole
-// MMAs, / 64): a tile of a slice with more coils takes more MMA and epilogue time,
-// and has a shorter ring beside its larger coefficient operand, so equal shares
-// would leave the CTAs of small coil arrays waiting for the large ones'.  With shares
-// that match, all slices also pass through the basis in step, so that it leaves DRAM
-// about once.  A slice's values do not depend on its share.
-void share_ctas(const mpi_batch_slice* sl, const Group& g, int total, float skew, float2* buf, int n_tiles,
-                std::vector<ExpandRow>* fwd, std::vector<ExpandRow>* adj) {
+// How a group's expansions are laid out: bundles of slices up to `chunks` x 8 coils
+// (0: every slice alone), `total` CTAs shared out over them with `skew`.
+struct Layout {
+  int chunks, total;
+  float skew;
+};
+
+int slice_chunks(const mpi_batch_slice& s) { return (s.C + 7) / 8; }
+
+// The launches' tables.  Slices are bundled (largest first, each into the first bundle
+// with room), since a bundle's CTAs load and split each tile of the basis once for all
+// of its slices; more columns leave less room for the ring beside the coefficients.
+// The CTAs, `total` of them (one per bundle at least), are shared out in proportion to
+// 1 + skew x (a bundle's columns / 64).  A slice's values do not depend on either.
+void layout_tables(const mpi_batch_slice* sl, Group& g, const Layout& lay, float2* buf, int n_tiles,
+                   std::vector<ExpandRow> (&ctas)[2], std::vector<ExpandSeg> (&segs)[2]) {
   const int n = (int)g.idx.size();
-  std::vector<float> w(n);
-  std::vector<int> share(n, 1);
-  for (int i = 0; i < n; ++i) w[i] = 1.f + skew * (float)((2 * sl[g.idx[i]].C + 15) / 16 * 16) / 64.f;
-  for (int used = n; used < total; ++used) {
+  const long N = sl[g.idx[0]].plan->N;
+  std::vector<long> off(n);
+  std::vector<int> order(n);
+  long sum = 0;
+  for (int i = 0; i < n; ++i) {
+    off[i] = sum;
+    order[i] = i;
+    sum += sl[g.idx[i]].C;
+  }
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return slice_chunks(sl[g.idx[a]]) > slice_chunks(sl[g.idx[b]]); });
+  struct Bundle {
+    std::vector<int> slices;
+    int chunks;
+  };
+  std::vector<Bundle> bundles;
+  for (int i : order) {
+    const int ch = slice_chunks(sl[g.idx[i]]);
+    size_t b = 0;
+    while (b < bundles.size() && bundles[b].chunks + ch > lay.chunks) ++b;
+    if (b == bundles.size()) bundles.push_back({{}, 0});
+    bundles[b].slices.push_back(i);
+    bundles[b].chunks += ch;
+  }
+  const int nb = (int)bundles.size();
+  std::vector<float> w(nb);
+  std::vector<int> share(nb, 1);
+  for (int b = 0; b < nb; ++b) w[b] = 1.f + lay.skew * (float)bundles[b].chunks / 4.f;
+  for (int used = nb; used < lay.total; ++used) {
     int most = -1;
-    for (int i = 0; i < n; ++i)
-      if (share[i] < n_tiles && (most < 0 || w[i] * share[most] > w[most] * share[i])) most = i;
+    for (int b = 0; b < nb; ++b)
+      if (share[b] < n_tiles && (most < 0 || w[b] * share[most] > w[most] * share[b])) most = b;
     if (most < 0) break;
     ++share[most];
   }
-  fwd->clear();
-  adj->clear();
-  long off = 0;
-  const long N = sl[g.idx[0]].plan->N;
-  for (int i = 0; i < n; ++i) {
-    const mpi_batch_slice& s = sl[g.idx[i]];
-    float2* W = buf + off * N;
-    for (int k = 0; k < share[i]; ++k) {
-      fwd->push_back(ExpandRow{(const float2*)s.alpha, (const float2*)s.p, nullptr, W, s.C, k, share[i], 0});
-      adj->push_back(ExpandRow{(const float2*)s.alpha, nullptr, W, (float2*)s.x, s.C, k, share[i], 0});
-    }
-    off += s.C;
+  g.coils = 0;
+  for (int d = 0; d < 2; ++d) {
+    ctas[d].clear();
+    segs[d].clear();
   }
+  for (int b = 0; b < nb; ++b) {
+    const size_t first = segs[0].size();
+    int chunk = 0;
+    for (int i : bundles[b].slices) {
+      const mpi_batch_slice& s = sl[g.idx[i]];
+      float2* W = buf + off[i] * N;
+      segs[0].push_back(ExpandSeg{(const float2*)s.alpha, (const float2*)s.p, nullptr, W, s.C, chunk});
+      segs[1].push_back(ExpandSeg{(const float2*)s.alpha, nullptr, W, (float2*)s.x, s.C, chunk});
+      chunk += slice_chunks(s);
+    }
+    g.coils = std::max(g.coils, 8 * chunk);
+    const int ns = (int)bundles[b].slices.size();
+    for (int k = 0; k < share[b]; ++k) {
+      ctas[0].push_back(ExpandRow{g.fwd_segs + first, ns, chunk, k, share[b]});
+      ctas[1].push_back(ExpandRow{g.adj_segs + first, ns, chunk, k, share[b]});
+    }
+  }
+  g.n_ctas = (int)ctas[0].size();
 }
 
 // The most CTAs a group's launch may have.
 int most_ctas(const mpi_ctx* ctx, const Group& g) { return std::max(2 * std::max(ctx->num_sms, 1), (int)g.idx.size()); }
 
-// CTAs of a group's expansions: every candidate timed over three launches of the
+// Layout of a group's expansions: every candidate timed over three launches of the
 // group's forward expansion (between events on the context's stream, after one
 // warm-up launch), the fastest kept.  FP32 CTAs fill an SM each, BF16 ones half.
-mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_precision prec, ExpandRow* ctas,
-                      float2* buf) {
+mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_precision prec, float2* buf) {
   const mpi_batch_slice& s0 = sl[g.idx[0]];
   const int nr = (int)g.idx.size(), n_tiles = (int)((s0.plan->N + 127) / 128);
   const int fill = std::max(ctx->num_sms, 1) * (prec == MPI_PREC_BF16 ? 2 : 1);
-  struct Cand {
-    int total;
-    float skew;
-  };
-  const Cand cands[4] = {{fill, 0.f}, {fill, 1.f}, {fill, 3.f}, {prec == MPI_PREC_BF16 ? fill / 2 : 2 * fill, 1.f}};
+  const int most = (g.Cmax + 7) / 8;
+  // An FP32 tile's time hardly depends on its coils: streaming and splitting U for every
+  // slice is most of it.  16 slices of 320^2, q = 160, with 8, 16 and 32 coils: 331 us with
+  // every slice in the largest one's operand, 296 alone in its own, 223 in bundles of 32
+  // coils; of 192^2, q = 96, 81 alone and 88 in bundles.  BF16 tiles are bound by their
+  // epilogues, which bundles do not share (120 us against 90): shares by coils instead.
+  std::vector<Layout> cands = {{0, fill, 0.f}, {0, fill, 1.f}};
+  if (prec == MPI_PREC_BF16) {
+    cands.push_back({0, fill, 3.f});
+  } else {
+    cands.push_back({most, fill, 0.f});
+    if (most < 4 && rows_supported(s0.basis, 32, prec)) cands.push_back({4, fill, 0.f});
+  }
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     cudaGetLastError();
@@ -242,24 +293,27 @@ mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_pre
   float best = 1e30f;
   int pick = 0;
   mpi_status st = MPI_OK;
-  std::vector<ExpandRow> fwd, adj;
-  auto upload = [&](const Cand& c) {
-    share_ctas(sl, g, c.total, c.skew, buf, n_tiles, &fwd, &adj);
-    cudaError_t e = cudaStreamSynchronize(ctx->stream);  // the launches that read the last table
-    if (e == cudaSuccess)
-      e = cudaMemcpy(ctas + g.fwd_ctas, fwd.data(), fwd.size() * sizeof(ExpandRow), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-      e = cudaMemcpy(ctas + g.adj_ctas, adj.data(), adj.size() * sizeof(ExpandRow), cudaMemcpyHostToDevice);
-    g.n_ctas = (int)fwd.size();
-    return cuda_check(ctx, e, "batch: CTA tables");
+  std::vector<ExpandRow> ctas[2];
+  std::vector<ExpandSeg> segs[2];
+  auto upload = [&](const Layout& lay) {
+    layout_tables(sl, g, lay, buf, n_tiles, ctas, segs);
+    cudaError_t e = cudaStreamSynchronize(ctx->stream);  // the launches that read the last tables
+    for (int d = 0; d < 2 && e == cudaSuccess; ++d) {
+      e = cudaMemcpy(d ? g.adj_ctas : g.fwd_ctas, ctas[d].data(), ctas[d].size() * sizeof(ExpandRow),
+                     cudaMemcpyHostToDevice);
+      if (e == cudaSuccess)
+        e = cudaMemcpy(d ? g.adj_segs : g.fwd_segs, segs[d].data(), segs[d].size() * sizeof(ExpandSeg),
+                       cudaMemcpyHostToDevice);
+    }
+    return cuda_check(ctx, e, "batch: expansion tables");
   };
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < (int)cands.size(); ++k) {
     st = upload(cands[k]);
-    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, ctas + g.fwd_ctas, g.n_ctas, g.Cmax, prec);
+    if (st == MPI_OK) st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, g.fwd_ctas, g.n_ctas, g.coils, prec);
     if (st) break;
     cudaEventRecord(e0, ctx->stream);
     for (int r = 0; r < 3 && st == MPI_OK; ++r)
-      st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, ctas + g.fwd_ctas, g.n_ctas, g.Cmax, prec);
+      st = expand_rows(ctx, s0.plan, s0.basis, EX_FWD, g.fwd_ctas, g.n_ctas, g.coils, prec);
     cudaEventRecord(e1, ctx->stream);
     if (st) break;
     if (cudaEventSynchronize(e1) != cudaSuccess) {
@@ -268,8 +322,9 @@ mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_pre
     }
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    char line[64];
-    snprintf(line, sizeof(line), " %d CTAs, skew %g: %.2f us;", g.n_ctas, cands[k].skew, ms / 3 * 1e3);
+    char line[96];
+    snprintf(line, sizeof(line), " %d CTAs, bundles of %d, skew %g: %.2f us;", g.n_ctas, 8 * cands[k].chunks,
+             cands[k].skew, ms / 3 * 1e3);
     rec += line;
     if (ms < best) {
       best = ms;
@@ -283,8 +338,9 @@ mpi_status tune_group(mpi_ctx* ctx, const mpi_batch_slice* sl, Group& g, mpi_pre
   mpi_ctx::TuneRecord tr{};
   tr.key[0] = -1;  // not a line-pass record
   tr.choice = g.n_ctas;
-  char line[64];
-  snprintf(line, sizeof(line), " chose %d, skew %g (%.2f us)", g.n_ctas, cands[pick].skew, best / 3 * 1e3);
+  char line[96];
+  snprintf(line, sizeof(line), " chose %d, bundles of %d, skew %g (%.2f us)", g.n_ctas, 8 * cands[pick].chunks,
+           cands[pick].skew, best / 3 * 1e3);
   tr.what = rec + line;
   ctx->tuned.push_back(tr);
   return MPI_OK;
@@ -363,21 +419,30 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
   bt->n = n;
   bt->groups = (int)groups.size();
   // the group buffer and the CTA tables
-  size_t buf_elems = 0, n_ctas = 0;
+  size_t buf_elems = 0, n_ctas = 0, n_segs = 0;
   for (Group& g : groups) {
     buf_elems = std::max(buf_elems, (size_t)g.sumC * slices[g.idx[0]].plan->N);
-    g.fwd_ctas = n_ctas;
-    g.adj_ctas = n_ctas + most_ctas(ctx, g);
     n_ctas += 2 * (size_t)most_ctas(ctx, g);
+    n_segs += 2 * g.idx.size();
   }
   cudaError_t e = cudaSuccess;
   if (!groups.empty()) {
     e = cudaMalloc(&bt->buf, buf_elems * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMalloc(&bt->ctas, n_ctas * sizeof(ExpandRow));
+    if (e == cudaSuccess) e = cudaMalloc(&bt->ctas, n_ctas * sizeof(ExpandRow) + n_segs * sizeof(ExpandSeg));
     if (e != cudaSuccess) {
       cudaGetLastError();
       mpi_batch_destroy(bt);
       return set_err(ctx, MPI_ERR_OOM, "batch: group buffers");
+    }
+    ExpandRow* ctas = (ExpandRow*)bt->ctas;
+    ExpandSeg* segs = (ExpandSeg*)(ctas + n_ctas);
+    for (Group& g : groups) {
+      g.fwd_ctas = ctas;
+      g.adj_ctas = ctas + most_ctas(ctx, g);
+      ctas += 2 * most_ctas(ctx, g);
+      g.fwd_segs = segs;
+      g.adj_segs = segs + g.idx.size();
+      segs += 2 * g.idx.size();
     }
     mpi_status st = group_tables(ctx, slices, groups, &bt->tabs);
     if (st) {
@@ -385,7 +450,7 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
       return st;
     }
     for (Group& g : groups) {
-      mpi_status st = tune_group(ctx, slices, g, prec, (ExpandRow*)bt->ctas, (float2*)bt->buf);
+      mpi_status st = tune_group(ctx, slices, g, prec, (float2*)bt->buf);
       const mpi_plan* pl = slices[g.idx[0]].plan;
       for (int dir = 0; dir < 2; ++dir)
         for (Group::Run& r : dir ? g.inv : g.fwd)
@@ -417,8 +482,7 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
   if (e == cudaSuccess) {
     for (size_t i = 0; i < seq.size() && st == MPI_OK; ++i) {
       if (seq[i].first == 0)
-        st = record_group(ctx, slices, groups[seq[i].second], kind, prec, (const ExpandRow*)bt->ctas,
-                          (float2*)bt->buf);
+        st = record_group(ctx, slices, groups[seq[i].second], kind, prec, (float2*)bt->buf);
       else
         st = record_slice(ctx, slices[seq[i].second], kind, prec);
     }

@@ -235,15 +235,21 @@ struct ScatterMap {
   bool bf16 = false;  // write BF16 values (the same element offsets) instead of FP32
 };
 
-// One CTA of a grouped expansion launch: a slice that shares the basis, with its own
-// coefficients, image, per-coil data and output, and the CTA's tiles t0, t0 + step, ...
-struct ExpandRow {
+// Grouped expansion launch.  A slice in it: its own coefficients, image, per-coil data
+// and output, and its first 16 accumulator columns (8 coils) in its bundle's operand.
+struct ExpandSeg {
   const float2* alpha;
   const float2* p;
   const float2* w;
   float2* out;
-  int C;
-  int t0, step, pad;
+  int C, chunk0;
+};
+// One CTA: the bundle of slices whose stacked coefficients it multiplies each tile of
+// the basis by, and its tiles t0, t0 + step, ...
+struct ExpandRow {
+  const ExpandSeg* segs;
+  int n_segs, chunks;
+  int t0, step;
 };
 
 struct ExpandArgs {

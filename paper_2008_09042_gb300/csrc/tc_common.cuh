@@ -44,11 +44,20 @@ struct TcArgs {
   int k_off;              // global K index of the coefficient image's first column
   int accumulate;         // EX_FWD / EX_JFWD: add into out instead of storing
   const ExpandRow* rows;  // grouped launch: CTA blockIdx.x's slice and tiles (nullptr: none)
+  const ExpandSeg* segs;  // the bundle of a grouped launch's CTA (set by the kernel)
+  int n_segs;
   int t0, tstep;          // this CTA's tiles t0, t0 + tstep, ... (set by the kernel)
   int smem;               // dynamic shared memory of the launch (3xTF32 kernel, grouped)
   long long wait_cycles;  // bounded-wait limit (SM clock cycles)
   int stall_after;        // fault injection: the producer stops after this many stages (-1: off)
 };
+
+// The slices a CTA works on: those of its bundle, or the call's own.
+template <bool BUNDLE>
+static __device__ __forceinline__ ExpandSeg tc_seg(const TcArgs& a, int i) {
+  if constexpr (BUNDLE) return a.segs[i];
+  return ExpandSeg{a.alpha, a.p, a.w, a.out, a.C, 0};
+}
 
 // Position in a ring of `n` shared-memory stages: slot and the parity of the
 // slot's current mbarrier phase.  Advanced one step at a time (no division on
@@ -245,7 +254,7 @@ static __device__ __forceinline__ float tf32_lo(float v) {
 // of q = 128 and 14,000 for 32, out of 28,000-36,000 for the whole expansion.
 // Ends with the writes made visible to the tensor core and one arrival per
 // warp on `ready`.
-template <bool SPLIT>
+template <bool SPLIT, bool BUNDLE = false>
 static __device__ void build_coef_smem(const TcArgs& a, unsigned char* sB, int Kp, bool with_dalpha, int etid,
                                        int nthr, uint64_t* ready) {
   constexpr int E = SPLIT ? 4 : 8;        // K values per 16-byte unit
@@ -253,76 +262,81 @@ static __device__ void build_coef_smem(const TcArgs& a, unsigned char* sB, int K
   constexpr int BATCH = SPLIT ? 4 : 2;    // tasks whose loads are in flight together
   const int rows = SPLIT ? 2 * a.n_gemm : a.n_gemm;
   const int units = Kp / E;               // units along K per row
-  const int n_coil = (with_dalpha ? 2 : 1) * a.C;  // coils of alpha, then of dalpha
   const int dc = nthr / units, du = nthr - dc * units;
-  int c = etid / units, u = etid - c * units;      // this thread's next task (coil, unit)
-  while (c < n_coil) {
-    float2 al[BATCH][E];
-    int tc[BATCH], tu[BATCH];
+  for (int sg = 0; sg < (BUNDLE ? a.n_segs : 1); ++sg) {
+    const ExpandSeg seg = tc_seg<BUNDLE>(a, sg);
+    const int C = seg.C, rb = 16 * seg.chunk0;       // the slice's first row
+    const int n_coil = (with_dalpha ? 2 : 1) * C;    // coils of alpha, then of dalpha
+    int c = etid / units, u = etid - c * units;      // this thread's next task (coil, unit)
+    while (c < n_coil) {
+      float2 al[BATCH][E];
+      int tc[BATCH], tu[BATCH];
 #pragma unroll
-    for (int j = 0; j < BATCH; ++j) {
-      tc[j] = c;
-      tu[j] = u;
-      if (c < n_coil) {
-        const float2* src = c < a.C ? a.alpha + (size_t)c * a.q : a.dalpha + (size_t)(c - a.C) * a.q;
+      for (int j = 0; j < BATCH; ++j) {
+        tc[j] = c;
+        tu[j] = u;
+        if (c < n_coil) {
+          const float2* src = c < C ? seg.alpha + (size_t)c * a.q : a.dalpha + (size_t)(c - C) * a.q;
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int k = u * E + e + a.k_off;
+            al[j][e] = make_float2(0.f, 0.f);
+            if (k < 2 * a.q) al[j][e] = src[k < a.q ? k : k - a.q];
+          }
+        }
+        c += dc;
+        u += du;
+        if (u >= units) {
+          u -= units;
+          ++c;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < BATCH; ++j) {
+        if (tc[j] >= n_coil) break;
+        const int r0 = tc[j] < C ? rb + 2 * tc[j] : a.half + 2 * (tc[j] - C), k0 = tu[j] * E;
+        float re[E], im[E];  // rows r0 and r0 + 1
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-          const int k = u * E + e + a.k_off;
-          al[j][e] = make_float2(0.f, 0.f);
-          if (k < 2 * a.q) al[j][e] = src[k < a.q ? k : k - a.q];
+          const bool first = k0 + e + a.k_off < a.q;  // past 2 q the loaded value is zero
+          re[e] = first ? al[j][e].x : -al[j][e].y;
+          im[e] = first ? al[j][e].y : al[j][e].x;
+        }
+        if (SPLIT) {
+          float4 h0, h1, l0, l1;
+          h0 = make_float4(tf32_hi(re[0]), tf32_hi(re[1]), tf32_hi(re[2]), tf32_hi(re[3]));
+          h1 = make_float4(tf32_hi(im[0]), tf32_hi(im[1]), tf32_hi(im[2]), tf32_hi(im[3]));
+          l0 = make_float4(tf32_lo(re[0]), tf32_lo(re[1]), tf32_lo(re[2]), tf32_lo(re[3]));
+          l1 = make_float4(tf32_lo(im[0]), tf32_lo(im[1]), tf32_lo(im[2]), tf32_lo(im[3]));
+          *reinterpret_cast<float4*>(sB + sw128_offset_e(r0, k0, rows, esize)) = h0;
+          *reinterpret_cast<float4*>(sB + sw128_offset_e(r0 + 1, k0, rows, esize)) = h1;
+          *reinterpret_cast<float4*>(sB + sw128_offset_e(r0 + a.n_gemm, k0, rows, esize)) = l0;
+          *reinterpret_cast<float4*>(sB + sw128_offset_e(r0 + 1 + a.n_gemm, k0, rows, esize)) = l1;
+        } else {
+          uint4 v0, v1;
+          __nv_bfloat162* p0 = reinterpret_cast<__nv_bfloat162*>(&v0);
+          __nv_bfloat162* p1 = reinterpret_cast<__nv_bfloat162*>(&v1);
+#pragma unroll
+          for (int e = 0; e < E / 2; ++e) {
+            p0[e] = __floats2bfloat162_rn(re[2 * e], re[2 * e + 1]);
+            p1[e] = __floats2bfloat162_rn(im[2 * e], im[2 * e + 1]);
+          }
+          *reinterpret_cast<uint4*>(sB + sw128_offset_e(r0, k0, rows, esize)) = v0;
+          *reinterpret_cast<uint4*>(sB + sw128_offset_e(r0 + 1, k0, rows, esize)) = v1;
         }
       }
-      c += dc;
-      u += du;
-      if (u >= units) {
-        u -= units;
-        ++c;
-      }
     }
-#pragma unroll
-    for (int j = 0; j < BATCH; ++j) {
-      if (tc[j] >= n_coil) break;
-      const int r0 = tc[j] < a.C ? 2 * tc[j] : a.half + 2 * (tc[j] - a.C), k0 = tu[j] * E;
-      float re[E], im[E];  // rows r0 and r0 + 1
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const bool first = k0 + e + a.k_off < a.q;  // past 2 q the loaded value is zero
-        re[e] = first ? al[j][e].x : -al[j][e].y;
-        im[e] = first ? al[j][e].y : al[j][e].x;
-      }
-      if (SPLIT) {
-        float4 h0, h1, l0, l1;
-        h0 = make_float4(tf32_hi(re[0]), tf32_hi(re[1]), tf32_hi(re[2]), tf32_hi(re[3]));
-        h1 = make_float4(tf32_hi(im[0]), tf32_hi(im[1]), tf32_hi(im[2]), tf32_hi(im[3]));
-        l0 = make_float4(tf32_lo(re[0]), tf32_lo(re[1]), tf32_lo(re[2]), tf32_lo(re[3]));
-        l1 = make_float4(tf32_lo(im[0]), tf32_lo(im[1]), tf32_lo(im[2]), tf32_lo(im[3]));
-        *reinterpret_cast<float4*>(sB + sw128_offset_e(r0, k0, rows, esize)) = h0;
-        *reinterpret_cast<float4*>(sB + sw128_offset_e(r0 + 1, k0, rows, esize)) = h1;
-        *reinterpret_cast<float4*>(sB + sw128_offset_e(r0 + a.n_gemm, k0, rows, esize)) = l0;
-        *reinterpret_cast<float4*>(sB + sw128_offset_e(r0 + 1 + a.n_gemm, k0, rows, esize)) = l1;
-      } else {
-        uint4 v0, v1;
-        __nv_bfloat162* p0 = reinterpret_cast<__nv_bfloat162*>(&v0);
-        __nv_bfloat162* p1 = reinterpret_cast<__nv_bfloat162*>(&v1);
-#pragma unroll
-        for (int e = 0; e < E / 2; ++e) {
-          p0[e] = __floats2bfloat162_rn(re[2 * e], re[2 * e + 1]);
-          p1[e] = __floats2bfloat162_rn(im[2 * e], im[2 * e + 1]);
-        }
-        *reinterpret_cast<uint4*>(sB + sw128_offset_e(r0, k0, rows, esize)) = v0;
-        *reinterpret_cast<uint4*>(sB + sw128_offset_e(r0 + 1, k0, rows, esize)) = v1;
-      }
+    // zero rows: [2C, half) always, [half + 2C, n_gemm) for the Jacobian, else [2C, the slice's last row)
+    const int last = BUNDLE ? (2 * C + 15) / 16 * 16 : a.n_gemm;
+    const int z0 = (with_dalpha ? a.half : last) - 2 * C;
+    const int z1 = with_dalpha ? a.n_gemm - a.half - 2 * C : 0;
+    for (int t = etid; t < (z0 + z1) * units; t += nthr) {
+      const int zr = t / units, zu = t - zr * units;
+      const int r = zr < z0 ? rb + 2 * C + zr : a.half + 2 * C + (zr - z0);
+      const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(sB + sw128_offset_e(r, zu * E, rows, esize)) = zero;
+      if (SPLIT) *reinterpret_cast<uint4*>(sB + sw128_offset_e(r + a.n_gemm, zu * E, rows, esize)) = zero;
     }
-  }
-  // zero rows: [2C, half) always, [half + 2C, n_gemm) for the Jacobian, [2C, n_gemm) otherwise
-  const int z0 = with_dalpha ? a.half - 2 * a.C : a.n_gemm - 2 * a.C;
-  const int z1 = with_dalpha ? a.n_gemm - a.half - 2 * a.C : 0;
-  for (int t = etid; t < (z0 + z1) * units; t += nthr) {
-    const int zr = t / units, zu = t - zr * units;
-    const int r = zr < z0 ? 2 * a.C + zr : a.half + 2 * a.C + (zr - z0);
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    *reinterpret_cast<uint4*>(sB + sw128_offset_e(r, zu * E, rows, esize)) = zero;
-    if (SPLIT) *reinterpret_cast<uint4*>(sB + sw128_offset_e(r + a.n_gemm, zu * E, rows, esize)) = zero;
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
   __syncwarp();
@@ -331,7 +345,7 @@ static __device__ void build_coef_smem(const TcArgs& a, unsigned char* sB, int K
 
 // Epilogue warps (4 of them, warp w owning TMEM lanes 32 (w % 4) ..): one pixel
 // per thread, reading the double-buffered accumulator of each tile this CTA owns.
-template <int MODE, bool SUM2 = false>
+template <int MODE, bool SUM2 = false, bool BUNDLE = false>
 static __device__ __forceinline__ void tc_epilogue(const TcArgs& a, uint32_t tmem, int warp, int lane,
                                                    uint64_t* acc_full, uint64_t* acc_empty, int n_tiles,
                                                    int* s_failed) {
@@ -340,6 +354,7 @@ static __device__ __forceinline__ void tc_epilogue(const TcArgs& a, uint32_t tme
     const int quarter = warp & 3;  // TMEM lanes 32 * quarter ..
     const int row = quarter * 32 + lane;
     int tc = 0;
+    const ExpandSeg first = tc_seg<BUNDLE>(a, 0);
     for (int t = a.t0; t < n_tiles; t += a.tstep, ++tc) {
       const int buf = tc & 1;
       const bool got = mpi_ptx::mbar_wait(&acc_full[buf], (uint32_t)((tc >> 1) & 1), a.err, a.wait_cycles);
@@ -354,7 +369,6 @@ static __device__ __forceinline__ void tc_epilogue(const TcArgs& a, uint32_t tme
       const int nn = valid ? n : 0;
       const float sg = (a.centre ? centre_sign(nn, a.nx, a.ny) : 1.f) * a.scale;
       constexpr bool kScatter = MODE == EX_SCATTER || MODE == EX_SCATTER_ADD;
-      const float2 pimg = (MODE != EX_MAPS && !kScatter) ? a.p[nn] : make_float2(0.f, 0.f);
       // maps mode: where coil c of pixel n goes ([C][N], or the Tucker remap)
       size_t maps_base = (size_t)n, maps_cstride = (size_t)a.N;
       if (MODE == EX_MAPS && a.tuck_B) {
@@ -370,107 +384,113 @@ static __device__ __forceinline__ void tc_epilogue(const TcArgs& a, uint32_t tme
         sc_base = (size_t)(q1 / a.sc_L1) * a.sc_hi + (size_t)(q1 % a.sc_L1) * a.sc_mid + lo +
                   (size_t)a.sc_col0 * a.sc_col;
       }
-      float2 pacc = make_float2(0.f, 0.f);
-      const int n_chunks = (2 * a.C + 15) / 16;
-      for (int ch = 0; ch < n_chunks; ++ch) {
-        // issue this chunk's per-coil loads before the accumulator reads
-        float2 wv[8];
-        if (MODE == EX_ADJ || MODE == EX_JADJ) {
+      for (int gi = 0; gi < (BUNDLE ? a.n_segs : 1); ++gi) {
+        const ExpandSeg g = !BUNDLE || gi == 0 ? first : tc_seg<BUNDLE>(a, gi);
+        const uint32_t tseg = tbase + (uint32_t)(16 * g.chunk0);
+        constexpr bool kImage = MODE == EX_FWD || MODE == EX_JFWD || MODE == EX_JADJ;
+        const float2 pimg = kImage ? g.p[nn] : make_float2(0.f, 0.f);
+        float2 pacc = make_float2(0.f, 0.f);
+        const int n_chunks = (2 * g.C + 15) / 16;
+        for (int ch = 0; ch < n_chunks; ++ch) {
+          // issue this chunk's per-coil loads before the accumulator reads
+          float2 wv[8];
+          if (MODE == EX_ADJ || MODE == EX_JADJ) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int c = min(ch * 8 + i, g.C - 1);
+              wv[i] = g.w[(size_t)c * a.N + nn];
+            }
+          }
+          // accumulator columns of this chunk (and of the Jacobian's second block), plus
+          // the second partial sums where the accumulation is split (a.lo_cols)
+          uint32_t v[16], vd[16], w2[16], wd2[16];
+          tmem_ld16_start(tseg + ch * 16, v);
+          if (MODE == EX_JFWD) tmem_ld16_start(tseg + a.half + ch * 16, vd);
+          if (SUM2) {
+            tmem_ld16_start(tseg + a.lo_cols + ch * 16, w2);
+            if (MODE == EX_JFWD) tmem_ld16_start(tseg + a.lo_cols + a.half + ch * 16, wd2);
+          }
+          tmem_wait_ld();
+          reg_fence16(v);
+          if (MODE == EX_JFWD) reg_fence16(vd);
+          if (SUM2) {
+            reg_fence16(w2);
+            if (MODE == EX_JFWD) reg_fence16(wd2);
+          }
+          float r[16], rd[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            r[i] = __uint_as_float(v[i]) + (SUM2 ? __uint_as_float(w2[i]) : 0.f);
+            if (MODE == EX_JFWD) rd[i] = __uint_as_float(vd[i]) + (SUM2 ? __uint_as_float(wd2[i]) : 0.f);
+          }
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            const int c = min(ch * 8 + i, a.C - 1);
-            wv[i] = a.w[(size_t)c * a.N + nn];
-          }
-        }
-        // accumulator columns of this chunk (and of the Jacobian's second block), plus
-        // the second partial sums where the accumulation is split (a.lo_cols)
-        uint32_t v[16], vd[16], w2[16], wd2[16];
-        tmem_ld16_start(tbase + ch * 16, v);
-        if (MODE == EX_JFWD) tmem_ld16_start(tbase + a.half + ch * 16, vd);
-        if (SUM2) {
-          tmem_ld16_start(tbase + a.lo_cols + ch * 16, w2);
-          if (MODE == EX_JFWD) tmem_ld16_start(tbase + a.lo_cols + a.half + ch * 16, wd2);
-        }
-        tmem_wait_ld();
-        reg_fence16(v);
-        if (MODE == EX_JFWD) reg_fence16(vd);
-        if (SUM2) {
-          reg_fence16(w2);
-          if (MODE == EX_JFWD) reg_fence16(wd2);
-        }
-        float r[16], rd[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          r[i] = __uint_as_float(v[i]) + (SUM2 ? __uint_as_float(w2[i]) : 0.f);
-          if (MODE == EX_JFWD) rd[i] = __uint_as_float(vd[i]) + (SUM2 ? __uint_as_float(wd2[i]) : 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int c = ch * 8 + i;
-          const bool cv = valid && c < a.C;
-          const float2 s = make_float2(r[2 * i], r[2 * i + 1]);
-          if (MODE == EX_MAPS) {
-            if (cv) a.out[maps_base + (size_t)c * maps_cstride] = s;
-          } else if (MODE == EX_SCATTER_ADD) {
-            if (cv) {
-              // partial sums of the K parts: added into a zeroed output; with two
-              // parts (0 + a) + b = (0 + b) + a exactly, so the result does not
-              // depend on which part lands first
-              float* o = reinterpret_cast<float*>(a.out) + sc_base + (size_t)c * a.sc_col;
-              atomicAdd(o, s.x);
-              atomicAdd(o + a.sc_im, s.y);
-            }
-          } else if (MODE == EX_SCATTER) {
-            if (cv && a.sc_bf16) {
-              __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(a.out) + sc_base + (size_t)c * a.sc_col;
-              o[0] = __float2bfloat16_rn(s.x);
-              o[a.sc_im] = __float2bfloat16_rn(s.y);
-            } else if (cv) {
-              float* o = reinterpret_cast<float*>(a.out) + sc_base + (size_t)c * a.sc_col;
-              o[0] = s.x;
-              o[a.sc_im] = s.y;
-            }
-          } else if (MODE == EX_FWD) {
-            const float2 v = cmul(s, pimg);
-            if (cv) {
-              float2* o = a.out + (size_t)c * a.N + n;
-              float2 r2 = make_float2(v.x * sg, v.y * sg);
-              if (a.accumulate) {
-                r2.x += o->x;
-                r2.y += o->y;
+            const int c = ch * 8 + i;
+            const bool cv = valid && c < g.C;
+            const float2 s = make_float2(r[2 * i], r[2 * i + 1]);
+            if (MODE == EX_MAPS) {
+              if (cv) g.out[maps_base + (size_t)c * maps_cstride] = s;
+            } else if (MODE == EX_SCATTER_ADD) {
+              if (cv) {
+                // partial sums of the K parts: added into a zeroed output; with two
+                // parts (0 + a) + b = (0 + b) + a exactly, so the result does not
+                // depend on which part lands first
+                float* o = reinterpret_cast<float*>(g.out) + sc_base + (size_t)c * a.sc_col;
+                atomicAdd(o, s.x);
+                atomicAdd(o + a.sc_im, s.y);
               }
-              *o = r2;
-            }
-          } else if (MODE == EX_JFWD) {
-            const float2 ds = make_float2(rd[2 * i], rd[2 * i + 1]);
-            const float2 v1 = cmul(s, dpi);
-            const float2 v2 = cmul(ds, pimg);
-            if (cv) {
-              float2* o = a.out + (size_t)c * a.N + n;
-              float2 r2 = make_float2((v1.x + v2.x) * sg, (v1.y + v2.y) * sg);
-              if (a.accumulate) {
-                r2.x += o->x;
-                r2.y += o->y;
+            } else if (MODE == EX_SCATTER) {
+              if (cv && a.sc_bf16) {
+                __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(g.out) + sc_base + (size_t)c * a.sc_col;
+                o[0] = __float2bfloat16_rn(s.x);
+                o[a.sc_im] = __float2bfloat16_rn(s.y);
+              } else if (cv) {
+                float* o = reinterpret_cast<float*>(g.out) + sc_base + (size_t)c * a.sc_col;
+                o[0] = s.x;
+                o[a.sc_im] = s.y;
               }
-              *o = r2;
-            }
-          } else {
-            if (cv) {
-              const float2 t2 = cmul_conj(s, wv[i]);
-              pacc.x += t2.x;
-              pacc.y += t2.y;
-              if (MODE == EX_JADJ) {
-                const float2 v = cmul_conj(pimg, wv[i]);
-                a.vout[(size_t)c * a.N + n] = make_float2(v.x * sg, v.y * sg);
+            } else if (MODE == EX_FWD) {
+              const float2 v = cmul(s, pimg);
+              if (cv) {
+                float2* o = g.out + (size_t)c * a.N + n;
+                float2 r2 = make_float2(v.x * sg, v.y * sg);
+                if (a.accumulate) {
+                  r2.x += o->x;
+                  r2.y += o->y;
+                }
+                *o = r2;
+              }
+            } else if (MODE == EX_JFWD) {
+              const float2 ds = make_float2(rd[2 * i], rd[2 * i + 1]);
+              const float2 v1 = cmul(s, dpi);
+              const float2 v2 = cmul(ds, pimg);
+              if (cv) {
+                float2* o = g.out + (size_t)c * a.N + n;
+                float2 r2 = make_float2((v1.x + v2.x) * sg, (v1.y + v2.y) * sg);
+                if (a.accumulate) {
+                  r2.x += o->x;
+                  r2.y += o->y;
+                }
+                *o = r2;
+              }
+            } else {
+              if (cv) {
+                const float2 t2 = cmul_conj(s, wv[i]);
+                pacc.x += t2.x;
+                pacc.y += t2.y;
+                if (MODE == EX_JADJ) {
+                  const float2 v = cmul_conj(pimg, wv[i]);
+                  a.vout[(size_t)c * a.N + n] = make_float2(v.x * sg, v.y * sg);
+                }
               }
             }
           }
         }
+        if ((MODE == EX_ADJ || MODE == EX_JADJ) && valid) g.out[n] = make_float2(pacc.x * sg, pacc.y * sg);
       }
       fence_before();
       __syncwarp();
       if (lane == 0) mpi_ptx::mbar_arrive(&acc_empty[buf]);
-      if ((MODE == EX_ADJ || MODE == EX_JADJ) && valid) a.out[n] = make_float2(pacc.x * sg, pacc.y * sg);
     }
   }
 }

@@ -37,21 +37,19 @@ constexpr int kKChunk = 64;  // BF16 elements per 128-byte swizzle row
 constexpr int kMaxStages = 12;
 constexpr int kThreads = 192;
 
-template <int MODE>
+template <int MODE, bool BUNDLE = false>
 __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant__ CUtensorMap tmap, TcArgs a_in,
                                                             int stages) {
   TcArgs a = a_in;
   a.t0 = (int)blockIdx.x;
   a.tstep = (int)gridDim.x;
-  if ((MODE == EX_FWD || MODE == EX_ADJ) && a.rows) {  // grouped launch: this CTA's slice
+  if constexpr (BUNDLE) {  // grouped launch: this CTA's bundle
     const ExpandRow r = a.rows[blockIdx.x];
+    a.segs = r.segs;
+    a.n_segs = r.n_segs;
     a.t0 = r.t0;
     a.tstep = r.step;
-    a.alpha = r.alpha;
-    a.p = r.p;
-    a.w = r.w;
-    a.out = r.out;
-    a.C = r.C;
+    a.n_gemm = a.half = 16 * r.chunks;
   }
   extern __shared__ unsigned char smem_raw[];
   // aligned by an offset from the shared array, so that accesses stay shared-memory ones
@@ -169,8 +167,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_expand_tc(const __grid_constant
     if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2) {
     mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
-    build_coef_smem<false>(a, sB, Kp, MODE == EX_JFWD, tid - 64, 128, bfull);
-    tc_epilogue<MODE>(a, tmem, warp, lane, acc_full, acc_empty, n_tiles, &s_failed);
+    build_coef_smem<false, BUNDLE>(a, sB, Kp, MODE == EX_JFWD, tid - 64, 128, bfull);
+    tc_epilogue<MODE, false, BUNDLE>(a, tmem, warp, lane, acc_full, acc_empty, n_tiles, &s_failed);
   }
   fence_before();
   __syncthreads();
@@ -340,24 +338,30 @@ mpi_status launch_expand_tc(mpi_ctx* ctx, const mpi_basis* b, int mode, const Ex
   const dim3 grid((unsigned)(x.rows ? x.n_ctas : std::min(n_tiles, per_sm * std::max(ctx->num_sms, 1))));
   const CUtensorMap& map = *(const CUtensorMap*)b->tmap;
   cudaError_t e = cudaSuccess;
-#define MPI_TC_CASE(m)                                                                                        \
-  case m:                                                                                                     \
-    e = smem_attr(ctx, (const void*)k_expand_tc<m>);                                                         \
-    if (e != cudaSuccess) return cuda_check(ctx, e, "tc smem attribute");                                    \
-    MPI_PROF(ctx, KF_EXPAND);                                                                                \
-    launch_pdl(ctx, k_expand_tc<m>, dim3(grid), dim3(kThreads), smem, map, a, stages);                                           \
-    break;
-  switch (mode) {
-    MPI_TC_CASE(EX_MAPS)
-    MPI_TC_CASE(EX_FWD)
-    MPI_TC_CASE(EX_JFWD)
-    MPI_TC_CASE(EX_ADJ)
-    MPI_TC_CASE(EX_JADJ)
-    MPI_TC_CASE(EX_SCATTER)
+#define MPI_TC_LAUNCH(...)                                                                \
+  do {                                                                                    \
+    e = smem_attr(ctx, (const void*)k_expand_tc<__VA_ARGS__>);                            \
+    if (e != cudaSuccess) return cuda_check(ctx, e, "tc smem attribute");                 \
+    MPI_PROF(ctx, KF_EXPAND);                                                             \
+    launch_pdl(ctx, k_expand_tc<__VA_ARGS__>, grid, dim3(kThreads), smem, map, a, stages); \
+  } while (0)
+  switch (x.rows && mode != EX_FWD && mode != EX_ADJ ? -1 : mode) {
+    case EX_MAPS: MPI_TC_LAUNCH(EX_MAPS); break;
+    case EX_FWD:
+      if (x.rows) MPI_TC_LAUNCH(EX_FWD, true);
+      else MPI_TC_LAUNCH(EX_FWD);
+      break;
+    case EX_JFWD: MPI_TC_LAUNCH(EX_JFWD); break;
+    case EX_ADJ:
+      if (x.rows) MPI_TC_LAUNCH(EX_ADJ, true);
+      else MPI_TC_LAUNCH(EX_ADJ);
+      break;
+    case EX_JADJ: MPI_TC_LAUNCH(EX_JADJ); break;
+    case EX_SCATTER: MPI_TC_LAUNCH(EX_SCATTER); break;
     default:
       return set_err(ctx, MPI_ERR_ARG, "unknown expansion mode");
   }
-#undef MPI_TC_CASE
+#undef MPI_TC_LAUNCH
   MPI_LAUNCH_CHECK(ctx, x.kname ? x.kname : "k_expand_tc");
   return MPI_OK;
 }

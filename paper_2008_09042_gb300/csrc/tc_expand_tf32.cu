@@ -96,7 +96,12 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) 
 // lo(U) per stage.
 // ODD: the K box count is odd, so the last ring stage of each tile holds one box
 // (a compile-time choice: with an even count the stage loop has no box test).
-template <int MODE, bool ODD = false>
+// GRP: coil groups as grid rows (1) or a grouped launch's bundles (2).  (Compile-time: with
+// the tests at run time, or either one's values in the arguments, the other launches lost
+// the arguments' place in the constant bank: Tucker core contraction 45 us instead of
+// 33.5.  Bundles with a ring of one-box stages, 64 KB beside 32 coils of q = 160 in four
+// parts instead of two, were slower: 235 against 230 us.)
+template <int MODE, bool ODD = false, int GRP = 0>
 __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_constant__ CUtensorMap tmap, TcArgs a_in,
                                                                 int stages) {
   // Coil groups: the CTAs of row blockIdx.y expand their group's coils.  The
@@ -105,20 +110,17 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
   TcArgs a = a_in;
   a.t0 = (int)blockIdx.x;
   a.tstep = (int)gridDim.x;
-  if ((MODE == EX_FWD || MODE == EX_ADJ) && a.rows) {  // grouped launch: this CTA's slice, with the operand, accumulators and ring of its own coil count
+  if constexpr (GRP == 2) {  // grouped launch: this CTA's bundle, with the operand, accumulators and ring of its own column count
     const ExpandRow r = a.rows[blockIdx.x];
+    a.segs = r.segs;
+    a.n_segs = r.n_segs;
     a.t0 = r.t0;
     a.tstep = r.step;
-    a.n_gemm = a.half = a.lo_cols = (2 * r.C + 15) / 16 * 16;
+    a.n_gemm = a.half = a.lo_cols = 16 * r.chunks;
     a.half_cols = tf32_acc_cols(a.n_gemm);
     stages = tf32_stages(a.n_gemm, a.KC * kKChunk32, (size_t)a.smem);
-    a.alpha = r.alpha;
-    a.p = r.p;
-    a.w = r.w;
-    a.out = r.out;
-    a.C = r.C;
   }
-  if (a.group_coils) {
+  if constexpr (GRP == 1) {
     const int c0 = (int)blockIdx.y * a.group_coils;
     a.C = min(a.group_coils, a.C_total - c0);
     a.alpha += (size_t)c0 * a.q;
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
     // operand, which every MMA waits for (one inlined copy for both: small
     // launches are short enough for the code they fetch to count)
     mpi_ptx::pdl_wait();  // alpha, p and w may come from the previous kernel
-    build_coef_smem<true>(a, sB, Kp, MODE == EX_JFWD, tid - 64, 256, bfull);
+    build_coef_smem<true, GRP == 2>(a, sB, Kp, MODE == EX_JFWD, tid - 64, 256, bfull);
   }
   if (warp == 0 && lane == 0) {
     // ---------------- producer: TMA tiles of U
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_expand_tf32x3(const __grid_co
     mbar_wait_warp(drain, 0, a.err, a.wait_cycles);
     if (!ok && lane == 0) s_failed = 1;
   } else if (warp >= 2 && warp <= 5) {
-    tc_epilogue<MODE, true>(a, tmem, warp, lane, acc_full, acc_empty, n_tiles, &s_failed);
+    tc_epilogue<MODE, true, GRP == 2>(a, tmem, warp, lane, acc_full, acc_empty, n_tiles, &s_failed);
   }
   fence_before();
   __syncthreads();
@@ -641,7 +643,7 @@ mpi_status launch_expand_tf32(mpi_ctx* ctx, const mpi_basis* b, int mode, const 
   const int nrows = ks > 1 ? ks : groups;
   const int per_row = std::max(std::max(ctx->num_sms, 1) / nrows, 1);
   dim3 grid((unsigned)std::min(n_tiles, per_row), (unsigned)nrows);
-  if (x.rows) {  // each CTA lays out its own slice's ring in all of the SM's memory
+  if (x.rows) {  // each CTA lays out its own bundle's ring in all of the SM's memory
     a.group_coils = 0;
     a.tmem_cols = 512;
     pl.smem = kSmemMax;
@@ -655,30 +657,45 @@ mpi_status launch_expand_tf32(mpi_ctx* ctx, const mpi_basis* b, int mode, const 
   const bool odd = a.KC % 2 != 0;
   if (odd && mode != EX_SCATTER && mode != EX_SCATTER_ADD)
     return set_err(ctx, MPI_ERR_UNSUPPORTED, "3xTF32 expansion: odd K box count in this mode");
-#define MPI_TF_LAUNCH(m, o)                                                                                   \
-  do {                                                                                                        \
-    e = smem_attr(ctx, (const void*)k_expand_tf32x3<m, o>);                                                     \
-    if (e != cudaSuccess) return cuda_check(ctx, e, "tf32 smem attribute");                                  \
-    MPI_PROF(ctx, KF_EXPAND);                                                                                \
-    launch_pdl(ctx, k_expand_tf32x3<m, o>, grid, dim3(kThreads32), pl.smem, map, a, pl.stages);            \
+#define MPI_TF_LAUNCH(...)                                                                               \
+  do {                                                                                                  \
+    e = smem_attr(ctx, (const void*)k_expand_tf32x3<__VA_ARGS__>);                                      \
+    if (e != cudaSuccess) return cuda_check(ctx, e, "tf32 smem attribute");                             \
+    MPI_PROF(ctx, KF_EXPAND);                                                                           \
+    launch_pdl(ctx, k_expand_tf32x3<__VA_ARGS__>, grid, dim3(kThreads32), pl.smem, map, a, pl.stages);  \
   } while (0)
+#define MPI_TF_GROUPS(m, o)                \
+  do {                                     \
+    if (a.group_coils) MPI_TF_LAUNCH(m, o, 1); \
+    else MPI_TF_LAUNCH(m, o, 0);           \
+  } while (0)
+  if ((x.rows && mode != EX_FWD && mode != EX_ADJ) ||
+      (a.group_coils && (mode == EX_ADJ || mode == EX_JADJ || mode == EX_SCATTER_ADD)))
+    return set_err(ctx, MPI_ERR_ARG, "3xTF32 expansion: groups in this mode");
   switch (mode) {
-    case EX_MAPS: MPI_TF_LAUNCH(EX_MAPS, false); break;
-    case EX_FWD: MPI_TF_LAUNCH(EX_FWD, false); break;
-    case EX_JFWD: MPI_TF_LAUNCH(EX_JFWD, false); break;
-    case EX_ADJ: MPI_TF_LAUNCH(EX_ADJ, false); break;
-    case EX_JADJ: MPI_TF_LAUNCH(EX_JADJ, false); break;
+    case EX_MAPS: MPI_TF_GROUPS(EX_MAPS, false); break;
+    case EX_FWD:
+      if (x.rows) MPI_TF_LAUNCH(EX_FWD, false, 2);
+      else MPI_TF_GROUPS(EX_FWD, false);
+      break;
+    case EX_JFWD: MPI_TF_GROUPS(EX_JFWD, false); break;
+    case EX_ADJ:
+      if (x.rows) MPI_TF_LAUNCH(EX_ADJ, false, 2);
+      else MPI_TF_LAUNCH(EX_ADJ, false, 0);
+      break;
+    case EX_JADJ: MPI_TF_LAUNCH(EX_JADJ, false, 0); break;
     case EX_SCATTER:
-      if (odd) MPI_TF_LAUNCH(EX_SCATTER, true);
-      else MPI_TF_LAUNCH(EX_SCATTER, false);
+      if (odd) MPI_TF_GROUPS(EX_SCATTER, true);
+      else MPI_TF_GROUPS(EX_SCATTER, false);
       break;
     case EX_SCATTER_ADD:
-      if (odd) MPI_TF_LAUNCH(EX_SCATTER_ADD, true);
-      else MPI_TF_LAUNCH(EX_SCATTER_ADD, false);
+      if (odd) MPI_TF_LAUNCH(EX_SCATTER_ADD, true, 0);
+      else MPI_TF_LAUNCH(EX_SCATTER_ADD, false, 0);
       break;
     default:
       return set_err(ctx, MPI_ERR_ARG, "unknown expansion mode");
   }
+#undef MPI_TF_GROUPS
 #undef MPI_TF_LAUNCH
   MPI_LAUNCH_CHECK(ctx, x.kname ? x.kname : "k_expand_tf32x3");
   return MPI_OK;
