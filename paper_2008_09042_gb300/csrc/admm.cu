@@ -26,7 +26,7 @@
 //   Reductions: partial sums per CTA, added in a fixed order by the kernels that use
 // them, so results do not depend on the order the CTAs run in.
 // At 256^2, 16 coils, q = 128 an outer step (5 CG, 10 TV iterations) went from 725
-// to 245 us, in 33 launches instead of 124.
+// to 215 us, in 33 launches instead of 124.
 #include <math.h>
 
 #include <algorithm>
@@ -119,6 +119,12 @@ __device__ __forceinline__ Sum2 warp_sum(Sum2 s) {
 }
 
 __device__ __forceinline__ float2 pack(Sum2 s) { return make_float2(s.h, s.l); }
+__device__ __forceinline__ Sum2 unpack(float2 v) {
+  Sum2 s;
+  s.h = v.x;
+  s.l = v.y;
+  return s;
+}
 __device__ __forceinline__ double to_double(Sum2 s) { return (double)s.h + (double)s.l; }
 
 // Sums over the CTA (valid in thread 0); sh holds NV values per warp.
@@ -280,9 +286,14 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
   const int t = tc / a.C, c = tc - t * a.C;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   float beta = 0.f;
-  if (!INV && a.r) {  // every warp adds the partial sums (a few per lane, L2 hits)
-    const Sum2 rr = partial_sum(a.rr, a.n_part), old = partial_sum(a.rr_old, a.n_part);
-    beta = pair_ratio(rr, old);
+  if (!INV && a.r) {  // a warp each for the two sums (all eight doing both: a third of the pass's instructions)
+    __shared__ float2 s_rr[2];
+    if (w < 2) {
+      const Sum2 sum = partial_sum(w ? a.rr_old : a.rr, a.n_part);
+      if (lane == 0) s_rr[w] = pack(sum);
+    }
+    __syncthreads();
+    beta = pair_ratio(unpack(s_rr[0]), unpack(s_rr[1]));
   }
   if constexpr (R1 > 0) {
     constexpr int G = kThreads / TILE;  // rows r (step 1) or k1 (step 2) at a time
