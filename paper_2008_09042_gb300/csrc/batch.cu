@@ -83,6 +83,13 @@ bool groupable(const mpi_batch_slice& s, mpi_precision prec) {
   return s.plan->kind == MPI_TRAJ_CARTESIAN && !s.basis->tucker && rows_supported(s.basis, s.C, prec);
 }
 
+// Whether two plans have the same grid: slices of equal N and nx may still be a 2D
+// slice and a volume, or volumes split differently into y and z, whose centring signs
+// and passes differ.
+bool same_grid(const mpi_plan* a, const mpi_plan* b) {
+  return a->ndim == b->ndim && a->nz == b->nz && a->ny == b->ny && a->nx == b->nx;
+}
+
 // The group's forward and adjoint expansions, and its slices' FFT passes.
 mpi_status record_group(mpi_ctx* ctx, const mpi_batch_slice* sl, const Group& g, int kind, mpi_precision prec, float2* buf) {
   const mpi_batch_slice& s0 = sl[g.idx[0]];
@@ -381,7 +388,7 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     int j = i;
     const mpi_batch_slice& a = slices[order[i]];
     while (j < n && slices[order[j]].basis == a.basis && groupable(slices[order[j]], prec) && groupable(a, prec) &&
-           slices[order[j]].plan->N == a.plan->N && slices[order[j]].plan->nx == a.plan->nx)
+           same_grid(slices[order[j]].plan, a.plan))
       ++j;
     if (j - i >= 2) {
       Group g;
@@ -401,9 +408,10 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     ++i;
   }
 
-  // grouped passes: slices in the order of the kinds of their passes along y
+  // grouped passes (2D; volumes keep the passes of their own calls): slices in the order
+  // of the kinds of their passes along y
   for (Group& g : groups) {
-    if ((int)g.idx.size() < kGroupedPasses || ctx->line_kernel) continue;
+    if ((int)g.idx.size() < kGroupedPasses || ctx->line_kernel || slices[g.idx[0]].plan->ndim != 2) continue;
     std::stable_sort(g.idx.begin(), g.idx.end(), [&](int a, int b) {
       const mpi_batch_slice &x = slices[a], &y = slices[b];
       const bool fa = fft_cols_in_registers(ctx, x.plan, x.C, false), fb = fft_cols_in_registers(ctx, y.plan, y.C, false);
