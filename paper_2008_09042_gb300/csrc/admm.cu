@@ -16,17 +16,18 @@
 //   k_maps_cols<inv>    inverse DFT along y, times conj(s) on store
 //   k_coil_sum          sum over coils, + d, and the CG's <d, A d>
 //   k_cg_update         x, r, |r|^2
-// and an outer step adds the ball projection inside the scatter of the k-space
-// rows (k_rows_scatter_ball), the dual update of the data blocks and their
-// residual norms inside the gather (k_rows_gather_dual) and the image's dual
-// update with the choice of rho (k_admm_dual).
+// and an outer step adds the norms of the ball projection (k_ball_norm), the
+// projection inside the scatter of the k-space rows (k_rows_scatter_ball), the dual
+// update of the data blocks and their residual norms inside the gather
+// (k_rows_gather_dual) and the image's dual update with the choice of rho
+// (k_admm_dual).
 //   The CG starts from the previous p, whose F_s S p is at hand (Apk), so its first
 // residual is one adjoint:  r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p.
 //   rho's rescaling of the scaled duals is applied where they are read (ufac).
 //   Reductions: partial sums per CTA, added in a fixed order by the kernels that use
 // them, so results do not depend on the order the CTAs run in.
 // At 256^2, 16 coils, q = 128 an outer step (5 CG, 10 TV iterations) went from 725
-// to 215 us, in 33 launches instead of 124.
+// to 224 us, in 33 launches instead of 124.
 #include <math.h>
 
 #include <algorithm>
@@ -52,119 +53,170 @@ enum { S_RHO = 0, S_UFAC, S_NUM };
 
 // ------------------------------------------------------------- reductions
 //
-// Sums are kept as pairs of FP32 values (h + l, about 48 bits) of exact differences
-// and products, from the threads to the partial sums: this GPU does two FP64
-// operations per clock and SM, and the fourteen per sample of the data blocks'
-// residuals took longer than everything else in their pass.  Every factor of a
-// product is multiplied by sum_scale first, a power of two that brings the data to
-// magnitude one (exact), since squares of FP32 values leave FP32's range long before
-// the values do; ratios of sums do not see it, norms are divided by it.
+// Sums are software floats of 58-bit mantissas with exponents of their own (Sum: v 2^e),
+// from the threads to the partial sums.  They are no less accurate than the FP64 sums of
+// the solve on the operator calls (errors of random dot products, and of sums of squared
+// differences of two and three terms, 0.06 to 0.6 of FP64's), and their range has no end,
+// where squares of FP32 values leave FP32's long before the values do: maps of magnitude
+// s make <d, A d> grow as s^4.  FP64 itself runs at two operations per clock and SM here:
+// an outer step at 256^2 and 16 coils took 290 us with it, 219 with pairs of FP32 values
+// (48 bits, FP32's range) and 224 this way.
 
-struct Sum2 {
-  float h = 0.f, l = 0.f;
+struct alignas(16) Sum {
+  long long v;  // |v| < 2^58
+  int e;
 };
+constexpr int kEmpty = -(1 << 22), kNotFinite = 1 << 24;  // exponents of zero, and of an infinity or NaN
 
-// s += p + e, e a small correction of p
-__device__ __forceinline__ void sum2_add(Sum2& s, float p, float e) {
-  const float t = s.h + p, z = t - s.h;
-  s.l += ((s.h - (t - z)) + (p - z)) + e;
-  s.h = t;
+__device__ __forceinline__ Sum sum_zero() { return Sum{0, kEmpty}; }
+__device__ __forceinline__ bool not_finite(Sum s) { return s.e >= kNotFinite / 2; }
+
+// |x| = m 2^e with m's leading bit at bit 23 (zero: m = 0)
+__device__ __forceinline__ void float_parts(float x, unsigned& m, int& e) {
+  const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+  m = (b & 0x7fffffu) | 0x800000u;
+  e = (int)(b >> 23) - 150;
+  if (b - 0x00800000u >= 0x7f000000u) {  // zero, subnormal, infinite or NaN
+    const int n = __clz(b) - 8;
+    m = b >= 0x7f800000u ? 0x800000u : (b ? b << n : 0u);
+    e = b >= 0x7f800000u ? kNotFinite : (b ? -149 - n : kEmpty);
+  }
 }
-// s += a b
-__device__ __forceinline__ void sum2_mul(Sum2& s, float a, float b) {
-  const float p = a * b;
-  sum2_add(s, p, fmaf(a, b, -p));
+// v with the sign of x y
+__device__ __forceinline__ long long signed_by(long long v, float x, float y = 0.f) {
+  return (int)(__float_as_uint(x) ^ __float_as_uint(y)) < 0 ? -v : v;
 }
-// s += (d + e)^2, e a small correction of d
-__device__ __forceinline__ void sum2_sq(Sum2& s, float d, float e) {
-  const float p = d * d;
-  sum2_add(s, p, fmaf(2.f * d, e, fmaf(d, d, -p)));
+__device__ __forceinline__ long long shift_down(long long v, int n) { return v >> min(n, 63); }
+
+__device__ __forceinline__ Sum sum_add(Sum a, Sum b) {
+  const int e = max(a.e, b.e);
+  const long long v = shift_down(a.v, e - a.e) + shift_down(b.v, e - b.e);
+  const int over = (int)((unsigned long long)(v + (1LL << 58)) >> 59) & 1;  // |v| reached 2^58
+  return Sum{v >> over, e + over};
 }
-// d + e = a - b exactly
+
+// Re(conj(a) b); the products' leading bit is bit 55 or 56
+__device__ __forceinline__ Sum sum_dot(float2 a, float2 b) {
+  unsigned m[4];
+  int e[4];
+  float_parts(a.x, m[0], e[0]);
+  float_parts(b.x, m[1], e[1]);
+  float_parts(a.y, m[2], e[2]);
+  float_parts(b.y, m[3], e[3]);
+  const long long px = signed_by((long long)((unsigned long long)m[0] * m[1] << 9), a.x, b.x);
+  const long long py = signed_by((long long)((unsigned long long)m[2] * m[3] << 9), a.y, b.y);
+  const int ex = e[0] + e[1] - 9, ey = e[2] + e[3] - 9, ec = max(ex, ey);
+  return Sum{shift_down(px, ec - ex) + shift_down(py, ec - ey), ec};
+}
+
+// d + e = a - b exactly (no overflow)
 __device__ __forceinline__ float diff_exact(float a, float b, float& e) {
   const float d = a - b, t = d - a;
   e = (a - (d - t)) - (b + t);
   return d;
 }
-// s += |k (a - b)|^2
-__device__ __forceinline__ void sum2_diff_sq(Sum2& s, float k, float2 a, float2 b) {
-  float e;
-  float d = diff_exact(a.x, b.x, e);
-  sum2_sq(s, k * d, k * e);
-  d = diff_exact(a.y, b.y, e);
-  sum2_sq(s, k * d, k * e);
-}
 
-// The power of two for the data's largest finite magnitude (its bits, k_data_max);
-// 2^-126 to 2^126, 1 for data that are all zero.
-__device__ __forceinline__ float sum_scale(const unsigned* __restrict__ ymax) {
-  const unsigned bits = *ymax, e = min(max(bits >> 23, 1u), 253u);
-  return bits ? __uint_as_float((254u - e) << 23) : 1.f;
-}
-
-// Sum over a warp (valid in every lane).
-__device__ __forceinline__ Sum2 warp_sum(Sum2 s) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float h = __shfl_xor_sync(0xffffffffu, s.h, o), l = __shfl_xor_sync(0xffffffffu, s.l, o);
-    // the lower lane's sum first in both lanes, so that all lanes agree
-    const bool up = threadIdx.x & o;
-    Sum2 a;
-    a.h = up ? h : s.h;
-    a.l = up ? l : s.l;
-    sum2_add(a, up ? s.h : h, up ? s.l : l);
-    s = a;
+// (d + c + b)^2, |c| and |b| at most about half a unit in the last place of d
+__device__ __forceinline__ Sum sum_sq(float d, float c, float b = 0.f) {
+  unsigned md, m;
+  int ed, e;
+  float_parts(d, md, ed);
+  long long v = signed_by((long long)md << 34, d);
+  if (c != 0.f) {  // mostly not: differences of values within a factor of two are exact
+    float_parts(c, m, e);
+    v += signed_by(shift_down((long long)m << 34, ed - e), c);
   }
-  return s;
+  if (b != 0.f) {
+    float_parts(b, m, e);
+    v += signed_by(shift_down((long long)m << 34, ed - e), b);
+  }
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v) << 5;  // leading bit 61 to 63
+  return Sum{(long long)(__umul64hi(u, u) >> 5), 2 * (ed - 39) + 69};
 }
 
-__device__ __forceinline__ float2 pack(Sum2 s) { return make_float2(s.h, s.l); }
-__device__ __forceinline__ Sum2 unpack(float2 v) {
-  Sum2 s;
-  s.h = v.x;
-  s.l = v.y;
-  return s;
+// |a - b|^2
+__device__ __forceinline__ Sum sum_diff_sq(float2 a, float2 b) {
+  float cx, cy;
+  const float dx = diff_exact(a.x, b.x, cx), dy = diff_exact(a.y, b.y, cy);
+  return sum_add(sum_sq(dx, cx), sum_sq(dy, cy));
 }
-__device__ __forceinline__ double to_double(Sum2 s) { return (double)s.h + (double)s.l; }
 
-// Sums over the CTA (valid in thread 0); sh holds NV values per warp.
-template <int NV>
-__device__ __forceinline__ void block_sums(const Sum2 (&v)[NV], float2* sh, Sum2 (&out)[NV]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// (a + b - c)^2
+__device__ __forceinline__ Sum sum_diff3_sq(float a, float b, float c) {
+  float c1, c2, c3;
+  float d = diff_exact(a, -b, c1);
+  d = diff_exact(d, c, c2);
+  d = diff_exact(d, -c1, c3);  // d + c3 + c2; where the second difference cancels, c2 = 0
+  return sum_sq(d, c3, c2);
+}
+
+// Sum of v over a warp, |v| < 2^58 (the same value in every lane).
+__device__ __forceinline__ long long warp_add(long long v) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x7ffffffu);
+  const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 27) & 0x7ffffffu);
+  const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 54));
+  return ((long long)hi << 54) + ((long long)mid << 27) + lo;
+}
+__device__ __forceinline__ Sum warp_sum(Sum s) {
+  const int e = __reduce_max_sync(0xffffffffu, s.e);
+  const long long v = warp_add(shift_down(s.v, e - s.e));  // below 2^63
+  const unsigned long long u = v < 0 ? -(unsigned long long)v : (unsigned long long)v;
+  const int n = max(6 - __clzll(u), 0);
+  return Sum{v >> n, e + n};
+}
+
+// out[j] = the sum of v[j] over the CTA's NT threads, by lane 0 of warp j; sh holds
+// NV x NT / 32 values.
+template <int NV, int NT>
+__device__ __forceinline__ void block_sums(const Sum (&v)[NV], Sum* sh, Sum* out) {
+  constexpr int NW = NT / 32;
+  static_assert(NV <= NW && NW <= 32, "a warp per sum");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
-    const Sum2 w = warp_sum(v[j]);
-    if (lane == 0) sh[warp * NV + j] = pack(w);
+    const Sum w = warp_sum(v[j]);
+    if (lane == 0) sh[j * NW + warp] = w;
   }
   __syncthreads();
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      Sum2 s;
-      for (int w = 0; w < nw; ++w) sum2_add(s, sh[w * NV + j].x, sh[w * NV + j].y);
-      out[j] = s;
-    }
-}
-
-// a / b to FP32 accuracy (0 where b <= 0), with the pairs' low parts.
-__device__ __forceinline__ float pair_ratio(Sum2 a, Sum2 b) {
-  const float bh = b.h + b.l, bl = b.l - (bh - b.h), ah = a.h + a.l, al = a.l - (ah - a.h);
-  if (!(bh > 0.f)) return 0.f;
-  const float q = ah / bh;
-  return q + (fmaf(-q, bh, ah) + fmaf(-q, bl, al)) / bh;
-}
-
-// The sum of n partial sums, by one warp in a fixed order (valid in every lane):
-// the kernels that use a reduction's result add its CTAs' partial sums themselves,
-// which is faster than having the last CTA of the reduction do it (its fence,
-// counter and second round trip were 3 us at the end of every such kernel).
-__device__ __forceinline__ Sum2 partial_sum(const float2* __restrict__ part, int n) {
-  Sum2 s;
-  for (int i = threadIdx.x & 31; i < n; i += 32) {
-    const float2 v = part[i];
-    sum2_add(s, v.x, v.y);
+  if (warp < NV) {
+    const Sum w = warp_sum(lane < NW ? sh[warp * NW + lane] : sum_zero());
+    if (lane == 0) out[warp] = w;
   }
-  return warp_sum(s);
+}
+
+// The sum of n <= kMaxElemBlocks partial sums, by one warp in a fixed order (valid in
+// every lane; |v| < 2^63): the kernels that use a reduction's result add its CTAs'
+// partial sums themselves, which is faster than having the last CTA of the reduction do
+// it (its fence, counter and second round trip were 3 us at the end of every such kernel).
+__device__ __forceinline__ Sum partial_sum(const Sum* __restrict__ part, int n) {
+  constexpr int PER = kMaxElemBlocks / 32;
+  static_assert(PER <= 16, "four bits of headroom in a lane");
+  Sum s[PER];
+  int e = kEmpty;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = (threadIdx.x & 31) + 32 * j;
+    s[j] = i < n ? part[i] : sum_zero();
+    e = max(e, s[j].e);
+  }
+  e = __reduce_max_sync(0xffffffffu, e) + 4;
+  long long v = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) v += shift_down(s[j].v, e - s[j].e);
+  return Sum{warp_add(v), e};
+}
+
+// 2^e, e within FP64's normal range
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + min(max(e, -1022), 1023)) << 20, 0); }
+__device__ __forceinline__ double to_double(Sum s) {
+  if (not_finite(s)) return __longlong_as_double(0x7ff8000000000000LL);
+  return (double)s.v * pow2(s.e);  // sums of squares of FP32 values: within FP64's range
+}
+
+// a / b, 0 unless b > 0
+__device__ __forceinline__ float sum_ratio(Sum a, Sum b) {
+  if (b.v <= 0 || not_finite(b)) return 0.f;
+  return (float)(to_double(a) / to_double(b));
 }
 
 // ------------------------------------------------------------ column passes
@@ -175,7 +227,7 @@ struct MapsCols {
   const float2* v;      // forward: image [T][N], or the CG's old direction
   const float2* r;      // forward, next CG direction d = r + beta d_old (null: v itself)
   float2* dnew;         // where that direction goes
-  const float2 *rr, *rr_old;  // partial sums of |r|^2, now and before the last update: beta = rr / rr_old
+  const Sum *rr, *rr_old;  // partial sums of |r|^2, now and before the last update: beta = rr / rr_old
   int n_part;
   int C, nx;
   size_t N;
@@ -202,7 +254,7 @@ constexpr int maps_cols_tile(int L) {
 // R values of one thread: rows y0 + step m of column x, formed from the image and
 // the map (forward) or read from the rows with samples (inverse).  All loads are
 // issued before the first use or store: a CTA has 8 warps and there are only
-// T C nx / 32 of them, so what a thread has in flight sets the time (the loads in
+// T C nx / 16 of them, so what a thread has in flight sets the time (the loads in
 // turn, with the store of the new direction between them: 30 us per pass at
 // 256^2 and 16 coils; batched: see the file header).
 template <int R, bool INV>
@@ -286,14 +338,17 @@ __global__ void __launch_bounds__(kThreads) k_maps_cols(MapsCols a) {
   const int t = tc / a.C, c = tc - t * a.C;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   float beta = 0.f;
-  if (!INV && a.r) {  // a warp each for the two sums (all eight doing both: a third of the pass's instructions)
-    __shared__ float2 s_rr[2];
+  if (!INV && a.r) {  // a warp each for the two sums (both by one: 2 us more per outer step)
+    __shared__ Sum s_rr[2];
+    __shared__ float s_beta;
     if (w < 2) {
-      const Sum2 sum = partial_sum(w ? a.rr_old : a.rr, a.n_part);
-      if (lane == 0) s_rr[w] = pack(sum);
+      const Sum sum = partial_sum(w ? a.rr_old : a.rr, a.n_part);
+      if (lane == 0) s_rr[w] = sum;
     }
     __syncthreads();
-    beta = pair_ratio(unpack(s_rr[0]), unpack(s_rr[1]));
+    if (tid == 0) s_beta = sum_ratio(s_rr[0], s_rr[1]);
+    __syncthreads();
+    beta = s_beta;
   }
   if constexpr (R1 > 0) {
     constexpr int G = kThreads / TILE;  // rows r (step 1) or k1 (step 2) at a time
@@ -397,11 +452,10 @@ struct MapsRows {
   float ksign;
   const float2* y;           // data [T][C][M]
   float2 *ap, *uk, *zk;      // F_s S p, the scaled duals, the projections [T][C][M]
-  const float2* ball;        // partial sums of the ball norms [T][C][kBallBlocks]
+  const Sum* ball;           // partial sums of the ball norms [T][C][kBallBlocks]
   const double* eps;         // ball radii [T][C]
   const double* sc;
-  const unsigned* ymax;      // see sum_scale
-  float2* partials;
+  Sum* partials;
 };
 
 // One sample's F_s S p, scaled dual and datum or projection.
@@ -496,32 +550,33 @@ template <int NX>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_scatter_ball(MapsRows a) {
   using F = Rows<NX>;
   __shared__ float2 buf[kRowWarps][F::kSmem];
+  __shared__ float s_f[kRowWarps];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
   const float fu = (float)a.sc[S_UFAC];
   float2* b = buf[warp];
   const int per = (a.n_list_max + F::R - 1) / F::R, total = a.TC * per;
-  for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
+  for (int g0 = blockIdx.x * kRowWarps; g0 < total; g0 += gridDim.x * kRowWarps) {
+    // f = eps / max(|.|, eps) of the warps' coils by one warp, a lane each: an FP64 root
+    // and division by every warp would take the pass longer than its rows
+    if (warp == 0 && lane < kRowWarps && g0 + lane < total) {
+      const int tc = (g0 + lane) / per;
+      Sum sq = sum_zero();
+#pragma unroll
+      for (int i = 0; i < kBallBlocks; ++i) sq = sum_add(sq, a.ball[(size_t)tc * kBallBlocks + i]);
+      const double nrm = sqrt(to_double(sq)), eps = a.eps[tc];
+      s_f[lane] = nrm > eps ? (float)(eps / nrm) : 1.f;
+    }
+    __syncthreads();
+    const float fc = s_f[warp];
+    __syncthreads();
+    const int gi = g0 + warp;
+    if (gi >= total) continue;  // warp-uniform, as below; every warp of the CTA runs all rounds
     const int tc = gi / per, j0 = (gi - tc * per) * F::R, t = tc / a.C;
     const int n_list = a.n_list[t];
-    if (j0 >= n_list) continue;  // warp-uniform
+    if (j0 >= n_list) continue;
     const int32_t* list = a.row_list + (size_t)t * a.ny;
-    // f = eps / max(|.|, eps): the root and the quotient corrected by their residues,
-    // so that FP32 arithmetic gives the FP64 value's rounding
-    Sum2 nrm;
-#pragma unroll
-    for (int i = 0; i < kBallBlocks; ++i) {
-      const float2 v = a.ball[(size_t)tc * kBallBlocks + i];
-      sum2_add(nrm, v.x, v.y);
-    }
-    const double eps = a.eps[tc] * sum_scale(a.ymax);
-    Sum2 root, radius;
-    root.h = sqrtf(nrm.h);
-    root.l = root.h > 0.f ? 0.5f * (fmaf(-root.h, root.h, nrm.h) + nrm.l) / root.h : 0.f;
-    radius.h = (float)eps;
-    radius.l = (float)(eps - radius.h);
-    const float fc = root.h > radius.h ? pair_ratio(radius, root) : 1.f;
     for (int i = lane; i < F::kSmem; i += 32) b[i] = make_float2(0.f, 0.f);
     __syncwarp();
     int row[F::R];  // the group's rows and the range of their samples
@@ -572,13 +627,13 @@ template <int NX>
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_gather_dual(MapsRows a) {
   using F = Rows<NX>;
   __shared__ float2 buf[kRowWarps][F::kSmem];
-  __shared__ float2 sh[2 * kRowWarps];
+  __shared__ Sum sh[2 * kRowWarps];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, p = lane % F::P;
-  const float fu = (float)a.sc[S_UFAC], ks = sum_scale(a.ymax);
+  const float fu = (float)a.sc[S_UFAC];
   float2* b = buf[warp];
-  Sum2 sums[2];
+  Sum sums[2] = {sum_zero(), sum_zero()};
   const int per = (a.n_list_max + F::R - 1) / F::R, total = a.TC * per;
   for (int gi = blockIdx.x * kRowWarps + warp; gi < total; gi += gridDim.x * kRowWarps) {
     const int tc = gi / per, j0 = (gi - tc * per) * F::R, t = tc / a.C;
@@ -629,17 +684,12 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_gather_dual(MapsRows a)
           const float2 ap = make_float2(e.x * sg, e.y * sg);
           a.ap[i0 + m] = ap;
           a.uk[i0 + m] = make_float2(fu * d.uk.x + ap.x - d.yz.x, fu * d.uk.y + ap.y - d.yz.y);
-          sum2_diff_sq(sums[0], ks, ap, d.yz);
-          sum2_diff_sq(sums[1], ks, ap, d.ap);
+          sums[0] = sum_add(sums[0], sum_diff_sq(ap, d.yz));
+          sums[1] = sum_add(sums[1], sum_diff_sq(ap, d.ap));
         });
     __syncwarp();
   }
-  Sum2 out[2];
-  block_sums(sums, sh, out);
-  if (threadIdx.x == 0) {
-    a.partials[2 * (size_t)blockIdx.x] = pack(out[0]);
-    a.partials[2 * (size_t)blockIdx.x + 1] = pack(out[1]);
-  }
+  block_sums<2, kRowWarps * 32>(sums, sh, a.partials + 2 * (size_t)blockIdx.x);
 }
 
 // ------------------------------------------------------- element-wise passes
@@ -653,19 +703,18 @@ struct CoilSum {
   const float2 *z0, *u0, *p;             // residual: sum + z0 - ufac u0 - p
   float2 *r, *p_prev;                    //   into r and d; p kept as p_prev
   const double* sc;
-  const unsigned* ymax;  // see sum_scale
-  float2* partials;  // per CTA: normal, <d, A d>; residual, |r|^2
+  Sum* partials;  // per CTA: normal, <d, A d>; residual, |r|^2
 };
 
 // sum over coils of conj(s_k) w_k with sign and scale.  NORMAL: A d and <d, A d>;
 // else the CG's first residual and |r|^2.
 template <bool NORMAL>
 __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
-  __shared__ float2 sh[kElemThreads / 32];
+  __shared__ Sum sh[kElemThreads / 32];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  const float fu = NORMAL ? 1.f : (float)a.sc[S_UFAC], ks = sum_scale(a.ymax);
-  Sum2 s[1];
+  const float fu = NORMAL ? 1.f : (float)a.sc[S_UFAC];
+  Sum s[1] = {sum_zero()};
   for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < a.total; i += (size_t)gridDim.x * kElemThreads) {
     const size_t t = i / a.N, n = i - t * a.N;
     const float2* w = a.W + t * a.C * a.N + n;
@@ -693,21 +742,17 @@ __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
       const float2 d = a.d[i];
       o = make_float2(o.x + d.x, o.y + d.y);
       a.Ad[i] = o;
-      sum2_mul(s[0], ks * d.x, ks * o.x);
-      sum2_mul(s[0], ks * d.y, ks * o.y);
+      s[0] = sum_add(s[0], sum_dot(d, o));
     } else {
       const float2 z = a.z0[i], u = a.u0[i], p = a.p[i];
       o = make_float2(o.x + z.x - fu * u.x - p.x, o.y + z.y - fu * u.y - p.y);
       a.r[i] = o;
       a.d[i] = o;
       a.p_prev[i] = p;
-      sum2_mul(s[0], ks * o.x, ks * o.x);
-      sum2_mul(s[0], ks * o.y, ks * o.y);
+      s[0] = sum_add(s[0], sum_dot(o, o));
     }
   }
-  Sum2 out[1];
-  block_sums(s, sh, out);
-  if (threadIdx.x == 0) a.partials[blockIdx.x] = pack(out[0]);
+  block_sums<1, kElemThreads>(s, sh, a.partials + blockIdx.x);
 }
 
 // x += a d, r -= a A d with a = |r|^2 / <d, A d>, and the new |r|^2 (partial sums in
@@ -715,17 +760,16 @@ __global__ void __launch_bounds__(kElemThreads) k_coil_sum(CoilSum a) {
 __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__ x, float2* __restrict__ r,
                                                             const float2* __restrict__ d,
                                                             const float2* __restrict__ Ad, size_t n,
-                                                            const float2* __restrict__ rr,
-                                                            const float2* __restrict__ dad, int n_part,
-                                                            const unsigned* __restrict__ ymax,
-                                                            float2* __restrict__ rr_new) {
-  __shared__ float2 sh[kElemThreads / 32];
+                                                            const Sum* __restrict__ rr,
+                                                            const Sum* __restrict__ dad, int n_part,
+                                                            Sum* __restrict__ rr_new) {
+  __shared__ Sum sh[kElemThreads / 32];
   __shared__ float s_a;
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  if (threadIdx.x < 32) {
-    const Sum2 num = partial_sum(rr, n_part), den = partial_sum(dad, n_part);
-    if (threadIdx.x == 0) s_a = pair_ratio(num, den);
+  if (threadIdx.x < 32) {  // (a warp per sum and a second barrier: slower by 1.5 us beside its neighbours)
+    const Sum num = partial_sum(rr, n_part), den = partial_sum(dad, n_part);
+    if (threadIdx.x == 0) s_a = sum_ratio(num, den);
   }
   const size_t i0 = (size_t)blockIdx.x * kElemThreads + threadIdx.x, step = (size_t)gridDim.x * kElemThreads;
   float2 dv, av, xv, rv;  // the first element's loads while the step size is formed
@@ -736,8 +780,8 @@ __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__
     rv = r[i0];
   }
   __syncthreads();
-  const float a = s_a, ks = sum_scale(ymax);
-  Sum2 s[1];
+  const float a = s_a;
+  Sum s[1] = {sum_zero()};
   for (size_t i = i0; i < n; i += step) {
     if (i != i0) {
       dv = d[i];
@@ -751,40 +795,27 @@ __global__ void __launch_bounds__(kElemThreads) k_cg_update(float2* __restrict__
     rv.y = fmaf(-a, av.y, rv.y);
     x[i] = xv;
     r[i] = rv;
-    sum2_mul(s[0], ks * rv.x, ks * rv.x);
-    sum2_mul(s[0], ks * rv.y, ks * rv.y);
+    s[0] = sum_add(s[0], sum_dot(rv, rv));
   }
-  Sum2 out[1];
-  block_sums(s, sh, out);
-  if (threadIdx.x == 0) rr_new[blockIdx.x] = pack(out[0]);
+  block_sums<1, kElemThreads>(s, sh, rr_new + blockIdx.x);
 }
 
 // |F_s S p + u_k - y|^2 of every (frame, coil): kBallBlocks partial sums each.
 __global__ void __launch_bounds__(kThreads) k_ball_norm(const float2* __restrict__ ap, const float2* __restrict__ uk,
                                                         const float2* __restrict__ y, int M,
-                                                        const double* __restrict__ sc,
-                                                        const unsigned* __restrict__ ymax,
-                                                        float2* __restrict__ partials) {
-  __shared__ float2 sh[kThreads / 32];
+                                                        const double* __restrict__ sc, Sum* __restrict__ partials) {
+  __shared__ Sum sh[kThreads / 32];
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
   const int c = blockIdx.y;
-  const float fu = (float)sc[S_UFAC], ks = sum_scale(ymax);
-  Sum2 s[1];
+  const float fu = (float)sc[S_UFAC];
+  Sum s[1] = {sum_zero()};
   for (int m = blockIdx.x * kThreads + threadIdx.x; m < M; m += gridDim.x * kThreads) {
     const size_t i = (size_t)c * M + m;
     const float2 av = ap[i], uv = uk[i], yv = y[i];
-    float e1, e2;  // ap + fu uk - y = d + e1 + e2 exactly
-    float d = diff_exact(av.x, -(fu * uv.x), e1);
-    d = diff_exact(d, yv.x, e2);
-    sum2_sq(s[0], ks * d, ks * (e1 + e2));
-    d = diff_exact(av.y, -(fu * uv.y), e1);
-    d = diff_exact(d, yv.y, e2);
-    sum2_sq(s[0], ks * d, ks * (e1 + e2));
+    s[0] = sum_add(s[0], sum_add(sum_diff3_sq(av.x, __fmul_rn(fu, uv.x), yv.x), sum_diff3_sq(av.y, __fmul_rn(fu, uv.y), yv.y)));
   }
-  Sum2 out[1];
-  block_sums(s, sh, out);
-  if (threadIdx.x == 0) partials[(size_t)c * kBallBlocks + blockIdx.x] = pack(out[0]);
+  block_sums<1, kThreads>(s, sh, partials + (size_t)c * kBallBlocks + blockIdx.x);
 }
 
 // u_0 += p - z_0; the residual norms of both blocks (row_part: the data blocks'
@@ -793,28 +824,25 @@ __global__ void __launch_bounds__(kThreads) k_ball_norm(const float2* __restrict
 __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__ u0, const float2* __restrict__ p,
                                                             const float2* __restrict__ z0,
                                                             const float2* __restrict__ p_prev, size_t n, double* sc,
-                                                            float2* partials, unsigned* counter,
-                                                            const float2* __restrict__ row_part, int n_row, double mu,
-                                                            double tau, const unsigned* __restrict__ ymax,
-                                                            double* __restrict__ hist) {
-  __shared__ float2 sh[2 * kElemThreads / 32];
+                                                            Sum* partials, unsigned* counter,
+                                                            const Sum* __restrict__ row_part, int n_row, double mu,
+                                                            double tau, double* __restrict__ hist) {
+  __shared__ Sum sh[2 * kElemThreads / 32], sums[2];
   __shared__ int last;
   mpi_ptx::pdl_trigger();
   mpi_ptx::pdl_wait();
-  const float fu = (float)sc[S_UFAC], ks = sum_scale(ymax);
-  Sum2 s[2];
+  const float fu = (float)sc[S_UFAC];
+  Sum s[2] = {sum_zero(), sum_zero()};
   for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
     const float2 pv = p[i], zv = z0[i], qv = p_prev[i];
     const float2 uv = u0[i];
     u0[i] = make_float2(fu * uv.x + pv.x - zv.x, fu * uv.y + pv.y - zv.y);
-    sum2_diff_sq(s[0], ks, pv, zv);
-    sum2_diff_sq(s[1], ks, pv, qv);
+    s[0] = sum_add(s[0], sum_diff_sq(pv, zv));
+    s[1] = sum_add(s[1], sum_diff_sq(pv, qv));
   }
-  Sum2 out[2];
-  block_sums(s, sh, out);
+  block_sums<2, kElemThreads>(s, sh, partials + 2 * (size_t)blockIdx.x);
+  __syncthreads();
   if (threadIdx.x == 0) {
-    partials[2 * (size_t)blockIdx.x] = pack(out[0]);
-    partials[2 * (size_t)blockIdx.x + 1] = pack(out[1]);
     __threadfence();
     last = atomicAdd(counter, 1u) == gridDim.x - 1;
     if (last) *counter = 0;
@@ -822,18 +850,19 @@ __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__
   __syncthreads();
   if (!last) return;
   __threadfence();
-  s[0] = s[1] = Sum2();
+  s[0] = s[1] = sum_zero();
   for (unsigned i = threadIdx.x; i < gridDim.x + n_row; i += kElemThreads) {
-    const float2* q = i < gridDim.x ? partials + 2 * (size_t)i : row_part + 2 * (size_t)(i - gridDim.x);
+    const Sum* q = i < gridDim.x ? partials + 2 * (size_t)i : row_part + 2 * (size_t)(i - gridDim.x);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const float2 v = __ldcg(q + j);
-      sum2_add(s[j], v.x, v.y);
+      const int4 w = __ldcg(reinterpret_cast<const int4*>(q + j));
+      s[j] = sum_add(s[j], Sum{(long long)((unsigned long long)(unsigned)w.y << 32 | (unsigned)w.x), w.z});
     }
   }
-  block_sums(s, sh, out);
+  block_sums<2, kElemThreads>(s, sh, sums);
+  __syncthreads();
   if (threadIdx.x) return;
-  const double prim = sqrt(to_double(out[0])) / ks, rho = sc[S_RHO], dual = rho * (sqrt(to_double(out[1])) / ks);
+  const double prim = sqrt(to_double(sums[0])), rho = sc[S_RHO], dual = rho * sqrt(to_double(sums[1]));
   hist[0] = prim;
   hist[1] = dual;
   hist[2] = rho;
@@ -851,19 +880,6 @@ __global__ void __launch_bounds__(kElemThreads) k_admm_dual(float2* __restrict__
 __global__ void k_admm_start(double* sc, double rho0) {
   sc[S_RHO] = rho0;
   sc[S_UFAC] = 1.0;
-}
-
-// The bits of the largest finite |Re| or |Im| of n values (*ymax cleared before).
-__global__ void __launch_bounds__(kElemThreads) k_data_max(const float2* __restrict__ y, size_t n, unsigned* ymax) {
-  unsigned m = 0;
-  for (size_t i = (size_t)blockIdx.x * kElemThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kElemThreads) {
-    const float2 v = y[i];
-    const unsigned a = __float_as_uint(v.x) & 0x7fffffffu, b = __float_as_uint(v.y) & 0x7fffffffu;
-    if (a < 0x7f800000u) m = max(m, a);
-    if (b < 0x7f800000u) m = max(m, b);
-  }
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(ymax, m);
 }
 
 // mask[t][idx[t][m]] = 1
@@ -978,18 +994,18 @@ size_t admm_maps_layout(const mpi_ctx* ctx, const mpi_plan* const* plans, int T,
   m->u0 = cplx(TN);
   m->ap = cplx(CM);
   m->uk = cplx(CM);
-  m->counters = (unsigned*)take(2 * sizeof(unsigned));
+  m->counter = (unsigned*)take(sizeof(unsigned));
   m->zero_bytes = (char*)mem + off - m->zero_begin;
   m->zk = cplx(CM);
   float2** img[] = {&m->z0, &m->r, &m->d[0], &m->d[1], &m->Ad, &m->p_prev};
   for (float2** b : img) *b = cplx(TN);
   m->tv = cplx(tv_scratch_elems(T > 1 ? 3 : 2, (long)TN));
   m->sc = (double*)take(S_NUM * sizeof(double));
-  m->ball_part = cplx((size_t)T * C * kBallBlocks);
-  m->part = cplx(5 * (size_t)kMaxElemBlocks);  // |r|^2 twice, <d, A d>, the dual's two
+  m->ball = take((size_t)T * C * kBallBlocks * sizeof(Sum));
+  m->part = take(5 * (size_t)kMaxElemBlocks * sizeof(Sum));  // |r|^2 twice, <d, A d>, the dual's two
   int n_list = 0;
   for (int t = 0; t < T; ++t) n_list = std::max(n_list, plans[t]->n_list);
-  m->row_part = cplx(2 * (size_t)row_blocks(ctx, (size_t)T * C, n_list, plans[0]->nx));
+  m->row_part = take(2 * (size_t)row_blocks(ctx, (size_t)T * C, n_list, plans[0]->nx) * sizeof(Sum));
   m->idx = (int32_t*)take((size_t)T * M * sizeof(int32_t));
   m->row_ptr = (int32_t*)take((size_t)T * (plans[0]->ny + 1) * sizeof(int32_t));
   m->row_list = (int32_t*)take((size_t)T * plans[0]->ny * sizeof(int32_t));
@@ -1044,15 +1060,12 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   int n_list = 0;
   for (int t = 0; t < T; ++t) n_list = std::max(n_list, plans[t]->n_list);
   const unsigned eblk = elem_blocks(TN), rblk = row_blocks(ctx, TC, n_list, nx);
-  float2 *rr[2] = {m.part, m.part + kMaxElemBlocks}, *dad = m.part + 2 * kMaxElemBlocks;
+  Sum* part = (Sum*)m.part;
+  Sum *rr[2] = {part, part + kMaxElemBlocks}, *dad = part + 2 * kMaxElemBlocks;
   TRY(cuda_check(ctx, cudaMemsetAsync(m.zero_begin, 0, m.zero_bytes, ctx->stream), "image solver start"));
   MPI_PROF(ctx, KF_SOLVER);
   k_admm_start<<<1, 1, 0, ctx->stream>>>(m.sc, prm->rho0);
   MPI_LAUNCH_CHECK(ctx, "k_admm_start");
-  const unsigned* ymax = m.counters + 1;
-  MPI_PROF(ctx, KF_SOLVER);
-  k_data_max<<<elem_blocks((size_t)TC * M), kElemThreads, 0, ctx->stream>>>(m.in_y, (size_t)TC * M, m.counters + 1);
-  MPI_LAUNCH_CHECK(ctx, "k_data_max");
   // MIXED: BF16 maps in the CG iterations; FP32 ones for the constraint-side
   // products and the CG's first residual
   TRY(mpi_basis_expand(ctx, basis, (const mpi_c32*)m.in_alpha, C, (mpi_c32*)m.S,
@@ -1103,11 +1116,10 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   rows.ap = m.ap;
   rows.uk = m.uk;
   rows.zk = m.zk;
-  rows.ball = m.ball_part;
+  rows.ball = (const Sum*)m.ball;
   rows.eps = m.in_eps;
   rows.sc = m.sc;
-  rows.ymax = ymax;
-  rows.partials = m.row_part;
+  rows.partials = (Sum*)m.row_part;
   CoilSum sum{};
   sum.W = m.W;
   sum.C = C;
@@ -1121,7 +1133,6 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   sum.r = m.r;
   sum.p_prev = m.p_prev;
   sum.sc = m.sc;
-  sum.ymax = ymax;
 
   for (int it = 0; it < prm->n_outer; ++it) {
     // z_0 = prox_{TV/rho}(p + u_0), z_k = Pi(F_s S p + u_k)
@@ -1129,7 +1140,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
                        prm->n_tv, m.tv, m.z0));
     MPI_PROF(ctx, KF_SOLVER);
     launch_pdl(ctx, k_ball_norm, dim3(kBallBlocks, (unsigned)TC), dim3(kThreads), 0, m.ap, m.uk, m.in_y, M,
-               m.sc, ymax, m.ball_part);
+               m.sc, (Sum*)m.ball);
     MPI_LAUNCH_CHECK(ctx, "k_ball_norm");
     TRY(launch_maps_rows(ctx, nx, ROWS_SCATTER, rows, rblk));
     // r = S^H F_s^H (z_k - u_k - F_s S p) + z_0 - u_0 - p
@@ -1158,7 +1169,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
       MPI_LAUNCH_CHECK(ctx, "k_coil_sum<normal>");
       MPI_PROF(ctx, KF_SOLVER);
       launch_pdl(ctx, k_cg_update, dim3(eblk), dim3(kElemThreads), 0, m.p, m.r, m.d[cur], m.Ad, TN, rr[par], dad,
-                 (int)eblk, ymax, rr[par ^ 1]);
+                 (int)eblk, rr[par ^ 1]);
       MPI_LAUNCH_CHECK(ctx, "k_cg_update");
       par ^= 1;
     }
@@ -1167,7 +1178,7 @@ mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     TRY(launch_maps_rows(ctx, nx, ROWS_GATHER, rows, rblk));
     MPI_PROF(ctx, KF_SOLVER);
     launch_pdl(ctx, k_admm_dual, dim3(eblk), dim3(kElemThreads), 0, m.u0, m.p, m.z0, m.p_prev, TN, m.sc,
-               m.part + 3 * kMaxElemBlocks, m.counters, m.row_part, (int)rblk, prm->mu, prm->tau, ymax,
+               part + 3 * kMaxElemBlocks, m.counter, (const Sum*)m.row_part, (int)rblk, prm->mu, prm->tau,
                m.hist + 3 * (size_t)it);
     MPI_LAUNCH_CHECK(ctx, "k_admm_dual");
   }

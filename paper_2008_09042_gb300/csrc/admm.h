@@ -14,11 +14,11 @@ struct AdmmMaps {
   float2* W;         // [T][C][N]
   float2 *p, *u0, *ap, *uk, *zk;
   float2 *z0, *r, *d[2], *Ad, *p_prev, *tv;
-  unsigned* counters;  // the dual's arrival counter, the data's largest magnitude
+  unsigned* counter;  // the dual's arrivals
   char* zero_begin;
   size_t zero_bytes;
   double* sc;
-  float2 *ball_part, *part, *row_part;  // partial sums as pairs
+  void *ball, *part, *row_part;  // partial sums (admm.cu)
   int32_t *idx, *row_ptr, *row_list, *n_list;
   uint8_t *rmask, *mask;
   bool whole_rows;  // every k-space row of every frame is sampled whole or not at all
