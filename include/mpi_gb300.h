@@ -145,8 +145,12 @@ mpi_status mpi_ctx_set_autotune(mpi_ctx* ctx, int enable);
  * the (coil, kz) planes unless the choice is -2 (separate, tuned passes): a
  * persistent kernel that streams the planes through shared memory in TMA
  * tiles where each plane's rows with samples fit beside the tiles, else, and
- * always with the choice -3, one CTA per plane.  MPI_ERR_ARG for other
- * values. */
+ * always with the choice -3, one CTA per plane.  A fixed choice of line passes
+ * also keeps mpi_image_solve and mpi_image_solve_dynamic on the operator calls
+ * (their fused passes for 2D Cartesian plans on dense bases have kernels of
+ * their own) and a batch's FFT passes slice by slice.  Solver graphs are kept
+ * per choice, so a solve after this call runs as chosen; recorded batches keep
+ * the kernels they were recorded with.  MPI_ERR_ARG for other values. */
 mpi_status mpi_ctx_set_line_kernel(mpi_ctx* ctx, int choice);
 mpi_status mpi_ctx_tuning_record(const mpi_ctx* ctx, int index, const char** text_out);
 /* Per-launch device timing: while enabled, every kernel the context launches is

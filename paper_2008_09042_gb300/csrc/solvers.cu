@@ -494,7 +494,9 @@ Grid3 grid_of(const mpi_plan* plan) {
 // precision and parameters), with its inputs copied into and its outputs
 // copied out of those buffers around one graph launch.  Destroying a plan or
 // basis drops the graphs that reference it; growing the context workspace
-// (which the graphs also reference) drops all of them.
+// (which the graphs also reference) drops all of them.  A graph serves the calls
+// under the kernel choice (mpi_ctx_set_line_kernel) it was recorded with, which
+// also decides the image solver's route.
 
 namespace {
 
@@ -504,6 +506,7 @@ struct SolverGraph {
   const mpi_basis* basis = nullptr;
   int C = 0;
   int prec = 0;
+  int choice = 0;  // kernel_choice() at capture time
   std::vector<unsigned char> key;
   std::vector<const mpi_plan*> others;  // every plan the graph reads (the frames of a dynamic solve)
   void* work = nullptr;  // ctx->work at capture time
@@ -533,13 +536,18 @@ SolverCache* cache_of(mpi_ctx* ctx) {
   return (SolverCache*)ctx->solver_cache;
 }
 
+// The context's choice of FFT kernels (mpi_ctx_set_line_kernel) as one value.
+int kernel_choice(const mpi_ctx* ctx) {
+  return 4 * ctx->line_kernel + 2 * (ctx->plane_pass ? 1 : 0) + (ctx->plane_pipe ? 1 : 0);
+}
+
 SolverGraph* cache_find(mpi_ctx* ctx, int kind, const mpi_plan* plan, const mpi_basis* basis, int C, int prec,
                         const void* prm, size_t prm_bytes) {
   SolverCache* c = cache_of(ctx);
   for (size_t i = 0; i < c->entries.size(); ++i) {
     SolverGraph* e = c->entries[i];
     if (e->kind == kind && e->plan == plan && e->basis == basis && e->C == C && e->prec == prec &&
-        e->key.size() == prm_bytes && memcmp(e->key.data(), prm, prm_bytes) == 0) {
+        e->choice == kernel_choice(ctx) && e->key.size() == prm_bytes && memcmp(e->key.data(), prm, prm_bytes) == 0) {
       if (e->work != ctx->work) {  // the workspace moved: the recorded kernels point at the old one
         delete e;
         c->entries.erase(c->entries.begin() + i);
@@ -720,6 +728,7 @@ mpi_status sm_estimate_impl(mpi_ctx* ctx, const mpi_plan* plan, const mpi_basis*
     g->basis = basis;
     g->C = C;
     g->prec = prec;
+    g->choice = kernel_choice(ctx);
     g->key.assign((const unsigned char*)prm, (const unsigned char*)prm + sizeof(*prm));
     // x, dx, res, d, Ad, h, b, spare (X each); ys, yt, r (CM each); in_y, out_alpha, out_p
     mpi_status st = alloc_solver(ctx, g->mem, 8 * X + 4 * CMs + Cq + N, prm->n_outer + 1, g->sv, &g->base, &g->dbase);
@@ -936,6 +945,7 @@ mpi_status image_solve_impl(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     g->basis = basis;
     g->C = C;
     g->prec = prec;
+    g->choice = kernel_choice(ctx);
     g->key = key;
     mpi_status st = MPI_OK;
     // 2D Cartesian with a dense basis: the fused solve with the maps kept (admm.cu),
