@@ -507,6 +507,7 @@ struct SolverGraph {
   int C = 0;
   int prec = 0;
   int choice = 0;  // kernel_choice() at capture time
+  bool fallback = false;  // MPI-L on the operator calls because the fused solve's buffers could not be allocated
   std::vector<unsigned char> key;
   std::vector<const mpi_plan*> others;  // every plan the graph reads (the frames of a dynamic solve)
   void* work = nullptr;  // ctx->work at capture time
@@ -557,6 +558,12 @@ SolverGraph* cache_find(mpi_ctx* ctx, int kind, const mpi_plan* plan, const mpi_
     }
   }
   return nullptr;
+}
+
+void cache_erase(mpi_ctx* ctx, SolverGraph* g) {
+  std::vector<SolverGraph*>& v = cache_of(ctx)->entries;
+  v.erase(std::remove(v.begin(), v.end(), g), v.end());
+  delete g;
 }
 
 void cache_insert(mpi_ctx* ctx, SolverGraph* g) {
@@ -937,6 +944,21 @@ mpi_status image_solve_impl(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
   key.insert(key.end(), (const unsigned char*)&T, (const unsigned char*)&T + sizeof(T));
   key.insert(key.end(), (const unsigned char*)plans, (const unsigned char*)(plans + T));
   SolverGraph* g = cache_find(ctx, 1, plans[0], basis, C, prec, key.data(), key.size());
+  // 2D Cartesian with a dense basis: the fused solve with the maps kept (admm.cu), where
+  // its buffers (T C N complex values and C N of maps beside the state) can be had; a
+  // solve that could not have them asks again the next time
+  AdmmMaps maps{};
+  const bool fusable = admm_maps_supported(ctx, plans, T, basis, C, prec);
+  void* fused_mem = nullptr;
+  if (fusable && (!g || g->fallback)) {
+    if (cudaMalloc(&fused_mem, admm_maps_layout(ctx, plans, T, basis, C, prm, prec, nullptr, &maps)) != cudaSuccess) {
+      cudaGetLastError();
+      fused_mem = nullptr;
+    } else if (g) {
+      cache_erase(ctx, g);
+      g = nullptr;
+    }
+  }
   if (!g) {
     g = new SolverGraph();
     g->kind = 1;
@@ -948,18 +970,10 @@ mpi_status image_solve_impl(mpi_ctx* ctx, const mpi_plan* const* plans, int T, c
     g->choice = kernel_choice(ctx);
     g->key = key;
     mpi_status st = MPI_OK;
-    // 2D Cartesian with a dense basis: the fused solve with the maps kept (admm.cu),
-    // where its buffers (T C N complex values and C N of maps beside the state) fit
-    AdmmMaps maps{};
-    bool fused = admm_maps_supported(ctx, plans, T, basis, C, prec);
-    if (fused && cudaMalloc(&g->mem.p, admm_maps_layout(ctx, plans, T, basis, C, prm, prec, nullptr, &maps)) !=
-                     cudaSuccess) {
-      cudaGetLastError();
-      g->mem.p = nullptr;
-      fused = false;
-    }
+    g->mem.p = fused_mem;
+    g->fallback = fusable && !fused_mem;
     g->work = ctx->work;
-    if (fused) {
+    if (fused_mem) {
       admm_maps_layout(ctx, plans, T, basis, C, prm, prec, g->mem.p, &maps);
       g->in_y = maps.in_y;
       g->in_alpha = maps.in_alpha;

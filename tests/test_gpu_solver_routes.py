@@ -45,3 +45,35 @@ def test_line_kernel_choice_between_solves():
         n, p = _solve(mp, ctx, problem)
         assert n == want[choice][0]
         assert torch.equal(p, want[choice][1])
+
+
+def test_solve_returns_to_the_fused_route_after_a_failed_allocation():
+    import paper_2008_09042_gb300 as mp
+
+    ctx = mp.Context(0)
+    fused, _ = _solve(mp, ctx, _problem(mp, ctx))
+    ctx.set_line_kernel(8)
+    calls, _ = _solve(mp, ctx, _problem(mp, ctx))  # both routes' kernels are loaded
+    ctx.set_line_kernel(0)
+    # 64 coils of 512^2: 268 MB of maps and coil images on the fused route, 50 MB on the operator calls
+    n, C = 512, 64
+    mask = np.zeros((n, n), dtype=bool)
+    mask[::64] = True
+    plan = mp.Plan(ctx, (n, n), sample_idx=np.flatnonzero(mask.ravel()).astype(np.int32))
+    basis = mp.Basis(ctx, w.smooth_orthonormal_basis(n, n, 4, seed=1).T * n)
+    alpha = torch.from_numpy(w.random_coefficients(C, 4, seed=2).astype(np.complex64)).cuda()
+    y = torch.from_numpy(w.random_image((C, plan.M), seed=3).astype(np.complex64)).cuda()
+    problem = plan, basis, alpha, y, np.full(C, 0.1 * np.sqrt(plan.M))
+    ctx.reserve(plan, basis, C)
+    mp.forward(ctx, plan, basis, alpha, torch.zeros(n * n, dtype=torch.complex64, device="cuda"))
+    ctx.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (150 << 20), dtype=torch.uint8, device="cuda")
+    n0, p0 = _solve(mp, ctx, problem)
+    assert n0 >= calls
+    del fill
+    torch.cuda.empty_cache()
+    n1, p1 = _solve(mp, ctx, problem)
+    assert n1 <= fused
+    a, b = p0.cpu().numpy(), p1.cpu().numpy()
+    assert np.linalg.norm(a - b) < 1e-4 * np.linalg.norm(a)  # the routes' bound (test_gpu_admm_fused.py)
