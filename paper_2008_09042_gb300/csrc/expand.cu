@@ -178,8 +178,7 @@ mpi_status launch_mode(mpi_ctx* ctx, const ExpandArgs& a) {
   const size_t smem = (size_t)q_pad * c_pad * sizeof(float2) * (MODE == EX_JFWD ? 2 : 1);
   if (smem > 200 * 1024) return set_err(ctx, MPI_ERR_UNSUPPORTED, "coefficient block too large for shared memory");
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_expand<MODE, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = smem_attr(ctx, (const void*)k_expand<MODE, CB>);
     if (e != cudaSuccess) return cuda_check(ctx, e, "expand smem attribute");
   }
   // every SM gets the same number of pixels: grid = k * SMs CTAs of a warp multiple
@@ -312,7 +311,7 @@ mpi_status launch_uh_v(mpi_ctx* ctx, const float2* U, int N, int q, const float2
     const int c_count = std::min(per_launch, C - c_begin);
     const int cpad = ((c_count + CT - 1) / CT) * CT;
     const size_t smem = ((size_t)q * (kUhvP + 1) + (size_t)kUhvP * cpad) * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_uh_v<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = smem_attr(ctx, (const void*)k_uh_v<CT>);
     if (e != cudaSuccess) return cuda_check(ctx, e, "uh_v smem attribute");
     MPI_PROF(ctx, KF_UHV);
   launch_pdl(ctx, k_uh_v<CT>, dim3(nblk), dim3(kUhvThreads), smem, U, N, q, V, C, c_begin, c_count, partials);

@@ -1342,7 +1342,7 @@ bool try_plane_pipe(mpi_ctx* ctx, const mpi_plan* plan, float2* data, int C, flo
   }
   if (!ok) return false;
   auto kern = inverse ? k_plane_pipe<NY, NX, true> : k_plane_pipe<NY, NX, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = smem_attr(ctx, (const void*)kern);
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPipeThreads, smem);
   if (e != cudaSuccess) {
@@ -1388,7 +1388,7 @@ mpi_status launch_plane_yx(mpi_ctx* ctx, const mpi_plan* plan, float2* data, int
   if (plan->ny == NY_ && plan->nx == NX_) {                                                                    \
     const size_t smem = plane_smem<NY_, NX_>();                                                                \
     auto kern = inverse ? k_plane_yx<NY_, NX_, true> : k_plane_yx<NY_, NX_, false>;                            \
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);                    \
+    e = smem_attr(ctx, (const void*)kern);                                                                      \
     if (e != cudaSuccess) return cuda_check(ctx, e, "plane pass smem attribute");                              \
     MPI_PROF(ctx, KF_FFT_ROWS);                                                                                \
     launch_pdl(ctx, kern, dim3((unsigned)planes), dim3(NX_ * 4), smem, data, y, plan->nz, plan->idx,           \

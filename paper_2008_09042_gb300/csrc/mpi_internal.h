@@ -197,7 +197,9 @@ inline cudaError_t launch_pdl(mpi_ctx* ctx, void (*kern)(KArgs...), dim3 grid, d
 
 // Lets `kern` be launched with any dynamic shared memory that the device has: set on a
 // context's first launch of it, to the same value by every context, rather than to each
-// launch's size before every launch (0.4 us of host time each, on calls of 15 to 50 us).
+// launch's size before every launch: the attribute belongs to the kernel on the device, so a
+// context on another thread could lower it between the two (and 0.4 us of host time each,
+// on calls of 15 to 50 us).
 inline cudaError_t smem_attr(mpi_ctx* ctx, const void* kern) {
   for (const void* k : ctx->smem_granted)
     if (k == kern) return cudaSuccess;

@@ -567,7 +567,7 @@ mpi_status tx_launch(mpi_ctx* ctx, const CUtensorMap* map, TxArgs& a, dim3 grid)
   a.stages = stages;
   const size_t smem = tx_smem<PREC, N1>(stages);
   auto kern = k_tucker_x1<PREC, MODE, N1>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = smem_attr(ctx, (const void*)kern);
   if (e != cudaSuccess) return cuda_check(ctx, e, "Tucker x1 smem attribute");
   MPI_PROF(ctx, KF_EXPAND);
   launch_pdl(ctx, kern, grid, dim3(kTxThreads), smem, *map, a);

@@ -345,8 +345,7 @@ mpi_status mode_last(mpi_ctx* ctx, bool adj, const float2* X, const float2* F, i
   const unsigned grid = (unsigned)((R + kLastRows - 1) / kLastRows);
   const size_t smem = ((size_t)P * I + (size_t)kLastRows * P) * sizeof(float2);
   if (smem > 232448 - 1024) return set_err(ctx, MPI_ERR_UNSUPPORTED, "Tucker last-mode product: factor too large");
-  cudaError_t e = adj ? cudaFuncSetAttribute(k_mode_last<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                      : cudaFuncSetAttribute(k_mode_last<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = smem_attr(ctx, adj ? (const void*)k_mode_last<true> : (const void*)k_mode_last<false>);
   if (e != cudaSuccess) return cuda_check(ctx, e, "k_mode_last smem attribute");
   MPI_PROF(ctx, KF_EXPAND);
   if (adj) launch_pdl(ctx, k_mode_last<true>, dim3(grid), dim3(256), smem, X, F, R, P, I, Y);

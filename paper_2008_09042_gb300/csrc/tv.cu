@@ -323,7 +323,7 @@ mpi_status launch_tv_prox(mpi_ctx* ctx, int nz, int ny, int nx, int nd, const fl
       }
     }
     const size_t side = t.ox + 2 * t.iters + t.last, smem = 6 * side * side * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(k_tv_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = smem_attr(ctx, (const void*)k_tv_tile);
     if (e != cudaSuccess) return cuda_check(ctx, e, "TV tile attributes");
     const dim3 grid((unsigned)((nx + t.ox - 1) / t.ox), (unsigned)((ny + t.oy - 1) / t.oy));
     const int cur = launch & 1;
