@@ -659,6 +659,23 @@ def radial_line(mp, ctx, dev, flush, stream, steps=10, warmup=3):
     return out
 
 
+def grouped_expansion(rec, hbm, bf16_peak):
+    """Figures of a batch's grouped expansion from the library's tuning record of it."""
+    m = re.match(r"grouped expansion \((\d+) slices, N=(\d+), q=(\d+), sumC=(\d+), (\w+)\):.* chose (\d+), bundles of "
+                 r"(\d+), skew ([\d.e+-]+) \(([\d.]+) us\)$", rec)
+    if not m:
+        return {"unparsed": rec}
+    ns, N, q, sumC, prec, ctas, bundle, _, us = m.groups()
+    N, q, sumC, us = int(N), int(q), int(sumC), float(us)
+    flops = 2.0 * N * (2 * q) * (2 * sumC)  # the real-ified GEMM, counted once
+    ub = (2 if prec == "bf16" else 4) * N * 2 * q
+    byts = ub + 8 * sumC * N + 8 * sumC * q + 8 * int(ns) * N  # basis, per-coil images out, alpha, images in
+    return {"slices": int(ns), "N": N, "q": q, "coils": sumC, "ctas": int(ctas), "bundle_coils": int(bundle),
+            "us_per_launch": us, "tflops": flops / (us * 1e-6) / 1e12,
+            "frac_of_bf16_tensor_peak": flops / (us * 1e-6) / 1e12 / bf16_peak,
+            "hbm_gbs": byts / (us * 1e-6) / 1e9, "frac_of_hbm_peak": byts / (us * 1e-6) / 1e9 / hbm}
+
+
 def batched_slices(mp, ctx, dev, flush, stream, steps=5, warmup=2):
     """The 64-slice mixed exam: grids from {128, 192, 256, 320}^2, coils from
     {8, 16, 32}, q by grid size, Poisson-disc R in 4..8; all slices' forward +
@@ -699,21 +716,8 @@ def batched_slices(mp, ctx, dev, flush, stream, steps=5, warmup=2):
         n_rec = len(ctx.tuning_records())
         batch = mp.Batch(ctx, slices, kind="pair", prec=prec)
         # the grouped expansions' timings from the batch's tuning records
-        grouped = []
-        for rec in ctx.tuning_records()[n_rec:]:
-            m = re.match(r"grouped expansion \((\d+) slices, N=(\d+), q=(\d+), sumC=(\d+), (\w+)\):.* chose (\d+) "
-                         r"\(([\d.]+) us\)", rec)
-            if not m:
-                continue
-            ns, N, q, sumC, pr, ctas, us = m.groups()
-            N, q, sumC, us = int(N), int(q), int(sumC), float(us)
-            flops = 2.0 * N * (2 * q) * (2 * sumC)  # the real-ified GEMM, counted once
-            ub = (2 if prec == "bf16" else 4) * N * 2 * q
-            byts = ub + 8 * sumC * N + 8 * sumC * q + 8 * int(ns) * N  # basis, per-coil images out, alpha, images in
-            grouped.append({"slices": int(ns), "N": N, "q": q, "coils": sumC, "ctas_per_row": int(ctas),
-                            "us_per_launch": us, "tflops": flops / (us * 1e-6) / 1e12,
-                            "frac_of_bf16_tensor_peak": flops / (us * 1e-6) / 1e12 / bf16_peak,
-                            "hbm_gbs": byts / (us * 1e-6) / 1e9, "frac_of_hbm_peak": byts / (us * 1e-6) / 1e9 / hbm})
+        grouped = [grouped_expansion(rec, hbm, bf16_peak) for rec in ctx.tuning_records()[n_rec:]
+                   if rec.startswith("grouped expansion")]
         for _ in range(warmup):
             batch.run()
         torch.cuda.synchronize()
