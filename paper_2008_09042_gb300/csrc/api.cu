@@ -490,7 +490,7 @@ extern "C" mpi_status mpi_ctx_set_line_kernel(mpi_ctx* ctx, int choice) {
   // -3: the plane kernel with one CTA per plane instead of the pipelined one
   ctx->plane_pass = choice != -2;
   ctx->plane_pipe = choice != -3;
-  ctx->line_kernel = choice == -2 ? 0 : choice;
+  ctx->line_kernel = choice <= -2 ? 0 : choice;  // the two 3D choices fix no line passes
   return MPI_OK;
 }
 

@@ -77,3 +77,20 @@ def test_solve_returns_to_the_fused_route_after_a_failed_allocation():
     assert n1 <= fused
     a, b = p0.cpu().numpy(), p1.cpu().numpy()
     assert np.linalg.norm(a - b) < 1e-4 * np.linalg.norm(a)  # the routes' bound (test_gpu_admm_fused.py)
+
+
+@pytest.mark.parametrize("choice", [-2, -3])
+def test_choices_for_volumes_leave_2d_calls_alone(choice):
+    import paper_2008_09042_gb300 as mp
+
+    def counts(c):
+        ctx = mp.Context(0)
+        ctx.set_line_kernel(c)
+        problem = _problem(mp, ctx)
+        n, p = _solve(mp, ctx, problem)
+        plan, basis, alpha, y, _ = problem
+        slices = [dict(plan=plan, basis=basis, alpha=alpha, p=p, y=y.clone(), x=torch.empty_like(p)) for _ in range(5)]
+        batch = mp.Batch(ctx, slices)
+        return n, batch.kernels()
+
+    assert counts(choice) == counts(0)
