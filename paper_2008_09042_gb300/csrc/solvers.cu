@@ -1079,7 +1079,13 @@ extern "C" mpi_status mpi_tv_prox(mpi_ctx* ctx, const mpi_plan* plan, const mpi_
   Solver sv;
   float2* base;
   double* dx;
-  TRY(alloc_solver(ctx, mem, tv_scratch_elems(g.nd, N), 0, sv, &base, &dx));
+  const size_t scratch = tv_scratch_elems(g.nd, N);
+  const bool in_place = x == v;
+  TRY(alloc_solver(ctx, mem, scratch + (in_place ? N : 0), 0, sv, &base, &dx));
+  if (in_place) {  // a tile of the image is written while its neighbours still read it
+    TRY(sv.lincomb(base + scratch, (const float2*)v, 1.f, nullptr, 0.f, N));
+    v = (const mpi_c32*)(base + scratch);
+  }
   if (lam == 0) {
     TRY(sv.lincomb((float2*)x, (const float2*)v, 1.f, nullptr, 0.f, N));
   } else {
