@@ -939,41 +939,6 @@ struct PipeLayout {
   static __host__ __device__ size_t total(int kmax) { return bars(kmax) + NB * sizeof(uint64_t) + 1024; }
 };
 
-// Rows of the compact store through the DFT along x: NX = 8 A, element n = p + 8 a,
-// output k1 + A k2, the two register steps of fft_rows.cuh in place in the store's
-// own padding (pad8: value (k1, p) at 9 k1 + p).  Half a warp per row: a plane has
-// some 16 rows for the CTA's 16 warps, so more rows per warp would only lengthen the
-// phase; the halves keep both steps free of bank conflicts whatever the row stride.
-template <int NX, bool INV>
-struct PlaneRows {
-  static constexpr int A = NX / 8;
-  static __device__ __forceinline__ int out_at(int x) { return x % A * 9 + x / A; }
-  // h: lane of the half warp; `in`: the half has a row
-  static __device__ __forceinline__ void go(float2* row, bool in, int h, const float2* tw) {
-    if (in && h < 8) {
-      float2 v[A];
-#pragma unroll
-      for (int a = 0; a < A; ++a) {
-        const float2 t = row[9 * a + h];
-        v[a] = INV ? make_float2(t.x, -t.y) : t;
-      }
-      mpi_dft::dft_r<A>(v);
-#pragma unroll
-      for (int k = 0; k < A; ++k) row[9 * k + h] = k ? mpi_dft::cmulf(v[k], tw[h * k]) : v[0];
-    }
-    __syncwarp();
-    if (in && h < A) {
-      float2 u[8];
-#pragma unroll
-      for (int p = 0; p < 8; ++p) u[p] = row[9 * h + p];
-      mpi_dft::dft8(u);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) row[9 * h + k] = INV ? make_float2(u[k].x, -u[k].y) : u[k];
-    }
-    __syncwarp();
-  }
-};
-
 template <int NY, int NX, bool INV>
 __global__ void __launch_bounds__(kPipeThreads, 1)
     k_plane_pipe(const __grid_constant__ CUtensorMap tmap, float2* __restrict__ y, int nz, int planes, int kmax,
