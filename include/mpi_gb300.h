@@ -127,19 +127,24 @@ enum { MPI_TF32_READ_FAILED = -2, MPI_TF32_READ_TRUNCATE = 0, MPI_TF32_READ_NEAR
        MPI_TF32_READ_NEAREST_AWAY = 2, MPI_TF32_READ_FULL = 3, MPI_TF32_READ_OTHER = 4 };
 int mpi_ctx_tf32_reading(const mpi_ctx* ctx);
 mpi_status mpi_ctx_set_tf32x3(mpi_ctx* ctx, int enable);
-/* Launch-shape autotuning (on by default).  The first operator call that runs an
- * FFT line pass of a new shape (length, stride, line count, row mask) times each
- * candidate tile width of that pass with CUDA events on a free workspace buffer
+/* Launch-shape autotuning (on by default).  Passes along y of 64, 96, 128, 192,
+ * 256 or 320 points over at most 64 MiB take the register two-step pass with 16
+ * columns per CTA untimed.  For any other FFT line pass, the first operator call
+ * that runs a new shape (length, stride, line count, row mask) times each
+ * candidate kernel of that pass with CUDA events on a free workspace buffer
  * (never while the stream is being captured, never in mpi_forward_noalloc) and
- * keeps the fastest for the context's later calls.  enable = 0 switches tuning
- * off (untuned shapes take a fixed default).  mpi_ctx_tuning_record returns the
+ * keeps the fastest for the context's later calls; mpi_batch_create times the
+ * layouts of its grouped expansions and the widths of its grouped passes.
+ * enable = 0 switches the timing of FFT passes off (untuned shapes take a fixed
+ * default).  mpi_ctx_tuning_record returns the
  * text of the `index`-th decision (shape, candidates and their times; valid for
  * the context's lifetime), MPI_ERR_ARG past the last.  Library machinery, no
  * paper passage. */
 mpi_status mpi_ctx_set_autotune(mpi_ctx* ctx, int enable);
 /* Fixes the FFT line passes' kernel instead of tuning it: 8, 16 or 32 lines per
  * CTA (shared-memory Stockham passes), -1 the register two-step pass along y
- * (lengths 64, 96, 128, 192, 256), 0 back to tuning.  A pass the choice does
+ * with 32 columns per CTA (lengths 64, 96, 128, 192, 256, 320), 0 back to the
+ * rules above.  A pass the choice does
  * not cover keeps its tuned or default kernel.  3D Tucker volumes with planes
  * of 64, 96 or 128 squared run the passes along y and x as one kernel over
  * the (coil, kz) planes unless the choice is -2 (separate, tuned passes): a
@@ -425,9 +430,9 @@ mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slices, int n, 
 mpi_status mpi_batch_run(mpi_ctx* ctx, mpi_batch* batch);
 /* Kernels one replay launches (-1 for a NULL batch). */
 int64_t mpi_batch_kernel_count(const mpi_batch* batch);
-/* Grouped expansion launches per direction in the batch (slices on Cartesian
- * plans sharing a dense basis, FP32 or BF16, are expanded by one launch per
- * group whose grid rows are the slices), or -1 for a null handle. */
+/* Grouped expansion launches per direction in the batch (consecutive slices on
+ * Cartesian plans of one grid that share a dense basis, FP32 or BF16, are
+ * expanded by one launch per group), or -1 for a null handle. */
 int mpi_batch_group_count(const mpi_batch* batch);
 mpi_status mpi_batch_destroy(mpi_batch* batch);
 

@@ -84,7 +84,8 @@ class Context:
 
     def set_line_kernel(self, choice=0):
         """Fix the FFT line passes' kernel: 8, 16, 32 (lines per CTA), -1 (register
-        two-step pass along y) or 0 (tuned)."""
+        two-step pass along y, 32 columns per CTA) or 0 (by rule or timed); -2 and -3
+        choose the passes of volumes (mpi_ctx_set_line_kernel)."""
         check(self.h, self.lib.mpi_ctx_set_line_kernel(self.h, int(choice)))
 
     def tuning_records(self):

@@ -8,20 +8,20 @@
 // context's stream.  The captured pointers are the caller's buffers, which must
 // stay valid for the life of the batch.
 //
-// Grouped expansion: consecutive slices on Cartesian plans that share a dense
-// basis (FP32 or BF16, every slice's coils within one tensor-core pass)
-// form a group.  The group's basis expansion is one launch over its slices (device
-// tables give each CTA its slices' coefficients, images, per-coil data and outputs);
-// the CTAs stream the same basis tiles in step, so the basis is read from DRAM
-// about once per group instead of once per slice, and slices of few coils are bundled,
-// their coefficients stacked into one operand, so that one CTA reads a tile for all.  Each slice's per-coil images live
-// in a batch-owned buffer between the expansion and the FFT passes.  From
-// kGroupedPasses slices on, the FFT passes take all coils of a group's slices in one
+// Grouped expansion: consecutive slices on Cartesian plans of one grid that share a
+// dense basis (FP32 or BF16, every slice's coils within one tensor-core pass) form a
+// group.  The group's basis expansion is one launch over its slices (device tables give
+// each CTA its slices' coefficients, images, per-coil data and outputs); the CTAs stream
+// the same basis tiles in step, so the basis is read from DRAM about once per group
+// instead of once per slice, and slices of few coils are bundled, their coefficients
+// stacked into one operand, so that one CTA reads a tile for all.  Each slice's per-coil
+// images live in a batch-owned buffer between the expansion and the FFT passes.  From
+// kGroupedPasses 2D slices on, the FFT passes take all coils of a group's slices in one
 // launch too (per run of slices whose pass along y is of the same kind, register or
-// Stockham, so that a slice's values stay those of its own call; its width is timed
-// for the group), with a table of every coil's sampling.  How the slices are bundled
-// and how many CTAs each bundle gets is chosen at creation by timing the candidates (an autotuner decision the context
-// records).
+// Stockham, so that a slice's values stay those of its own call; its width is timed for
+// the group), with a table of every coil's sampling.  How the slices are bundled and how
+// many CTAs each bundle gets is chosen at creation by timing the candidates (an
+// autotuner decision the context records).
 #include <algorithm>
 #include <cstdio>
 #include <numeric>

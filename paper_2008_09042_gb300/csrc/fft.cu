@@ -1234,7 +1234,7 @@ mpi_status launch_fft_cols_window(mpi_ctx* ctx, float2* grid, int C, int G, cons
   }
 #undef MPI_WIN_CASE
 #undef MPI_WIN_REG
-  MPI_LAUNCH_CHECK(ctx, "k_fft_lines_win");
+  MPI_LAUNCH_CHECK(ctx, G < 64 ? "k_fft_lines_win" : "k_fft_cols_win");
   return MPI_OK;
 }
 

@@ -184,7 +184,7 @@ int spread_coils_padded(int C, int G) {
 }
 
 // ys[cell_rank[m]][c] = ksign * y[c][m] for c < C, zero for C <= c < Cp (C
-// padded to a multiple of four): the samples in first-tap-cell order, the
+// padded to whole spreading threads, see spread_groups): the samples in first-tap-cell order, the
 // coils of one sample contiguous.  Reads follow y's layout; writes scatter.
 __global__ void k_nufft_sort_y(const float2* __restrict__ y, int C, int Cp, int M,
                                const int32_t* __restrict__ cell_rank, float ksign, float2* __restrict__ ys) {

@@ -11,7 +11,7 @@
 //
 // Same real-ified GEMM as the BF16 kernel: 128-pixel tiles of U are the A
 // operand, the coefficient rows B, with a TMA ring (128-byte swizzle), one MMA
-// thread, a double-buffered TMEM accumulator and four epilogue warps.  Per
+// warp, a double-buffered TMEM accumulator and four epilogue warps.  Per
 // 8-element K step it issues two kind::tf32 MMAs:
 //  - U_hi against the stacked rows [A_hi; A_lo] (N = 2 n), which writes U_hi A_hi
 //    and U_hi A_lo into two column blocks that the epilogue adds.  U_hi is the
@@ -23,9 +23,9 @@
 //    memory: four converter warps read each landed tile from shared memory and
 //    store lo(x) with tcgen05.st into a TMEM slot of the stage, so the split
 //    costs no shared-memory writes and each ring stage is one 16 KB slot.
-// A tcgen05.mma costs about the same to issue for any N up to 64, so stacking
-// the coefficient rows saves a third of the instructions.  The stacked
-// coefficient image is built once per call.  Every mbarrier wait is bounded.
+// Stacking the coefficient rows makes two MMAs of a K step's three products; an MMA
+// takes some 39 cycles from issue to issue, of which the tensor core needs 32
+// (tc_common.cuh).  The stacked coefficient image is built once per call.  Every mbarrier wait is bounded.
 // Operands whose K box count is odd end each tile with a one-box stage (a
 // compile-time variant).  EX_SCATTER_ADD splits K over the grid rows: each
 // row's coefficient image covers its part of K, and its partial products are
