@@ -117,6 +117,7 @@ struct mpi_plan {
   float* cell_w = nullptr;
   int32_t* cell_dense = nullptr;
   int n_dense = 0;
+  int dense_max = 0;  // samples in the fullest cell's window
   // Interpolation work list: the samples sorted by the 32 x 32 tile of their
   // first tap (tile_samples [M]); items [n_tile_items][3] = (tile, first
   // sorted sample, count), dense tiles split into chunks.

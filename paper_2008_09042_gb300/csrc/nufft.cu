@@ -167,19 +167,28 @@ constexpr int kSpreadCoils = 4;   // coils of a group; a spreading thread accumu
 constexpr int kSpreadGroups = 3;
 constexpr int kSpreadDense = 24;  // cells with more samples in their window go to the warp kernel
 
-// Groups per spreading thread for C coils on a G x G grid: as many as leave 131,072
-// threads (some 860 per SM; a 192^2 grid with 5 coils is slower with two groups per
-// thread, 11.5 against 9.3 us), at most kSpreadGroups, in as few passes over the
-// samples and with as few padded coils as that allows.
-int spread_groups(int C, int G) {
+// Groups per spreading thread (and per warp of a dense cell) for C coils: as many as
+// leave 131,072 threads (some 860 per SM; a 192^2 grid with 5 coils is slower with two
+// groups per thread, 11.5 against 9.3 us), at most kSpreadGroups, in as few passes over
+// the samples as that allows and with at most a quarter more padded coils than single
+// groups have (12 coils of 256^2 in two groups of eight: 91 against 81 us).  One group
+// where the fullest cell is a large part of the work: a warp takes 12 ns per sample of it
+// with three groups and 5 with one, the rest some 3e-6 us per sample, tap and coil and
+// 5e-6 us per grid cell and coil.  Adjoint at G = 512, W = 6, 12 coils, 40,000 samples
+// with 861, 3,028 and 10,913 in the fullest cell: three groups 72, 96 and 235 us, one group
+// 94, 106 and 183.  A coil's values do not depend on it.
+int spread_groups(const mpi_plan* plan, int C) {
   const int g = (C + kSpreadCoils - 1) / kSpreadCoils;
-  int ng = std::min(kSpreadGroups, g);
-  while (ng > 1 && (long)G * G * ((g + ng - 1) / ng) < 131072) --ng;
-  const int z = (g + ng - 1) / ng;
-  return (g + z - 1) / z;
+  const double cells = (double)plan->G * plan->G;
+  if (plan->dense_max > (double)plan->M * plan->W * plan->W * C / 9260 + cells * C / 5555 + 360) return 1;
+  for (int ng = std::min(kSpreadGroups, g); ng > 1; --ng) {
+    const int z = (g + ng - 1) / ng, even = (g + z - 1) / z;
+    if (cells * z >= 131072 && 4 * even * z <= 5 * g) return even;
+  }
+  return 1;
 }
-int spread_coils_padded(int C, int G) {
-  const int per = kSpreadCoils * spread_groups(C, G);
+int spread_coils_padded(const mpi_plan* plan, int C) {
+  const int per = kSpreadCoils * spread_groups(plan, C);
   return (C + per - 1) / per * per;
 }
 
@@ -307,7 +316,10 @@ __device__ __forceinline__ void spread_sparse(const SpreadArgs& s, int gx, int g
 
 // Output-driven spreading, dense cells (the plan's list of cells whose window
 // holds more than kSpreadDense samples): warp (cell i, 4 NG coils), the lanes
-// taking every 32nd sample of each row range, then a butterfly sum.
+// taking every 32nd sample of each row range, then a butterfly sum.  With one group the
+// loads of four samples are in flight (a cell of thousands of samples is a chain of
+// them: 40,000 samples towards the centre of a 96^2 grid 126 -> 76 us); with more, a
+// sample's own loads are as many.
 template <int W, int NG>
 __device__ __forceinline__ void spread_dense(const SpreadArgs& s, int i, int c0) {
   const int C = s.C, Cp = s.Cp, G = s.G;
@@ -320,12 +332,14 @@ __device__ __forceinline__ void spread_dense(const SpreadArgs& s, int i, int c0)
   const int ystride = Cp / 2;
   const float4* yc = s.ys + c0 / 2;
   float acc[8 * NG] = {};
+  constexpr int kUnroll = NG == 1 ? 4 : 1;
 #pragma unroll
   for (int a = 0; a < W; ++a) {
     int sy = gy - a;
     if (sy < 0) sy += G;
     int r[4];
     spread_row_ranges<W>(cell_ptr + sy * G, gx, G, r);
+#pragma unroll kUnroll
     for (int k = r[0] + lane; k < r[1]; k += 32) spread_term<W, NG>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
     for (int k = r[2] + lane; k < r[3]; k += 32) spread_term<W, NG>(cell_w, cell_sx, yc, ystride, k, gx, a, G, acc);
   }
@@ -339,9 +353,9 @@ __device__ __forceinline__ void spread_dense(const SpreadArgs& s, int i, int c0)
 // Both kinds of cells in one launch, the dense ones' CTAs (a warp per cell) first: a
 // grid cell has one kind, so they need no order, and neither fills the chip by itself
 // (the dense cells of a radial trajectory's centre are few and long, most sparse ones
-// are empty).
+// are empty).  One group: four CTAs per SM (G = 96 as above 96 -> 76 us).
 template <int W, int NG>
-__global__ void __launch_bounds__(256) k_nufft_spread(SpreadArgs s, int dense_ctas) {
+__global__ void __launch_bounds__(256, NG == 1 ? 4 : 0) k_nufft_spread(SpreadArgs s, int dense_ctas) {
   mpi_ptx::pdl_trigger();
   const int c0 = blockIdx.y * kSpreadCoils * NG, warp = threadIdx.x >> 5;
   if ((int)blockIdx.x < dense_ctas) {
@@ -364,7 +378,7 @@ mpi_status launch_fft_rows_inplace(mpi_ctx* ctx, float2* data, long n_rows, int 
                                    int load_hi = -1, int keep_lo = 0, int keep_hi = -1);
 
 size_t nufft_grid_elems(const mpi_plan* plan, int C) {
-  return (size_t)C * plan->G * plan->G + (size_t)spread_coils_padded(C, plan->G) * plan->M;
+  return (size_t)C * plan->G * plan->G + (size_t)spread_coils_padded(plan, C) * plan->M;
 }
 
 mpi_status nufft_plan_init(mpi_ctx* ctx, mpi_plan* plan, const float* traj_host) {
@@ -426,6 +440,7 @@ mpi_status nufft_plan_init(mpi_ctx* ctx, mpi_plan* plan, const float* traj_host)
           }
         }
         if (cnt > kSpreadDense) dense.push_back(gy * G + gx);
+        plan->dense_max = std::max(plan->dense_max, (int)cnt);
       }
     plan->n_dense = (int)dense.size();
     e = cudaMalloc(&plan->cell_ptr, ptr.size() * sizeof(int32_t));
@@ -504,13 +519,13 @@ mpi_status nufft_adjoint(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, in
     if (e != cudaSuccess) return cuda_check(ctx, e, "grid clear");
   } else {
     const float ks = axis_sign(G) * axis_sign(G);
-    const int Cp = spread_coils_padded(C, G);
+    const int Cp = spread_coils_padded(plan, C);
     float2* ys = grid + total;  // nufft_grid_elems reserves the sorted copy after the grid
     MPI_PROF(ctx, KF_NUFFT);
     launch_pdl(ctx, k_nufft_sort_y, dim3(blocks_for((size_t)M * Cp, 256)), dim3(256), 0, y, C, Cp, M,
                plan->cell_rank, ks, ys);
     MPI_LAUNCH_CHECK(ctx, "k_nufft_sort_y");
-    const int ng = spread_groups(C, G);
+    const int ng = spread_groups(plan, C);
     const unsigned groups = (unsigned)(Cp / (kSpreadCoils * ng));
     const int dense_ctas = (plan->n_dense + 7) / 8;
     const dim3 sgrid((unsigned)(dense_ctas + (G + 31) / 32 * ((G + 7) / 8)), groups);
