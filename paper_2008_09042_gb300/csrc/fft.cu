@@ -641,8 +641,9 @@ __global__ void __launch_bounds__(kLineWarps * 32, (L * 8 <= 2048) ? 4 : (L * 8 
 // The windowed pass along y as a two-step register FFT (G = R1 R2, see
 // k_fft_cols_reg), 16 adjacent columns per CTA (two rows per warp step): one write
 // and read of shared memory per element instead of one per radix stage and two
-// transposes, and the padded rows are never loaded.  256^2, 12 coils, G = 512:
-// 17.6 -> 12.4 us.  Tiles wholly outside the window are not launched.
+// transposes, and the padded rows are never loaded.  Tiles wholly outside the window are
+// not launched.  256^2, 12 coils, G = 512: 17.6 -> 12.4 us; small grids and few coils have
+// too few of these CTAs, of too much work each (see kWinReg).
 template <int R1, int R2, bool INV>
 __global__ void __launch_bounds__(256) k_fft_cols_win(float2* __restrict__ grid, int C, LineWin win, int x_first,
                                                       int x_tiles, const float2* __restrict__ tw_g) {
@@ -1188,6 +1189,15 @@ mpi_status launch_fft_cols(mpi_ctx* ctx, float2* data, int C, int nz, int ny, in
   return lines_dispatch<false>(ctx, "k_fft_lines<y,fwd>", data, ny, nx, nx, C * nz, 1, plane, 0, row_has, nz);
 }
 
+namespace {
+// Grid points along y times coils from which the windowed pass is the register one (at
+// G >= 128): both directions in us, Stockham lines against registers, with 4, 12 and 32
+// coils: G = 96 12.6/14.9, 12.9/15.0, 14.6/14.6; 128 13.7/14.0, 13.4/15.2, 16.2/14.8; 192
+// 15.5/16.4, 16.2/16.5, 19.7/17.1; 256 16.5/16.9, 18.8/17.0, 20.7/19.1; 320 18.8/19.9,
+// 22.0/20.1, 32.6/24.5; 512 24.2/22.3, 34.9/24.6, 59.6/38.2.
+constexpr int kWinReg = 2048;
+}  // namespace
+
 mpi_status launch_fft_cols_window(mpi_ctx* ctx, float2* grid, int C, int G, const float2* src, float2* dst,
                                   const float* deap, int n, bool inverse) {
   if (C == 0) return MPI_OK;
@@ -1196,6 +1206,7 @@ mpi_status launch_fft_cols_window(mpi_ctx* ctx, float2* grid, int C, int G, cons
   const float2* tw = twiddle_table(ctx, G);
   if (!tw) return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
   const LineWin win{src, dst, deap, n, G / 2 - n / 2};
+  const bool reg = G >= 128 && C >= (kWinReg + G - 1) / G;
 #define MPI_WIN_CASE(L)                                                                                    \
   case L:                                                                                                  \
     if (inverse)                                                                                           \
@@ -1218,23 +1229,35 @@ mpi_status launch_fft_cols_window(mpi_ctx* ctx, float2* grid, int C, int G, cons
     break;                                                                                                          \
   }
   MPI_PROF(ctx, KF_FFT_LINES);
-  switch (G) {
-    MPI_WIN_CASE(16)
-    MPI_WIN_CASE(32)
-    MPI_WIN_CASE(48)
-    MPI_WIN_REG(64, 8, 8)
-    MPI_WIN_REG(96, 8, 12)
-    MPI_WIN_REG(128, 8, 16)
-    MPI_WIN_REG(192, 16, 12)
-    MPI_WIN_REG(256, 16, 16)
-    MPI_WIN_REG(320, 16, 20)
-    MPI_WIN_REG(512, 16, 32)
-    default:
-      return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+  if (reg) {
+    switch (G) {
+      MPI_WIN_REG(128, 8, 16)
+      MPI_WIN_REG(192, 16, 12)
+      MPI_WIN_REG(256, 16, 16)
+      MPI_WIN_REG(320, 16, 20)
+      MPI_WIN_REG(512, 16, 32)
+      default:
+        return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+    }
+  } else {
+    switch (G) {
+      MPI_WIN_CASE(16)
+      MPI_WIN_CASE(32)
+      MPI_WIN_CASE(48)
+      MPI_WIN_CASE(64)
+      MPI_WIN_CASE(96)
+      MPI_WIN_CASE(128)
+      MPI_WIN_CASE(192)
+      MPI_WIN_CASE(256)
+      MPI_WIN_CASE(320)
+      MPI_WIN_CASE(512)
+      default:
+        return set_err(ctx, MPI_ERR_SHAPE, "unsupported FFT length");
+    }
   }
 #undef MPI_WIN_CASE
 #undef MPI_WIN_REG
-  MPI_LAUNCH_CHECK(ctx, G < 64 ? "k_fft_lines_win" : "k_fft_cols_win");
+  MPI_LAUNCH_CHECK(ctx, reg ? "k_fft_cols_win" : "k_fft_lines_win");
   return MPI_OK;
 }
 
