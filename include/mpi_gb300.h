@@ -422,8 +422,9 @@ typedef struct mpi_batch mpi_batch;
  * forward followed by the adjoint of its output) into one CUDA graph.  Slices
  * are ordered by basis so that a shared basis stays L2-resident; the context
  * workspace is sized first, so replays allocate nothing.  The slice descriptors
- * are copied; their buffers must stay valid while the batch exists.  Waits for
- * the context's stream once. */
+ * are copied; their buffers must stay valid while the batch exists.  A workspace
+ * that a later call outgrows is kept for the batches that were recorded on it.
+ * Waits for the context's stream once. */
 mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slices, int n, int kind,
                             mpi_precision prec, mpi_batch** out);
 /* Launch the recorded graph once on the context's stream (asynchronous). */

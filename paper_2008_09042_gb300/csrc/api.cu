@@ -50,7 +50,8 @@ mpi_status ensure_work(mpi_ctx* ctx, size_t bytes) {
   if (bytes <= ctx->work_bytes) return MPI_OK;
   cudaError_t e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_check(ctx, e, "workspace sync");
-  if (ctx->work) cudaFree(ctx->work);
+  if (ctx->work && std::find(ctx->work_users.begin(), ctx->work_users.end(), ctx->work) == ctx->work_users.end())
+    cudaFree(ctx->work);
   ctx->work = nullptr;
   ctx->work_bytes = 0;
   ctx->tune_scratch = nullptr;
@@ -63,6 +64,14 @@ mpi_status ensure_work(mpi_ctx* ctx, size_t bytes) {
   }
   ctx->work_bytes = want;
   return MPI_OK;
+}
+
+void work_release(mpi_ctx* ctx, void* work) {
+  std::vector<void*>& v = ctx->work_users;
+  auto it = std::find(v.begin(), v.end(), work);
+  if (it == v.end()) return;
+  v.erase(it);
+  if (work != ctx->work && std::find(v.begin(), v.end(), work) == v.end()) cudaFree(work);
 }
 
 void prof_begin(mpi_ctx* ctx, int family) {
@@ -323,6 +332,7 @@ extern "C" mpi_status mpi_ctx_destroy(mpi_ctx* ctx) {
   }
   solver_cache_clear(ctx);
   for (mpi_ctx** slot : ctx->children) *slot = nullptr;  // orphan the children still alive
+  while (!ctx->work_users.empty()) work_release(ctx, ctx->work_users.back());
   if (ctx->work) cudaFree(ctx->work);
   if (ctx->stage) cudaFree(ctx->stage);
   if (ctx->twiddles) cudaFree(ctx->twiddles);

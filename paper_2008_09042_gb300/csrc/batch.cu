@@ -36,6 +36,7 @@ struct mpi_batch {
   cudaGraphExec_t exec = nullptr;
   int n = 0;
   int64_t kernels = 0;  // kernels per replay
+  void* work = nullptr;  // the context's workspace block that the recorded kernels use
   void* buf = nullptr;   // per-coil images of one group [sum C][N]
   void* ctas = nullptr;  // CTA and slice tables of every group's expansions (device)
   void* tabs = nullptr;  // sampling tables and row masks of the grouped passes (device)
@@ -516,6 +517,10 @@ extern "C" mpi_status mpi_batch_create(mpi_ctx* ctx, const mpi_batch_slice* slic
     return st;
   }
   ctx_adopt(ctx, &bt->ctx);
+  if (ctx->work) {
+    bt->work = ctx->work;
+    ctx->work_users.push_back(bt->work);
+  }
   *out = bt;
   return MPI_OK;
 }
@@ -537,6 +542,7 @@ extern "C" int mpi_batch_group_count(const mpi_batch* bt) { return bt ? bt->grou
 extern "C" mpi_status mpi_batch_destroy(mpi_batch* bt) {
   if (!bt) return MPI_ERR_ARG;
   if (bt->ctx && (bt->buf || bt->ctas || bt->tabs)) cudaStreamSynchronize(bt->ctx->stream);  // a replay may still run
+  if (bt->ctx && bt->work) work_release(bt->ctx, bt->work);
   ctx_release(&bt->ctx);
   if (bt->exec) cudaGraphExecDestroy(bt->exec);
   if (bt->graph) cudaGraphDestroy(bt->graph);

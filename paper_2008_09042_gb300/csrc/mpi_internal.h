@@ -39,6 +39,9 @@ struct mpi_ctx {
   // its context (in any order a caller's garbage collector picks) only frees
   // the child's own memory.
   std::vector<mpi_ctx**> children;
+  // Workspace blocks that recorded batches' kernels point at, one entry per batch: a
+  // block the workspace has outgrown lives until its last batch is destroyed.
+  std::vector<void*> work_users;
   std::string err;
   // profiling: event pairs around launches while enabled
   bool profiling = false;
@@ -290,6 +293,8 @@ struct ExpandArgs {
 mpi_status launch_expand(mpi_ctx* ctx, int mode, const ExpandArgs& a);
 // Precision dispatch over the FFMA, 3xTF32 and BF16 expansion kernels.
 mpi_status expand(mpi_ctx* ctx, const mpi_basis* basis, int mode, const ExpandArgs& a, mpi_precision prec);
+// The end of one batch's use of a workspace block (see mpi_ctx::work_users).
+void work_release(mpi_ctx* ctx, void* work);
 // Child bookkeeping (see mpi_ctx::children).
 void ctx_adopt(mpi_ctx* ctx, mpi_ctx** slot);
 void ctx_release(mpi_ctx** slot);
