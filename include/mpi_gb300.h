@@ -89,8 +89,8 @@ const char* mpi_last_error(const mpi_ctx* ctx);
 /* Number of kernels this context has launched since creation (for accounting). */
 int64_t mpi_ctx_launch_count(const mpi_ctx* ctx);
 /* Bytes of device memory the context currently holds for its growable workspace
- * and host-call staging buffer (0 until an operator call or mpi_ctx_reserve
- * grows them); -1 for a null context.  Library bookkeeping, no paper passage. */
+ * and host-call staging buffer (0 until an operator call, mpi_tv_prox or
+ * mpi_ctx_reserve grows them); -1 for a null context.  Library bookkeeping, no paper passage. */
 int64_t mpi_ctx_workspace_bytes(const mpi_ctx* ctx);
 /* Bounded waits.  Every mbarrier wait of the tensor-core kernels gives up after
  * `cycles` SM clock cycles (default 2^32, about 2 s at 2 GHz; at least 1000):
@@ -497,7 +497,8 @@ mpi_status mpi_image_solve_dynamic(mpi_ctx* ctx, const mpi_plan* const* plans, i
                                    mpi_precision prec);
 
 /* TV prox alone: x = argmin (1/2)||x - v||^2 + lam TV(x) by n_iter FGP
- * iterations (the z0 update of Eq. 11).  v, x device [N] on the plan's grid. */
+ * iterations (the z0 update of Eq. 11).  v, x device [N] on the plan's grid (x may
+ * be v).  Scratch comes from the context's workspace. */
 mpi_status mpi_tv_prox(mpi_ctx* ctx, const mpi_plan* plan, const mpi_c32* v, double lam,
                        int n_iter, mpi_c32* x);
 

@@ -999,7 +999,7 @@ size_t admm_maps_layout(const mpi_ctx* ctx, const mpi_plan* const* plans, int T,
   m->zk = cplx(CM);
   float2** img[] = {&m->z0, &m->r, &m->d[0], &m->d[1], &m->Ad, &m->p_prev};
   for (float2** b : img) *b = cplx(TN);
-  m->tv = cplx(tv_scratch_elems(T > 1 ? 3 : 2, (long)TN));
+  m->tv = cplx(tv_scratch_elems(T > 1 ? 3 : 2, (long)TN, prm->n_tv));
   m->sc = (double*)take(S_NUM * sizeof(double));
   m->ball = take((size_t)T * C * kBallBlocks * sizeof(Sum));
   m->part = take(5 * (size_t)kMaxElemBlocks * sizeof(Sum));  // |r|^2 twice, <d, A d>, the dual's two

@@ -410,8 +410,8 @@ void solver_cache_clear(mpi_ctx* ctx);
 // out = argmin_x 1/2 ||x - b||^2 + lam TV(x) by n_iter FGP iterations on the
 // (nz, ny, nx) grid, nd = 2 or 3 axes (tv.cu); b = p + ufac u (u and its device
 // factor may be null), lam = 1 / *rho (device) or the host value where rho is
-// null.  scratch holds tv_scratch_elems complex values.
-size_t tv_scratch_elems(int nd, long N);
+// null.  scratch holds tv_scratch_elems complex values; neither it nor p or u is out.
+size_t tv_scratch_elems(int nd, long N, int n_iter);
 mpi_status launch_tv_prox(mpi_ctx* ctx, int nz, int ny, int nx, int nd, const float2* p, const float2* u,
                           const double* ufac, const double* rho, float lam, int n_iter, float2* scratch, float2* out);
 

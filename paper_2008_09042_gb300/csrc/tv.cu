@@ -14,9 +14,13 @@
 //    of radius one), so ten iterations are one launch.  The halo is recomputed
 //    by its neighbours: at 32 x 32 outputs and ten iterations a CTA works on
 //    about 42 x 42 pixels on average (1.7 times its own).
-//  - 3D (k_tv_step): the halo of several iterations would be most of the work,
-//    so one launch per iteration, both updates fused: each thread forms x at its
-//    pixel and at its forward neighbours from R.
+//  - 3D: the halo of several iterations would be most of the work.  Up to
+//    kFusedBytes of P and two R (k_tv_step) an iteration is one launch, both updates
+//    fused: each thread forms x at its pixel and at its forward neighbours from R.
+//    Beyond, where the third array leaves L2, x is formed first (k_tv_out) and P and R
+//    are updated in place (k_tv_dual).  An iteration takes, fused and not, 8.7 and 15 us
+//    at 16 x 32 x 32, 15 and 27 at 64^3, 40 and 54 at 96^3 (64 MB), 134 and 80 at
+//    96 x 96 x 128 (85 MB), 235 and 174 at 96 x 128 x 128.
 #include <math.h>
 
 #include <algorithm>
@@ -28,6 +32,7 @@ namespace {
 
 constexpr int kTvThreads = 512;
 constexpr int kTileIters = 10;
+constexpr size_t kFusedBytes = (size_t)64 << 20;
 
 // lam = 1 / rho and the dual step rho / L, L = 4 nd, formed by one thread (an FP64
 // division per thread costs more than the pixel's arithmetic at this GPU's FP64 rate).
@@ -256,6 +261,41 @@ __global__ void __launch_bounds__(256) k_tv_step(TvIn in, TvGrid g, size_t N, co
   }
 }
 
+// P and R of one FGP iteration from x, in place (first: P = R = 0).
+__global__ void __launch_bounds__(256) k_tv_dual(TvIn in, TvGrid g, size_t N, const float2* __restrict__ x,
+                                                 float2* __restrict__ P, float2* __restrict__ R, int first, float c) {
+  mpi_ptx::pdl_trigger();
+  mpi_ptx::pdl_wait();
+  const float stp = tv_scalars(in, 3).step;
+  const size_t stride[3] = {1, (size_t)g.n[0], (size_t)g.n[0] * g.n[1]};
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
+    const unsigned j = (unsigned)i, r = j / (unsigned)g.n[0], z = r / (unsigned)g.n[1];  // N < 2^31
+    const int pos[3] = {(int)(j - r * g.n[0]), (int)(r - z * g.n[1]), (int)z};
+    const float2 xi = x[i];
+    float2 q[3];
+    float mag2 = 0.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float2 gd = make_float2(0.f, 0.f);
+      if (pos[d] <= g.n[d] - 2) {
+        const float2 xn = x[i + stride[d]];
+        gd = make_float2(xn.x - xi.x, xn.y - xi.y);
+      }
+      const float2 rv = first ? make_float2(0.f, 0.f) : R[d * N + i];
+      q[d] = make_float2(fmaf(stp, gd.x, rv.x), fmaf(stp, gd.y, rv.y));
+      mag2 += q[d].x * q[d].x + q[d].y * q[d].y;
+    }
+    const float inv = 1.0f / fmaxf(1.0f, sqrtf(mag2));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float2 o = first ? make_float2(0.f, 0.f) : P[d * N + i];
+      const float2 nv = make_float2(q[d].x * inv, q[d].y * inv);
+      P[d * N + i] = nv;
+      R[d * N + i] = make_float2(nv.x + c * (nv.x - o.x), nv.y + c * (nv.y - o.y));
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256) k_tv_out(TvIn in, TvGrid g, size_t N, const float2* __restrict__ P,
                                                 float2* __restrict__ out) {
   mpi_ptx::pdl_trigger();
@@ -271,7 +311,14 @@ __global__ void __launch_bounds__(256) k_tv_out(TvIn in, TvGrid g, size_t N, con
 
 }  // namespace
 
-size_t tv_scratch_elems(int nd, long N) { return nd == 3 ? 9 * (size_t)N : 8 * (size_t)N; }
+namespace {
+bool tv_fused(size_t N) { return 9 * N * sizeof(float2) <= kFusedBytes; }
+}  // namespace
+
+size_t tv_scratch_elems(int nd, long N, int n_iter) {
+  if (nd == 3) return (size_t)N * (tv_fused((size_t)N) ? 9 : 6);
+  return (size_t)N * 4 * std::clamp((n_iter + kTileIters - 1) / kTileIters - 1, 0, 2);  // P and R between launches
+}
 
 mpi_status launch_tv_prox(mpi_ctx* ctx, int nz, int ny, int nx, int nd, const float2* p, const float2* u,
                           const double* ufac, const double* rho, float lam, int n_iter, float2* scratch, float2* out) {
@@ -287,10 +334,19 @@ mpi_status launch_tv_prox(mpi_ctx* ctx, int nz, int ny, int nx, int nd, const fl
   if (nd == 3) {
     const TvGrid g{{nx, ny, nz}};
     const unsigned blocks = (unsigned)std::min<size_t>((N + 255) / 256, 16 * (size_t)std::max(ctx->num_sms, 1));
-    float2 *P = scratch, *R[2] = {P + 3 * N, P + 6 * N};
+    const bool fused = tv_fused(N);
+    float2 *P = scratch, *R[2] = {P + 3 * N, fused ? P + 6 * N : nullptr};
     for (int it = 0; it < n_iter; ++it) {
       const float c = momentum();
       MPI_PROF(ctx, KF_SOLVER);
+      if (!fused) {
+        launch_pdl(ctx, k_tv_out, dim3(blocks), dim3(256), 0, in, g, N, it ? R[0] : nullptr, out);
+        MPI_LAUNCH_CHECK(ctx, "k_tv_out");
+        MPI_PROF(ctx, KF_SOLVER);
+        launch_pdl(ctx, k_tv_dual, dim3(blocks), dim3(256), 0, in, g, N, out, P, R[0], it == 0, c);
+        MPI_LAUNCH_CHECK(ctx, "k_tv_dual");
+        continue;
+      }
       launch_pdl(ctx, k_tv_step, dim3(blocks), dim3(256), 0, in, g, N, it ? R[(it - 1) & 1] : nullptr, P, R[it & 1], c);
       MPI_LAUNCH_CHECK(ctx, "k_tv_step");
     }
@@ -302,7 +358,7 @@ mpi_status launch_tv_prox(mpi_ctx* ctx, int nz, int ny, int nx, int nd, const fl
   // 2D: launches of up to kTileIters iterations.  Output tile: 16 x 16 where that
   // is fewer pixels (halo included) for the busiest SM, else 32 x 32: at ten
   // iterations 37^2 against 53^2 pixels per tile.
-  float2 *P[2] = {scratch, scratch + 2 * N}, *R[2] = {scratch + 4 * N, scratch + 6 * N};
+  float2 *P[2] = {scratch, scratch + 4 * N}, *R[2] = {P[0] + 2 * N, P[1] + 2 * N};  // as many as there are launches to come
   int done = 0, launch = 0;
   do {
     TvTile t;
