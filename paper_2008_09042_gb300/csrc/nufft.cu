@@ -81,7 +81,7 @@ __global__ void k_nufft_deap(int n, int G, int W, double beta, float* __restrict
 constexpr int kInterpTile = 32;    // first-tap tile of the shared-memory interpolation
 constexpr int kInterpChunk = 256;  // samples per interpolation work item (one per thread)
 
-// Interpolation through shared memory: CTA (item, group of kInterpCoils coils) takes
+// Interpolation through shared memory: CTA (item, group of `per` coils) takes
 // a chunk of at most kInterpChunk of the samples whose first tap lies in one 32 x 32
 // tile (the plan's tile-sorted list).  Each thread loads its sample's first tap
 // and weights (before waiting on the kernel that writes the grid) and forms the
@@ -90,8 +90,15 @@ constexpr int kInterpChunk = 256;  // samples per interpolation work item (one p
 // shared memory, the next coil's loads in flight while each thread forms its
 // sample's W x W sum there.  The set-up (divisions by the tile width, wraps,
 // scattered weights) was most of the kernel when every CTA did one coil:
-// 256^2, 12 coils, 64 spokes 26.2 -> 22.4 us.
-constexpr int kInterpCoils = 4;
+// 256^2, 12 coils, 64 spokes 26.2 -> 22.4 us.  With few items there are too few such
+// CTAs, and started early they share a few SMs: a forward takes, with 1, 2 and 4 coils per
+// CTA, 30, 33 and 43 us with 810 (item, coil) pairs (G = 96, W = 8, 30 coils), 28, 30 and
+// 33 with 1,020, 34, 33 and 36 with 2,040, 45, 40 and 36 with 2,608, 54, 45 and 42 with
+// 5,312.
+int interp_coils(const mpi_ctx* ctx, int items, int C) {
+  const long pairs = (long)items * C, sms = std::max(ctx->num_sms, 1);
+  return pairs < 7 * sms ? 1 : (pairs < 16 * sms ? 2 : 4);
+}
 
 template <int W>
 __global__ void __launch_bounds__(kInterpChunk) k_nufft_interp_tiled(const float2* __restrict__ grid, int C, int G,
@@ -99,12 +106,12 @@ __global__ void __launch_bounds__(kInterpChunk) k_nufft_interp_tiled(const float
                                                                      const float* __restrict__ gw, float ksign,
                                                                      const int32_t* __restrict__ items,
                                                                      const int32_t* __restrict__ samples,
-                                                                     float2* __restrict__ y) {
+                                                                     float2* __restrict__ y, int per) {
   mpi_ptx::pdl_trigger();
   constexpr int TT = kInterpTile + W - 1;
   constexpr int PER = (TT * TT + kInterpChunk - 1) / kInterpChunk;  // cells per thread
   __shared__ float2 tile[TT * TT];
-  const int it = blockIdx.x, c0 = blockIdx.y * kInterpCoils, c1 = min(c0 + kInterpCoils, C);
+  const int it = blockIdx.x, c0 = blockIdx.y * per, c1 = min(c0 + per, C);
   const int t = items[3 * it], s0 = items[3 * it + 1], cnt = items[3 * it + 2];
   const int tpr = (G + kInterpTile - 1) / kInterpTile;
   const int oy = (t / tpr) * kInterpTile, ox = (t % tpr) * kInterpTile;
@@ -494,13 +501,14 @@ mpi_status nufft_forward(mpi_ctx* ctx, const mpi_plan* plan, const float2* v, in
   if (st) return st;
   if (M == 0) return MPI_OK;
   const float ks = axis_sign(G) * axis_sign(G);
-  const dim3 igrid((unsigned)plan->n_tile_items, (unsigned)((C + kInterpCoils - 1) / kInterpCoils));
+  const int per = interp_coils(ctx, plan->n_tile_items, C);
+  const dim3 igrid((unsigned)plan->n_tile_items, (unsigned)((C + per - 1) / per));
   MPI_PROF(ctx, KF_NUFFT);
   switch (plan->W) {
 #define MPI_W_CASE(w)                                                                                \
   case w:                                                                                            \
     launch_pdl(ctx, k_nufft_interp_tiled<w>, igrid, dim3(kInterpChunk), 0,                                         \
-               grid, C, G, M, plan->gstart, plan->gw, ks, plan->tile_items, plan->tile_samples, y);         \
+               grid, C, G, M, plan->gstart, plan->gw, ks, plan->tile_items, plan->tile_samples, y, per);    \
     break;
     MPI_W_CASE(2) MPI_W_CASE(3) MPI_W_CASE(4) MPI_W_CASE(5) MPI_W_CASE(6) MPI_W_CASE(7) MPI_W_CASE(8)
 #undef MPI_W_CASE
