@@ -189,6 +189,10 @@ mpi_status launch_mode(mpi_ctx* ctx, const ExpandArgs& a) {
   const bool adj_like = (MODE == EX_ADJ || MODE == EX_JADJ);
   const int gy = adj_like ? 1 : (a.C + CB - 1) / CB;
   const long gx = std::min(grid, ((long)a.N + block - 1) / block);
+  // the adjoint's CTAs (a pass over all coils, one per SM or a few) take the same time each:
+  // 512 x 16, q = 50, 33 coils 70 us started early, 47 after the pass along y; 96 x 128,
+  // q = 40, 65 coils 84 and 51
+  const NoEarlyStart late(ctx, adj_like);
   MPI_PROF(ctx, KF_EXPAND);
   launch_pdl(ctx, k_expand<MODE, CB>, dim3((unsigned)gx, gy), dim3(block), smem, a, q_pad, c_pad);
   MPI_LAUNCH_CHECK(ctx, a.kname ? a.kname : "k_expand");

@@ -199,6 +199,16 @@ inline cudaError_t launch_pdl(mpi_ctx* ctx, void (*kern)(KArgs...), dim3 grid, d
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// While it lives (and `on`), launch_pdl's kernels start after the previous one, not early:
+// for grids that fit the chip at once and whose CTAs are long.  Started early, they are
+// placed while the previous kernel holds SMs and pile up on the others for good.
+struct NoEarlyStart {
+  mpi_ctx* ctx;
+  bool pdl;
+  NoEarlyStart(mpi_ctx* c, bool on) : ctx(c), pdl(c->pdl) { ctx->pdl = pdl && !on; }
+  ~NoEarlyStart() { ctx->pdl = pdl; }
+};
+
 // Lets `kern` be launched with any dynamic shared memory that the device has: set on a
 // context's first launch of it, to the same value by every context, rather than to each
 // launch's size before every launch: the attribute belongs to the kernel on the device, so a

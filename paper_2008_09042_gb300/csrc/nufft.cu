@@ -539,11 +539,9 @@ mpi_status nufft_adjoint(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, in
     const dim3 sgrid((unsigned)(dense_ctas + (G + 31) / 32 * ((G + 7) / 8)), groups);
     const SpreadArgs sa{(const float4*)ys, C, Cp, G, plan->cell_ptr, plan->cell_sx, plan->cell_w, plan->cell_dense,
                         plan->n_dense, grid};
-    // CTAs of crowded cells that fit the chip at once must not be placed while the sort
-    // still holds SMs: they would pile up on the others (G = 32, W = 8, 9 coils, 40,000
-    // samples: adjoint 122 us started early, 74 after the sort; small work gains 2-3 us by it)
-    const bool pdl = ctx->pdl;
-    ctx->pdl = pdl && !(plan->dense_max >= 1024 && (long)sgrid.x * sgrid.y <= 4L * std::max(ctx->num_sms, 1));
+    // crowded cells (G = 32, W = 8, 9 coils, 40,000 samples: adjoint 122 us started early, 74
+    // after the sort; small work gains 2-3 us by an early start)
+    const NoEarlyStart late(ctx, plan->dense_max >= 1024 && (long)sgrid.x * sgrid.y <= 4L * std::max(ctx->num_sms, 1));
     MPI_PROF(ctx, KF_NUFFT);
 #define MPI_SPREAD(w, g) \
   if (plan->W == w && ng == g) launch_pdl(ctx, k_nufft_spread<w, g>, sgrid, dim3(256), 0, sa, dense_ctas);
@@ -551,7 +549,6 @@ mpi_status nufft_adjoint(mpi_ctx* ctx, const mpi_plan* plan, const float2* y, in
     MPI_W_CASE(2) MPI_W_CASE(3) MPI_W_CASE(4) MPI_W_CASE(5) MPI_W_CASE(6) MPI_W_CASE(7) MPI_W_CASE(8)
 #undef MPI_W_CASE
 #undef MPI_SPREAD
-    ctx->pdl = pdl;
     if (plan->W < 2 || plan->W > 8) return set_err(ctx, MPI_ERR_ARG, "kernel width");
     MPI_LAUNCH_CHECK(ctx, "k_nufft_spread");
   }
