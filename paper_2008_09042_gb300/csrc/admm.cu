@@ -27,7 +27,7 @@
 //   Reductions: partial sums per CTA, added in a fixed order by the kernels that use
 // them, so results do not depend on the order the CTAs run in.
 // At 256^2, 16 coils, q = 128 an outer step (5 CG, 10 TV iterations) went from 725
-// to 224 us, in 33 launches instead of 124.
+// to 195 us, in 33 launches instead of 124.
 #include <math.h>
 
 #include <algorithm>
@@ -60,7 +60,8 @@ enum { S_RHO = 0, S_UFAC, S_NUM };
 // where squares of FP32 values leave FP32's long before the values do: maps of magnitude
 // s make <d, A d> grow as s^4.  FP64 itself runs at two operations per clock and SM here:
 // an outer step at 256^2 and 16 coils took 290 us with it, 219 with pairs of FP32 values
-// (48 bits, FP32's range) and 224 this way.
+// (48 bits, FP32's range) and 225 this way (all with passes started early, see
+// admm_maps_record).
 
 struct alignas(16) Sum {
   long long v;  // |v| < 2^58
@@ -1054,6 +1055,11 @@ mpi_status admm_maps_tables(mpi_ctx* ctx, const mpi_plan* const* plans, int T, A
 
 mpi_status admm_maps_record(mpi_ctx* ctx, const mpi_plan* const* plans, int T, const mpi_basis* basis, int C,
                             const mpi_admm_params* prm, mpi_precision prec, const AdmmMaps& m) {
+  // In the graph a kernel's start costs little, and started early the passes' CTAs, some 120
+  // to 500 that fit the chip at once, pile up on the SMs that the pass before has left: 256^2
+  // and 16 coils 225 us per outer step started early, 195 not (rows alone not 211), 4 frames
+  // of 128^2 91 and 68, 192^2 and 10 coils 195 and 146.
+  const NoEarlyStart late(ctx, true);
   const int ny = plans[0]->ny, nx = plans[0]->nx, M = plans[0]->M, TC = T * C;
   const size_t N = plans[0]->N, TN = (size_t)T * N;
   const float scale = 1.0f / sqrtf((float)N);
